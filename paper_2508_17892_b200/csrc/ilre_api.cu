@@ -31,11 +31,16 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 constexpr int kNumStages = 4;            // timed stages (see ilre_recall_stage_times)
 constexpr int kProfRing = 32;            // runs whose stage events are kept for averaging
 constexpr int kMaxSinkStaging = 65536;
+constexpr int kPairMinTiles = 32;        // accumulators per CTA pair from which the paired scores pass is used
 static constexpr int kHostPieces = 16;              // most pieces of a pipelined host upload
 static constexpr long long kHostPieceMinKeys = 65536;   // no piece shorter than this (128-key multiple)
 
+struct PassGeometry {
+  int pair, n_rb, rb_rows, n_groups, cpg, n_tiles, stages;
+};
 struct Geometry {
-  int group_size, n_rb, rb_rows, n_groups, cpg, n_tiles, stages;
+  int group_size, kv_rows;             // kv_rows: rows of one kv head in the packed query
+  PassGeometry stats, scores;
 };
 
 }  // namespace
@@ -136,6 +141,14 @@ struct DeviceGuard {
   ~DeviceGuard() { if (prev >= 0) cudaSetDevice(prev); }
 };
 
+// Splits the rows of one kv head into blocks of at most max_rows, padded to a multiple of `unit`.
+void split_rows(int rows, int max_rows, int unit, PassGeometry* g) {
+  g->n_rb = (rows + max_rows - 1) / max_rows;
+  const int per = (rows + g->n_rb - 1) / g->n_rb;
+  g->rb_rows = ((per + unit - 1) / unit) * unit;
+}
+
+// Upper bound of the packed rows of one kv head, for any query of up to q_len tokens.
 int rows_padded_bound(int group_size, int q_len) {
   const long long rg = static_cast<long long>(group_size) * q_len;
   const long long n_rb = (rg + kMaxRbRows - 1) / kMaxRbRows;
@@ -146,18 +159,37 @@ Geometry make_geometry(const ilre_recall_config_t& c, int n_sm, long long L, int
   Geometry g;
   g.group_size = c.n_q_heads / c.n_kv_heads;
   const int rg = g.group_size * q_len;
-  g.n_rb = (rg + kMaxRbRows - 1) / kMaxRbRows;
-  const int per = (rg + g.n_rb - 1) / g.n_rb;
-  g.rb_rows = ((per + 127) / 128) * 128;
-  g.n_groups = c.n_kv_heads * g.n_rb;
-  g.n_tiles = static_cast<int>((L + kTileKeys - 1) / kTileKeys);
-  g.cpg = n_sm / g.n_groups;
-  if (g.cpg < 1) g.cpg = 1;
-  if (g.cpg > g.n_tiles) g.cpg = g.n_tiles;
-  const long long fixed = static_cast<long long>(g.rb_rows) * 256 + kSmemTailBytes +
-                          static_cast<long long>(g.rb_rows) * 4;
-  g.stages = static_cast<int>((kMaxDynSmem - fixed) / kStageBytes);
-  if (g.stages > kMaxStages) g.stages = kMaxStages;
+  auto finish = [&](PassGeometry* p, int tile_keys, int workers) {
+    p->n_groups = c.n_kv_heads * p->n_rb;
+    p->n_tiles = static_cast<int>((L + tile_keys - 1) / tile_keys);
+    p->cpg = workers / p->n_groups;
+    if (p->cpg < 1) p->cpg = 1;
+    if (p->cpg > p->n_tiles) p->cpg = p->n_tiles;
+    const long long fixed = static_cast<long long>(p->rb_rows) * 256 + kSmemTailBytes +
+                            static_cast<long long>(p->rb_rows) * 4;
+    p->stages = static_cast<int>((kMaxDynSmem - fixed) / kStageBytes);
+    if (p->stages > kMaxStages) p->stages = kMaxStages;
+  };
+  g.stats.pair = 0;
+  split_rows(rg, kMaxRbRows, 128, &g.stats);
+  finish(&g.stats, kTileKeys, n_sm);
+  // Scores by CTA pairs: where padding the rows of a kv head to a multiple of 256 instead of 128 adds
+  // none (every padded row costs tensor time), and where a pair has at least kPairMinTiles
+  // accumulators to compute, which pay for the cluster launch.  Scores pass, pairs / single CTAs:
+  // L = 1M, 1024 rows per kv head 1414 / 1568 us; 512K, 512 rows 372 / 390; 128K, 256 rows
+  // 53.9 / 56.7; 300K, 700 rows 151 / 223 (two blocks of 384 rows fill a 256-column tile badly); at
+  // the line 32K, 1024 rows (57 accumulators) 55.2 / 56.4, 32K, 512 rows (28) 37.9 / 37.7, and
+  // below it 32K, 256 rows (14) 22.7 / 22.4, 8K, 1024 rows (14) 24.4 / 23.4.
+  PassGeometry pair;
+  split_rows(rg, kMaxPairRows, 256, &pair);
+  pair.pair = 1;
+  finish(&pair, kPairTileKeys, n_sm / 2);
+  pair.stages = 2;                       // the launcher sizes the ring
+  const long long accumulators = static_cast<long long>(pair.n_tiles) * (pair.rb_rows / 256);
+  const bool use_pair = pair.n_rb * pair.rb_rows <= g.stats.n_rb * g.stats.rb_rows &&
+                        accumulators >= static_cast<long long>(kPairMinTiles) * pair.cpg;
+  g.scores = use_pair ? pair : g.stats;
+  g.kv_rows = g.stats.n_rb * g.stats.rb_rows;
   return g;
 }
 
@@ -377,7 +409,7 @@ int recall_impl(ilre_recall_t* h, const void* k_cache_dev, int64_t L, const void
   if (!guard.ok) return ILRE_ERR_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
   const Geometry g = make_geometry(h->cfg, h->n_sm, L, q_len);
-  if (g.stages < 2) return ILRE_ERR_UNSUPPORTED;
+  if (g.stats.stages < 2 || g.scores.stages < 2) return ILRE_ERR_UNSUPPORTED;
 
   // combination table (Algorithm 1 loop order: max sizes outer, window sizes inner)
   ComboTable tbl;
@@ -429,12 +461,15 @@ int recall_impl(ilre_recall_t* h, const void* k_cache_dev, int64_t L, const void
   if (with_qk &&
       (!encode_2d(h->encode, &map_k, k_cache_dev, static_cast<uint64_t>(h->cfg.n_kv_heads) * 128,
                   static_cast<uint64_t>(L), static_cast<uint64_t>(h->cfg.n_kv_heads) * 256) ||
-       !encode_2d(h->encode, &map_q, h->qp, 128, static_cast<uint64_t>(g.n_groups) * g.rb_rows, 256)))
+       !encode_2d(h->encode, &map_q, h->qp, 128, static_cast<uint64_t>(h->cfg.n_kv_heads) * g.kv_rows, 256)))
     return ILRE_ERR_CUDA;
 
   QkParams qk;
-  qk.L = L; qk.n_tiles = g.n_tiles; qk.n_groups = g.n_groups; qk.n_rb = g.n_rb;
-  qk.rb_rows = g.rb_rows; qk.cpg = g.cpg; qk.stages = g.stages;
+  auto set_pass = [&](const PassGeometry& pg) {
+    qk.pair = pg.pair; qk.n_tiles = pg.n_tiles; qk.n_groups = pg.n_groups; qk.n_rb = pg.n_rb;
+    qk.rb_rows = pg.rb_rows; qk.cpg = pg.cpg; qk.stages = pg.stages;
+  };
+  qk.L = L; qk.kv_rows = g.kv_rows;
   qk.c2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(kHeadDim)));
   qk.partial = h->partial; qk.enc = h->enc; qk.status = h->status;
   qk.clk = h->profiling ? h->clk : nullptr;
@@ -444,7 +479,7 @@ int recall_impl(ilre_recall_t* h, const void* k_cache_dev, int64_t L, const void
   PrepParams pp;
   std::memset(&pp, 0, sizeof(pp));
   pp.n_kv = h->cfg.n_kv_heads; pp.n_q = h->cfg.n_q_heads; pp.group_size = g.group_size;
-  pp.q_len = q_len; pp.n_rb = g.n_rb; pp.rb_rows = g.rb_rows; pp.L = L; pp.n_sink = spec->n_sink;
+  pp.q_len = q_len; pp.kv_rows = g.kv_rows; pp.L = L; pp.n_sink = spec->n_sink;
   pp.enc = h->enc; pp.bitmap = h->bitmap; pp.hist = h->hist;
   pp.n_comb = tbl.n_comb;
   pp.hist_words = static_cast<long long>(kSelectPasses) * tbl.n_comb * kHistBins;
@@ -452,7 +487,7 @@ int recall_impl(ilre_recall_t* h, const void* k_cache_dev, int64_t L, const void
   pp.sel_state_words = 4 * kMaxCombos;
 
   MergeParams mp;
-  mp.n_groups = g.n_groups; mp.n_rb = g.n_rb; mp.rb_rows = g.rb_rows; mp.cpg = g.cpg;
+  mp.n_kv = h->cfg.n_kv_heads; mp.n_rb = g.stats.n_rb; mp.rb_rows = g.stats.rb_rows; mp.cpg = g.stats.cpg;
   mp.group_size = g.group_size; mp.q_len = q_len; mp.n_q = h->cfg.n_q_heads;
   mp.partial = h->partial; mp.row_lse = h->row_lse;
 
@@ -491,7 +526,7 @@ int recall_impl(ilre_recall_t* h, const void* k_cache_dev, int64_t L, const void
   cudaEvent_t* ev = h->ev[h->prof_runs % kProfRing];
 #define ILRE_MARK(i) do { if (prof) ILRE_CUDA(cudaEventRecord(ev[i], st)); } while (0)
 
-  if (!with_qk) pp.n_rb = 0;                             // no query to pack
+  if (!with_qk) pp.kv_rows = 0;                          // no query to pack
   mp.ext_stats = io.ext_stats; mp.n_ext = io.n_ext;
   if (io.scores_in) { sp.scores = const_cast<float*>(io.scores_in); sp.scores_given = 1; }
   ILRE_MARK(0);
@@ -502,12 +537,14 @@ int recall_impl(ilre_recall_t* h, const void* k_cache_dev, int64_t L, const void
   ILRE_MARK(1);
   if (io.stages & kStageStats) {
     TraceRange r("ilre: row statistics (Eq. 4)");
+    set_pass(g.stats);
     ILRE_CUDA(launch_row_stats(map_k, map_q, qk, st)); ++launches;
     if (io.stats_out) { ILRE_CUDA(launch_export_stats(mp, io.stats_out, st)); ++launches; }
   }
   ILRE_MARK(2);
   if (io.stages & kStageScores) {
     TraceRange r("ilre: scores (Eq. 5)");
+    set_pass(g.scores);
     ILRE_CUDA(launch_scores(map_k, map_q, qk, mp, st)); ++launches;
     if (io.shard_scores_out) {
       ILRE_CUDA(launch_decode_scores(h->enc, io.shard_scores_out, L, st)); ++launches;

@@ -33,10 +33,10 @@ struct CtaItem {
   int tile_begin, n_tiles;
 };
 
-__device__ __forceinline__ CtaItem decode_item(const QkParams& p) {
+__device__ __forceinline__ CtaItem decode_item(const QkParams& p, int item) {
   CtaItem it;
-  it.chunk = blockIdx.x / p.n_groups;
-  it.group = blockIdx.x % p.n_groups;
+  it.chunk = item / p.n_groups;
+  it.group = item % p.n_groups;
   it.g = it.group / p.n_rb;
   const long long t0 = static_cast<long long>(it.chunk) * p.n_tiles / p.cpg;
   const long long t1 = static_cast<long long>(it.chunk + 1) * p.n_tiles / p.cpg;
@@ -97,7 +97,7 @@ __device__ __forceinline__ void producer_loop(const CUtensorMap* tmapK, const CU
   for (int kb = 0; kb < 2; ++kb)
     for (int mt = 0; mt < p.rb_rows / 128; ++mt)
       tma_load_2d(q_s + kb * p.rb_rows * 128 + mt * 16384, tmapQ, kb * 64,
-                  it.group * p.rb_rows + mt * 128, qf);
+                  it.g * p.kv_rows + (it.group % p.n_rb) * p.rb_rows + mt * 128, qf);
   // ring position as (stage, phase) counters: no division by the run-time stage count
   int s = 0;
   uint32_t phase = 0;
@@ -175,7 +175,7 @@ row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
   SmemTail* tail = reinterpret_cast<SmemTail*>(smem + MT * 128 * 256 + p.stages * kStageBytes);
   volatile int* abort_flag = &tail->abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const CtaItem it = decode_item(p);
+  const CtaItem it = decode_item(p, blockIdx.x);
 
   const uint32_t tmem_base = cta_setup(tail, smem_base, p.stages, 4, 4, p.status);
   const bool run = (it.n_tiles > 0) && (*abort_flag == 0);
@@ -339,13 +339,10 @@ row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
   cta_teardown(tmem_base);
 }
 
-// Combines the partial statistics of one row (per key chunk of this launch, or per key shard)
-// into (max in log2 units, sum); -lse in log2 units for the scores pass (-inf marks a padding
-// row); `publish` also stores the user-visible natural-log lse.
-__device__ __forceinline__ float2 merged_stats(const MergeParams& p, int group, int within,
-                                               int* user_row) {
-  const int g = group / p.n_rb, rb = group % p.n_rb;
-  const int rg = rb * p.rb_rows + within;
+// Combines the partial statistics of one row (per key chunk of the statistics pass, or per key
+// shard) into (max in log2 units, sum); -lse in log2 units for the scores pass (-inf marks a
+// padding row); `publish` also stores the user-visible natural-log lse.  rg: row of kv head g.
+__device__ __forceinline__ float2 merged_stats(const MergeParams& p, int g, int rg, int* user_row) {
   *user_row = -1;
   if (rg >= p.group_size * p.q_len) return make_float2(-INFINITY, 0.f);
   const int i = rg / p.group_size, j = rg % p.group_size;
@@ -357,9 +354,10 @@ __device__ __forceinline__ float2 merged_stats(const MergeParams& p, int group, 
     part = p.ext_stats + *user_row;
     stride = static_cast<size_t>(p.q_len) * p.n_q;
     n = p.n_ext;
-  } else {                               // one entry per key chunk of this launch
+  } else {                               // one entry per key chunk of the statistics pass
+    const int group = g * p.n_rb + rg / p.rb_rows;
     part = reinterpret_cast<const float2*>(p.partial) +
-           static_cast<size_t>(group) * p.cpg * p.rb_rows + within;
+           static_cast<size_t>(group) * p.cpg * p.rb_rows + rg % p.rb_rows;
     stride = p.rb_rows;
     n = p.cpg;
   }
@@ -373,10 +371,9 @@ __device__ __forceinline__ float2 merged_stats(const MergeParams& p, int group, 
   return make_float2(mm, zz);
 }
 
-__device__ __forceinline__ float merged_neg_lse2(const MergeParams& p, int group, int within,
-                                                 bool publish) {
+__device__ __forceinline__ float merged_neg_lse2(const MergeParams& p, int g, int rg, bool publish) {
   int user_row;
-  const float2 st = merged_stats(p, group, within, &user_row);
+  const float2 st = merged_stats(p, g, rg, &user_row);
   if (user_row < 0) return -INFINITY;
   const float lse2 = st.x + log2f(st.y);
   if (publish) p.row_lse[user_row] = lse2 * 0.69314718055994530942f;
@@ -384,10 +381,11 @@ __device__ __forceinline__ float merged_neg_lse2(const MergeParams& p, int group
 }
 
 __global__ void export_stats_kernel(MergeParams p, float2* __restrict__ out) {
-  const int prow = blockIdx.x * blockDim.x + threadIdx.x;
-  if (prow >= p.n_groups * p.rb_rows) return;
+  const int rows = p.group_size * p.q_len;
+  const int row = blockIdx.x * blockDim.x + threadIdx.x;
+  if (row >= p.n_kv * rows) return;
   int user_row;
-  const float2 st = merged_stats(p, prow / p.rb_rows, prow % p.rb_rows, &user_row);
+  const float2 st = merged_stats(p, row / rows, row % rows, &user_row);
   if (user_row >= 0) out[user_row] = st;
 }
 
@@ -411,7 +409,7 @@ scores_kernel(const __grid_constant__ CUtensorMap tmapK,
   float* nl = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(tail) + kSmemTailBytes);
   volatile int* abort_flag = &tail->abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const CtaItem it = decode_item(p);
+  const CtaItem it = decode_item(p, blockIdx.x);
   const int n_nh = (p.rb_rows + 255) / 256;
 
   // Two MMA-issuing threads (warps 1 and 2), one per accumulator buffer: tcgen05.mma holds its
@@ -475,7 +473,7 @@ scores_kernel(const __grid_constant__ CUtensorMap tmapK,
     // (the set-up above does not wait for it).
     grid_dep_wait();
     for (int i = threadIdx.x - 128; i < p.rb_rows; i += kConsumerWarps * 32)
-      nl[i] = merged_neg_lse2(mp, it.group, i, it.chunk == 0);
+      nl[i] = merged_neg_lse2(mp, it.g, (it.group % p.n_rb) * p.rb_rows + i, it.chunk == 0);
     asm volatile("bar.sync 2, %0;" ::"r"(kConsumerWarps * 32) : "memory");
     const int wg = (warp - 4) >> 2;
     const int quad = warp & 3;
@@ -523,10 +521,237 @@ scores_kernel(const __grid_constant__ CUtensorMap tmapK,
 }
 
 // ---------------------------------------------------------------------------------------
+// Pass B by CTA pairs, for long query parts
+// ---------------------------------------------------------------------------------------
+// Two CTAs of a cluster share tensor-core tiles of M = 256 keys by N = 256 query rows (tcgen05
+// cta_group::2): each keeps half of the query rows resident and loads half of the keys of every
+// 256-key tile.  Per instruction an SM reads 8 KB of operands for 128 cycles of math where the
+// one-CTA form reads 12 KB, a key tile crosses from L2 to the SMs once per pair instead of once
+// per CTA, and twice the query rows stay resident, so that half as many CTAs read each key tile.
+// Bound by the tensor pipe and the board's power: L = 1M, 1024 rows per kv head 1414 us = 1.56
+// PFLOP/s (one-CTA kernel 1568 us = 1.40).
+struct PairTail {
+  uint64_t q_full;                   // q_full, k_full and acc_empty: used in the first CTA only
+  uint64_t k_full[kMaxUnits];
+  uint64_t k_empty[kMaxUnits];       // both CTAs
+  uint64_t acc_full[2];              // both CTAs
+  uint64_t acc_empty[2];
+  uint32_t tmem_base;
+  int abort_flag;
+};
+static_assert(sizeof(PairTail) <= kSmemTailBytes, "tail too large");
+
+// TMA producer of one CTA: its 128 keys of every key tile in units of 64 channels, and its half of
+// the query rows once.  Both CTAs' bytes are counted on the first CTA's barriers, whose producer
+// announces the sum.  The keys are the caller's and final since before this launch, so a ring's
+// worth of them is on its way before the wait for the kernel that packs the query.
+template <int MT>
+__device__ __forceinline__ void pair_producer_loop(const CUtensorMap* tmapK, const CUtensorMap* tmapQ,
+                                                   const QkParams& p, const CtaItem& it, bool wait_for_query,
+                                                   PairTail* tail, uint32_t rank, uint32_t q_s, uint32_t k_s) {
+  volatile int* abort_flag = &tail->abort_flag;
+  const int units = p.stages, n_units = 2 * it.n_tiles;
+  int s = 0;
+  uint32_t phase = 0;
+  auto load_unit = [&](int n) -> bool {
+    if (!mbar_wait(smem_u32(&tail->k_empty[s]), phase ^ 1u, abort_flag, p.status, kDevWaitKEmpty))
+      return false;
+    const uint32_t kf = smem_u32(&tail->k_full[s]);
+    if (rank == 0) mbar_arrive_expect_tx(kf, 2 * kUnitBytes);
+    const int row = (it.tile_begin + (n >> 1)) * kPairTileKeys + static_cast<int>(rank) * kTileKeys;
+    tma_load_2d_pair(k_s + s * kUnitBytes, tmapK, it.g * 128 + (n & 1) * 64, row, cluster_addr(kf, 0));
+    if (++s == units) { s = 0; phase ^= 1u; }
+    return true;
+  };
+  const int ahead = min(units, n_units);
+  int n = 0;
+  bool ok = true;
+  for (; n < ahead && ok; ++n) ok = load_unit(n);
+  if (wait_for_query) grid_dep_wait();
+  grid_dep_launch();                       // the next kernel's CTAs may come in as SMs fall free
+  if (!ok) return;
+  const uint32_t qf = smem_u32(&tail->q_full);
+  if (rank == 0) mbar_arrive_expect_tx(qf, 2u * MT * 128 * 256);
+  for (int kb = 0; kb < 2; ++kb)
+    for (int mt = 0; mt < MT; ++mt)
+      tma_load_2d_pair(q_s + kb * (MT * 16384) + mt * 16384, tmapQ, kb * 64,
+                       it.g * p.kv_rows + (it.group % p.n_rb) * p.rb_rows +
+                           (static_cast<int>(rank) * MT + mt) * 128, cluster_addr(qf, 0));
+  for (; n < n_units && ok; ++n) ok = load_unit(n);
+}
+
+// One of the two MMA-issuing threads of a pair (first CTA, warps 1 and 2), one per accumulator:
+// tcgen05.mma holds its issuing thread until the tensor pipe takes the instruction, so the waits
+// and commits of one thread overlap the MMAs of the other.  With several row tiles per CTA each
+// thread issues every other one and both release a key tile; with one row tile they take the key
+// tiles in turn.
+template <int MT>
+__device__ __forceinline__ void pair_issue_loop(const QkParams& p, const CtaItem& it, PairTail* tail,
+                                                uint32_t tmem_base, uint32_t q_s, uint32_t k_s,
+                                                uint32_t mine) {
+  volatile int* abort_flag = &tail->abort_flag;
+  constexpr uint32_t idesc = umma_idesc_bf16(256, 256);
+  bool ok = mbar_wait(smem_u32(&tail->q_full), 0, abort_flag, p.status, kDevWaitQFull);
+  tc_fence_after();
+  uint32_t u = 0;
+  int s = 0;
+  uint32_t kphase = 0;
+#pragma unroll 1
+  for (int i = 0; i < it.n_tiles && ok; ++i) {
+    const int s0 = s;
+    const uint32_t ph0 = kphase;
+    if (++s == p.stages) { s = 0; kphase ^= 1u; }
+    const int s1 = s;
+    const uint32_t ph1 = kphase;
+    if (++s == p.stages) { s = 0; kphase ^= 1u; }
+    if (MT == 1 && ((static_cast<uint32_t>(i) & 1u) != mine)) { ++u; continue; }
+    ok = mbar_wait(smem_u32(&tail->k_full[s0]), ph0, abort_flag, p.status, kDevWaitKFull) &&
+         mbar_wait(smem_u32(&tail->k_full[s1]), ph1, abort_flag, p.status, kDevWaitKFull);
+    if (!ok) break;
+    const uint64_t kd[2] = {umma_desc_sw128(k_s + s0 * kUnitBytes), umma_desc_sw128(k_s + s1 * kUnitBytes)};
+#pragma unroll 1
+    for (int mt = 0; mt < MT; ++mt, ++u) {
+      const uint32_t b = u & 1u, use = u >> 1;
+      if (b != mine) continue;
+      ok = mbar_wait(smem_u32(&tail->acc_empty[b]), (use & 1u) ^ 1u, abort_flag, p.status, kDevWaitAccEmpty);
+      if (!ok) break;
+      tc_fence_after();
+      const uint64_t qd = umma_desc_sw128(q_s + mt * 16384);
+#pragma unroll
+      for (int kb = 0; kb < 2; ++kb)
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks)
+          umma_bf16_pair(tmem_base + b * 256, kd[kb] + ((ks * 32) >> 4),
+                         qd + ((kb * (MT * 16384) + ks * 32) >> 4), idesc, (kb | ks) != 0);
+      umma_commit_pair(smem_u32(&tail->acc_full[b]));
+    }
+    umma_commit_pair(smem_u32(&tail->k_empty[s0]));
+    umma_commit_pair(smem_u32(&tail->k_empty[s1]));
+  }
+}
+
+// D is 256 keys (128 in each CTA) by 256 query rows (columns 0..127 from the first CTA's row tile
+// nh, 128..255 from the second's); consumer warpgroup w of a CTA takes columns [64 w, 64 w + 64) of
+// its 128 keys.  MT: row tiles of 128 in each CTA.
+template <int MT>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
+scores_pair_kernel(const __grid_constant__ CUtensorMap tmapK,
+                   const __grid_constant__ CUtensorMap tmapQ, const QkParams p, const MergeParams mp) {
+  extern __shared__ __align__(1024) uint8_t smem[];
+  const uint32_t smem_base = smem_u32(smem);
+  const uint32_t q_s = smem_base;
+  const uint32_t k_s = smem_base + MT * 128 * 256;
+  PairTail* tail = reinterpret_cast<PairTail*>(smem + MT * 128 * 256 + p.stages * kUnitBytes);
+  float* nl = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(tail) + kSmemTailBytes);
+  volatile int* abort_flag = &tail->abort_flag;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_ctarank();
+  const CtaItem it = decode_item(p, blockIdx.x >> 1);
+
+  if (threadIdx.x == 0) {
+    tail->abort_flag = 0;
+    if (smem_base & 1023u) {                       // swizzled tiles need 1024-byte alignment
+      tail->abort_flag = 1;
+      atomicCAS(p.status, 0, kDevSmemAlign);
+    }
+    mbar_init(smem_u32(&tail->q_full), 1);
+    for (int s = 0; s < p.stages; ++s) {
+      mbar_init(smem_u32(&tail->k_full[s]), 1);
+      mbar_init(smem_u32(&tail->k_empty[s]), (MT >= 2) ? 2 : 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(smem_u32(&tail->acc_full[b]), 1);
+      mbar_init(smem_u32(&tail->acc_empty[b]), 2 * kPairConsumerWarps);
+    }
+    fence_mbar_init();
+  }
+  if (warp == 1) {
+    tmem_alloc_pair(smem_u32(&tail->tmem_base), 512);
+    tmem_relinquish_pair();
+  }
+  tc_fence_before();
+  __syncwarp();
+  cluster_sync_all();                      // from here on either CTA may signal the other's barriers
+  tc_fence_after();
+  const uint32_t tmem_base = tail->tmem_base;
+  const bool run = (it.n_tiles > 0) && (*abort_flag == 0);
+
+  if (warp == 0) {
+    // The query was packed by the kernel before the statistics kernel, which had completed before
+    // the statistics kernel let this one start.  A launch without the statistics kernel waits.
+    if (lane == 0 && run)
+      pair_producer_loop<MT>(&tmapK, &tmapQ, p, it, mp.n_ext > 0, tail, rank, q_s, k_s);
+  } else if (warp == 1 || warp == 2) {
+    if (lane == 0 && run && rank == 0)
+      pair_issue_loop<MT>(p, it, tail, tmem_base, q_s, k_s, static_cast<uint32_t>(warp - 1));
+  } else if (warp >= 4) {
+    // merge the per-key-chunk statistics of the pair's rows (see the one-CTA kernel)
+    grid_dep_wait();
+    for (int i = threadIdx.x - 128; i < p.rb_rows; i += kPairConsumerWarps * 32)
+      nl[i] = merged_neg_lse2(mp, it.g, (it.group % p.n_rb) * p.rb_rows + i, it.chunk == 0 && rank == 0);
+    asm volatile("bar.sync 2, %0;" ::"r"(kPairConsumerWarps * 32) : "memory");
+    const int wg = (warp - 4) >> 2;
+    const int quad = warp & 3;
+    const float c2 = p.c2;
+    const uint32_t full_bar = smem_u32(&tail->acc_full[0]);
+    const uint32_t empty_bar = cluster_addr(smem_u32(&tail->acc_empty[0]), 0);
+    const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + wg * 64;
+    // columns 64 wg ..: rows of CTA wg / 2 of the pair
+    const float4* nl4 = reinterpret_cast<const float4*>(nl + (wg >> 1) * (MT * 128) + (wg & 1) * 64);
+    bool ok = run;
+    uint32_t u = 0;
+    for (int i = 0; i < it.n_tiles && ok; ++i) {
+      float b0 = -INFINITY, b1 = -INFINITY, b2 = -INFINITY, b3 = -INFINITY;
+#pragma unroll 1
+      for (int nh = 0; nh < MT; ++nh, ++u) {
+        const uint32_t b = u & 1u;
+        ok = mbar_wait(full_bar + 8 * b, (u >> 1) & 1u, abort_flag, p.status, kDevWaitAccFull);
+        if (!ok) break;
+        tc_fence_after();
+        float va[32], vb[32];
+        tmem_ld32(taddr + b * 256, va);
+        tmem_ld32(taddr + b * 256 + 32, vb);
+        tmem_ld_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(empty_bar + 8 * b);     // the arithmetic runs under the next MMAs
+#pragma unroll
+        for (int j = 0; j < 32; j += 4) {
+          const float4 n4 = nl4[nh * 32 + (j >> 2)];
+          b0 = fmaxf(b0, fmaf(va[j], c2, n4.x));
+          b1 = fmaxf(b1, fmaf(va[j + 1], c2, n4.y));
+          b2 = fmaxf(b2, fmaf(va[j + 2], c2, n4.z));
+          b3 = fmaxf(b3, fmaf(va[j + 3], c2, n4.w));
+        }
+#pragma unroll
+        for (int j = 0; j < 32; j += 4) {
+          const float4 n4 = nl4[nh * 32 + 8 + (j >> 2)];
+          b0 = fmaxf(b0, fmaf(vb[j], c2, n4.x));
+          b1 = fmaxf(b1, fmaf(vb[j + 1], c2, n4.y));
+          b2 = fmaxf(b2, fmaf(vb[j + 2], c2, n4.z));
+          b3 = fmaxf(b3, fmaf(vb[j + 3], c2, n4.w));
+        }
+      }
+      const long long t = static_cast<long long>(it.tile_begin + i) * kPairTileKeys +
+                          static_cast<int>(rank) * kTileKeys + quad * 32 + lane;
+      if (ok && t < p.L) atomicMax(p.enc + t, float_to_ordered(fmaxf(fmaxf(b0, b1), fmaxf(b2, b3))));
+    }
+  }
+  // Neither CTA may leave while the other can still signal its barriers or read its operands.
+  tc_fence_before();
+  __syncwarp();
+  cluster_sync_all();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc_pair(tmem_base, 512);
+  }
+}
+
+// ---------------------------------------------------------------------------------------
 // small kernels around the two passes
 // ---------------------------------------------------------------------------------------
 
-// Packs the query rows of every (kv head, row block) contiguously, zero-padded to rb_rows,
+// Packs the query rows of every kv head contiguously, zero-padded to kv_rows,
 // and clears the per-run state (encoded scores, bitmap with the sink bits set, selection
 // state).
 __global__ void prepare_kernel(const uint4* __restrict__ q, uint4* __restrict__ qp, PrepParams p) {
@@ -534,14 +759,11 @@ __global__ void prepare_kernel(const uint4* __restrict__ q, uint4* __restrict__ 
   const long long tid = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   const long long nthreads = static_cast<long long>(gridDim.x) * blockDim.x;
   // packed query: 16 x uint4 per 128-element row
-  const long long n_pack = static_cast<long long>(p.n_kv) * p.n_rb * p.rb_rows * 16;
+  const long long n_pack = static_cast<long long>(p.n_kv) * p.kv_rows * 16;
   for (long long e = tid; e < n_pack; e += nthreads) {
     const int part = static_cast<int>(e & 15);
     const long long prow = e >> 4;
-    const int within = static_cast<int>(prow % p.rb_rows);
-    const int group = static_cast<int>(prow / p.rb_rows);
-    const int g = group / p.n_rb, rb = group % p.n_rb;
-    const int rg = rb * p.rb_rows + within;               // row inside the kv head's group
+    const int g = static_cast<int>(prow / p.kv_rows), rg = static_cast<int>(prow % p.kv_rows);
     uint4 val = make_uint4(0, 0, 0, 0);
     if (rg < p.group_size * p.q_len) {
       const int i = rg / p.group_size, j = rg % p.group_size;
@@ -614,7 +836,7 @@ cudaError_t launch_row_stats(const CUtensorMap& tk, const CUtensorMap& tq, const
 }
 
 cudaError_t launch_export_stats(const MergeParams& p, float2* out, cudaStream_t st) {
-  const int n = p.n_groups * p.rb_rows;
+  const int n = p.n_kv * p.group_size * p.q_len;
   export_stats_kernel<<<(n + 127) / 128, 128, 0, st>>>(p, out);
   return cudaGetLastError();
 }
@@ -624,8 +846,30 @@ cudaError_t launch_decode_scores(const uint32_t* enc, float* out, long long L, c
   return cudaGetLastError();
 }
 
+template <int MT>
+static cudaError_t launch_scores_pair_mt(const CUtensorMap& tk, const CUtensorMap& tq, QkParams p,
+                                         const MergeParams& mp, cudaStream_t st) {
+  constexpr int kFixed = MT * 128 * 256 + kSmemTailBytes + MT * 256 * static_cast<int>(sizeof(float));
+  constexpr int kUnits = (kMaxDynSmem - kFixed) / kUnitBytes;
+  p.stages = kUnits > kMaxUnits ? kMaxUnits : kUnits;
+  const size_t smem = static_cast<size_t>(kFixed) + static_cast<size_t>(p.stages) * kUnitBytes;
+  cudaError_t e = cudaFuncSetAttribute(scores_pair_kernel<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem);
+  if (e != cudaSuccess) return e;
+  return launch_after_previous(scores_pair_kernel<MT>, 2 * p.n_groups * p.cpg, kPairThreads, smem, st, tk, tq, p, mp);
+}
+
 cudaError_t launch_scores(const CUtensorMap& tk, const CUtensorMap& tq, const QkParams& p,
                           const MergeParams& mp, cudaStream_t st) {
+  if (p.pair) {
+    switch (p.rb_rows / 256) {
+      case 1: return launch_scores_pair_mt<1>(tk, tq, p, mp, st);
+      case 2: return launch_scores_pair_mt<2>(tk, tq, p, mp, st);
+      case 3: return launch_scores_pair_mt<3>(tk, tq, p, mp, st);
+      case 4: return launch_scores_pair_mt<4>(tk, tq, p, mp, st);
+      default: return cudaErrorInvalidValue;
+    }
+  }
   const size_t smem = scores_smem_bytes(p.rb_rows, p.stages);
   cudaError_t e = cudaFuncSetAttribute(scores_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);

@@ -23,20 +23,29 @@ static constexpr int kStatsConsumerWarps = 4 * kStatsWarpgroups;
 static constexpr int kStatsThreads = 64 + 32 * kStatsConsumerWarps;
 static constexpr int kSmemTailBytes = 256;
 static constexpr int kMaxDynSmem = 232448;         // 227 KB per CTA on sm_100
+// Paired scores pass: two CTAs of a cluster share every tensor-core tile of 256 keys x 256 rows.
+static constexpr int kPairTileKeys = 256;          // keys per key tile, 128 in each CTA
+static constexpr int kUnitBytes = kTileKeys * 64 * 2;    // ring unit: 128 keys x 64 channels
+static constexpr int kMaxUnits = 12;
+static constexpr int kMaxPairRows = 1024;          // query rows resident in a pair
+static constexpr int kPairConsumerWarps = 16;
+static constexpr int kPairThreads = 640;           // warp 0 TMA, warps 1-2 MMA, warps 4..19 consumers
 
 // Row statistics: how many of every 16 logit pairs take 2^x from the FMA-pipe polynomial
 // instead of the special-function unit (0 = none).  Balances the two pipes.
 static constexpr int kRowStatsPolyPairs = 4;
 
-// Geometry of one recall, shared by both passes.
+// Geometry of one pass.
 struct QkParams {
   long long L;
-  int n_tiles;       // ceil(L / kTileKeys)
+  int pair;          // 1: scores by CTA pairs
+  int n_tiles;       // key tiles of kTileKeys keys (pair: of kPairTileKeys)
   int n_groups;      // n_kv_heads * n_rb
   int n_rb;          // row blocks per kv head
-  int rb_rows;       // rows per block, multiple of 128, <= kMaxRbRows
-  int cpg;           // key chunks (CTAs) per group
-  int stages;
+  int rb_rows;       // rows per block: multiple of 128 up to kMaxRbRows (pair: of 256 up to kMaxPairRows)
+  int kv_rows;       // rows of one kv head in the packed query (>= n_rb * rb_rows)
+  int cpg;           // key chunks (CTAs or CTA pairs) per group
+  int stages;        // ring depth in key tiles (pair: in units, set by the launcher)
   float c2;          // log2(e) / sqrt(d)
   float* partial;    // [n_groups][cpg][rb_rows][2]: (max * c2, sum-exp) per key chunk
   uint32_t* enc;     // [L]: order-preserving uint of max_r log2 p_rt
@@ -53,7 +62,7 @@ struct QkParams {
 };
 
 struct PrepParams {
-  int n_kv, n_q, group_size, q_len, n_rb, rb_rows;
+  int n_kv, n_q, group_size, q_len, kv_rows;   // kv_rows = 0: no query to pack
   long long L;
   int n_sink;
   uint32_t* enc;
@@ -67,7 +76,7 @@ struct PrepParams {
 };
 
 struct MergeParams {
-  int n_groups, n_rb, rb_rows, cpg, group_size, q_len, n_q;
+  int n_kv, n_rb, rb_rows, cpg, group_size, q_len, n_q;    // n_rb, rb_rows, cpg: the statistics pass's
   const float* partial;
   float* row_lse;    // [q_len][n_q] natural-log lse
   // Key-range sharding: when n_ext > 0 the statistics come from ext_stats

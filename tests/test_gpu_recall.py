@@ -129,6 +129,33 @@ BIG = [
 ]
 
 
+# Query and key sizes of the paired scores pass: 1 to 4 row tiles per CTA, two row blocks per kv
+# head, contexts that end in the first or the second CTA's keys of the last tile, padded rows, and
+# the sizes one step below the dispatch's line (single CTAs).  (L, q_len, n_kv, n_q)
+PAIRED = [(75777, 64, 8, 32), (75649, 33, 8, 64), (39001, 128, 8, 32), (26113, 192, 8, 32),
+          (25801, 100, 4, 28), (20479, 256, 8, 32), (16640, 511, 4, 16), (9472, 512, 4, 16)]
+
+
+@pytest.mark.parametrize("case", PAIRED, ids=lambda c: f"L{c[0]}_q{c[1]}_kv{c[2]}_h{c[3]}")
+def test_paired_scores_pass_matches_oracle(case):
+    L, q_len, n_kv, n_q = case
+    x = make_inputs(small_workload(L, q_len, seed=L, n_kv_heads=n_kv, n_q_heads=n_q, budget=300,
+                                   win_sizes=(1, 7)))
+    eng = _engine(x.workload)
+    idx, sc = _run(eng, x)
+    parity.check_recall(x.K, x.Q, x.workload, idx, sc)
+    # given statistics instead of this launch's own (key shards): the same scores but for the
+    # rounding of the merged sums
+    K, Q = x.K.cuda(), x.Q.cuda()
+    cut = (L // 2) & ~127
+    st = torch.stack([eng.shard_stats(k, Q) for k in (K[:cut], K[cut:])])
+    sc2 = eng.shard_scores(K, Q, st).cpu().numpy()
+    eng.check_status()
+    assert np.abs(sc2 - sc).max() <= 1e-5 * np.abs(sc).max()
+    assert eng.check_guards() == 0, "a kernel wrote past the end of a workspace buffer"
+    eng.close()
+
+
 @pytest.mark.parametrize("case", BIG, ids=lambda c: f"L{c[0]}_q{c[1]}_B{c[2]}_m{len(c[3])}")
 def test_selection_kernel_edge_paths(case):
     L, q_len, budget, max_sizes, win_sizes, win_op, n_sink = case
