@@ -8,8 +8,8 @@
 namespace ilre {
 
 static constexpr int kFillBlockK = 64;          // model channels per pipeline stage (128 B rows)
-static constexpr int kFillTileM = 128;          // tokens per output tile
-static constexpr int kFillThreads = 192;        // warp 0 TMA, warp 1 MMA, warps 2..5 epilogue
+static constexpr int kFillTileM = 256;          // tokens per output tile (128 in each CTA of the pair)
+static constexpr int kFillThreads = 256;        // warps 0 and 2 TMA, warp 1 MMA, warps 4..7 epilogue
 static constexpr int kRopeLoRows = 1024;        // position = hi * kRopeLoRows + lo
 
 struct FillParams {
@@ -21,16 +21,19 @@ struct FillParams {
   const float2* rope_lo;  // [kRopeLoRows][64]: (cos, sin) of lo * theta^(-2c/128)
   const float2* rope_hi;  // [..][64]: (cos, sin) of hi * kRopeLoRows * theta^(-2c/128)
   uint16_t* k_cache;      // bf16 [L][n_kv][128]
-  int stages;
   int* status;
+  // Work split (fill_plan): tiles 0 .. n_wide - 1 are whole units of kFillTileM tokens by unit_width
+  // channels, the others parts of units, tail_width channels wide.
+  int unit_width, tail_width;
+  int n_wide, n_tiles;
 };
 
-size_t fill_smem_bytes(int tile_n, int stages);
-int fill_max_stages(int tile_n);
+// Fills in the work split from n_tok and n_kv.
+void fill_plan(int n_sm, FillParams* p);
 cudaError_t launch_rope_pos_tables(float2* lo, float2* hi, int hi_rows, double theta,
                                    cudaStream_t st);
-// tile_n = 128 (one head per tile) or 256 (two heads per tile)
-cudaError_t launch_fill(const CUtensorMap& map_x, const CUtensorMap& map_w, const FillParams& p,
-                        int tile_n, int grid, cudaStream_t st);
+// The box of map_w has unit_width / 2 weight rows, that of map_w_tail tail_width / 2.
+cudaError_t launch_fill(const CUtensorMap& map_x, const CUtensorMap& map_w, const CUtensorMap& map_w_tail,
+                        const FillParams& p, int n_sm, cudaStream_t st);
 
 }  // namespace ilre

@@ -726,26 +726,20 @@ int ilre_recall_fill_keys(ilre_recall_t* h, const void* x_dev, int64_t n_tok, in
     ILRE_CUDA(wait_for_tables(st, h->pos_ready));
   }
   const int n_out = h->cfg.n_kv_heads * kHeadDim;
-  const long long m_tiles = (n_tok + kFillTileM - 1) / kFillTileM;
-  // two heads per tile when that still gives every SM a tile, one head per tile otherwise
-  const int tile_n = (n_out % 256 == 0 && m_tiles * (n_out / 256) >= h->n_sm) ? 256 : 128;
-  const long long n_tiles = m_tiles * (n_out / tile_n);
-  CUtensorMap map_x, map_w;
-  if (!encode_2d(h->encode, &map_x, x_dev, static_cast<uint64_t>(d_model),
-                 static_cast<uint64_t>(n_tok), static_cast<uint64_t>(d_model) * 2, kFillTileM))
-    return ILRE_ERR_CUDA;
-  if (!encode_2d(h->encode, &map_w, w_k_dev, static_cast<uint64_t>(d_model),
-                 static_cast<uint64_t>(n_out), static_cast<uint64_t>(d_model) * 2, tile_n))
-    return ILRE_ERR_CUDA;
   FillParams fp;
   fp.n_tok = n_tok; fp.d_model = d_model; fp.n_kv = h->cfg.n_kv_heads; fp.pos0 = pos0;
   fp.bias = static_cast<const uint16_t*>(bias_dev);
   fp.rope_lo = h->pos_lo; fp.rope_hi = h->pos_hi;
   fp.k_cache = static_cast<uint16_t*>(k_cache_dev);
-  fp.stages = fill_max_stages(tile_n);
   fp.status = h->status;
-  const int grid = static_cast<int>(n_tiles < h->n_sm ? n_tiles : h->n_sm);
-  ILRE_CUDA(launch_fill(map_x, map_w, fp, tile_n, grid, st)); ++launches;
+  fill_plan(h->n_sm, &fp);
+  CUtensorMap map_x, map_w, map_w_tail;
+  const uint64_t inner = static_cast<uint64_t>(d_model);
+  if (!encode_2d(h->encode, &map_x, x_dev, inner, static_cast<uint64_t>(n_tok), inner * 2, kFillTileM / 2) ||
+      !encode_2d(h->encode, &map_w, w_k_dev, inner, static_cast<uint64_t>(n_out), inner * 2, fp.unit_width / 2) ||
+      !encode_2d(h->encode, &map_w_tail, w_k_dev, inner, static_cast<uint64_t>(n_out), inner * 2, fp.tail_width / 2))
+    return ILRE_ERR_CUDA;
+  ILRE_CUDA(launch_fill(map_x, map_w, map_w_tail, fp, h->n_sm, st)); ++launches;
   h->last_launches = launches;
   return ILRE_OK;
 }

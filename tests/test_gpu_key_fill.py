@@ -68,6 +68,20 @@ def test_fill_matches_oracle(case):
     eng.close()
 
 
+# Work splits of the paired kernel: tile widths 32, 64, 128 and 256, whole units with and without a
+# rest that is cut along the channels, an odd number of heads (units of one head), token counts at
+# the edges of a CTA's 128 and a pair's 256 tokens, and fewer or more 64-channel blocks than a
+# loading thread tests at once.  (n_tok, d_model, n_kv, pos0, bias)
+SPLITS = [(127, 192, 3, 5, True), (129, 320, 8, 0, False), (256, 64, 7, 5, True), (257, 128, 5, 5, False),
+          (1000, 192, 8, 1000, True), (2047, 64, 8, 5, False), (4400, 64, 8, 5, True),
+          (4865, 192, 8, 5, True), (9800, 64, 7, 5, False), (5121, 448, 4, 5, False)]
+
+
+@pytest.mark.parametrize("case", SPLITS, ids=lambda c: f"n{c[0]}_d{c[1]}_kv{c[2]}")
+def test_fill_work_splits_match_oracle(case):
+    test_fill_matches_oracle(case)
+
+
 def test_chunked_fill_equals_one_call_and_feeds_the_recall():
     from paper_2508_17892_b200 import IlreRecall
     n_kv, d_model, L, chunk = 8, 256, 3000, 1024
