@@ -3,7 +3,9 @@
 // where the first n_prefix rows of K/V are the cached sink and sliding-window tokens (visible
 // to every query of the chunk) and the remaining c rows the chunk's own (visible causally).
 //
-// One CTA per (128 query tokens, pair of query heads that share a kv head).  Both contractions
+// One CTA per (128 query tokens, pair of query heads that share a kv head); an odd group leaves one
+// head per kv head over, which gets a CTA of its own (28 / 4 heads, 16384 tokens behind 516 rows:
+// 2557 us with one CTA per head, 1894 with three pairs and a single one; 1024 tokens 44.7, 37.4).  Both contractions
 // run on the tensor cores: S = Q K^T into tensor memory, and O += P V with P written to shared
 // memory as bf16 by the softmax warps (four per head, one thread per query row).  The two heads
 // are two independent streams over the same key/value tiles (one TMA ring feeds both): while
@@ -65,20 +67,23 @@ chunk_attention_kernel(const __grid_constant__ CUtensorMap map_q,
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   // Work items in launch order, heaviest first (later query tiles see more keys): the query
-  // tiles from split_from on with one CTA per head, then the others with one CTA per head pair.
+  // tiles from split_from on with one CTA per head, then the others with one CTA per pair of heads
+  // of a kv head (and one for the head that an odd group leaves over).
   int qt, h0, n_streams;
   {
-    const int n_single = p.pair ? (p.n_qt - p.split_from) * p.n_q : p.n_qt * p.n_q;
+    const int group = p.n_q / p.n_kv, per_kv = (group + 1) / 2;
+    const int n_single = (p.n_qt - p.split_from) * p.n_q;
     const int b = blockIdx.x;
     if (b < n_single) {
       qt = p.n_qt - 1 - b / p.n_q;
       h0 = b % p.n_q;
       n_streams = 1;
     } else {
-      const int n_pairs = p.n_q / 2, r = b - n_single;
-      qt = p.split_from - 1 - r / n_pairs;
-      h0 = 2 * (r % n_pairs);                            // head of stream 0; stream 1 = h0 + 1
-      n_streams = 2;
+      const int per_qt = p.n_kv * per_kv, r = b - n_single;
+      qt = p.split_from - 1 - r / per_qt;
+      const int i = r % per_qt, k = i / p.n_kv;          // the left-over heads last: they take less time
+      h0 = (i % p.n_kv) * group + 2 * k;                 // head of stream 0; stream 1 = h0 + 1
+      n_streams = (2 * k + 1 < group) ? 2 : 1;
     }
   }
   const int j0 = qt * 128;                               // first query token
@@ -397,16 +402,15 @@ cudaError_t launch_chunk_attention(const CUtensorMap& map_q, const CUtensorMap& 
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
+  const int per_qt = p.n_kv * ((p.n_q / p.n_kv + 1) / 2);        // CTAs of a query tile
   p.n_qt = (p.c + 127) / 128;
   p.split_from = p.n_qt;
-  long long n_cta = static_cast<long long>(p.n_qt) * (p.pair ? p.n_q / 2 : p.n_q);
-  if (p.pair) {
-    // A short chunk leaves SMs idle while the wave lasts as long as its heaviest CTA: give the
-    // heaviest query tiles one CTA per head for as long as everything still fits one wave.
-    while (p.split_from > 0 && n_cta + p.n_q / 2 <= n_sm) {
-      --p.split_from;
-      n_cta += p.n_q / 2;
-    }
+  long long n_cta = static_cast<long long>(p.n_qt) * per_qt;
+  // A short chunk leaves SMs idle while the wave lasts as long as its heaviest CTA: give the
+  // heaviest query tiles one CTA per head for as long as everything still fits one wave.
+  while (p.split_from > 0 && n_cta + p.n_q - per_qt <= n_sm) {
+    --p.split_from;
+    n_cta += p.n_q - per_qt;
   }
   chunk_attention_kernel<<<static_cast<unsigned>(n_cta), kAttnThreads, smem, st>>>(map_q, map_k, map_v, p);
   return cudaGetLastError();

@@ -14,9 +14,8 @@ struct AttnParams {
   int c;             // query tokens of the chunk
   int n_prefix;      // rows of K/V visible to every query (sink + sliding window)
   int n_q, n_kv;     // query heads, kv heads
-  int pair;          // 1: a CTA serves two query heads of one kv head; 0: one head
   int n_qt;          // query tiles of 128 tokens
-  int split_from;    // query tiles >= split_from get one CTA per head (pair mode only; n_qt = none)
+  int split_from;    // query tiles >= split_from get one CTA per head (n_qt = none)
   float c2;          // log2(e) / sqrt(d)
   uint16_t* out;     // bf16 [c][n_q][128]
   int* status;

@@ -54,3 +54,13 @@ def test_chunk_attention_matches_oracle(case):
     assert err.mean() < 2e-3 * vmax
     assert eng.check_guards() == 0, "a kernel wrote past the end of a workspace buffer"
     eng.close()
+
+
+# Odd groups of query heads: pairs of heads and one left over share a launch, with and without
+# query tiles that get one CTA per head.  (c, n_prefix, n_q, n_kv)
+ODD = [(300, 60, 3, 1), (1300, 5, 10, 2), (700, 516, 28, 4), (129, 0, 7, 7), (1500, 516, 20, 4)]
+
+
+@pytest.mark.parametrize("case", ODD, ids=lambda c: f"c{c[0]}_p{c[1]}_h{c[2]}_kv{c[3]}")
+def test_odd_groups_match_oracle(case):
+    test_chunk_attention_matches_oracle(case)
