@@ -79,7 +79,7 @@ struct ilre_recall {
   cudaStream_t pos_stream;
   unsigned long long* cand;
   uint32_t* cand_count;
-  unsigned long long* pending;
+  uint32_t* cand_seg;
   int* ranked;
   uint32_t* bitmap;
   int* status;
@@ -102,6 +102,7 @@ struct ilre_recall {
   int last_q_len;
   cudaStream_t last_stream;
   int cand_stride;
+  long long pooled_stride;
   int select_max_grid;                  // co-resident CTAs of the selection kernel
   long long wait_limit;                 // spin budget of the device waits, SM cycles
   int inject;                           // failure-detection self test: which wait cannot complete
@@ -211,7 +212,7 @@ void free_all(ilre_recall* h) {
   cudaFree(h->qp); cudaFree(h->partial); cudaFree(h->row_lse);
   cudaFree(h->enc); cudaFree(h->scores); cudaFree(h->pooled); cudaFree(h->maxpooled); cudaFree(h->hist);
   cudaFree(h->tile_ties); cudaFree(h->grid_barrier); cudaFree(h->rope_table); cudaFree(h->pos_lo); cudaFree(h->pos_hi);
-  cudaFree(h->cand); cudaFree(h->cand_count); cudaFree(h->pending); cudaFree(h->ranked); cudaFree(h->bitmap);
+  cudaFree(h->cand); cudaFree(h->cand_count); cudaFree(h->cand_seg); cudaFree(h->ranked); cudaFree(h->bitmap);
   cudaFree(h->status); cudaFree(h->clk); cudaFree(h->stage_k); cudaFree(h->stage_q); cudaFree(h->stage_idx);
   cudaFree(h->piece_stats);
   if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
@@ -320,7 +321,8 @@ int ilre_recall_create(const ilre_recall_config_t* cfg, ilre_recall_t** out) {
   const size_t max_items = max_groups > static_cast<size_t>(h->n_sm) ? max_groups : h->n_sm;
   const size_t maxL = static_cast<size_t>(cfg->max_L);
   const size_t ncomb = static_cast<size_t>(cfg->max_combinations);
-  h->cand_stride = (cfg->max_budget + 2 + 3) & ~3;    // rows of the ranked lists start 16-byte aligned
+  h->cand_stride = (cfg->max_budget + 2 + kCandSlack + 3) & ~3;    // rows of the ranked lists start 16-byte aligned
+  h->pooled_stride = (cfg->max_L + 3) & ~3ll;                      // and the pooled arrays, read four at a time
 
   bool ok = true;
   ok = ok && dev_alloc(h, reinterpret_cast<uint8_t**>(&h->qp), cfg->n_kv_heads * rows_pad * 256);
@@ -328,9 +330,9 @@ int ilre_recall_create(const ilre_recall_config_t* cfg, ilre_recall_t** out) {
   ok = ok && dev_alloc(h, &h->row_lse, static_cast<size_t>(cfg->max_q_len) * cfg->n_q_heads);
   ok = ok && dev_alloc(h, &h->enc, maxL);
   ok = ok && dev_alloc(h, &h->scores, maxL);
-  ok = ok && dev_alloc(h, &h->pooled, ncomb * maxL);
+  ok = ok && dev_alloc(h, &h->pooled, ncomb * static_cast<size_t>(h->pooled_stride));
   ok = ok && dev_alloc(h, &h->maxpooled, ncomb * (maxL / 2 + 1));   // one array per distinct m > 1
-  ok = ok && dev_alloc(h, &h->hist, static_cast<size_t>(kSelectPasses) * kMaxCombos * kHistBins);
+  ok = ok && dev_alloc(h, &h->hist, static_cast<size_t>(2 + kSelectPasses) * kMaxCombos * kHistBins);
   ok = ok && dev_alloc(h, &h->tile_ties, ncomb * (maxL / kSelTile + 1));
   ok = ok && dev_alloc(h, &h->grid_barrier, 1);
   ok = ok && dev_alloc(h, &h->rope_table, static_cast<size_t>(kRopeTableRows) * kRopeHalfDim);
@@ -339,7 +341,7 @@ int ilre_recall_create(const ilre_recall_config_t* cfg, ilre_recall_t** out) {
   ok = ok && dev_alloc(h, &h->pos_hi, static_cast<size_t>(h->pos_hi_rows) * 64);
   ok = ok && dev_alloc(h, &h->cand, ncomb * h->cand_stride);
   ok = ok && dev_alloc(h, &h->cand_count, 4 * static_cast<size_t>(kMaxCombos));
-  ok = ok && dev_alloc(h, &h->pending, ncomb * kPendCap);
+  ok = ok && dev_alloc(h, &h->cand_seg, ncomb * h->cand_stride);
   ok = ok && dev_alloc(h, &h->ranked, ncomb * h->cand_stride);
   ok = ok && dev_alloc(h, &h->bitmap, (maxL + 31) / 32 + 4);    // read four words at a time
   ok = ok && dev_alloc(h, &h->status, 1);
@@ -482,7 +484,7 @@ int recall_impl(ilre_recall_t* h, const void* k_cache_dev, int64_t L, const void
   pp.q_len = q_len; pp.kv_rows = g.kv_rows; pp.L = L; pp.n_sink = spec->n_sink;
   pp.enc = h->enc; pp.bitmap = h->bitmap; pp.hist = h->hist;
   pp.n_comb = tbl.n_comb;
-  pp.hist_words = static_cast<long long>(kSelectPasses) * tbl.n_comb * kHistBins;
+  pp.hist_words = 2ll * tbl.n_comb * kHistBins;
   pp.cand_count = h->cand_count; pp.grid_barrier = h->grid_barrier;
   pp.sel_state_words = 4 * kMaxCombos;
 
@@ -495,11 +497,11 @@ int recall_impl(ilre_recall_t* h, const void* k_cache_dev, int64_t L, const void
   std::memset(&sp, 0, sizeof(sp));
   sp.enc = h->enc; sp.scores = h->scores; sp.user_scores = out_scores_dev;
   sp.L = L; sp.n_sink = spec->n_sink; sp.win_op = spec->win_op;
-  sp.pooled = h->pooled; sp.pooled_stride = h->cfg.max_L; sp.hist = h->hist;
+  sp.pooled = h->pooled; sp.pooled_stride = h->pooled_stride; sp.hist = h->hist;
   sp.maxpooled = h->maxpooled; sp.maxpooled_stride = h->cfg.max_L / 2 + 1;
   sp.tile_ties = h->tile_ties;
   sp.cand = h->cand; sp.cand_stride = h->cand_stride;
-  sp.cand_count = h->cand_count; sp.pending = h->pending; sp.ranked = h->ranked; sp.bitmap = h->bitmap;
+  sp.cand_count = h->cand_count; sp.cand_seg = h->cand_seg; sp.ranked = h->ranked; sp.bitmap = h->bitmap;
   sp.out_idx = out_idx_dev; sp.budget = budget; sp.barrier = h->grid_barrier;
   sp.status = h->status;
   sp.wait_limit = h->wait_limit;

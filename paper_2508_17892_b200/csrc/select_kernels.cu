@@ -3,19 +3,19 @@
 //
 //   A  A^C[t] = exp2(max_r log2 p_rt) from the scores pass' encoded maxima (Eq. 5);
 //   B  MaxPooling(size = stride = m), once per distinct m, then the stride-1 window pooling
-//      (average or max) of every (m, n) combination, and a histogram of the top 11 bits of
-//      the 64-bit key (pooled value, then lower cell index first);
-//   C  every CTA finds, for the combinations it scans, the histogram bin that holds the
-//      K_m-th largest key;
-//   D  one scan gathers the candidates: cells above that bin, the bin's cells too when all of
-//      them are wanted; otherwise the bin's cells (at most kPendCap) are set aside and one CTA
-//      per combination picks the wanted number of highest keys among them with a radix select
-//      over the remaining 53 bits in shared memory.  Only a plateau of more than kPendCap
-//      cells in the bin (exactly equal pooled values, mostly) takes the long way: two more
-//      histogram passes over the array, then the ties in cell order (the tiles are in cell
-//      order, so a count of the holders per tile plus an ordered rank inside the tile settle
-//      which cells win);
-//   E  ranking (value descending, cell ascending) by counting, spread over the grid;
+//      (average or max) of every (m, n) combination, and a histogram of the pooled values in
+//      kHistBins logarithmic bins;
+//   C  every CTA finds, for each combination it scans, the bin that holds the K_m-th largest value
+//      and how many values lie in the bins above each bin;
+//   D  one scan gathers the candidates, the cells of that bin and of the bins above it, sorted by
+//      bin: the place of a cell is the number of values in higher bins plus a counter of its own
+//      bin.  The threshold bin brings a few cells more than K_m; only when it brings more than
+//      kCandSlack of them (a plateau of equal values, mostly) does the combination take the long
+//      way: a radix select of the K_m-th value in three histogram passes over the array, then the
+//      ties in cell order (the tiles are in cell order, so a count of the holders per tile plus an
+//      ordered rank inside the tile settle which cells win);
+//   E  ranking (value descending, cell ascending): a candidate is compared with the candidates of
+//      its own bin only, spread over the grid;
 //   F  one CTA walks the combinations in loop order: maps cells back to tokens, skips tokens
 //      already allocated, stops each combination at its quota B_c, then writes the allocated
 //      positions in ascending order.
@@ -38,15 +38,25 @@ __device__ __forceinline__ void pass_bits(int pass, int& shift, int& bits) {
   bits = bt[pass];
 }
 
+// Bin of a pooled value: kHistBins logarithmic bins, 32 per power of two, from 2^-63 to 2 (the scores are
+// probabilities); values outside fall into the first and the last one.
+static constexpr int kBinShift = 18;
+static constexpr int kFirstBin = (64 << 5) + 8192;       // float_to_ordered(2^-63) >> kBinShift
+__device__ __forceinline__ int bin_of_ordered(uint32_t o) {
+  return min(max(static_cast<int>(o >> kBinShift) - kFirstBin, 0), kHistBins - 1);
+}
+
 struct SelShared {
   uint32_t hist[kHistBins];
+  uint32_t above[kHistBins + 1];           // of one combination: [b + 1] values in the bins above bin b; [0] all
   uint32_t scan[33];
   int flag;
-  unsigned long long prefix[kMaxCombos];   // per combination: radix prefix found so far
-  uint32_t state[kMaxCombos];              // per combination: threshold settled / candidate count
-  uint32_t krem[kMaxCombos];               // per combination: keys still wanted inside the prefix
-  uint8_t mode[kMaxCombos];                // per combination, after the first pass: 0 settled,
-                                           // 1 threshold bin handed to one CTA, 2 full-scan passes
+  int threshold;                           // the bin of its K_m-th largest value
+  int plateau;                             // it brings too many cells: full-scan passes
+  unsigned long long prefix[kMaxCombos];   // full-scan passes, per combination: radix prefix found so far,
+  uint32_t state[kMaxCombos];              // whether the K_m-th value is settled,
+  uint32_t krem[kMaxCombos];               // and the keys still wanted inside the prefix
+  uint8_t mode[kMaxCombos];                // 1: the combination takes the full-scan passes
   uint32_t tot[2][32];                     // warp totals of the one-barrier block scan
 };
 
@@ -88,7 +98,8 @@ __device__ __forceinline__ bool grid_sync(const SelectParams& p, SelShared* sh, 
 }
 
 // Exclusive prefix sum over the block of kSelThreads threads; *total receives the block sum.
-__device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* sh_warp,
+// Not inlined: the kernel meets its code cold, and every phase after the first use finds this one warm.
+__device__ __noinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* sh_warp,
                                                          uint32_t* total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t incl = v;
@@ -143,7 +154,10 @@ __device__ __forceinline__ int combo_of_tile(const ComboTable& tbl, int tile, in
 
 static constexpr int kTilePer = kSelTile / kSelThreads;
 static constexpr int kMaxWalkWarps = kSelThreads / 32;
-static constexpr int kScanGroup = 4;      // tiles whose loads are issued together
+static constexpr int kWalkCells = 2;      // ranked cells per thread of the quota walk, for the longest list
+static constexpr int kMinWalkers = 128;   // fewest threads that walk
+static constexpr int kScanGroup = 4;      // tiles whose loads are issued together (long way)
+static constexpr int kGatherGroup = 4;    // the same in the gather
 
 // Pooled values of one tile, kTilePer per thread, all loads in flight together.
 __device__ __forceinline__ void fetch_tile(const ComboTable& tbl, const SelectParams& p, int tile,
@@ -193,8 +207,8 @@ __device__ __forceinline__ void maxpool_tile(const ComboTable& tbl, const Select
 }
 
 // Phase B2 for one tile: pooled cells [c0, c0 + n_out) of `combo` from its max-pooled source
-// (the scores themselves for m = 1), written to p.pooled; the first-pass radix digit of every
-// cell goes to the shared histogram.  `buf0`/`buf1` hold kSelTile + kMaxWin floats each.
+// (the scores themselves for m = 1), written to p.pooled; the bin of every cell goes to the shared
+// histogram.  `buf0`/`buf1` hold kSelTile + kMaxWin floats each.
 __device__ __forceinline__ void pool_tile(const ComboTable& tbl, const SelectParams& p, int combo,
                                           int c0, float* buf0, float* buf1, uint32_t* sh_hist) {
   const int n = tbl.n[combo], len = tbl.len[combo];
@@ -249,23 +263,95 @@ __device__ __forceinline__ void pool_tile(const ComboTable& tbl, const SelectPar
         acc = fmaxf(src[i], src[i + n - w]);
       }
       out[c0 + i] = acc;
-      digit = static_cast<uint32_t>(make_key(acc, static_cast<uint32_t>(c0 + i)) >> 53);
+      digit = static_cast<uint32_t>(bin_of_ordered(float_to_ordered(acc)));
     }
     hist_add(sh_hist, digit);
   }
   __syncthreads();
 }
 
-// Locates the bin of pass `pass` that holds the k-th largest key of `combo` among those that
-// match the prefix so far and extends the prefix.  Every CTA does this for the combinations
-// whose tiles it scans, from the same global histogram, so all of them reach the same answer.
-// The state lives in shared memory.  A combination is settled (state = 1) when every key of
-// the chosen bin is wanted: then "key >= prefix" selects exactly K_m keys.
-__device__ __forceinline__ void bin_search(const SelectParams& p, int n_comb, int combo, int pass,
+// Phase C for one combination: the bin of its K_m-th largest value, and for every bin the number of
+// values in the bins above it.  Every CTA does this for the combinations whose tiles it scans, from the
+// same global histogram, so all of them reach the same answer.
+__device__ __forceinline__ void find_threshold(const SelectParams& p, const ComboTable& tbl, int combo, SelShared* sh) {
+  const uint32_t* gh = p.hist + static_cast<long long>(combo) * kHistBins;
+  const uint32_t k = static_cast<uint32_t>(tbl.k_m[combo]);
+  static_assert(kHistBins == 2 * kSelThreads, "two bins per thread");
+  const int hi = kHistBins - 1 - 2 * threadIdx.x;           // bins in descending order
+  const uint2 h = __ldcg(reinterpret_cast<const uint2*>(gh + hi - 1));      // (lower, higher) bin
+  uint32_t grand;
+  const uint32_t excl = block_exclusive_scan(h.x + h.y, sh->scan, &grand);   // begins with a barrier
+  sh->above[hi + 1] = excl;
+  sh->above[hi] = excl + h.y;
+  if (threadIdx.x == 0) sh->above[0] = grand;
+  if (excl < k && k <= excl + h.x + h.y) {
+    const bool in_hi = k <= excl + h.y;
+    const uint32_t total = in_hi ? excl + h.y : excl + h.x + h.y;
+    sh->threshold = in_hi ? hi : hi - 1;
+    sh->plateau = total > k + static_cast<uint32_t>(kCandSlack);
+    if (total > k + static_cast<uint32_t>(kCandSlack)) {
+      p.cand_count[kMaxCombos + combo] = 1u;
+      p.cand_count[3 * kMaxCombos] = 1u;
+    } else {
+      p.cand_count[combo] = total;                          // the same from every CTA
+    }
+  }
+  __syncthreads();
+}
+
+// Phase D for the tiles [tile0, tile1) of one combination: the cells of its threshold bin and of the bins
+// above, sorted by bin.  Four consecutive cells per thread and tile; most warps find none.
+__device__ __forceinline__ void gather_combination(const SelectParams& p, const ComboTable& tbl, int combo, int tile0,
+                                                   int tile1, const SelShared* sh) {
+  const float* w = p.pooled + static_cast<long long>(combo) * p.pooled_stride;
+  unsigned long long* cand = p.cand + static_cast<long long>(combo) * p.cand_stride;
+  uint32_t* seg = p.cand_seg + static_cast<long long>(combo) * p.cand_stride;
+  uint32_t* slots = p.hist + static_cast<long long>(tbl.n_comb + combo) * kHistBins;
+  const int len = tbl.len[combo], threshold = sh->threshold;
+  const uint32_t lowest = (threshold == 0) ? 0u : static_cast<uint32_t>(threshold + kFirstBin) << kBinShift;
+  for (int tile = tile0; tile < tile1; tile += kGatherGroup) {
+    float4 v[kGatherGroup];
+    int c[kGatherGroup];
+#pragma unroll
+    for (int g = 0; g < kGatherGroup; ++g) {
+      c[g] = (tile + g < tile1) ? (tile + g - tbl.tile_begin[combo]) * kSelTile + 4 * static_cast<int>(threadIdx.x) : len;
+      if (c[g] < len) v[g] = __ldcg(reinterpret_cast<const float4*>(w + c[g]));
+    }
+#pragma unroll 1
+    for (int g = 0; g < kGatherGroup; ++g) {
+      uint32_t o[4];
+      float4 x = v[0];
+      int cell = c[0];
+#pragma unroll
+      for (int i = 1; i < kGatherGroup; ++i)
+        if (g == i) { x = v[i]; cell = c[i]; }
+      o[0] = float_to_ordered(x.x); o[1] = float_to_ordered(x.y);
+      o[2] = float_to_ordered(x.z); o[3] = float_to_ordered(x.w);
+#pragma unroll 1
+      for (int i = 0; i < 4; ++i) {
+        const uint32_t mine = (i == 0) ? o[0] : (i == 1) ? o[1] : (i == 2) ? o[2] : o[3];
+        if (cell + i < len && mine >= lowest) {
+          const int bin = bin_of_ordered(mine);
+          const uint32_t start = sh->above[bin + 1], count = sh->above[bin] - start;
+          const uint32_t at = start + atomicAdd(&slots[bin], 1u);
+          if (at < static_cast<uint32_t>(p.cand_stride)) {
+            cand[at] = (static_cast<unsigned long long>(mine) << 32) | (0xFFFFFFFFu - static_cast<uint32_t>(cell + i));
+            seg[at] = start | (count << 16);
+          }
+        }
+      }
+    }
+  }
+}
+
+// One pass of the long way: locates the digit of pass `pass` that holds the k-th largest key of `combo`
+// among those that match the prefix so far and extends the prefix.  The state lives in shared memory.
+// A combination is settled (state = 1) when every key of the chosen digit is wanted: then
+// "key >= prefix" selects exactly K_m keys.
+__device__ __forceinline__ void bin_search(const SelectParams& p, const uint32_t* gh, int combo, int pass,
                                            SelShared* sh) {
   int shift, bits;
   pass_bits(pass, shift, bits);
-  const uint32_t* gh = p.hist + (static_cast<long long>(pass) * n_comb + combo) * kHistBins;
   const unsigned long long prefix = sh->prefix[combo];
   const uint32_t k_rem = sh->krem[combo];
   constexpr int kPer = kHistBins / kSelThreads;
@@ -288,18 +374,6 @@ __device__ __forceinline__ void bin_search(const SelectParams& p, int n_comb, in
         sh->prefix[combo] = prefix | (static_cast<unsigned long long>(bin) << shift);
         sh->krem[combo] = new_k;
         sh->state[combo] = (h[j] == new_k) ? 1u : 0u;
-        if (pass == 0 && h[j] != new_k) {
-          // The threshold bin holds more cells than are wanted from it.  Few enough: they are
-          // set aside during the gather and one CTA picks the new_k highest of them; too many
-          // (a plateau across the bin): the remaining passes scan the whole array.
-          if (h[j] <= static_cast<uint32_t>(kPendCap)) {
-            sh->mode[combo] = 1;
-            p.cand_count[2 * kMaxCombos + combo] = new_k;
-          } else {
-            sh->mode[combo] = 2;
-            p.cand_count[3 * kMaxCombos] = 1u;
-          }
-        }
       }
       cum += h[j];
     }
@@ -309,261 +383,58 @@ __device__ __forceinline__ void bin_search(const SelectParams& p, int n_comb, in
   __syncthreads();
 }
 
-// Phase E: ranks the candidates [lo, hi) of `combo` among all of its n candidates by counting
-// the keys above each (keys are distinct).
-//
-// Lists of kRankBucketMin..kRankChunk keys are first split into kRankBuckets value ranges, so
-// that a candidate is compared with its own range only: kRankSamples keys taken at even
-// strides are ranked among themselves, every fourth of them becomes a splitter, every key of
-// the list goes to the bucket "number of splitters above it" (bucket 0 holds the largest
-// keys) and is stored bucket by bucket in shared memory.  rank = keys in the buckets before
-// + keys above inside the bucket.  The result does not depend on which keys were sampled,
-// only the work per candidate does; every CTA samples for itself.
-//
-// Other lists take the plain form: the keys are staged in shared memory (at most kRankChunk
-// at a time), a thread owns one candidate and one slice of the keys, the threads of a warp
-// share the slice, so every key is one broadcast read for 32 comparisons; the slices' counts
-// meet in shared-memory counters.
+// Phase E: ranks the candidates [lo, hi) of `combo`, which are sorted by bin: the rank of a candidate is
+// where its bin's segment begins plus the keys of the segment above its own (keys are distinct).  The
+// segments that the range touches are staged in shared memory, kRankChunk keys at a time; several
+// threads share a candidate when there are threads to spare.  Ranks past K_m are not wanted.
 static constexpr int kRankChunk = 8192;
-static constexpr int kRankSamples = 128;
-static constexpr int kRankBuckets = 32;
-static constexpr int kRankBucketMin = 1024;
 
-struct RankScratch {
-  unsigned long long samp[kRankSamples];
-  unsigned long long spl[kRankBuckets];    // splitters, descending; the last entry is unused
-  uint32_t srank[kRankSamples];
-  uint32_t count[kRankBuckets];
-  uint32_t start[kRankBuckets + 1];
-};
-
-// Number of splitters above `key`.
-__device__ __forceinline__ int rank_bucket(const unsigned long long* spl, unsigned long long key) {
-  int b = 0;
-#pragma unroll
-  for (int step = kRankBuckets / 2; step >= 1; step >>= 1)
-    if (spl[b + step - 1] > key) b += step;
-  return b;
-}
-
-__device__ __forceinline__ void rank_range_bucketed(const unsigned long long* cand, int* ranked, int n,
-                                                    int lo, int hi, unsigned long long* grouped,
-                                                    RankScratch* rs) {
-  constexpr int kLd = kRankChunk / kSelThreads;
-  const int tid = threadIdx.x;
-  unsigned long long v[kLd];
-#pragma unroll
-  for (int k = 0; k < kLd; ++k) {
-    const int i = k * kSelThreads + tid;
-    v[k] = (i < n) ? __ldcg(&cand[i]) : 0ull;
-  }
-  __syncthreads();                                          // previous users of rs / grouped
-  if (tid < kRankSamples) {
-    rs->samp[tid] = __ldcg(&cand[static_cast<int>((static_cast<long long>(tid) * n) / kRankSamples)]);
-    rs->srank[tid] = 0;
-  }
-  if (tid < kRankBuckets) rs->count[tid] = 0;
-  __syncthreads();
-  {                                                         // rank the samples among themselves
-    constexpr int kPer = kRankSamples / (kSelThreads / kRankSamples);
-    const int si = tid % kRankSamples, j0 = (tid / kRankSamples) * kPer;
-    const unsigned long long mine = rs->samp[si];
-    uint32_t above = 0;
-#pragma unroll
-    for (int j = 0; j < kPer; ++j) above += (rs->samp[j0 + j] > mine) ? 1u : 0u;
-    if (above) atomicAdd(&rs->srank[si], above);
-  }
-  __syncthreads();
-  if (tid < kRankSamples) {
-    const uint32_t r = rs->srank[tid];
-    if ((r & 3u) == 3u) rs->spl[r >> 2] = rs->samp[tid];
-  }
-  __syncthreads();
-  uint32_t where[kLd];                                      // bucket << 16 | slot inside the bucket
-#pragma unroll
-  for (int k = 0; k < kLd; ++k) {
-    const int i = k * kSelThreads + tid;
-    if (i < n) {
-      const int b = rank_bucket(rs->spl, v[k]);
-      where[k] = (static_cast<uint32_t>(b) << 16) | atomicAdd(&rs->count[b], 1u);
-    }
-  }
-  __syncthreads();
-  if (tid < 32) {
-    const uint32_t c = rs->count[tid];
-    uint32_t incl = c;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-      if (tid >= d) incl += o;
-    }
-    rs->start[tid] = incl - c;
-    if (tid == 31) rs->start[32] = incl;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < kLd; ++k) {
-    const int i = k * kSelThreads + tid;
-    if (i < n) grouped[rs->start[where[k] >> 16] + (where[k] & 0xFFFFu)] = v[k];
-  }
-  __syncthreads();
+__device__ __forceinline__ void rank_range(const SelectParams& p, const ComboTable& tbl, int combo, int n, int lo, int hi,
+                                           unsigned long long* chunk) {
+  const unsigned long long* cand = p.cand + static_cast<long long>(combo) * p.cand_stride;
+  const uint32_t* seg = p.cand_seg + static_cast<long long>(combo) * p.cand_stride;
+  int* ranked = p.ranked + static_cast<long long>(combo) * p.cand_stride;
+  const bool unsorted = __ldcg(&p.cand_count[kMaxCombos + combo]) != 0u;     // came the long way: one segment
+  const int k_m = tbl.k_m[combo];
   for (int c0 = lo; c0 < hi; c0 += kSelThreads) {
     const int nc = min(kSelThreads, hi - c0);
     int g = 1;                                              // threads per candidate
     while (g < 32 && 2 * g * nc <= kSelThreads) g <<= 1;
-    const int local = tid / g, sub = tid % g;
+    const int local = threadIdx.x / g, sub = threadIdx.x % g;
     const bool active = local < nc;
+    const uint32_t whole = static_cast<uint32_t>(n) << 16;  // start | length << 16
+    const uint32_t s_first = unsorted ? whole : __ldcg(&seg[c0]);
+    const uint32_t s_last = unsorted ? whole : __ldcg(&seg[c0 + nc - 1]);
+    const uint32_t s_mine = (active && !unsorted) ? __ldcg(&seg[c0 + local]) : whole;
     const unsigned long long key = active ? __ldcg(&cand[c0 + local]) : ~0ull;
-    int j = 0, j1 = 0, first = 0;
-    if (active) {
-      const int b = rank_bucket(rs->spl, key);
-      first = static_cast<int>(rs->start[b]);
-      j = first + sub;
-      j1 = static_cast<int>(rs->start[b + 1]);
-    }
+    const int begin = static_cast<int>(s_first & 0xFFFFu);
+    const int end = static_cast<int>((s_last & 0xFFFFu) + (s_last >> 16));
+    const int first = static_cast<int>(s_mine & 0xFFFFu), last = first + static_cast<int>(s_mine >> 16);
     int above = 0;
-    for (; j < j1; j += g) above += (grouped[j] > key) ? 1 : 0;
+    for (int base = begin; base < end; base += kRankChunk) {
+      const int cnt = min(kRankChunk, end - base);
+      __syncthreads();                                      // previous users of the chunk
+      for (int i = threadIdx.x; i < cnt; i += kSelThreads) chunk[i] = __ldcg(&cand[base + i]);
+      __syncthreads();
+      if (active) {
+        const int j1 = min(last, base + cnt) - base;
+#pragma unroll 4
+        for (int j = max(first, base) - base + sub; j < j1; j += g) above += (chunk[j] > key) ? 1 : 0;
+      }
+    }
     for (int d = 1; d < g; d <<= 1) above += __shfl_xor_sync(0xFFFFFFFFu, above, d);
-    if (active && sub == 0)
+    if (active && sub == 0 && first + above < k_m)
       ranked[first + above] = static_cast<int>(0xFFFFFFFFu - static_cast<uint32_t>(key & 0xFFFFFFFFull));
   }
 }
 
-__device__ __forceinline__ void rank_range(const SelectParams& p, int combo, int n, int lo, int hi,
-                                           unsigned long long* chunk, int* count_s, RankScratch* rs) {
-  const unsigned long long* cand = p.cand + static_cast<long long>(combo) * p.cand_stride;
-  int* ranked = p.ranked + static_cast<long long>(combo) * p.cand_stride;
-  if (n >= kRankBucketMin && n <= kRankChunk) {
-    rank_range_bucketed(cand, ranked, n, lo, hi, chunk, rs);
-    return;
-  }
-  for (int c0 = lo; c0 < hi; c0 += kSelThreads) {
-    const int nc = min(kSelThreads, hi - c0);               // candidates of this round
-    const int cpad = (nc + 31) & ~31;
-    const int n_slices = kSelThreads / cpad;                // >= 1; whole warps per slice
-    const int local = threadIdx.x % cpad, slice = threadIdx.x / cpad;
-    const bool active = slice < n_slices && local < nc;
-    const unsigned long long key = active ? __ldcg(&cand[c0 + local]) : ~0ull;
-    __syncthreads();                                        // previous users of count_s / chunk
-    if (threadIdx.x < cpad) count_s[threadIdx.x] = 0;
-    int above = 0;
-    for (int base = 0; base < n; base += kRankChunk) {
-      const int cnt = min(kRankChunk, n - base);
-      if (base > 0) __syncthreads();
-      constexpr int kLd = kRankChunk / kSelThreads;         // all loads in flight together
-      unsigned long long v[kLd];
-#pragma unroll
-      for (int k = 0; k < kLd; ++k) {
-        const int i = k * kSelThreads + threadIdx.x;
-        v[k] = (i < cnt) ? __ldcg(&cand[base + i]) : 0ull;
-      }
-#pragma unroll
-      for (int k = 0; k < kLd; ++k) {
-        const int i = k * kSelThreads + threadIdx.x;
-        if (i < cnt) chunk[i] = v[k];
-      }
-      __syncthreads();
-      const int per = (cnt + n_slices - 1) / n_slices;
-      const int j0 = min(cnt, slice * per), j1 = min(cnt, j0 + per);
-      if (slice < n_slices) {                               // warp-uniform
-        int j = j0;
-        for (; j + 4 <= j1; j += 4) {
-          above += (chunk[j] > key) ? 1 : 0;
-          above += (chunk[j + 1] > key) ? 1 : 0;
-          above += (chunk[j + 2] > key) ? 1 : 0;
-          above += (chunk[j + 3] > key) ? 1 : 0;
-        }
-        for (; j < j1; ++j) above += (chunk[j] > key) ? 1 : 0;
-      }
-    }
-    if (active && above) atomicAdd(&count_s[local], above);
-    __syncthreads();
-    if (threadIdx.x < nc)                                   // slice 0 holds candidate c0 + threadIdx.x
-      ranked[count_s[threadIdx.x]] = static_cast<int>(0xFFFFFFFFu - static_cast<uint32_t>(key & 0xFFFFFFFFull));
-  }
+// Shared memory of the allocation phase: the bitmap and its summary lie behind the work area of the
+// other phases, which the staged cells and the output list reuse.
+__device__ __forceinline__ uint32_t* smem_bitmap(uint8_t* dyn_smem) {
+  return reinterpret_cast<uint32_t*>(dyn_smem + kSelWorkBytes);
 }
-
-// One CTA picks the `wanted` highest of the n_p keys that the gather set aside for `combo`
-// (all of them share the top 11 bits) and appends them to the combination's candidates.
-// Radix select over the remaining 53 bits, 11/10/11/11/10 per pass, histograms in shared memory.
-__device__ __forceinline__ void resolve_pending(const SelectParams& p, const ComboTable& tbl,
-                                                int combo, int n_p, SelShared* sh) {
-  constexpr int kPer = kPendCap / kSelThreads;
-  const unsigned long long* pend = p.pending + static_cast<long long>(combo) * kPendCap;
-  unsigned long long* cand = p.cand + static_cast<long long>(combo) * p.cand_stride;
-  const uint32_t wanted = __ldcg(&p.cand_count[2 * kMaxCombos + combo]);
-  const uint32_t base = __ldcg(&p.cand_count[combo]);
-  __shared__ unsigned long long s_prefix;
-  __shared__ uint32_t s_krem, s_slot;
-  __shared__ int s_done;
-  unsigned long long key[kPer];
-#pragma unroll
-  for (int j = 0; j < kPer; ++j) {
-    const int i = j * kSelThreads + threadIdx.x;
-    key[j] = (i < n_p) ? __ldcg(&pend[i]) : 0ull;
-  }
-  __syncthreads();                                         // earlier users of the shared words are done
-  if (threadIdx.x == 0) {
-    s_prefix = (key[0] >> 53) << 53;                       // thread 0 holds key 0 (n_p >= 1)
-    s_krem = wanted;
-    s_done = (wanted >= static_cast<uint32_t>(n_p)) || wanted == 0u;
-    s_slot = 0u;
-  }
-  for (int b = threadIdx.x; b < kHistBins; b += kSelThreads) sh->hist[b] = 0u;
-  __syncthreads();
-  const int shifts[5] = {42, 32, 21, 10, 0};
-  const int widths[5] = {11, 10, 11, 11, 10};
-  for (int pass = 0; pass < 5; ++pass) {
-    if (s_done) break;                                     // uniform: read after a barrier
-    const int shift = shifts[pass], bits = widths[pass];
-    const unsigned long long prefix = s_prefix;
-    const uint32_t k_rem = s_krem;
-#pragma unroll
-    for (int j = 0; j < kPer; ++j) {
-      if (j * kSelThreads >= n_p) break;                   // uniform
-      const int i = j * kSelThreads + threadIdx.x;
-      uint32_t digit = 0xFFFFFFFFu;
-      if (i < n_p && ((key[j] ^ prefix) >> (shift + bits)) == 0ull)
-        digit = static_cast<uint32_t>(key[j] >> shift) & ((1u << bits) - 1u);
-      hist_add(sh->hist, digit);
-    }
-    __syncthreads();
-    const uint32_t h0 = sh->hist[kHistBins - 1 - 2 * threadIdx.x];   // bins in descending order
-    const uint32_t h1 = sh->hist[kHistBins - 2 - 2 * threadIdx.x];
-    uint32_t total;
-    const uint32_t excl = block_exclusive_scan(h0 + h1, sh->scan, &total);
-    sh->hist[kHistBins - 1 - 2 * threadIdx.x] = 0u;
-    sh->hist[kHistBins - 2 - 2 * threadIdx.x] = 0u;
-    if (k_rem > excl && k_rem <= excl + h0 + h1) {
-      const bool first = k_rem <= excl + h0;
-      const uint32_t bin = first ? kHistBins - 1 - 2 * threadIdx.x : kHistBins - 2 - 2 * threadIdx.x;
-      const uint32_t above = first ? excl : excl + h0;
-      const uint32_t cnt = first ? h0 : h1;
-      s_prefix = prefix | (static_cast<unsigned long long>(bin) << shift);
-      s_krem = k_rem - above;
-      s_done = (cnt == k_rem - above) || pass == 4;
-    }
-    __syncthreads();
-  }
-  // every key at or above the threshold is wanted: exactly `wanted` of them (keys are distinct)
-  const unsigned long long threshold = (wanted >= static_cast<uint32_t>(n_p)) ? 0ull : s_prefix;
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int j = 0; j < kPer; ++j) {
-    if (j * kSelThreads >= n_p) break;                     // uniform
-    const int i = j * kSelThreads + threadIdx.x;
-    const bool take = wanted != 0u && i < n_p && key[j] >= threshold;
-    const uint32_t votes = __ballot_sync(0xFFFFFFFFu, take);
-    if (votes) {
-      uint32_t slot = 0;
-      if (lane == __ffs(votes) - 1) slot = atomicAdd(&s_slot, __popc(votes));
-      slot = base + __shfl_sync(0xFFFFFFFFu, slot, __ffs(votes) - 1) + __popc(votes & ((1u << lane) - 1u));
-      if (take && slot < static_cast<uint32_t>(tbl.k_m[combo])) cand[slot] = key[j];
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) p.cand_count[combo] = base + s_slot;
-  __syncthreads();
+__device__ __forceinline__ uint32_t* smem_summary(uint8_t* dyn_smem, long long L) {
+  return reinterpret_cast<uint32_t*>(dyn_smem + kSelWorkBytes) + (((L + 31) / 32 + 3) & ~3ll);
 }
 
 // Bitmap word access of the quota walk.  The bitmap lives in shared memory on the common path;
@@ -588,36 +459,103 @@ __device__ __forceinline__ void bitmap_set(uint32_t* bm, int w, uint32_t bits) {
 }
 
 // Tokens of cell `cell` (size m) that are not allocated yet, as a bit mask (bit j = token j).
-// Positions fit 32 bits (L < 2^31).
-template <bool kSmem>
-__device__ __forceinline__ unsigned long long fresh_tokens(const uint32_t* bm, int cell, int m,
-                                                           int Lp, int n_sink) {
-  if (m == 1) {
-    const int pos = n_sink + cell;
-    return ((bitmap_word<kSmem>(bm, pos >> 5) >> (pos & 31)) & 1u) ^ 1u;
-  }
+// Positions fit 32 bits (L < 2^31).  m <= 32: at most 32 consecutive bits, two bitmap words and one
+// funnel shift; kWide, m <= 64: at most three words.  A word past the bitmap's end may be read (there is
+// memory behind it) but its bits are masked.
+template <bool kWide, bool kSmem>
+__device__ __forceinline__ auto fresh_tokens(const uint32_t* bm, int cell, int m, int Lp, int n_sink) {
   const int t0 = cell * m;
   const int cnt = min(m, Lp - t0);
   const int pos0 = n_sink + t0;
   const int w0 = pos0 >> 5, sh = pos0 & 31;
-  if (m <= 32) {
-    // at most 32 consecutive bits: two bitmap words, one funnel shift (the bitmap has
-    // ceil(L / 32) words; a word past its end is not read)
-    const uint32_t lo = bitmap_word<kSmem>(bm, w0);
-    const uint32_t hi = (sh + cnt > 32) ? bitmap_word<kSmem>(bm, w0 + 1) : 0u;
-    const uint32_t taken32 = __funnelshift_r(lo, hi, sh);
-    const uint32_t mask32 = (cnt >= 32) ? 0xFFFFFFFFu : ((1u << cnt) - 1u);
-    return static_cast<unsigned long long>(~taken32 & mask32);
+  if constexpr (!kWide) {
+    const uint32_t taken = __funnelshift_r(bitmap_word<kSmem>(bm, w0), bitmap_word<kSmem>(bm, w0 + 1), sh);
+    return ~taken & (0xFFFFFFFFu >> (32 - cnt));
+  } else {
+    unsigned long long taken = bitmap_word<kSmem>(bm, w0);
+    taken |= static_cast<unsigned long long>(bitmap_word<kSmem>(bm, w0 + 1)) << 32;
+    taken >>= sh;
+    if (sh) taken |= static_cast<unsigned long long>(bitmap_word<kSmem>(bm, w0 + 2)) << (64 - sh);
+    return ~taken & (~0ull >> (64 - cnt));
   }
-  // up to 64 consecutive bits sit in at most three bitmap words
-  const int last_w = (pos0 + cnt - 1) >> 5;
-  unsigned long long taken = bitmap_word<kSmem>(bm, w0);
-  if (last_w > w0) taken |= static_cast<unsigned long long>(bitmap_word<kSmem>(bm, w0 + 1)) << 32;
-  taken >>= sh;
-  if (last_w > w0 + 1)                                    // only with sh > 0 and cnt > 64 - sh
-    taken |= static_cast<unsigned long long>(bitmap_word<kSmem>(bm, w0 + 2)) << (64 - sh);
-  const unsigned long long mask = (cnt >= 64) ? ~0ull : ((1ull << cnt) - 1ull);
-  return ~taken & mask;
+}
+
+// Marks the fresh tokens `f` of a cell that starts at position pos0, and in the summary (one bit per
+// bitmap word; null: none) the words that were touched.
+template <bool kWide, bool kSmem, class Mask>
+__device__ __forceinline__ void mark_tokens(uint32_t* bm, uint32_t* summary, int pos0, Mask f) {
+  const int w0 = pos0 >> 5, sft = pos0 & 31;
+  auto set = [&](int w, uint32_t bits) {
+    if (!bits) return;
+    bitmap_set<kSmem>(bm, w, bits);
+    if constexpr (kSmem) {
+      if (summary) bitmap_set<true>(summary, w >> 5, 1u << (w & 31));
+    }
+  };
+  if constexpr (!kWide) {
+    set(w0, f << sft);
+    set(w0 + 1, __funnelshift_l(f, 0u, sft));
+  } else {
+    const unsigned long long shifted = f << sft;
+    set(w0, static_cast<uint32_t>(shifted));
+    set(w0 + 1, static_cast<uint32_t>(shifted >> 32));
+    set(w0 + 2, sft ? static_cast<uint32_t>(f >> (64 - sft)) : 0u);
+  }
+}
+
+// One combination of the quota walk.  Thread t owns the ranks [t * per, (t + 1) * per).  Only the warp in
+// which the quota ends needs the order of its cells' tokens: the warps before it take all of theirs,
+// so the counts are added up with one reduction per warp instead of a prefix sum.  `totals`: one word
+// per walking warp, of this combination only.  The barrier separates counting from marking.  The
+// loops are not unrolled: the kernel meets every instruction cold, and the fetch of unrolled code
+// costs more than the loops do.
+template <bool kWide, bool kSmem, class Barrier>
+__device__ __forceinline__ void walk_combination(const SelectParams& p, const int* cells, int K, int m, uint32_t quota,
+                                                 uint32_t* bm, uint32_t* summary, uint32_t* totals, int n_walk,
+                                                 Barrier walk_barrier) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int Lp = static_cast<int>(p.L - p.n_sink), n_sink = p.n_sink;
+  auto count = [](auto f) -> uint32_t {
+    if constexpr (kWide) return __popcll(f); else return __popc(f);
+  };
+  const int per = (K + n_walk - 1) / n_walk;
+  const int r0 = min(K, static_cast<int>(threadIdx.x) * per), r1 = min(K, r0 + per);
+  uint32_t mine = 0;
+#pragma unroll 1
+  for (int r = r0; r < r1; ++r) mine += count(fresh_tokens<kWide, kSmem>(bm, cells[r], m, Lp, n_sink));
+  const uint32_t warp_sum = __reduce_add_sync(0xFFFFFFFFu, mine);
+  if (lane == 0) totals[warp] = warp_sum;
+  walk_barrier();
+  const uint32_t wt = (lane < n_walk / 32) ? totals[lane] : 0u;
+  const uint32_t before = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? wt : 0u);
+  if (warp == 0 && __reduce_add_sync(0xFFFFFFFFu, wt) < quota && lane == 0) atomicCAS(p.status, 0, kDevQuota);
+  if (before >= quota) return;
+  uint32_t room = 0xFFFFFFFFu;                                 // tokens that this thread may take
+  if (before + warp_sum > quota) {                             // the quota ends inside this warp
+    uint32_t incl = mine;
+#pragma unroll 1
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+      if (lane >= o) incl += t;
+    }
+    const uint32_t ord = before + incl - mine;
+    room = (ord < quota) ? quota - ord : 0u;
+  }
+  // rank order; inside a cell in ascending position
+#pragma unroll 1
+  for (int r = r0; r < r1 && room > 0; ++r) {
+    const int c = cells[r];
+    auto f = fresh_tokens<kWide, kSmem>(bm, c, m, Lp, n_sink);
+    const uint32_t n_new = count(f);
+    if (n_new == 0) continue;
+    if (n_new > room) {                                        // the quota ends inside this cell
+      auto rest = f;
+      for (uint32_t k = 0; k < room; ++k) rest &= rest - 1;    // without its lowest `room` tokens
+      f ^= rest;
+    }
+    room = (n_new > room) ? 0u : room - n_new;
+    mark_tokens<kWide, kSmem>(bm, summary, n_sink + c * m, f);
+  }
 }
 
 // Exclusive prefix sum over the block with a single barrier: every warp scans the 32 warp
@@ -646,43 +584,39 @@ __device__ __forceinline__ uint32_t block_exclusive_scan_1(uint32_t v, uint32_t 
 }
 
 // Phase F (one CTA): quota walk over the ranked cells of every combination, then the
-// ascending list of allocated positions.  The bitmap lives in shared memory when it fits,
-// else in global memory.  Every thread owns a run of consecutive ranks; the cells of one combination are disjoint, so the new-token counts of all its cells
-// can be taken before any of them is marked.
+// ascending list of allocated positions.  The bitmap lives in shared memory when it fits
+// (cleared at the start of the kernel, beside the memory of the other phases), else in global
+// memory.  Every thread owns a run of consecutive ranks; the cells of one combination are
+// disjoint, so the new-token counts of all its cells can be taken before any of them is marked.
 template <bool kBitmapInSmem>
 __device__ __forceinline__ void allocate(const ComboTable& tbl, const SelectParams& p,
                                          uint8_t* dyn_smem, SelShared* sh) {
   // Two instantiations, so that the compiler knows the bitmap's address space on the common
   // path (shared memory) instead of going through generic loads and atomics.
-  uint32_t* bm;
-  int* staged;
-  if constexpr (kBitmapInSmem) {
-    bm = reinterpret_cast<uint32_t*>(dyn_smem);
-    staged = reinterpret_cast<int*>(dyn_smem + ((((p.L + 31) / 32) * 4 + 15) & ~15ll));
-  } else {
-    bm = p.bitmap;
-    staged = reinterpret_cast<int*>(dyn_smem);
-  }
+  uint32_t* bm = kBitmapInSmem ? smem_bitmap(dyn_smem) : p.bitmap;
+  // (the output pass takes a thread per bitmap word, without the summary, up to kSelThreads words)
+  uint32_t* summary = (kBitmapInSmem && (p.L + 31) / 32 > kSelThreads) ? smem_summary(dyn_smem, p.L) : nullptr;
+  int* staged = reinterpret_cast<int*>(dyn_smem);
   __shared__ uint32_t warp_totals[2][kMaxWalkWarps];
   const int n_walk = p.walk_threads;                       // multiple of 32, <= kSelThreads
-  const int Lp = static_cast<int>(p.L - p.n_sink);
+  // (m, quota, ranked cells) per combination: an indexed read of the kernel's parameters costs
+  // hundreds of cycles in the walk's dependent chain
+  __shared__ int4 walk_table[kMaxCombos];
   for (int combo = threadIdx.x; combo < tbl.n_comb; combo += kSelThreads)
-    sh->state[combo] = __ldcg(&p.cand_count[combo]);
+    walk_table[combo] = make_int4(tbl.m[combo], tbl.quota[combo],
+                                  min(static_cast<int>(min(__ldcg(&p.cand_count[combo]), static_cast<uint32_t>(kMaxKm))),
+                                      tbl.k_m[combo]), 0);
   __syncthreads();
   // The walk is a chain of short dependent steps per combination, so what it costs is the
-  // number of warps that have to issue them: walk_threads threads walk (about two ranked
-  // cells each for the longest list, at least 256), the others wait for the output pass.  The ranked cells of a combination reach shared memory by 16-byte
-  // asynchronous copies, one combination ahead when two staging buffers fit.
+  // number of warps that have to issue them and the length of the chain: walk_threads threads walk
+  // (kWalkCells ranked cells each for the longest list), the others wait for the output pass.  The
+  // ranked cells of a combination reach shared memory by 16-byte asynchronous copies, one
+  // combination ahead when two staging buffers fit.
   if (static_cast<int>(threadIdx.x) < n_walk) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     auto walk_barrier = [&] { asm volatile("bar.sync 1, %0;" ::"r"(n_walk) : "memory"); };
-    auto candidates = [&](int combo) {
-      return min(static_cast<int>(min(sh->state[combo], static_cast<uint32_t>(kMaxKm))),
-                 tbl.k_m[combo]);
-    };
     const bool two = p.stage_double != 0;
     auto issue_copy = [&](int combo) {
-      const int K = candidates(combo);
+      const int K = walk_table[combo].z;
       const int* ranked = p.ranked + static_cast<long long>(combo) * p.cand_stride;
       int* dst = staged + ((two && (combo & 1)) ? p.stage_capacity : 0);
       for (int r = 4 * threadIdx.x; r < K; r += 4 * n_walk)
@@ -693,77 +627,22 @@ __device__ __forceinline__ void allocate(const ComboTable& tbl, const SelectPara
     if (tbl.n_comb > 0) issue_copy(0);
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     walk_barrier();
-    for (int combo = 0; combo < tbl.n_comb; ++combo) {
-      const int m = tbl.m[combo];
-      const uint32_t quota = static_cast<uint32_t>(tbl.quota[combo]);
-      const int K = candidates(combo);
+    const int n_comb = tbl.n_comb;
+    for (int combo = 0; combo < n_comb; ++combo) {
+      const int4 entry = walk_table[combo];
+      const int m = entry.x, K = entry.z;
+      const uint32_t quota = static_cast<uint32_t>(entry.y);
       const int* cells = staged + ((two && (combo & 1)) ? p.stage_capacity : 0);
       // the other buffer last served combination combo - 1, which every thread has left
-      if (two && combo + 1 < tbl.n_comb) issue_copy(combo + 1);
-      // thread t owns the ranks [t * per, (t + 1) * per)
-      const int per = (K + n_walk - 1) / n_walk;
-      const int r0 = min(K, static_cast<int>(threadIdx.x) * per), r1 = min(K, r0 + per);
-      uint32_t mine = 0;
-      int r = r0;
-      for (; r + 4 <= r1; r += 4) {                            // four cells' loads in flight together
-        const int c0 = cells[r], c1 = cells[r + 1], c2 = cells[r + 2], c3 = cells[r + 3];
-        const unsigned long long f0 = fresh_tokens<kBitmapInSmem>(bm, c0, m, Lp, p.n_sink);
-        const unsigned long long f1 = fresh_tokens<kBitmapInSmem>(bm, c1, m, Lp, p.n_sink);
-        const unsigned long long f2 = fresh_tokens<kBitmapInSmem>(bm, c2, m, Lp, p.n_sink);
-        const unsigned long long f3 = fresh_tokens<kBitmapInSmem>(bm, c3, m, Lp, p.n_sink);
-        mine += __popcll(f0) + __popcll(f1) + __popcll(f2) + __popcll(f3);
-      }
-      for (; r < r1; ++r)
-        mine += __popcll(fresh_tokens<kBitmapInSmem>(bm, cells[r], m, Lp, p.n_sink));
-      // exclusive prefix over the walking threads: tokens that higher-ranked cells bring
-      uint32_t incl = mine;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= o) incl += t;
-      }
-      if (lane == 31) warp_totals[combo & 1][warp] = incl;
-      walk_barrier();
-      const uint32_t wt = (lane < n_walk / 32) ? warp_totals[combo & 1][lane] : 0u;
-      uint32_t wi = wt;
-#pragma unroll
-      for (int o = 1; o < kMaxWalkWarps; o <<= 1) {
-        const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, wi, o);
-        if (lane >= o) wi += t;
-      }
-      const uint32_t total = __shfl_sync(0xFFFFFFFFu, wi, 31);
-      uint32_t ord = __shfl_sync(0xFFFFFFFFu, wi - wt, warp) + incl - mine;
-      // accept in rank order while the quota lasts; inside a cell in ascending position; the
-      // tokens of a cell are marked with one atomic per bitmap word (at most three words)
-      for (r = r0; r < r1 && ord < quota; ++r) {
-        const int cell = cells[r];
-        unsigned long long f = fresh_tokens<kBitmapInSmem>(bm, cell, m, Lp, p.n_sink);
-        if (f == 0ull) continue;
-        uint32_t n_new = __popcll(f);
-        if (ord + n_new > quota) {                             // the quota ends inside this cell
-          unsigned long long kept = 0ull;
-          for (uint32_t k = quota - ord; k > 0; --k) {
-            const unsigned long long lowest = f & (0ull - f);
-            kept |= lowest;
-            f ^= lowest;
-          }
-          f = kept;
-          n_new = quota - ord;
-        }
-        ord += n_new;
-        const int pos0 = p.n_sink + cell * m;
-        const int w0 = pos0 >> 5, sft = pos0 & 31;
-        const unsigned long long shifted = f << sft;
-        const uint32_t b0 = static_cast<uint32_t>(shifted), b1 = static_cast<uint32_t>(shifted >> 32);
-        const uint32_t b2 = sft ? static_cast<uint32_t>(f >> (64 - sft)) : 0u;
-        if (b0) bitmap_set<kBitmapInSmem>(bm, w0, b0);
-        if (b1) bitmap_set<kBitmapInSmem>(bm, w0 + 1, b1);
-        if (b2) bitmap_set<kBitmapInSmem>(bm, w0 + 2, b2);
-      }
-      if (total < quota && threadIdx.x == 0) atomicCAS(p.status, 0, kDevQuota);
+      if (two && combo + 1 < n_comb) issue_copy(combo + 1);
+      uint32_t* totals = warp_totals[combo & 1];
+      if (m <= 32)
+        walk_combination<false, kBitmapInSmem>(p, cells, K, m, quota, bm, summary, totals, n_walk, walk_barrier);
+      else
+        walk_combination<true, kBitmapInSmem>(p, cells, K, m, quota, bm, summary, totals, n_walk, walk_barrier);
       if (!two) {                                              // one buffer: copy only once it is free
         walk_barrier();
-        if (combo + 1 < tbl.n_comb) issue_copy(combo + 1);
+        if (combo + 1 < n_comb) issue_copy(combo + 1);
       }
       asm volatile("cp.async.wait_group 0;" ::: "memory");
       walk_barrier();                                          // bitmap updates and the next cells visible
@@ -773,12 +652,12 @@ __device__ __forceinline__ void allocate(const ComboTable& tbl, const SelectPara
 
   // Ascending output.  One SM does this, so what counts is the number of instructions it has
   // to issue.  Up to kSelThreads bitmap words (32K positions) a thread takes one word.  Longer
-  // contexts: the sink part is the identity; for the rest the bitmap is read four words per
-  // lane and load (a warp owns a contiguous run of words), twice: to count the words that hold
-  // an allocated position outside the sink part, then to list them in ascending order in
-  // shared memory (where the staged cells were; they are done with).  There are at most
-  // `budget` such words, usually a few hundred: the threads share them out evenly, take the
-  // prefix of their position counts and write the positions.
+  // contexts: the sink part is the identity; for the rest the words that hold an allocated position
+  // (at most `budget`, usually a few hundred) are listed in ascending order in shared memory (where
+  // the staged cells were; they are done with): from the summary, 32 words per summary word, or,
+  // with the bitmap in global memory, from the bitmap, four words per lane and load, read twice.
+  // The threads share the list out evenly, take the prefix of the words' position counts and
+  // write the positions.
   const long long n_words = (p.L + 31) / 32;
   const uint32_t cap = static_cast<uint32_t>(p.n_sink + p.budget);
   if (n_words <= kSelThreads) {
@@ -797,10 +676,6 @@ __device__ __forceinline__ void allocate(const ComboTable& tbl, const SelectPara
     return;
   }
   const int n_w = static_cast<int>(n_words);                // L < 2^31: word and quad numbers fit an int
-  const int n_quads = (n_w + 3) / 4;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int rounds = (n_quads + kSelThreads - 1) / kSelThreads;      // per warp
-  const int q_begin = warp * rounds * 32;
   int* list = staged;
   // bits of word w that stand for allocated positions outside the sink part
   const int sink_words = p.n_sink >> 5;                     // words that lie in the sink part entirely
@@ -808,48 +683,64 @@ __device__ __forceinline__ void allocate(const ComboTable& tbl, const SelectPara
   auto outside_sink = [&](uint32_t bits, int w) -> uint32_t {
     return (w > sink_words) ? bits : ((w < sink_words) ? 0u : (bits & sink_tail));
   };
-  const int plain_from = sink_words / 4 + 1, plain_to = n_w / 4;      // quads that need no fixing
-  auto load_quad = [&](int q) -> uint4 {
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (q >= n_quads) return v;
-    if constexpr (kBitmapInSmem) {
-      asm volatile("ld.volatile.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-                   : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(smem_u32(bm) + 16u * q) : "memory");
-    } else {
-      v = __ldcg(reinterpret_cast<const uint4*>(bm) + q);
-    }
-    if (q >= plain_from && q < plain_to) return v;
-    const int w0 = 4 * q;
-    if (w0 + 1 >= n_w) v.y = 0u;                            // words past the end hold nothing
-    if (w0 + 2 >= n_w) v.z = 0u;
-    if (w0 + 3 >= n_w) v.w = 0u;
-    v.x = outside_sink(v.x, w0); v.y = outside_sink(v.y, w0 + 1);
-    v.z = outside_sink(v.z, w0 + 2); v.w = outside_sink(v.w, w0 + 3);
-    return v;
-  };
   for (int j = threadIdx.x; j < p.n_sink; j += kSelThreads) p.out_idx[j] = j;
-  uint32_t n_mine = 0;
-  for (int k = 0; k < rounds; ++k) {
-    const uint4 v = load_quad(q_begin + k * 32 + lane);
-    n_mine += (v.x != 0u) + (v.y != 0u) + (v.z != 0u) + (v.w != 0u);
-  }
   uint32_t n_entries;
-  uint32_t running = block_exclusive_scan(n_mine, sh->scan, &n_entries);
-  running = __shfl_sync(0xFFFFFFFFu, running, 0);            // entries of the warps before this one
-  const uint32_t lt = (1u << lane) - 1u;
-  for (int k = 0; k < rounds; ++k) {
-    const int q = q_begin + k * 32 + lane;
-    const uint4 v = load_quad(q);
-    if (__ballot_sync(0xFFFFFFFFu, (v.x | v.y | v.z | v.w) != 0u) == 0u) continue;
-    const uint32_t b0 = __ballot_sync(0xFFFFFFFFu, v.x != 0u), b1 = __ballot_sync(0xFFFFFFFFu, v.y != 0u);
-    const uint32_t b2 = __ballot_sync(0xFFFFFFFFu, v.z != 0u), b3 = __ballot_sync(0xFFFFFFFFu, v.w != 0u);
-    uint32_t at = running + __popc(b0 & lt) + __popc(b1 & lt) + __popc(b2 & lt) + __popc(b3 & lt);
-    const uint32_t room = static_cast<uint32_t>(p.budget);  // the list's size; never short unless a quota was overrun
-    if (v.x) { if (at < room) list[at] = 4 * q; ++at; }
-    if (v.y) { if (at < room) list[at] = 4 * q + 1; ++at; }
-    if (v.z) { if (at < room) list[at] = 4 * q + 2; ++at; }
-    if (v.w) { if (at < room) list[at] = 4 * q + 3; ++at; }
-    running += __popc(b0) + __popc(b1) + __popc(b2) + __popc(b3);
+  if constexpr (kBitmapInSmem) {
+    const int n_sum = (n_w + 31) / 32, per = (n_sum + kSelThreads - 1) / kSelThreads;
+    const int s0 = min(n_sum, static_cast<int>(threadIdx.x) * per), s1 = min(n_sum, s0 + per);
+    uint32_t n_mine = 0;
+    for (int k = s0; k < s1; ++k) n_mine += __popc(bitmap_word<true>(summary, k));
+    uint32_t at = block_exclusive_scan(n_mine, sh->scan, &n_entries);
+    for (int k = s0; k < s1; ++k) {
+      uint32_t words = bitmap_word<true>(summary, k);
+      while (words) {
+        const int b = __ffs(words) - 1;
+        words &= words - 1;
+        if (at < static_cast<uint32_t>(p.budget)) list[at] = k * 32 + b;    // never short unless a quota was overrun
+        ++at;
+      }
+    }
+  } else {
+    const int n_quads = (n_w + 3) / 4;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rounds = (n_quads + kSelThreads - 1) / kSelThreads;      // per warp
+    const int q_begin = warp * rounds * 32;
+    const int plain_from = sink_words / 4 + 1, plain_to = n_w / 4;      // quads that need no fixing
+    auto load_quad = [&](int q) -> uint4 {
+      uint4 v = make_uint4(0u, 0u, 0u, 0u);
+      if (q >= n_quads) return v;
+      v = __ldcg(reinterpret_cast<const uint4*>(bm) + q);
+      if (q >= plain_from && q < plain_to) return v;
+      const int w0 = 4 * q;
+      if (w0 + 1 >= n_w) v.y = 0u;                            // words past the end hold nothing
+      if (w0 + 2 >= n_w) v.z = 0u;
+      if (w0 + 3 >= n_w) v.w = 0u;
+      v.x = outside_sink(v.x, w0); v.y = outside_sink(v.y, w0 + 1);
+      v.z = outside_sink(v.z, w0 + 2); v.w = outside_sink(v.w, w0 + 3);
+      return v;
+    };
+    uint32_t n_mine = 0;
+    for (int k = 0; k < rounds; ++k) {
+      const uint4 v = load_quad(q_begin + k * 32 + lane);
+      n_mine += (v.x != 0u) + (v.y != 0u) + (v.z != 0u) + (v.w != 0u);
+    }
+    uint32_t running = block_exclusive_scan(n_mine, sh->scan, &n_entries);
+    running = __shfl_sync(0xFFFFFFFFu, running, 0);            // entries of the warps before this one
+    const uint32_t lt = (1u << lane) - 1u;
+    for (int k = 0; k < rounds; ++k) {
+      const int q = q_begin + k * 32 + lane;
+      const uint4 v = load_quad(q);
+      if (__ballot_sync(0xFFFFFFFFu, (v.x | v.y | v.z | v.w) != 0u) == 0u) continue;
+      const uint32_t b0 = __ballot_sync(0xFFFFFFFFu, v.x != 0u), b1 = __ballot_sync(0xFFFFFFFFu, v.y != 0u);
+      const uint32_t b2 = __ballot_sync(0xFFFFFFFFu, v.z != 0u), b3 = __ballot_sync(0xFFFFFFFFu, v.w != 0u);
+      uint32_t at = running + __popc(b0 & lt) + __popc(b1 & lt) + __popc(b2 & lt) + __popc(b3 & lt);
+      const uint32_t room = static_cast<uint32_t>(p.budget);  // the list's size; never short unless a quota was overrun
+      if (v.x) { if (at < room) list[at] = 4 * q; ++at; }
+      if (v.y) { if (at < room) list[at] = 4 * q + 1; ++at; }
+      if (v.z) { if (at < room) list[at] = 4 * q + 2; ++at; }
+      if (v.w) { if (at < room) list[at] = 4 * q + 3; ++at; }
+      running += __popc(b0) + __popc(b1) + __popc(b2) + __popc(b3);
+    }
   }
   __syncthreads();
   n_entries = min(n_entries, static_cast<uint32_t>(p.budget));
@@ -885,6 +776,14 @@ select_kernel(const ComboTable tbl, const SelectParams p) {
   const int t_begin = static_cast<int>(static_cast<long long>(blockIdx.x) * n_tiles / gridDim.x);
   const int t_end = static_cast<int>(static_cast<long long>(blockIdx.x + 1) * n_tiles / gridDim.x);
   for (int b = threadIdx.x; b < kHistBins; b += kSelThreads) sh.hist[b] = 0u;
+  if (blockIdx.x == 0 && p.bitmap_in_smem) {               // for phase F: empty but for the sink part
+    uint32_t* bm = smem_bitmap(dyn_smem);
+    const int n_words = static_cast<int>((p.L + 31) / 32), sink_words = p.n_sink >> 5;
+    for (int w = threadIdx.x; w < n_words; w += kSelThreads)
+      bm[w] = (w < sink_words) ? 0xFFFFFFFFu : ((w == sink_words) ? (1u << (p.n_sink & 31)) - 1u : 0u);
+    uint32_t* summary = smem_summary(dyn_smem, p.L);
+    for (int k = threadIdx.x; k < (n_words + 31) / 32; k += kSelThreads) summary[k] = 0u;
+  }
   uint32_t epoch = 0;
   grid_dep_wait();       // the kernel before this one (scores, state cleared for this run) is done
 
@@ -930,107 +829,41 @@ select_kernel(const ComboTable tbl, const SelectParams p) {
   }
   if (!grid_sync<kCluster>(p, &sh, epoch)) return;
 
-  // ---- C: radix select of the K_m-th largest value ----
-  // combinations whose tiles this CTA scans
+  // ---- C, D: the threshold bin of every combination this CTA scans, and the gather ----
   int c_lo = 0, c_hi = -1;
   if (t_begin < t_end) {
     int cursor = 0;
     c_lo = combo_of_tile(tbl, t_begin, cursor);
     c_hi = combo_of_tile(tbl, t_end - 1, cursor);
   }
-  for (int combo = c_lo + threadIdx.x; combo <= c_hi; combo += kSelThreads) {
-    sh.prefix[combo] = 0ull;
-    sh.krem[combo] = static_cast<uint32_t>(tbl.k_m[combo]);
-    sh.state[combo] = 0u;
-    sh.mode[combo] = 0;
-  }
-  __syncthreads();
-  for (int combo = c_lo; combo <= c_hi; ++combo) bin_search(p, tbl.n_comb, combo, 0, &sh);
-
-  // ---- D: the gather.  After the first pass a combination knows the bin (top 11 bits of the
-  // key) that holds its K_m-th value.  One scan settles almost everything: cells above that
-  // bin are candidates; where every cell of the bin is wanted too (or few cells exist), the
-  // bin's cells are candidates as well; otherwise the bin's cells are set aside (at most
-  // kPendCap of them) and one CTA picks the wanted number of highest keys among them.
-  {
-    const int lane = threadIdx.x & 31;
-    int load_cursor = 0, cursor = 0;
-    for (int t0 = t_begin; t0 < t_end; t0 += kScanGroup) {
-      float wv[kScanGroup][kTilePer];
-#pragma unroll
-      for (int g = 0; g < kScanGroup; ++g)
-        if (t0 + g < t_end) fetch_tile(tbl, p, t0 + g, load_cursor, nullptr, wv[g]);
-#pragma unroll
-      for (int g = 0; g < kScanGroup; ++g) {
-        const int tile = t0 + g;
-        if (tile >= t_end) break;
-        const int combo = combo_of_tile(tbl, tile, cursor);
-        const int mode = sh.mode[combo];
-        if (mode == 2) continue;                             // left to the full-scan passes
-        const unsigned long long threshold = sh.prefix[combo];
-        const uint32_t bin = static_cast<uint32_t>(threshold >> 53);
-        unsigned long long* cand = p.cand + static_cast<long long>(combo) * p.cand_stride;
-        unsigned long long* pend = p.pending + static_cast<long long>(combo) * kPendCap;
-        const int c0 = (tile - tbl.tile_begin[combo]) * kSelTile;
-        const int c1 = min(tbl.len[combo], c0 + kSelTile);
-#pragma unroll
-        for (int k = 0; k < kTilePer; ++k) {
-          const int c = c0 + k * kSelThreads + threadIdx.x;
-          unsigned long long key = 0ull;
-          bool take = false, aside = false;
-          if (c < c1) {
-            key = make_key(wv[g][k], static_cast<uint32_t>(c));
-            if (mode == 0) {
-              take = key >= threshold;
-            } else {
-              const uint32_t digit = static_cast<uint32_t>(key >> 53);
-              take = digit > bin;
-              aside = digit == bin;
-            }
-          }
-          const uint32_t votes = __ballot_sync(0xFFFFFFFFu, take);
-          if (votes) {
-            uint32_t slot = 0;
-            if (lane == __ffs(votes) - 1) slot = atomicAdd(&p.cand_count[combo], __popc(votes));
-            slot = __shfl_sync(0xFFFFFFFFu, slot, __ffs(votes) - 1) +
-                   __popc(votes & ((1u << lane) - 1u));
-            if (take && slot < static_cast<uint32_t>(tbl.k_m[combo])) cand[slot] = key;
-          }
-          const uint32_t held = __ballot_sync(0xFFFFFFFFu, aside);
-          if (held) {
-            uint32_t slot = 0;
-            if (lane == __ffs(held) - 1)
-              slot = atomicAdd(&p.cand_count[kMaxCombos + combo], __popc(held));
-            slot = __shfl_sync(0xFFFFFFFFu, slot, __ffs(held) - 1) +
-                   __popc(held & ((1u << lane) - 1u));
-            if (aside && slot < static_cast<uint32_t>(kPendCap)) pend[slot] = key;
-          }
-        }
-      }
-    }
+  for (int combo = c_lo; combo <= c_hi; ++combo) {
+    find_threshold(p, tbl, combo, &sh);
+    if (threadIdx.x == 0) sh.mode[combo] = static_cast<uint8_t>(sh.plateau);
+    if (!sh.plateau)                                         // uniform
+      gather_combination(p, tbl, combo, max(t_begin, tbl.tile_begin[combo]), min(t_end, tbl.tile_begin[combo + 1]), &sh);
+    __syncthreads();                                         // readers of the threshold words
   }
   if (!grid_sync<kCluster>(p, &sh, epoch)) return;
 
-  // The cells set aside: one CTA per combination selects the highest `wanted` keys among them
-  // (radix select over the remaining 53 bits of the key in shared memory) and appends them.
-  for (int combo = blockIdx.x; combo < tbl.n_comb; combo += gridDim.x) {
-    const int n_p = static_cast<int>(min(__ldcg(&p.cand_count[kMaxCombos + combo]),
-                                         static_cast<uint32_t>(kPendCap)));
-    if (n_p == 0) continue;                                  // uniform
-    resolve_pending(p, tbl, combo, n_p, &sh);
-  }
-
-  // A plateau across a whole bin (more than kPendCap equal-digit cells): the remaining passes
-  // over the array, for those combinations only.  The flag is the same for every CTA.
+  // The long way, for the combinations whose threshold bin is a plateau.  The flag is the same for every
+  // CTA.  The histograms of its passes are cleared here: they are hardly ever needed.
   if (__ldcg(&p.cand_count[3 * kMaxCombos]) != 0u) {
-    for (int combo = c_lo + threadIdx.x; combo <= c_hi; combo += kSelThreads)
-      if (sh.mode[combo] != 2) sh.state[combo] = 1u;         // nothing left to do for these
-    __syncthreads();
-    for (int pass = 1; pass < kSelectPasses; ++pass) {
+    uint32_t* pass_hist = p.hist + 2ll * tbl.n_comb * kHistBins;
+    const long long n_hist = static_cast<long long>(kSelectPasses) * tbl.n_comb * kHistBins;
+    for (long long i = static_cast<long long>(blockIdx.x) * kSelThreads + threadIdx.x; i < n_hist;
+         i += static_cast<long long>(gridDim.x) * kSelThreads)
+      pass_hist[i] = 0u;
+    for (int combo = c_lo + threadIdx.x; combo <= c_hi; combo += kSelThreads) {
+      sh.prefix[combo] = 0ull;
+      sh.krem[combo] = static_cast<uint32_t>(tbl.k_m[combo]);
+      sh.state[combo] = sh.mode[combo] ? 0u : 1u;            // nothing left to do for the others
+    }
+    if (!grid_sync<kCluster>(p, &sh, epoch)) return;
+    for (int pass = 0; pass < kSelectPasses; ++pass) {
       int shift, bits;
       pass_bits(pass, shift, bits);
       const uint32_t mask = (1u << bits) - 1u;
-      uint32_t* hist_pass = p.hist + static_cast<long long>(pass) * tbl.n_comb * kHistBins;
+      uint32_t* hist_pass = pass_hist + static_cast<long long>(pass) * tbl.n_comb * kHistBins;
       int cur = -1, load_cursor = 0, cursor = 0;
       for (int t0 = t_begin; t0 < t_end; t0 += kScanGroup) {
         float wv[kScanGroup][kTilePer];
@@ -1055,7 +888,7 @@ select_kernel(const ComboTable tbl, const SelectParams p) {
             uint32_t digit = 0xFFFFFFFFu;                    // sentinel: does not take part
             if (c < c1) {
               const unsigned long long key = make_key(wv[g][k], static_cast<uint32_t>(c));
-              if (((key ^ prefix) >> (shift + bits)) == 0ull)
+              if (pass == 0 || ((key ^ prefix) >> (shift + bits)) == 0ull)
                 digit = static_cast<uint32_t>(key >> shift) & mask;
             }
             hist_add(sh.hist, digit);
@@ -1065,7 +898,8 @@ select_kernel(const ComboTable tbl, const SelectParams p) {
       if (cur >= 0) hist_flush(sh.hist, hist_pass + static_cast<long long>(cur) * kHistBins);
       if (!grid_sync<kCluster>(p, &sh, epoch)) return;
       for (int combo = c_lo; combo <= c_hi; ++combo)
-        if (sh.state[combo] == 0u) bin_search(p, tbl.n_comb, combo, pass, &sh);
+        if (sh.state[combo] == 0u)
+          bin_search(p, hist_pass + static_cast<long long>(combo) * kHistBins, combo, pass, &sh);
     }
 
     // ---- D: ties at the K_m-th value, then the gather ----
@@ -1113,7 +947,7 @@ select_kernel(const ComboTable tbl, const SelectParams p) {
           const int tile = t0 + g;
           if (tile >= t_end) break;
           const int combo = combo_of_tile(tbl, tile, cursor);
-          if (sh.mode[combo] != 2) continue;                   // gathered in the first scan
+          if (!sh.mode[combo]) continue;                       // gathered in the first scan
           const bool settled = sh.state[combo] != 0u;
           const unsigned long long threshold = sh.prefix[combo];
           const uint32_t v_star = static_cast<uint32_t>(threshold >> 32);
@@ -1164,17 +998,14 @@ select_kernel(const ComboTable tbl, const SelectParams p) {
         }
       }
     }
+    if (!grid_sync<kCluster>(p, &sh, epoch)) return;
   }
-  if (!grid_sync<kCluster>(p, &sh, epoch)) return;
 
   // ---- E: ranking ----
   {
     unsigned long long* chunk = reinterpret_cast<unsigned long long*>(dyn_smem);
-    __shared__ int rank_count[kSelThreads];
-    __shared__ RankScratch rank_scratch;
     for (int combo = threadIdx.x; combo < tbl.n_comb; combo += kSelThreads)
-      sh.state[combo] = min(min(__ldcg(&p.cand_count[combo]), static_cast<uint32_t>(kMaxKm)),
-                            static_cast<uint32_t>(tbl.k_m[combo]));
+      sh.state[combo] = min(__ldcg(&p.cand_count[combo]), static_cast<uint32_t>(p.cand_stride));
     __syncthreads();
     const int grid = static_cast<int>(gridDim.x), bid = static_cast<int>(blockIdx.x);
     if (tbl.rank_by_list) {
@@ -1186,7 +1017,7 @@ select_kernel(const ComboTable tbl, const SelectParams p) {
         if (bid < b0 || bid >= b1) continue;
         const uint32_t n = sh.state[combo], share = b1 - b0, k = bid - b0;
         const int lo = static_cast<int>(n * k / share), hi = static_cast<int>(n * (k + 1) / share);
-        if (lo < hi) rank_range(p, combo, static_cast<int>(n), lo, hi, chunk, rank_count, &rank_scratch);
+        if (lo < hi) rank_range(p, tbl, combo, static_cast<int>(n), lo, hi, chunk);
       }
     } else {
       // fewer CTAs than lists: every CTA takes a contiguous run of all candidates
@@ -1198,7 +1029,7 @@ select_kernel(const ComboTable tbl, const SelectParams p) {
       for (int combo = 0; combo < tbl.n_comb; ++combo) {
         const int n = static_cast<int>(sh.state[combo]);
         const int lo = max(i_begin, first) - first, hi = min(i_end, first + n) - first;
-        if (lo < hi) rank_range(p, combo, n, lo, hi, chunk, rank_count, &rank_scratch);
+        if (lo < hi) rank_range(p, tbl, combo, n, lo, hi, chunk);
         first += n;
       }
     }
@@ -1208,15 +1039,6 @@ select_kernel(const ComboTable tbl, const SelectParams p) {
   // ---- F: allocation and ascending output (one CTA) ----
   if (blockIdx.x != 0) return;
   if (p.bitmap_in_smem) {
-    uint32_t* bm = reinterpret_cast<uint32_t*>(dyn_smem);
-    const long long n_words = (p.L + 31) / 32;
-    for (long long w = threadIdx.x; w < n_words; w += kSelThreads) {
-      const long long lo = w * 32;
-      uint32_t bits = 0;
-      if (p.n_sink > lo) bits = (p.n_sink - lo >= 32) ? 0xFFFFFFFFu : ((1u << (p.n_sink - lo)) - 1u);
-      bm[w] = bits;
-    }
-    __syncthreads();
     allocate<true>(tbl, p, dyn_smem, &sh);
   } else {
     allocate<false>(tbl, p, dyn_smem, &sh);
@@ -1227,28 +1049,17 @@ select_kernel(const ComboTable tbl, const SelectParams p) {
 // host side
 // ---------------------------------------------------------------------------------------
 size_t select_smem_bytes(long long L, int max_km, int budget, SelectParams* p) {
-  size_t bytes = 2 * static_cast<size_t>(kSelTile + kMaxWin) * sizeof(float);  // pooling tiles
-  if (kSrcTileTokens * sizeof(float) > bytes) bytes = kSrcTileTokens * sizeof(float);
-  if (kRankChunk * sizeof(unsigned long long) > bytes) bytes = kRankChunk * sizeof(unsigned long long);
-  // quota walk: bitmap (when it fits) + one or two staging buffers of max_km cell ids
+  (void)budget;                                             // the output list (<= kMaxKm) fits the work area
+  // quota walk: one or two staging buffers of max_km cell ids in the work area, the bitmap and its
+  // summary (when they fit) behind it
   const size_t cap = (static_cast<size_t>(max_km < 1 ? 1 : max_km) + 3) & ~size_t(3);
-  const size_t bm_bytes = (static_cast<size_t>((L + 31) / 32) * sizeof(uint32_t) + 15) & ~size_t(15);
-  p->bitmap_in_smem = bm_bytes <= static_cast<size_t>(kSelBitmapSmemBytes) ? 1 : 0;
-  const size_t base = p->bitmap_in_smem ? bm_bytes : 0;
-  int walkers = ((max_km + 1) / 2 + 31) & ~31;               // about two ranked cells per thread
-  p->walk_threads = walkers < 256 ? 256 : (walkers > kSelThreads ? kSelThreads : walkers);
+  const size_t words = (static_cast<size_t>((L + 31) / 32) + 3) & ~size_t(3);
+  p->bitmap_in_smem = words * sizeof(uint32_t) <= static_cast<size_t>(kSelBitmapSmemBytes) ? 1 : 0;
+  int walkers = ((max_km + kWalkCells - 1) / kWalkCells + 31) & ~31;
+  p->walk_threads = walkers < kMinWalkers ? kMinWalkers : (walkers > kSelThreads ? kSelThreads : walkers);
   p->stage_capacity = static_cast<int>(cap);
-  p->stage_double = (base + 2 * cap * sizeof(int) <= static_cast<size_t>(kSelMaxDynSmemBytes)) ? 1 : 0;
-  size_t after_bitmap = (p->stage_double ? 2 : 1) * cap * sizeof(int);
-  // the output pass lists the bitmap words that hold allocated positions (at most `budget`)
-  // where the staged cells were
-  size_t list_bytes = static_cast<size_t>((L + 31) / 32);
-  if (list_bytes > static_cast<size_t>(budget < 0 ? 0 : budget)) list_bytes = budget < 0 ? 0 : budget;
-  list_bytes *= sizeof(int);
-  if (list_bytes > after_bitmap) after_bitmap = list_bytes;
-  const size_t alloc_bytes = base + after_bitmap;
-  if (alloc_bytes > bytes) bytes = alloc_bytes;
-  return bytes;
+  p->stage_double = (2 * cap * sizeof(int) <= static_cast<size_t>(kSelWorkBytes)) ? 1 : 0;
+  return kSelWorkBytes + (p->bitmap_in_smem ? (words + (words + 31) / 32) * sizeof(uint32_t) : 0);
 }
 
 cudaError_t select_max_grid(int n_sm, int* max_grid) {

@@ -11,14 +11,19 @@ static constexpr int kHistBins = 2048;
 static constexpr int kMaxWin = 1024;        // largest stride-1 window size
 static constexpr int kMaxMaxSize = 64;      // largest strided max-pool size
 static constexpr int kMaxKm = 16384;        // largest K_m (bounds the candidate lists)
-static constexpr int kSelectPasses = 3;     // 32 value bits of the key in 11/11/10-bit digits
+static constexpr int kSelectPasses = 3;     // long way: 32 value bits of the key in 11/11/10-bit digits
 static constexpr int kSelThreads = 1024;    // threads per CTA of the selection kernel
 static constexpr int kSelTile = 4096;       // cells of one combination per work tile
 static constexpr int kSrcTileTokens = 8192; // tokens per work tile of the strided max-pool
 static constexpr int kSelClusterMax = 8;     // grids up to this size run as one thread-block cluster
-static constexpr int kPendCap = 8192;        // cells of the threshold bin resolved by one CTA (else: more passes)
+static constexpr int kCandSlack = 4096;      // candidates past K_m that the threshold bin may bring
 static constexpr int kSelBitmapSmemBytes = 136 * 1024;   // bitmap kept in shared memory up to this
-static constexpr int kSelMaxDynSmemBytes = kSelBitmapSmemBytes + kMaxKm * 4;
+// Work area in front of the bitmap: pooling tiles, the keys of a ranking list, the staged cells of the
+// quota walk and the list of the output pass, one after another.
+static constexpr int kSelWorkBytes = 64 * 1024;
+static_assert(kSelWorkBytes >= 2 * (kSelTile + kMaxWin) * 4 && kSelWorkBytes >= kSrcTileTokens * 4 &&
+              kSelWorkBytes >= kMaxKm * 4, "work area too small");
+static constexpr int kSelMaxDynSmemBytes = kSelWorkBytes + kSelBitmapSmemBytes + kSelBitmapSmemBytes / 32 + 64;
 
 // One entry per (m_i, n_j) combination, in Algorithm 1's loop order.
 struct ComboTable {
@@ -54,15 +59,15 @@ struct SelectParams {
   long long maxpooled_stride;
   float* pooled;           // [n_comb][pooled_stride]
   long long pooled_stride;
-  uint32_t* hist;          // [kSelectPasses][n_comb][kHistBins], zero on entry
+  uint32_t* hist;          // [2 + kSelectPasses][n_comb][kHistBins]: values per bin and candidates placed per
+                           // bin, zero on entry; then the passes of the long way
   int* tile_ties;          // [work tiles]: cells of a tile that hold the K_m-th value
-  unsigned long long* cand;   // [n_comb][cand_stride] selected 64-bit keys
-  int cand_stride;
+  unsigned long long* cand;   // [n_comb][cand_stride] 64-bit keys of the candidates, sorted by bin
+  uint32_t* cand_seg;      // [n_comb][cand_stride] start | length << 16 of a candidate's bin
+  int cand_stride;         // at least K_m + kCandSlack, a multiple of 4, below 2^16
   uint32_t* cand_count;    // [4 * kMaxCombos]: candidates gathered per combination; then, at
-                           // kMaxCombos, 2 kMaxCombos and 3 kMaxCombos: cells pending in the
-                           // threshold bin, keys still wanted from it, and one flag word
-                           // (some combination needs the full-scan passes); zero on entry
-  unsigned long long* pending;   // [n_comb][kPendCap] keys of the threshold bin
+                           // kMaxCombos, whether the combination took the long way, and at
+                           // 3 kMaxCombos one flag word (some combination did); zero on entry
   int* ranked;             // [n_comb][cand_stride] cell ids in rank order (cand_stride: multiple of 4)
   uint32_t* bitmap;        // [ceil(L/32)] in global memory, used when it does not fit shared memory
   int bitmap_in_smem;
