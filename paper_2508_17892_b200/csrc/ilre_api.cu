@@ -495,7 +495,7 @@ int recall_impl(ilre_recall_t* h, const void* k_cache_dev, int64_t L, const void
 
   SelectParams sp;
   std::memset(&sp, 0, sizeof(sp));
-  sp.enc = h->enc; sp.scores = h->scores; sp.user_scores = out_scores_dev;
+  sp.enc = h->enc; sp.user_scores = out_scores_dev;
   sp.L = L; sp.n_sink = spec->n_sink; sp.win_op = spec->win_op;
   sp.pooled = h->pooled; sp.pooled_stride = h->pooled_stride; sp.hist = h->hist;
   sp.maxpooled = h->maxpooled; sp.maxpooled_stride = h->cfg.max_L / 2 + 1;
@@ -530,7 +530,7 @@ int recall_impl(ilre_recall_t* h, const void* k_cache_dev, int64_t L, const void
 
   if (!with_qk) pp.kv_rows = 0;                          // no query to pack
   mp.ext_stats = io.ext_stats; mp.n_ext = io.n_ext;
-  if (io.scores_in) { sp.scores = const_cast<float*>(io.scores_in); sp.scores_given = 1; }
+  if (io.scores_in) { sp.scores = io.scores_in; sp.scores_given = 1; }
   ILRE_MARK(0);
   {
     TraceRange r("ilre: prepare");
@@ -629,8 +629,8 @@ int ilre_recall_run_host(ilre_recall_t* h, const void* k_cache_host, int64_t L,
   int rc;
   if (n_pieces < 2) {
     ILRE_CUDA(cudaMemcpyAsync(h->stage_k, k_cache_host, k_bytes, cudaMemcpyHostToDevice, st));
-    rc = ilre_recall_run(h, h->stage_k, L, h->stage_q, q_len, budget, spec, h->stage_idx, nullptr,
-                         st);
+    rc = ilre_recall_run(h, h->stage_k, L, h->stage_q, q_len, budget, spec, h->stage_idx,
+                         out_scores_host ? h->scores : nullptr, st);
   } else {
     const size_t row_bytes = static_cast<size_t>(h->cfg.n_kv_heads) * 256;
     const size_t n_rows = static_cast<size_t>(q_len) * h->cfg.n_q_heads;
@@ -651,8 +651,8 @@ int ilre_recall_run_host(ilre_recall_t* h, const void* k_cache_host, int64_t L,
     if (rc == ILRE_OK) {
       const RunIo io = {kStageScores | kStageSelect, nullptr, h->piece_stats, n_pieces, nullptr,
                         nullptr};
-      rc = recall_impl(h, h->stage_k, L, h->stage_q, q_len, budget, spec, h->stage_idx, nullptr, st,
-                       io);
+      rc = recall_impl(h, h->stage_k, L, h->stage_q, q_len, budget, spec, h->stage_idx,
+                       out_scores_host ? h->scores : nullptr, st, io);
     }
     if (rc != ILRE_OK) cudaStreamSynchronize(h->copy_stream);   // nothing in flight on return
   }

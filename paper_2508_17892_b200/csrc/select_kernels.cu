@@ -1,10 +1,12 @@
 // Algorithm 1 ("Context Allocation") on the device, as ONE cooperative kernel whose CTAs
 // meet at grid barriers between the phases:
 //
-//   A  A^C[t] = exp2(max_r log2 p_rt) from the scores pass' encoded maxima (Eq. 5);
-//   B  MaxPooling(size = stride = m), once per distinct m, then the stride-1 window pooling
-//      (average or max) of every (m, n) combination, and a histogram of the pooled values in
+//   A  MaxPooling(size = stride = m), once per distinct m > 1;
+//   B  the stride-1 window pooling (average or max) of every (m, n) combination, up to kPoolGroup
+//      windows of one m from one load of the cells, and a histogram of the pooled values in
 //      kHistBins logarithmic bins;
+//   (A and B take A^C[t] = exp2(max_r log2 p_rt) from the scores pass' encoded maxima, Eq. 5, as they
+//   read them;)
 //   C  every CTA finds, for each combination it scans, the bin that holds the K_m-th largest value
 //      and how many values lie in the bins above each bin;
 //   D  one scan gathers the candidates, the cells of that bin and of the bins above it, sorted by
@@ -20,8 +22,8 @@
 //      already allocated, stops each combination at its quota B_c, then writes the allocated
 //      positions in ascending order.
 //
-// Work of phases B-D is cut into tiles of kSelTile cells of one combination; every CTA owns a
-// contiguous run of tiles, the same in every phase.
+// Work of phase B is cut into tiles of cells of one group of windows, work of phase D into tiles of
+// kSelTile cells of one combination; every CTA owns a contiguous run of tiles.
 #include "select_kernels.cuh"
 #include "sm100_ptx.cuh"
 
@@ -174,100 +176,147 @@ __device__ __forceinline__ void fetch_tile(const ComboTable& tbl, const SelectPa
   }
 }
 
-// Phase B1 for one tile of source `src`: cells of MaxPooling(size = stride = m), a shorter
+// Score of position t (Eq. 5).
+__device__ __forceinline__ float score_at(const SelectParams& p, long long t) {
+  return p.scores_given ? __ldcg(&p.scores[t]) : exp2f(ordered_to_float(__ldcg(&p.enc[t])));
+}
+
+// Phase A for one tile of source `src`: cells of MaxPooling(size = stride = m), a shorter
 // last cell where m does not divide the length.  The tokens are read coalesced into `buf`
-// (kSrcTileTokens floats), all loads in flight together.
+// (kSrcTileTokens words), all loads in flight together; the maximum is taken of the encoded
+// scores, whose order is the scores', and one exponential per cell.
 __device__ __forceinline__ void maxpool_tile(const ComboTable& tbl, const SelectParams& p, int src,
-                                             int tile_in_src, float* buf) {
+                                             int tile_in_src, uint32_t* buf) {
   const int m = tbl.src_m[src], len = tbl.src_len[src];
   const long long Lp = p.L - p.n_sink;
-  const float* a = p.scores + p.n_sink;
+  const uint32_t* a = (p.scores_given ? reinterpret_cast<const uint32_t*>(p.scores) : p.enc) + p.n_sink;
   const int cells_per_tile = kSrcTileTokens / m;
   const int c0 = tile_in_src * cells_per_tile;
   const int n_cells = min(cells_per_tile, len - c0);
   const long long t0 = static_cast<long long>(c0) * m;
   const int n_tok = static_cast<int>(min(static_cast<long long>(n_cells) * m, Lp - t0));
   constexpr int kLd = kSrcTileTokens / kSelThreads;
-  float v[kLd];
+  uint32_t v[kLd];
 #pragma unroll
   for (int k = 0; k < kLd; ++k) {
     const int i = k * kSelThreads + threadIdx.x;
-    v[k] = (i < n_tok) ? __ldcg(a + t0 + i) : -INFINITY;
+    v[k] = (i < n_tok) ? __ldcg(a + t0 + i) : 0u;
+    if (p.scores_given && i < n_tok) v[k] = float_to_ordered(__uint_as_float(v[k]));
   }
 #pragma unroll
-  for (int k = 0; k < kLd; ++k) buf[k * kSelThreads + threadIdx.x] = v[k];
+  for (int k = 0; k < kLd; ++k) buf[k * kSelThreads + threadIdx.x] = v[k];      // 0: below every score
   __syncthreads();
   float* out = p.maxpooled + static_cast<long long>(src) * p.maxpooled_stride;
   for (int c = threadIdx.x; c < n_cells; c += kSelThreads) {
-    float acc = buf[c * m];
-    for (int j = 1; j < m; ++j) acc = fmaxf(acc, buf[c * m + j]);
-    out[c0 + c] = acc;
+    uint32_t acc = buf[c * m];
+    for (int j = 1; j < m; ++j) acc = max(acc, buf[c * m + j]);
+    out[c0 + c] = p.scores_given ? ordered_to_float(acc) : exp2f(ordered_to_float(acc));
   }
   __syncthreads();
 }
 
-// Phase B2 for one tile: pooled cells [c0, c0 + n_out) of `combo` from its max-pooled source
-// (the scores themselves for m = 1), written to p.pooled; the bin of every cell goes to the shared
-// histogram.  `buf0`/`buf1` hold kSelTile + kMaxWin floats each.
-__device__ __forceinline__ void pool_tile(const ComboTable& tbl, const SelectParams& p, int combo,
-                                          int c0, float* buf0, float* buf1, uint32_t* sh_hist) {
-  const int n = tbl.n[combo], len = tbl.len[combo];
-  const int source = tbl.src[combo];
-  const float* a = (source < 0)
-      ? p.scores + p.n_sink
-      : p.maxpooled + static_cast<long long>(source) * p.maxpooled_stride;
-  const int lo = c0 - n / 2;
-  const int n_out = min(kSelTile, len - c0);
-  const int span = n_out + n - 1;
+// Counts the bin of one cell per lane (-1: none).  Neighbouring cells of a window maximum are often
+// equal: the first lane of a run of equal bins adds the whole run.
+__device__ __forceinline__ void count_bins(uint32_t* hist, int bin) {
+  const int lane = threadIdx.x & 31;
+  const int left = __shfl_up_sync(0xFFFFFFFFu, bin, 1);
+  const bool leader = lane == 0 || left != bin;
+  const uint32_t leaders = __ballot_sync(0xFFFFFFFFu, leader);
+  if (leader && bin >= 0) {
+    const uint32_t after = (lane == 31) ? 0u : leaders >> (lane + 1);
+    atomicAdd(&hist[bin], after ? static_cast<uint32_t>(__ffs(after)) : static_cast<uint32_t>(32 - lane));
+  }
+}
+
+// Phase B for one tile: cells [c0, c0 + n_out) of every combination of group `grp` from their common
+// source (the scores themselves for m = 1), written to p.pooled; the bins of the cells are counted in
+// the group's histograms.  `buf0` / `buf1` hold the tile and the widest window's margin; hists[k] belongs
+// to the group's k-th combination (ascending window sizes).
+__device__ __forceinline__ void pool_tile(const ComboTable& tbl, const SelectParams& p, int grp, int c0, int n_out,
+                                          float* buf0, float* buf1, uint32_t* hist0, uint32_t* hist1) {
+  const int first = tbl.grp_first[grp], n_win = tbl.grp_first[grp + 1] - first;
+  const int some = tbl.grp_combo[first];
+  const int n_max = tbl.n[tbl.grp_combo[first + n_win - 1]], len = tbl.len[some];
+  const int source = tbl.src[some];
+  const float* a = (source < 0) ? nullptr : p.maxpooled + static_cast<long long>(source) * p.maxpooled_stride;
+  const int lo = c0 - n_max / 2;
+  const int span = n_out + n_max - 1;
   const float pad = (p.win_op == 0) ? 0.f : -INFINITY;
-  {
-    constexpr int kLd = (kSelTile + kMaxWin + kSelThreads - 1) / kSelThreads;
-    float v[kLd];
+  for (int base = 0; base < span; base += 4 * kSelThreads) {
+    float v[4];                                            // all loads in flight together
 #pragma unroll
-    for (int k = 0; k < kLd; ++k) {
-      const int idx = k * kSelThreads + threadIdx.x, u = lo + idx;
-      v[k] = (idx < span && u >= 0 && u < len) ? __ldcg(a + u) : pad;
+    for (int k = 0; k < 4; ++k) {
+      const int idx = base + k * kSelThreads + threadIdx.x, u = lo + idx;
+      v[k] = (idx < span && u >= 0 && u < len) ? (a ? __ldcg(a + u) : score_at(p, p.n_sink + u)) : pad;
     }
 #pragma unroll
-    for (int k = 0; k < kLd; ++k) {
-      const int idx = k * kSelThreads + threadIdx.x;
+    for (int k = 0; k < 4; ++k) {
+      const int idx = base + k * kSelThreads + threadIdx.x;
       if (idx < span) buf0[idx] = v[k];
     }
   }
   __syncthreads();
-  // Window maximum by doubling: after the step of width w, src[i] = max of cells [i, i + w);
-  // a window of n cells is then the maximum of two overlapping runs of width w <= n < 2w.
-  float* src = buf0;
-  int w = 1;
   if (p.win_op != 0) {
-    float* dst = buf1;
-    while (2 * w <= n) {
-      const int cnt = span - 2 * w + 1;
-      for (int i = threadIdx.x; i < cnt; i += kSelThreads) dst[i] = fmaxf(src[i], src[i + w]);
-      __syncthreads();
-      float* t = src; src = dst; dst = t;
-      w *= 2;
-    }
-  }
-  float* out = p.pooled + static_cast<long long>(combo) * p.pooled_stride;
-  for (int base = 0; base < n_out; base += kSelThreads) {
-    const int i = base + threadIdx.x;
-    uint32_t digit = 0xFFFFFFFFu;
-    if (i < n_out) {
-      float acc;
-      if (p.win_op == 0) {
-        acc = 0.f;
-        for (int j = 0; j < n; ++j) acc += src[i + j];       // left to right, as the definition
-        acc = acc / static_cast<float>(n);
-      } else {
-        acc = fmaxf(src[i], src[i + n - w]);
+    // Window maximum by doubling: after the step of width w, src[i] = max of cells [i, i + w);
+    // a window of n cells is then the maximum of two overlapping runs of width w <= n < 2w.
+    float *src = buf0, *dst = buf1;
+    int w = 1;
+#pragma unroll 1
+    for (int k = 0; k < n_win; ++k) {
+      const int combo = tbl.grp_combo[first + k], n = tbl.n[combo];
+#pragma unroll 1
+      for (; 2 * w <= n; w *= 2) {
+        const int cnt = span - 2 * w + 1;
+#pragma unroll 4
+        for (int i = threadIdx.x; i < cnt; i += kSelThreads) dst[i] = fmaxf(src[i], src[i + w]);
+        __syncthreads();
+        float* t = src; src = dst; dst = t;
       }
-      out[c0 + i] = acc;
-      digit = static_cast<uint32_t>(bin_of_ordered(float_to_ordered(acc)));
+      float* out = p.pooled + static_cast<long long>(combo) * p.pooled_stride + c0;
+      uint32_t* hist = (k == 0) ? hist0 : hist1 + (k - 1) * kHistBins;
+      const float* s0 = src + (n_max / 2 - n / 2);
+#pragma unroll 1
+      for (int base = 0; base < n_out; base += kSelThreads) {
+        const int i = base + threadIdx.x;
+        int bin = -1;
+        if (i < n_out) {
+          const float acc = fmaxf(s0[i], s0[i + n - w]);
+          out[i] = acc;
+          bin = bin_of_ordered(float_to_ordered(acc));
+        }
+        count_bins(hist, bin);
+      }
+      // the next doubling step writes the other buffer, which everyone has left at its last barrier
     }
-    hist_add(sh_hist, digit);
+    __syncthreads();
+  } else {
+    // Window averages: the sum of n cells from cell u on is the sum of n - 1 cells from u on plus one,
+    // added left to right as in the definition, so one pass serves all windows that start at u.
+#pragma unroll 1
+    for (int base = 0; base < span; base += kSelThreads) {
+      const int i = base + threadIdx.x;
+      float acc = 0.f;
+      int j = 0;
+#pragma unroll 1
+      for (int k = 0; k < n_win; ++k) {
+        const int combo = tbl.grp_combo[first + k], n = tbl.n[combo];
+        if (i + n <= span) {
+#pragma unroll 4
+          for (int jj = j; jj < n; ++jj) acc += buf0[i + jj];
+        }
+        j = n;
+        const int c = i - (n_max / 2 - n / 2);             // cell of the window that starts here
+        int bin = -1;
+        if (c >= 0 && c < n_out) {
+          const float avg = acc / static_cast<float>(n);
+          p.pooled[static_cast<long long>(combo) * p.pooled_stride + c0 + c] = avg;
+          bin = bin_of_ordered(float_to_ordered(avg));
+        }
+        count_bins((k == 0) ? hist0 : hist1 + (k - 1) * kHistBins, bin);
+      }
+    }
+    __syncthreads();
   }
-  __syncthreads();
 }
 
 // Phase C for one combination: the bin of its K_m-th largest value, and for every bin the number of
@@ -300,7 +349,8 @@ __device__ __forceinline__ void find_threshold(const SelectParams& p, const Comb
 }
 
 // Phase D for the tiles [tile0, tile1) of one combination: the cells of its threshold bin and of the bins
-// above, sorted by bin.  Four consecutive cells per thread and tile; most warps find none.
+// above, sorted by bin.  Four consecutive cells per thread and tile; few of them are candidates, which
+// are read once more.
 __device__ __forceinline__ void gather_combination(const SelectParams& p, const ComboTable& tbl, int combo, int tile0,
                                                    int tile1, const SelShared* sh) {
   const float* w = p.pooled + static_cast<long long>(combo) * p.pooled_stride;
@@ -308,37 +358,34 @@ __device__ __forceinline__ void gather_combination(const SelectParams& p, const 
   uint32_t* seg = p.cand_seg + static_cast<long long>(combo) * p.cand_stride;
   uint32_t* slots = p.hist + static_cast<long long>(tbl.n_comb + combo) * kHistBins;
   const int len = tbl.len[combo], threshold = sh->threshold;
-  const uint32_t lowest = (threshold == 0) ? 0u : static_cast<uint32_t>(threshold + kFirstBin) << kBinShift;
+  const float lowest = (threshold == 0) ? -INFINITY
+                                        : ordered_to_float(static_cast<uint32_t>(threshold + kFirstBin) << kBinShift);
   for (int tile = tile0; tile < tile1; tile += kGatherGroup) {
+    const int cell0 = (tile - tbl.tile_begin[combo]) * kSelTile + 4 * static_cast<int>(threadIdx.x);
+    const int end = min(len, (tile1 - tbl.tile_begin[combo]) * kSelTile);
     float4 v[kGatherGroup];
-    int c[kGatherGroup];
 #pragma unroll
     for (int g = 0; g < kGatherGroup; ++g) {
-      c[g] = (tile + g < tile1) ? (tile + g - tbl.tile_begin[combo]) * kSelTile + 4 * static_cast<int>(threadIdx.x) : len;
-      if (c[g] < len) v[g] = __ldcg(reinterpret_cast<const float4*>(w + c[g]));
+      v[g] = make_float4(NAN, NAN, NAN, NAN);
+      if (cell0 + g * kSelTile < end) v[g] = __ldcg(reinterpret_cast<const float4*>(w + cell0 + g * kSelTile));
     }
-#pragma unroll 1
-    for (int g = 0; g < kGatherGroup; ++g) {
-      uint32_t o[4];
-      float4 x = v[0];
-      int cell = c[0];
+    uint32_t found = 0;
 #pragma unroll
-      for (int i = 1; i < kGatherGroup; ++i)
-        if (g == i) { x = v[i]; cell = c[i]; }
-      o[0] = float_to_ordered(x.x); o[1] = float_to_ordered(x.y);
-      o[2] = float_to_ordered(x.z); o[3] = float_to_ordered(x.w);
-#pragma unroll 1
-      for (int i = 0; i < 4; ++i) {
-        const uint32_t mine = (i == 0) ? o[0] : (i == 1) ? o[1] : (i == 2) ? o[2] : o[3];
-        if (cell + i < len && mine >= lowest) {
-          const int bin = bin_of_ordered(mine);
-          const uint32_t start = sh->above[bin + 1], count = sh->above[bin] - start;
-          const uint32_t at = start + atomicAdd(&slots[bin], 1u);
-          if (at < static_cast<uint32_t>(p.cand_stride)) {
-            cand[at] = (static_cast<unsigned long long>(mine) << 32) | (0xFFFFFFFFu - static_cast<uint32_t>(cell + i));
-            seg[at] = start | (count << 16);
-          }
-        }
+    for (int g = 0; g < kGatherGroup; ++g)
+      found |= ((v[g].x >= lowest ? 1u : 0u) | (v[g].y >= lowest ? 2u : 0u) | (v[g].z >= lowest ? 4u : 0u) |
+                (v[g].w >= lowest ? 8u : 0u)) << (4 * g);
+    while (found) {
+      const int e = __ffs(found) - 1;
+      found &= found - 1;
+      const int cell = cell0 + (e >> 2) * kSelTile + (e & 3);
+      if (cell >= len) continue;
+      const uint32_t o = float_to_ordered(__ldcg(w + cell));
+      const int bin = bin_of_ordered(o);
+      const uint32_t start = sh->above[bin + 1], count = sh->above[bin] - start;
+      const uint32_t at = start + atomicAdd(&slots[bin], 1u);
+      if (at < static_cast<uint32_t>(p.cand_stride)) {
+        cand[at] = (static_cast<unsigned long long>(o) << 32) | (0xFFFFFFFFu - static_cast<uint32_t>(cell));
+        seg[at] = start | (count << 16);
       }
     }
   }
@@ -787,45 +834,39 @@ select_kernel(const ComboTable tbl, const SelectParams p) {
   uint32_t epoch = 0;
   grid_dep_wait();       // the kernel before this one (scores, state cleared for this run) is done
 
-  // ---- A: scores from the encoded maxima, one exp per position ----
-  if (!p.scores_given) {
-    const long long stride = static_cast<long long>(gridDim.x) * kSelThreads;
-    for (long long t = static_cast<long long>(blockIdx.x) * kSelThreads + threadIdx.x; t < p.L;
-         t += stride) {
-      const float a = exp2f(ordered_to_float(__ldcg(&p.enc[t])));
-      p.scores[t] = a;
-      if (p.user_scores) p.user_scores[t] = a;
-    }
-  }
-  if (!grid_sync<kCluster>(p, &sh, epoch)) return;
-
-  // ---- B1: strided max-pool arrays, one per distinct m > 1 ----
+  // ---- A: strided max-pool arrays, one per distinct m > 1 ----
   if (tbl.n_src > 0) {
-    float* buf = reinterpret_cast<float*>(dyn_smem);
     const int n_st = tbl.src_tile_begin[tbl.n_src];
     const int s_begin = static_cast<int>(static_cast<long long>(blockIdx.x) * n_st / gridDim.x);
     const int s_end = static_cast<int>(static_cast<long long>(blockIdx.x + 1) * n_st / gridDim.x);
     int src = 0;
     for (int tile = s_begin; tile < s_end; ++tile) {
       while (src + 1 < tbl.n_src && tile >= tbl.src_tile_begin[src + 1]) ++src;
-      maxpool_tile(tbl, p, src, tile - tbl.src_tile_begin[src], buf);
+      maxpool_tile(tbl, p, src, tile - tbl.src_tile_begin[src], reinterpret_cast<uint32_t*>(dyn_smem));
     }
     if (!grid_sync<kCluster>(p, &sh, epoch)) return;
   }
 
-  // ---- B2: window pooling of every combination + first histogram ----
+  // ---- B: window pooling of every combination + histograms ----
   {
-    float* buf0 = reinterpret_cast<float*>(dyn_smem);
-    float* buf1 = buf0 + (kSelTile + kMaxWin);
-    int cur = -1, cursor = 0;
-    for (int tile = t_begin; tile < t_end; ++tile) {
-      const int combo = combo_of_tile(tbl, tile, cursor);
-      if (combo != cur && cur >= 0)
-        hist_flush(sh.hist, p.hist + static_cast<long long>(cur) * kHistBins);
-      cur = combo;
-      pool_tile(tbl, p, combo, (tile - tbl.tile_begin[combo]) * kSelTile, buf0, buf1, sh.hist);
+    uint32_t* hist1 = reinterpret_cast<uint32_t*>(dyn_smem);          // of the group's combinations after the first
+    float* buf0 = reinterpret_cast<float*>(hist1 + (kPoolGroup - 1) * kHistBins);
+    float* buf1 = buf0 + (kPoolTileMax + kMaxWin);
+    for (int i = threadIdx.x; i < (kPoolGroup - 1) * kHistBins; i += kSelThreads) hist1[i] = 0u;
+    __syncthreads();
+    const int n_pt = tbl.grp_tile_begin[tbl.n_grp], per = tbl.pool_tile;
+    const int p_begin = static_cast<int>(static_cast<long long>(blockIdx.x) * n_pt / gridDim.x);
+    const int p_end = static_cast<int>(static_cast<long long>(blockIdx.x + 1) * n_pt / gridDim.x);
+    int grp = 0;
+    for (int tile = p_begin; tile < p_end; ++tile) {
+      while (grp + 1 < tbl.n_grp && tile >= tbl.grp_tile_begin[grp + 1]) ++grp;
+      const int c0 = (tile - tbl.grp_tile_begin[grp]) * per, first = tbl.grp_first[grp];
+      pool_tile(tbl, p, grp, c0, min(per, tbl.len[tbl.grp_combo[first]] - c0), buf0, buf1, sh.hist, hist1);
+      if (tile + 1 == p_end || tile + 1 == tbl.grp_tile_begin[grp + 1])        // the CTA's last tile of this group
+        for (int k = 0; first + k < tbl.grp_first[grp + 1]; ++k)
+          hist_flush((k == 0) ? sh.hist : hist1 + (k - 1) * kHistBins,
+                     p.hist + static_cast<long long>(tbl.grp_combo[first + k]) * kHistBins);
     }
-    if (cur >= 0) hist_flush(sh.hist, p.hist + static_cast<long long>(cur) * kHistBins);
   }
   if (!grid_sync<kCluster>(p, &sh, epoch)) return;
 
@@ -1036,7 +1077,12 @@ select_kernel(const ComboTable tbl, const SelectParams p) {
   }
   if (!grid_sync<kCluster>(p, &sh, epoch)) return;
 
-  // ---- F: allocation and ascending output (one CTA) ----
+  // ---- F: allocation and ascending output (one CTA); the others write the scores if asked ----
+  if (p.user_scores && (blockIdx.x != 0 || gridDim.x == 1)) {
+    const long long writers = gridDim.x == 1 ? 1 : gridDim.x - 1, mine = gridDim.x == 1 ? 0 : blockIdx.x - 1;
+    for (long long t = mine * kSelThreads + threadIdx.x; t < p.L; t += writers * kSelThreads)
+      p.user_scores[t] = score_at(p, t);
+  }
   if (blockIdx.x != 0) return;
   if (p.bitmap_in_smem) {
     allocate<true>(tbl, p, dyn_smem, &sh);
@@ -1105,9 +1151,42 @@ static void assign_ranking(ComboTable* t, int grid) {
   t->rank_cta_begin[t->n_comb] = b0;
 }
 
+// Groups the combinations for the pooling phase and cuts the groups into tiles: equal shares of the
+// grid's CTAs, rounded up to whole warps.
+static void assign_pooling(ComboTable* t, int grid) {
+  t->n_grp = 0;
+  int n = 0;
+  long long cells = 0;
+  for (int src = -1; src < t->n_src; ++src) {
+    int list[kMaxCombos], cnt = 0;
+    for (int c = 0; c < t->n_comb; ++c)
+      if (t->src[c] == src) list[cnt++] = c;
+    for (int i = 1; i < cnt; ++i)                           // by window size
+      for (int j = i; j > 0 && t->n[list[j]] < t->n[list[j - 1]]; --j) {
+        const int x = list[j]; list[j] = list[j - 1]; list[j - 1] = x;
+      }
+    const int n_groups = (cnt + kPoolGroup - 1) / kPoolGroup;
+    for (int g = 0; g < n_groups; ++g) {                    // groups of even size
+      t->grp_first[t->n_grp++] = n;
+      for (int i = g * cnt / n_groups; i < (g + 1) * cnt / n_groups; ++i) t->grp_combo[n++] = list[i];
+      cells += t->len[list[0]];
+    }
+  }
+  t->grp_first[t->n_grp] = n;
+  const long long rounds = (cells + static_cast<long long>(grid) * kPoolTileMax - 1) / (static_cast<long long>(grid) * kPoolTileMax);
+  const long long workers = static_cast<long long>(grid) * (rounds < 1 ? 1 : rounds);
+  long long tile = ((cells + workers - 1) / workers + 31) & ~31ll;
+  t->pool_tile = static_cast<int>(tile < 256 ? 256 : (tile > kPoolTileMax ? kPoolTileMax : tile));
+  t->grp_tile_begin[0] = 0;
+  for (int g = 0; g < t->n_grp; ++g)
+    t->grp_tile_begin[g + 1] = t->grp_tile_begin[g] +
+        (t->len[t->grp_combo[t->grp_first[g]]] + t->pool_tile - 1) / t->pool_tile;
+}
+
 cudaError_t launch_select(const ComboTable& table, const SelectParams& p, int grid, size_t smem,
                           cudaStream_t st) {
   ComboTable tbl = table;
+  assign_pooling(&tbl, grid);
   assign_ranking(&tbl, grid);
   // Short contexts need few CTAs: up to kSelClusterMax of them run as one thread-block cluster,
   // whose hardware barrier costs a fraction of a trip to the L2 (not with the self test's

@@ -13,7 +13,9 @@ static constexpr int kMaxMaxSize = 64;      // largest strided max-pool size
 static constexpr int kMaxKm = 16384;        // largest K_m (bounds the candidate lists)
 static constexpr int kSelectPasses = 3;     // long way: 32 value bits of the key in 11/11/10-bit digits
 static constexpr int kSelThreads = 1024;    // threads per CTA of the selection kernel
-static constexpr int kSelTile = 4096;       // cells of one combination per work tile
+static constexpr int kSelTile = 4096;       // cells of one combination per work tile of the gather
+static constexpr int kPoolGroup = 5;        // window sizes of one strided max-pool that are pooled together
+static constexpr int kPoolTileMax = 3072;   // cells of a group of windows per work tile, at most
 static constexpr int kSrcTileTokens = 8192; // tokens per work tile of the strided max-pool
 static constexpr int kSelClusterMax = 8;     // grids up to this size run as one thread-block cluster
 static constexpr int kCandSlack = 4096;      // candidates past K_m that the threshold bin may bring
@@ -21,7 +23,7 @@ static constexpr int kSelBitmapSmemBytes = 136 * 1024;   // bitmap kept in share
 // Work area in front of the bitmap: pooling tiles, the keys of a ranking list, the staged cells of the
 // quota walk and the list of the output pass, one after another.
 static constexpr int kSelWorkBytes = 64 * 1024;
-static_assert(kSelWorkBytes >= 2 * (kSelTile + kMaxWin) * 4 && kSelWorkBytes >= kSrcTileTokens * 4 &&
+static_assert(kSelWorkBytes >= (kPoolGroup - 1) * kHistBins * 4 + 2 * (kPoolTileMax + kMaxWin) * 4 && kSelWorkBytes >= kSrcTileTokens * 4 &&
               kSelWorkBytes >= kMaxKm * 4, "work area too small");
 static constexpr int kSelMaxDynSmemBytes = kSelWorkBytes + kSelBitmapSmemBytes + kSelBitmapSmemBytes / 32 + 64;
 
@@ -41,6 +43,12 @@ struct ComboTable {
   int src_m[kMaxCombos];
   int src_len[kMaxCombos];
   int src_tile_begin[kMaxCombos + 1];   // tiles of kSrcTileTokens / m cells each
+  // Groups of combinations of one source (up to kPoolGroup, ascending window sizes) that are pooled
+  // together, and their work tiles of pool_tile cells (filled in by launch_select).
+  int n_grp, pool_tile;
+  int grp_first[kMaxCombos + 1];        // first entry of each group in grp_combo
+  int grp_combo[kMaxCombos];
+  int grp_tile_begin[kMaxCombos + 1];
   // Ranking phase (filled in by launch_select): with rank_by_list, combination c is ranked by
   // the CTAs [rank_cta_begin[c], rank_cta_begin[c + 1]).
   int rank_by_list;
@@ -49,9 +57,9 @@ struct ComboTable {
 
 struct SelectParams {
   const uint32_t* enc;     // [L] order-preserving uint of max_r log2 p_rt (scores pass output)
-  float* scores;           // A^C [L]
-  float* user_scores;      // optional copy of A^C for the caller, or null
-  int scores_given;        // 1: `scores` already holds A^C (phase A is skipped)
+  const float* scores;     // A^C [L], with scores_given
+  float* user_scores;      // A^C [L] for the caller, or null
+  int scores_given;        // 1: `scores` holds A^C (else it comes from `enc`)
   long long L;
   int n_sink;
   int win_op;              // 0 average, 1 max

@@ -171,6 +171,27 @@ def test_selection_kernel_edge_paths(case):
     eng.close()
 
 
+# Groups of windows that are pooled together: unsorted sizes, more windows of one max size than a group
+# holds, sizes up to the largest, contexts shorter than a window or a tile, one cell more than a whole
+# number of tiles.  (L, budget, max_sizes, win_sizes, win_op, n_sink)
+GROUPS = [(5000, 300, (1,), (63, 1, 200, 7, 31, 15), 1, 0), (3073, 200, (3, 1, 2), (16, 5, 1, 9, 2, 1024), 0, 4),
+          (260, 20, (4, 1), (1024, 3, 2, 600, 1, 5, 9), 1, 3), (40, 9, (1, 64), (7, 100, 1), 0, 0),
+          (33025, 700, (1, 2), (31, 4, 8, 16, 2, 64, 1, 128, 256, 512, 1024), 1, 1),
+          (150000, 4096, (1,), (5, 4, 3, 2, 1, 6, 7), 0, 0)]
+
+
+@pytest.mark.parametrize("case", GROUPS, ids=lambda c: f"L{c[0]}_m{len(c[2])}_n{len(c[3])}_op{c[4]}")
+def test_window_groups_match_oracle(case):
+    L, budget, max_sizes, win_sizes, win_op, n_sink = case
+    x = make_inputs(small_workload(L, 2, seed=L, budget=budget, max_sizes=max_sizes, win_sizes=win_sizes,
+                                   win_op=win_op, n_sink=n_sink, n_spans=2 if L > 100 else 0))
+    eng = _engine(x.workload)
+    idx, sc = _run(eng, x)
+    parity.check_recall(x.K, x.Q, x.workload, idx, sc)
+    assert eng.check_guards() == 0, "a kernel wrote past the end of a workspace buffer"
+    eng.close()
+
+
 @pytest.mark.parametrize("pattern", ["all_equal", "two_levels", "blocks_of_equal", "all_equal_40k",
                                      "blocks_of_equal_40k", "all_equal_40k_B6000",
                                      "blocks_of_equal_40k_B6000"])
