@@ -790,7 +790,7 @@ scores_pair_kernel(const __grid_constant__ CUtensorMap tmapK,
 // ---------------------------------------------------------------------------------------
 
 // Packs the query rows of every kv head contiguously, zero-padded to kv_rows,
-// and clears the per-run state (encoded scores, bitmap with the sink bits set, selection
+// and clears the per-run state (encoded scores, empty bitmap, selection
 // state).
 __global__ void prepare_kernel(const uint4* __restrict__ q, uint4* __restrict__ qp, PrepParams p) {
   grid_dep_launch();                     // the statistics kernel sets itself up meanwhile
@@ -812,9 +812,8 @@ __global__ void prepare_kernel(const uint4* __restrict__ q, uint4* __restrict__ 
   for (long long t = tid; t < p.L; t += nthreads) p.enc[t] = 0u;
   const long long n_words = (p.L + 31) / 32;
   for (long long w = tid; w < n_words; w += nthreads) {
-    const long long lo = w * 32;
-    uint32_t bits = 0;
-    if (p.n_sink > lo) bits = (p.n_sink - lo >= 32) ? 0xFFFFFFFFu : ((1u << (p.n_sink - lo)) - 1u);
+    const long long left = p.L - p.n_sink - w * 32;       // bits past the end never look free
+    const uint32_t bits = (left >= 32) ? 0u : (left <= 0) ? 0xFFFFFFFFu : 0xFFFFFFFFu << left;
     p.bitmap[w] = bits;
   }
   for (long long e = tid; e < p.hist_words; e += nthreads) p.hist[e] = 0u;

@@ -55,6 +55,7 @@ struct SelShared {
   int flag;
   int threshold;                           // the bin of its K_m-th largest value
   int plateau;                             // it brings too many cells: full-scan passes
+  uint32_t n_listed;                       // candidates of this CTA listed in shared memory
   unsigned long long prefix[kMaxCombos];   // full-scan passes, per combination: radix prefix found so far,
   uint32_t state[kMaxCombos];              // whether the K_m-th value is settled,
   uint32_t krem[kMaxCombos];               // and the keys still wanted inside the prefix
@@ -330,6 +331,7 @@ __device__ __forceinline__ void find_threshold(const SelectParams& p, const Comb
   const uint2 h = __ldcg(reinterpret_cast<const uint2*>(gh + hi - 1));      // (lower, higher) bin
   uint32_t grand;
   const uint32_t excl = block_exclusive_scan(h.x + h.y, sh->scan, &grand);   // begins with a barrier
+  if (threadIdx.x == 0) sh->n_listed = 0u;
   sh->above[hi + 1] = excl;
   sh->above[hi] = excl + h.y;
   if (threadIdx.x == 0) sh->above[0] = grand;
@@ -349,10 +351,11 @@ __device__ __forceinline__ void find_threshold(const SelectParams& p, const Comb
 }
 
 // Phase D for the tiles [tile0, tile1) of one combination: the cells of its threshold bin and of the bins
-// above, sorted by bin.  Four consecutive cells per thread and tile; few of them are candidates, which
-// are read once more.
+// above, sorted by bin.  Four consecutive cells per thread and tile; few of them are candidates, and
+// those come in runs, so they are listed in shared memory first and then placed a cell per thread
+// (one after another in the thread that found them, each waited for its counter: up to 3 us).
 __device__ __forceinline__ void gather_combination(const SelectParams& p, const ComboTable& tbl, int combo, int tile0,
-                                                   int tile1, const SelShared* sh) {
+                                                   int tile1, SelShared* sh, int* list) {
   const float* w = p.pooled + static_cast<long long>(combo) * p.pooled_stride;
   unsigned long long* cand = p.cand + static_cast<long long>(combo) * p.cand_stride;
   uint32_t* seg = p.cand_seg + static_cast<long long>(combo) * p.cand_stride;
@@ -360,6 +363,16 @@ __device__ __forceinline__ void gather_combination(const SelectParams& p, const 
   const int len = tbl.len[combo], threshold = sh->threshold;
   const float lowest = (threshold == 0) ? -INFINITY
                                         : ordered_to_float(static_cast<uint32_t>(threshold + kFirstBin) << kBinShift);
+  auto place = [&](int cell) {
+    const uint32_t o = float_to_ordered(__ldcg(w + cell));
+    const int bin = bin_of_ordered(o);
+    const uint32_t start = sh->above[bin + 1], count = sh->above[bin] - start;
+    const uint32_t at = start + atomicAdd(&slots[bin], 1u);
+    if (at < static_cast<uint32_t>(p.cand_stride)) {
+      cand[at] = (static_cast<unsigned long long>(o) << 32) | (0xFFFFFFFFu - static_cast<uint32_t>(cell));
+      seg[at] = start | (count << 16);
+    }
+  };
   for (int tile = tile0; tile < tile1; tile += kGatherGroup) {
     const int cell0 = (tile - tbl.tile_begin[combo]) * kSelTile + 4 * static_cast<int>(threadIdx.x);
     const int end = min(len, (tile1 - tbl.tile_begin[combo]) * kSelTile);
@@ -374,21 +387,20 @@ __device__ __forceinline__ void gather_combination(const SelectParams& p, const 
     for (int g = 0; g < kGatherGroup; ++g)
       found |= ((v[g].x >= lowest ? 1u : 0u) | (v[g].y >= lowest ? 2u : 0u) | (v[g].z >= lowest ? 4u : 0u) |
                 (v[g].w >= lowest ? 8u : 0u)) << (4 * g);
+    if (!found) continue;
+    int at = static_cast<int>(atomicAdd(&sh->n_listed, static_cast<uint32_t>(__popc(found))));
     while (found) {
       const int e = __ffs(found) - 1;
       found &= found - 1;
       const int cell = cell0 + (e >> 2) * kSelTile + (e & 3);
-      if (cell >= len) continue;
-      const uint32_t o = float_to_ordered(__ldcg(w + cell));
-      const int bin = bin_of_ordered(o);
-      const uint32_t start = sh->above[bin + 1], count = sh->above[bin] - start;
-      const uint32_t at = start + atomicAdd(&slots[bin], 1u);
-      if (at < static_cast<uint32_t>(p.cand_stride)) {
-        cand[at] = (static_cast<unsigned long long>(o) << 32) | (0xFFFFFFFFu - static_cast<uint32_t>(cell));
-        seg[at] = start | (count << 16);
-      }
+      if (at < kSelWorkBytes / 4) list[at++] = (cell < len) ? cell : -1;
+      else if (cell < len) place(cell);                      // more than the list holds
     }
   }
+  __syncthreads();
+  const int n = static_cast<int>(min(sh->n_listed, static_cast<uint32_t>(kSelWorkBytes / 4)));
+  for (int i = threadIdx.x; i < n; i += kSelThreads)
+    if (list[i] >= 0) place(list[i]);
 }
 
 // One pass of the long way: locates the digit of pass `pass` that holds the k-th largest key of `combo`
@@ -505,33 +517,46 @@ __device__ __forceinline__ void bitmap_set(uint32_t* bm, int w, uint32_t bits) {
   }
 }
 
-// Tokens of cell `cell` (size m) that are not allocated yet, as a bit mask (bit j = token j).
-// Positions fit 32 bits (L < 2^31).  m <= 32: at most 32 consecutive bits, two bitmap words and one
-// funnel shift; kWide, m <= 64: at most three words.  A word past the bitmap's end may be read (there is
-// memory behind it) but its bits are masked.
-template <bool kWide, bool kSmem>
-__device__ __forceinline__ auto fresh_tokens(const uint32_t* bm, int cell, int m, int Lp, int n_sink) {
+// The bitmap of allocated tokens covers the context without its sink part: bit t = token t, t < Lp; the
+// bits past the end are set from the start, so that they never look free.
+__device__ __forceinline__ uint32_t empty_bitmap_word(int w, int Lp) {
+  const int left = Lp - 32 * w;
+  return (left >= 32) ? 0u : (left <= 0) ? 0xFFFFFFFFu : 0xFFFFFFFFu << left;
+}
+
+// How the cells of a combination lie in the bitmap words.
+enum : int {
+  kCellsAligned = 0,      // m divides 32: inside one word
+  kCellsShort = 1,        // m <= 32: in at most two words (one funnel shift)
+  kCellsLong = 2          // m <= 64: in at most three words
+};
+
+// Tokens of cell `cell` (size m) that are not allocated yet, as a bit mask (bit j = token j).  Positions
+// fit 32 bits (L < 2^31).  Words past the bitmap's end may be read (there is memory behind it) but
+// their bits are masked.
+template <int kCells, bool kSmem>
+__device__ __forceinline__ auto fresh_tokens(const uint32_t* bm, int cell, int m, int Lp) {
   const int t0 = cell * m;
-  const int cnt = min(m, Lp - t0);
-  const int pos0 = n_sink + t0;
-  const int w0 = pos0 >> 5, sh = pos0 & 31;
-  if constexpr (!kWide) {
+  const int w0 = t0 >> 5, sh = t0 & 31;
+  if constexpr (kCells == kCellsAligned) {
+    return (~bitmap_word<kSmem>(bm, w0) >> sh) & (0xFFFFFFFFu >> (32 - m));
+  } else if constexpr (kCells == kCellsShort) {
     const uint32_t taken = __funnelshift_r(bitmap_word<kSmem>(bm, w0), bitmap_word<kSmem>(bm, w0 + 1), sh);
-    return ~taken & (0xFFFFFFFFu >> (32 - cnt));
+    return ~taken & (0xFFFFFFFFu >> (32 - min(m, Lp - t0)));
   } else {
     unsigned long long taken = bitmap_word<kSmem>(bm, w0);
     taken |= static_cast<unsigned long long>(bitmap_word<kSmem>(bm, w0 + 1)) << 32;
     taken >>= sh;
     if (sh) taken |= static_cast<unsigned long long>(bitmap_word<kSmem>(bm, w0 + 2)) << (64 - sh);
-    return ~taken & (~0ull >> (64 - cnt));
+    return ~taken & (~0ull >> (64 - min(m, Lp - t0)));
   }
 }
 
-// Marks the fresh tokens `f` of a cell that starts at position pos0, and in the summary (one bit per
-// bitmap word; null: none) the words that were touched.
-template <bool kWide, bool kSmem, class Mask>
-__device__ __forceinline__ void mark_tokens(uint32_t* bm, uint32_t* summary, int pos0, Mask f) {
-  const int w0 = pos0 >> 5, sft = pos0 & 31;
+// Marks the fresh tokens `f` of a cell that starts at token t0, and in the summary (one bit per bitmap
+// word; null: none) the words that were touched.
+template <int kCells, bool kSmem, class Mask>
+__device__ __forceinline__ void mark_tokens(uint32_t* bm, uint32_t* summary, int t0, Mask f) {
+  const int w0 = t0 >> 5, sft = t0 & 31;
   auto set = [&](int w, uint32_t bits) {
     if (!bits) return;
     bitmap_set<kSmem>(bm, w, bits);
@@ -539,7 +564,9 @@ __device__ __forceinline__ void mark_tokens(uint32_t* bm, uint32_t* summary, int
       if (summary) bitmap_set<true>(summary, w >> 5, 1u << (w & 31));
     }
   };
-  if constexpr (!kWide) {
+  if constexpr (kCells == kCellsAligned) {
+    set(w0, f << sft);
+  } else if constexpr (kCells == kCellsShort) {
     set(w0, f << sft);
     set(w0 + 1, __funnelshift_l(f, 0u, sft));
   } else {
@@ -556,20 +583,20 @@ __device__ __forceinline__ void mark_tokens(uint32_t* bm, uint32_t* summary, int
 // per walking warp, of this combination only.  The barrier separates counting from marking.  The
 // loops are not unrolled: the kernel meets every instruction cold, and the fetch of unrolled code
 // costs more than the loops do.
-template <bool kWide, bool kSmem, class Barrier>
+template <int kCells, bool kSmem, class Barrier>
 __device__ __forceinline__ void walk_combination(const SelectParams& p, const int* cells, int K, int m, uint32_t quota,
                                                  uint32_t* bm, uint32_t* summary, uint32_t* totals, int n_walk,
                                                  Barrier walk_barrier) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int Lp = static_cast<int>(p.L - p.n_sink), n_sink = p.n_sink;
+  const int Lp = static_cast<int>(p.L - p.n_sink);
   auto count = [](auto f) -> uint32_t {
-    if constexpr (kWide) return __popcll(f); else return __popc(f);
+    if constexpr (kCells == kCellsLong) return __popcll(f); else return __popc(f);
   };
   const int per = (K + n_walk - 1) / n_walk;
   const int r0 = min(K, static_cast<int>(threadIdx.x) * per), r1 = min(K, r0 + per);
   uint32_t mine = 0;
 #pragma unroll 1
-  for (int r = r0; r < r1; ++r) mine += count(fresh_tokens<kWide, kSmem>(bm, cells[r], m, Lp, n_sink));
+  for (int r = r0; r < r1; ++r) mine += count(fresh_tokens<kCells, kSmem>(bm, cells[r], m, Lp));
   const uint32_t warp_sum = __reduce_add_sync(0xFFFFFFFFu, mine);
   if (lane == 0) totals[warp] = warp_sum;
   walk_barrier();
@@ -592,7 +619,7 @@ __device__ __forceinline__ void walk_combination(const SelectParams& p, const in
 #pragma unroll 1
   for (int r = r0; r < r1 && room > 0; ++r) {
     const int c = cells[r];
-    auto f = fresh_tokens<kWide, kSmem>(bm, c, m, Lp, n_sink);
+    auto f = fresh_tokens<kCells, kSmem>(bm, c, m, Lp);
     const uint32_t n_new = count(f);
     if (n_new == 0) continue;
     if (n_new > room) {                                        // the quota ends inside this cell
@@ -601,7 +628,7 @@ __device__ __forceinline__ void walk_combination(const SelectParams& p, const in
       f ^= rest;
     }
     room = (n_new > room) ? 0u : room - n_new;
-    mark_tokens<kWide, kSmem>(bm, summary, n_sink + c * m, f);
+    mark_tokens<kCells, kSmem>(bm, summary, c * m, f);
   }
 }
 
@@ -642,7 +669,7 @@ __device__ __forceinline__ void allocate(const ComboTable& tbl, const SelectPara
   // path (shared memory) instead of going through generic loads and atomics.
   uint32_t* bm = kBitmapInSmem ? smem_bitmap(dyn_smem) : p.bitmap;
   // (the output pass takes a thread per bitmap word, without the summary, up to kSelThreads words)
-  uint32_t* summary = (kBitmapInSmem && (p.L + 31) / 32 > kSelThreads) ? smem_summary(dyn_smem, p.L) : nullptr;
+  uint32_t* summary = (kBitmapInSmem && (p.L - p.n_sink + 31) / 32 > kSelThreads) ? smem_summary(dyn_smem, p.L) : nullptr;
   int* staged = reinterpret_cast<int*>(dyn_smem);
   __shared__ uint32_t warp_totals[2][kMaxWalkWarps];
   const int n_walk = p.walk_threads;                       // multiple of 32, <= kSelThreads
@@ -683,10 +710,12 @@ __device__ __forceinline__ void allocate(const ComboTable& tbl, const SelectPara
       // the other buffer last served combination combo - 1, which every thread has left
       if (two && combo + 1 < n_comb) issue_copy(combo + 1);
       uint32_t* totals = warp_totals[combo & 1];
-      if (m <= 32)
-        walk_combination<false, kBitmapInSmem>(p, cells, K, m, quota, bm, summary, totals, n_walk, walk_barrier);
+      if (32 % m == 0)
+        walk_combination<kCellsAligned, kBitmapInSmem>(p, cells, K, m, quota, bm, summary, totals, n_walk, walk_barrier);
+      else if (m <= 32)
+        walk_combination<kCellsShort, kBitmapInSmem>(p, cells, K, m, quota, bm, summary, totals, n_walk, walk_barrier);
       else
-        walk_combination<true, kBitmapInSmem>(p, cells, K, m, quota, bm, summary, totals, n_walk, walk_barrier);
+        walk_combination<kCellsLong, kBitmapInSmem>(p, cells, K, m, quota, bm, summary, totals, n_walk, walk_barrier);
       if (!two) {                                              // one buffer: copy only once it is free
         walk_barrier();
         if (combo + 1 < n_comb) issue_copy(combo + 1);
@@ -698,39 +727,34 @@ __device__ __forceinline__ void allocate(const ComboTable& tbl, const SelectPara
   __syncthreads();
 
   // Ascending output.  One SM does this, so what counts is the number of instructions it has
-  // to issue.  Up to kSelThreads bitmap words (32K positions) a thread takes one word.  Longer
-  // contexts: the sink part is the identity; for the rest the words that hold an allocated position
+  // to issue.  The sink part is the identity.  Up to kSelThreads bitmap words (32K positions) a thread
+  // takes one word.  Longer contexts: the words that hold an allocated position
   // (at most `budget`, usually a few hundred) are listed in ascending order in shared memory (where
   // the staged cells were; they are done with): from the summary, 32 words per summary word, or,
   // with the bitmap in global memory, from the bitmap, four words per lane and load, read twice.
   // The threads share the list out evenly, take the prefix of the words' position counts and
   // write the positions.
-  const long long n_words = (p.L + 31) / 32;
+  const int Lp = static_cast<int>(p.L - p.n_sink);
+  const long long n_words = (Lp + 31ll) / 32;
   const uint32_t cap = static_cast<uint32_t>(p.n_sink + p.budget);
+  for (int j = threadIdx.x; j < p.n_sink; j += kSelThreads) p.out_idx[j] = j;
   if (n_words <= kSelThreads) {
-    // short context: a thread per bitmap word (sink bits included), one prefix sum
-    uint32_t bits = (static_cast<long long>(threadIdx.x) < n_words)
-                        ? bitmap_word<kBitmapInSmem>(bm, static_cast<int>(threadIdx.x)) : 0u;
+    // short context: a thread per bitmap word, one prefix sum
+    const int w = static_cast<int>(threadIdx.x);
+    uint32_t bits = (w < n_words) ? bitmap_word<kBitmapInSmem>(bm, w) & ~empty_bitmap_word(w, Lp) : 0u;
     uint32_t total;
-    uint32_t at = block_exclusive_scan(__popc(bits), sh->scan, &total);
+    uint32_t at = p.n_sink + block_exclusive_scan(__popc(bits), sh->scan, &total);
     while (bits) {
       const int b = __ffs(bits) - 1;
       bits &= bits - 1;
-      if (at < cap) p.out_idx[at] = static_cast<int>(threadIdx.x) * 32 + b;
+      if (at < cap) p.out_idx[at] = p.n_sink + w * 32 + b;
       ++at;
     }
-    if (threadIdx.x == 0 && total != cap) atomicCAS(p.status, 0, kDevQuota);
+    if (threadIdx.x == 0 && total != static_cast<uint32_t>(p.budget)) atomicCAS(p.status, 0, kDevQuota);
     return;
   }
   const int n_w = static_cast<int>(n_words);                // L < 2^31: word and quad numbers fit an int
   int* list = staged;
-  // bits of word w that stand for allocated positions outside the sink part
-  const int sink_words = p.n_sink >> 5;                     // words that lie in the sink part entirely
-  const uint32_t sink_tail = ~((1u << (p.n_sink & 31)) - 1u);         // the word after them: its bits outside
-  auto outside_sink = [&](uint32_t bits, int w) -> uint32_t {
-    return (w > sink_words) ? bits : ((w < sink_words) ? 0u : (bits & sink_tail));
-  };
-  for (int j = threadIdx.x; j < p.n_sink; j += kSelThreads) p.out_idx[j] = j;
   uint32_t n_entries;
   if constexpr (kBitmapInSmem) {
     const int n_sum = (n_w + 31) / 32, per = (n_sum + kSelThreads - 1) / kSelThreads;
@@ -752,18 +776,17 @@ __device__ __forceinline__ void allocate(const ComboTable& tbl, const SelectPara
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rounds = (n_quads + kSelThreads - 1) / kSelThreads;      // per warp
     const int q_begin = warp * rounds * 32;
-    const int plain_from = sink_words / 4 + 1, plain_to = n_w / 4;      // quads that need no fixing
+    const int plain_to = Lp / 128;                            // quads that lie inside the context
     auto load_quad = [&](int q) -> uint4 {
       uint4 v = make_uint4(0u, 0u, 0u, 0u);
       if (q >= n_quads) return v;
       v = __ldcg(reinterpret_cast<const uint4*>(bm) + q);
-      if (q >= plain_from && q < plain_to) return v;
-      const int w0 = 4 * q;
-      if (w0 + 1 >= n_w) v.y = 0u;                            // words past the end hold nothing
-      if (w0 + 2 >= n_w) v.z = 0u;
-      if (w0 + 3 >= n_w) v.w = 0u;
-      v.x = outside_sink(v.x, w0); v.y = outside_sink(v.y, w0 + 1);
-      v.z = outside_sink(v.z, w0 + 2); v.w = outside_sink(v.w, w0 + 3);
+      if (q < plain_to) return v;
+      const int w0 = 4 * q;                                   // bits past the end stand for nothing
+      v.x &= ~empty_bitmap_word(w0, Lp);
+      v.y &= ~empty_bitmap_word(w0 + 1, Lp);
+      v.z &= ~empty_bitmap_word(w0 + 2, Lp);
+      v.w &= ~empty_bitmap_word(w0 + 3, Lp);
       return v;
     };
     uint32_t n_mine = 0;
@@ -797,17 +820,17 @@ __device__ __forceinline__ void allocate(const ComboTable& tbl, const SelectPara
   uint32_t mine = 0;
   for (int e = e_begin; e < e_end; ++e) {
     const int w = list[e];
-    mine += __popc(outside_sink(bitmap_word<kBitmapInSmem>(bm, w), w));
+    mine += __popc(bitmap_word<kBitmapInSmem>(bm, w) & ~empty_bitmap_word(w, Lp));
   }
   uint32_t total;
   uint32_t at = static_cast<uint32_t>(p.n_sink) + block_exclusive_scan(mine, sh->scan, &total);
   for (int e = e_begin; e < e_end; ++e) {
     const int w = list[e];
-    uint32_t bits = outside_sink(bitmap_word<kBitmapInSmem>(bm, w), w);
+    uint32_t bits = bitmap_word<kBitmapInSmem>(bm, w) & ~empty_bitmap_word(w, Lp);
     while (bits) {
       const int b = __ffs(bits) - 1;
       bits &= bits - 1;
-      if (at < cap) p.out_idx[at] = w * 32 + b;
+      if (at < cap) p.out_idx[at] = p.n_sink + w * 32 + b;
       ++at;
     }
   }
@@ -823,11 +846,10 @@ select_kernel(const ComboTable tbl, const SelectParams p) {
   const int t_begin = static_cast<int>(static_cast<long long>(blockIdx.x) * n_tiles / gridDim.x);
   const int t_end = static_cast<int>(static_cast<long long>(blockIdx.x + 1) * n_tiles / gridDim.x);
   for (int b = threadIdx.x; b < kHistBins; b += kSelThreads) sh.hist[b] = 0u;
-  if (blockIdx.x == 0 && p.bitmap_in_smem) {               // for phase F: empty but for the sink part
+  if (blockIdx.x == 0 && p.bitmap_in_smem) {               // for phase F: empty
     uint32_t* bm = smem_bitmap(dyn_smem);
-    const int n_words = static_cast<int>((p.L + 31) / 32), sink_words = p.n_sink >> 5;
-    for (int w = threadIdx.x; w < n_words; w += kSelThreads)
-      bm[w] = (w < sink_words) ? 0xFFFFFFFFu : ((w == sink_words) ? (1u << (p.n_sink & 31)) - 1u : 0u);
+    const int n_words = static_cast<int>((p.L + 31) / 32), Lp = static_cast<int>(p.L - p.n_sink);
+    for (int w = threadIdx.x; w < n_words; w += kSelThreads) bm[w] = empty_bitmap_word(w, Lp);
     uint32_t* summary = smem_summary(dyn_smem, p.L);
     for (int k = threadIdx.x; k < (n_words + 31) / 32; k += kSelThreads) summary[k] = 0u;
   }
@@ -881,7 +903,8 @@ select_kernel(const ComboTable tbl, const SelectParams p) {
     find_threshold(p, tbl, combo, &sh);
     if (threadIdx.x == 0) sh.mode[combo] = static_cast<uint8_t>(sh.plateau);
     if (!sh.plateau)                                         // uniform
-      gather_combination(p, tbl, combo, max(t_begin, tbl.tile_begin[combo]), min(t_end, tbl.tile_begin[combo + 1]), &sh);
+      gather_combination(p, tbl, combo, max(t_begin, tbl.tile_begin[combo]), min(t_end, tbl.tile_begin[combo + 1]), &sh,
+                         reinterpret_cast<int*>(dyn_smem));
     __syncthreads();                                         // readers of the threshold words
   }
   if (!grid_sync<kCluster>(p, &sh, epoch)) return;
