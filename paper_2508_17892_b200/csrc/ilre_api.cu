@@ -31,6 +31,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 constexpr int kNumStages = 4;            // timed stages (see ilre_recall_stage_times)
 constexpr int kProfRing = 32;            // runs whose stage events are kept for averaging
 constexpr int kMaxSinkStaging = 65536;
+constexpr int kPairMinRows = 192;        // query rows per kv head above which the paired scores pass is used
 constexpr int kPairMinTiles = 32;        // accumulators per CTA pair from which the paired scores pass is used
 static constexpr int kHostPieces = 16;              // most pieces of a pipelined host upload
 static constexpr long long kHostPieceMinKeys = 65536;   // no piece shorter than this (128-key multiple)
@@ -152,8 +153,9 @@ void split_rows(int rows, int max_rows, int unit, PassGeometry* g) {
 // Upper bound of the packed rows of one kv head, for any query of up to q_len tokens.
 int rows_padded_bound(int group_size, int q_len) {
   const long long rg = static_cast<long long>(group_size) * q_len;
-  const long long n_rb = (rg + kMaxRbRows - 1) / kMaxRbRows;
-  return static_cast<int>(rg + 128 * (n_rb + 1));
+  const long long n_rb = (rg + kMaxRbRows - 1) / kMaxRbRows, n_pair = (rg + kMaxPairRows - 1) / kMaxPairRows;
+  const long long stats = 128 * (n_rb + 1), pair = 256 * (n_pair + 1);     // paddings
+  return static_cast<int>(rg + (stats > pair ? stats : pair));
 }
 
 Geometry make_geometry(const ilre_recall_config_t& c, int n_sm, long long L, int q_len) {
@@ -174,23 +176,24 @@ Geometry make_geometry(const ilre_recall_config_t& c, int n_sm, long long L, int
   g.stats.pair = 0;
   split_rows(rg, kMaxRbRows, 128, &g.stats);
   finish(&g.stats, kTileKeys, n_sm);
-  // Scores by CTA pairs: where padding the rows of a kv head to a multiple of 256 instead of 128 adds
-  // none (every padded row costs tensor time), and where a pair has at least kPairMinTiles
-  // accumulators to compute, which pay for the cluster launch.  Scores pass, pairs / single CTAs:
-  // L = 1M, 1024 rows per kv head 1414 / 1568 us; 512K, 512 rows 372 / 390; 128K, 256 rows
-  // 53.9 / 56.7; 300K, 700 rows 151 / 223 (two blocks of 384 rows fill a 256-column tile badly); at
-  // the line 32K, 1024 rows (57 accumulators) 55.2 / 56.4, 32K, 512 rows (28) 37.9 / 37.7, and
-  // below it 32K, 256 rows (14) 22.7 / 22.4, 8K, 1024 rows (14) 24.4 / 23.4.
+  // Scores by CTA pairs, which pad the rows of a kv head to a multiple of 256 (single CTAs: to 32), where
+  // there are more than kPairMinRows rows, and where a pair has at least kPairMinTiles accumulators to
+  // compute, which pay for the cluster launch.  Scores pass, pairs / single CTAs, us:
+  //   rows, 128K keys: 148: 53.4 / 47.4; 192: 53.5 / 50.0; 256: 53.7 / 56.1; 280: 93.7 / 100.6;
+  //   400: 94.6 / 101.7; 560: 129.7 / 194.8; 800: 169 / 189 (a second tile of few rows starves the two
+  //   issuing threads of the single form); L = 1M, 1024 rows: 1414 / 1568.
+  //   accumulators: 57 (32K keys, 1024 rows) 55.2 / 56.4; 28 (32K, 512) 37.9 / 37.7; 14 (8K, 1024)
+  //   24.4 / 23.4.
   PassGeometry pair;
   split_rows(rg, kMaxPairRows, 256, &pair);
   pair.pair = 1;
   finish(&pair, kPairTileKeys, n_sm / 2);
   pair.stages = 2;                       // the launcher sizes the ring
   const long long accumulators = static_cast<long long>(pair.n_tiles) * (pair.rb_rows / 256);
-  const bool use_pair = pair.n_rb * pair.rb_rows <= g.stats.n_rb * g.stats.rb_rows &&
-                        accumulators >= static_cast<long long>(kPairMinTiles) * pair.cpg;
+  const bool use_pair = rg > kPairMinRows && accumulators >= static_cast<long long>(kPairMinTiles) * pair.cpg;
   g.scores = use_pair ? pair : g.stats;
-  g.kv_rows = g.stats.n_rb * g.stats.rb_rows;
+  const int a = g.stats.n_rb * g.stats.rb_rows, b = g.scores.n_rb * g.scores.rb_rows;
+  g.kv_rows = a > b ? a : b;
   return g;
 }
 
@@ -471,7 +474,7 @@ int recall_impl(ilre_recall_t* h, const void* k_cache_dev, int64_t L, const void
     qk.pair = pg.pair; qk.n_tiles = pg.n_tiles; qk.n_groups = pg.n_groups; qk.n_rb = pg.n_rb;
     qk.rb_rows = pg.rb_rows; qk.cpg = pg.cpg; qk.stages = pg.stages;
   };
-  qk.L = L; qk.kv_rows = g.kv_rows;
+  qk.L = L; qk.kv_rows = g.kv_rows; qk.rows_per_kv = g.group_size * q_len;
   qk.c2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(kHeadDim)));
   qk.partial = h->partial; qk.enc = h->enc; qk.status = h->status;
   qk.clk = h->profiling ? h->clk : nullptr;

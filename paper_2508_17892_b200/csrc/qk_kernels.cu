@@ -273,6 +273,7 @@ row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
 #pragma unroll
     for (int j = 0; j < kStates; ++j) { m[j] = -1e30f; z[j] = 0.f; }
     const float c2 = p.c2;
+    const int live_rows = min(p.rb_rows, p.rows_per_kv - (it.group % p.n_rb) * p.rb_rows);
     const uint32_t n_acc = run ? static_cast<uint32_t>(it.n_tiles) * MT : 0u;
     // One copy of the loop body serves every (key tile, row tile): the warpgroups run at
     // different places of the loop, and a body unrolled over the row tiles would not fit the
@@ -287,6 +288,12 @@ row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
                      kDevWaitAccFull, p.wait_limit))
         break;
       tc_fence_after();
+      if (mt * 128 + quad * 32 >= live_rows) {                 // padding rows only: nothing to compute
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&tail->acc_empty[b]));
+        continue;
+      }
       float mr = m[0], zr = z[0];
       if (kStates > 1) {
 #pragma unroll
@@ -448,7 +455,9 @@ scores_kernel(const __grid_constant__ CUtensorMap tmapK,
   volatile int* abort_flag = &tail->abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const CtaItem it = decode_item(p, blockIdx.x);
-  const int n_nh = (p.rb_rows + 255) / 256;
+  // query rows of the block, rounded up to the consumers' step of 32: the tensor time goes with them
+  const int n_rows = (min(p.rb_rows, p.rows_per_kv - (it.group % p.n_rb) * p.rb_rows) + 31) & ~31;
+  const int n_nh = (n_rows + 255) / 256;
 
   // Two MMA-issuing threads (warps 1 and 2), one per accumulator buffer: tcgen05.mma holds its
   // issuing thread until the tensor pipe takes the instruction, so the waits and commits of
@@ -483,7 +492,7 @@ scores_kernel(const __grid_constant__ CUtensorMap tmapK,
         tc_fence_after();
         for (int nh = 0; nh < n_nh; ++nh, ++u) {
           if ((u & 1u) != mine) continue;
-          const int N = min(256, p.rb_rows - nh * 256);
+          const int N = min(256, n_rows - nh * 256);
           const uint32_t idesc = umma_idesc_bf16(128, N);
           const uint32_t b = u & 1u, use = u >> 1;
           ok = mbar_wait(smem_u32(&tail->acc_empty[b]), (use & 1u) ^ 1u, abort_flag, p.status,
@@ -521,19 +530,18 @@ scores_kernel(const __grid_constant__ CUtensorMap tmapK,
     for (int i = 0; i < it.n_tiles && ok; ++i) {
       float best = -INFINITY;
       for (int nh = 0; nh < n_nh && ok; ++nh) {
-        const int N = min(256, p.rb_rows - nh * 256);
-        const int half = N >> 1;
+        const int N = min(256, n_rows - nh * 256);
         const uint32_t b = u & 1u, use = u >> 1;
         ++u;
         ok = mbar_wait(smem_u32(&tail->acc_full[b]), use & 1u, abort_flag, p.status,
                        kDevWaitAccFull);
         if (!ok) break;
         tc_fence_after();
-        const int col0 = wg * half;
-        const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + b * 256 + col0;
-        const float4* nl4 = reinterpret_cast<const float4*>(nl + nh * 256 + col0);
+        // the warpgroups take the 32-column steps in turn, first one and then the other begins
+        const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + b * 256;
+        const float4* nl4 = reinterpret_cast<const float4*>(nl + nh * 256);
         float b0 = -INFINITY, b1 = -INFINITY, b2 = -INFINITY, b3 = -INFINITY;
-        for (int c = 0; c < half; c += 32) {
+        for (int c = ((wg ^ i) & 1) * 32; c < N; c += 64) {
           float v[32];
           tmem_ld32(taddr + c, v);
           tmem_ld_wait();

@@ -44,6 +44,7 @@ struct QkParams {
   int n_rb;          // row blocks per kv head
   int rb_rows;       // rows per block: multiple of 128 up to kMaxRbRows (pair: of 256 up to kMaxPairRows)
   int kv_rows;       // rows of one kv head in the packed query (>= n_rb * rb_rows)
+  int rows_per_kv;   // those that are not padding
   int cpg;           // key chunks (CTAs or CTA pairs) per group
   int stages;        // ring depth in key tiles (pair: in units, set by the launcher)
   float c2;          // log2(e) / sqrt(d)

@@ -133,7 +133,10 @@ BIG = [
 # head, contexts that end in the first or the second CTA's keys of the last tile, padded rows, and
 # the sizes one step below the dispatch's line (single CTAs).  (L, q_len, n_kv, n_q)
 PAIRED = [(75777, 64, 8, 32), (75649, 33, 8, 64), (39001, 128, 8, 32), (26113, 192, 8, 32),
-          (25801, 100, 4, 28), (20479, 256, 8, 32), (16640, 511, 4, 16), (9472, 512, 4, 16)]
+          (25801, 100, 4, 28), (20479, 256, 8, 32), (16640, 511, 4, 16), (9472, 512, 4, 16),
+          # padded to more rows than the statistics pass; up to 192 rows single CTAs, in steps of 32 rows
+          (40001, 70, 8, 32), (60001, 129, 2, 8), (75001, 48, 8, 32), (75001, 49, 8, 32), (20001, 8, 8, 32),
+          (20001, 9, 8, 32), (20001, 37, 8, 32), (3001, 24, 4, 28), (3001, 19, 1, 7)]
 
 
 @pytest.mark.parametrize("case", PAIRED, ids=lambda c: f"L{c[0]}_q{c[1]}_kv{c[2]}_h{c[3]}")
