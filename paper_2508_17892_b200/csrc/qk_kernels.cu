@@ -12,6 +12,20 @@
 
 namespace ilre {
 
+// Clears the per-run state: encoded scores, empty bitmap, selection state.
+__device__ __forceinline__ void clear_state(const PrepParams& p, long long tid, long long nthreads) {
+  for (long long t = tid; t < p.L; t += nthreads) p.enc[t] = 0u;
+  const long long n_words = (p.L + 31) / 32;
+  for (long long w = tid; w < n_words; w += nthreads) {
+    const long long left = p.L - p.n_sink - w * 32;       // bits past the end never look free
+    const uint32_t bits = (left >= 32) ? 0u : (left <= 0) ? 0xFFFFFFFFu : 0xFFFFFFFFu << left;
+    p.bitmap[w] = bits;
+  }
+  for (long long e = tid; e < p.hist_words; e += nthreads) p.hist[e] = 0u;
+  if (tid == 0) *p.grid_barrier = 0u;
+  for (long long c = tid; c < p.sel_state_words; c += nthreads) p.cand_count[c] = 0u;
+}
+
 // ---------------------------------------------------------------------------------------
 // shared-memory tail layout (after the Q block and the K stages)
 // ---------------------------------------------------------------------------------------
@@ -89,6 +103,14 @@ __device__ __forceinline__ void cta_teardown(uint32_t tmem_base) {
   }
 }
 
+// 128 query rows of kv head g from row `row` on, channels 64 kb ..: from the packed copy, or straight from
+// the caller's [q_len][n_q][128] array, whose rows of one kv head are `group` heads of consecutive tokens.
+__device__ __forceinline__ void load_query_tile(const CUtensorMap* tmapQ, const QkParams& p, int g, int row, int kb,
+                                                uint32_t dst, uint32_t bar) {
+  if (p.group > 0) tma_load_3d(dst, tmapQ, kb * 64, g * p.group, row / p.group, bar);
+  else tma_load_2d(dst, tmapQ, kb * 64, g * p.kv_rows + row, bar);
+}
+
 // TMA producer: the resident Q block once, then the K tiles of this CTA's key range.
 __device__ __forceinline__ void producer_loop(const CUtensorMap* tmapK, const CUtensorMap* tmapQ,
                                               const QkParams& p, const CtaItem& it,
@@ -99,8 +121,8 @@ __device__ __forceinline__ void producer_loop(const CUtensorMap* tmapK, const CU
   mbar_arrive_expect_tx(qf, static_cast<uint32_t>(p.rb_rows) * 256u);
   for (int kb = 0; kb < 2; ++kb)
     for (int mt = 0; mt < p.rb_rows / 128; ++mt)
-      tma_load_2d(q_s + kb * p.rb_rows * 128 + mt * 16384, tmapQ, kb * 64,
-                  it.g * p.kv_rows + (it.group % p.n_rb) * p.rb_rows + mt * 128, qf);
+      load_query_tile(tmapQ, p, it.g, (it.group % p.n_rb) * p.rb_rows + mt * 128, kb,
+                      q_s + kb * p.rb_rows * 128 + mt * 16384, qf);
   // ring position as (stage, phase) counters: no division by the run-time stage count
   int s = 0;
   uint32_t phase = 0;
@@ -197,7 +219,7 @@ __device__ __forceinline__ void row_update64(const float (&va)[32], const float 
 template <int MT, int NPOLY>
 __global__ void __launch_bounds__(kStatsThreads, 1)
 row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
-                 const __grid_constant__ CUtensorMap tmapQ, const QkParams p) {
+                 const __grid_constant__ CUtensorMap tmapQ, const QkParams p, const PrepParams pp) {
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t smem_base = smem_u32(smem);
   const uint32_t q_s = smem_base;
@@ -219,7 +241,8 @@ row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
 
   if (warp == 0) {
     if (lane == 0 && run) {
-      // The packed query comes from the kernel before this one, which may still be running.
+      // The packed query comes from the kernel before this one, which may still be running (as the
+      // first kernel of a run this one does not overlap anything and the wait returns at once).
       // After that the next kernel's CTAs may come in as SMs fall free.
       grid_dep_wait();
       grid_dep_launch();
@@ -265,6 +288,9 @@ row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
     // at L = 1M, q_len 256 -- more registers' worth of independent work beats the prefetch).
     const int wg = (warp - 2) >> 2;
     const int quad = warp & 3;               // TMEM lane quadrant this warp may read
+    if (pp.clear)                            // while the first tiles are on their way
+      clear_state(pp, static_cast<long long>(blockIdx.x) * (kStatsConsumerWarps * 32) + threadIdx.x - 64,
+                  static_cast<long long>(gridDim.x) * (kStatsConsumerWarps * 32));
     // Accumulator u belongs to warpgroup u % 4 and holds row tile u % MT.  With 1, 2 or 4 row
     // tiles a warpgroup therefore always meets the same row tile (wg % MT) and a thread keeps
     // one (max, sum) pair; only with 3 row tiles does it meet all of them in turn.
@@ -471,7 +497,9 @@ scores_kernel(const __grid_constant__ CUtensorMap tmapK,
 
   if (warp == 0) {
     if (lane == 0 && run) {
-      grid_dep_wait();                   // the kernel before this one (it packed the query or made the statistics) is done
+      // keys and query are the caller's; a packed query comes from a kernel that the kernel before this
+      // one waited for, unless that was the prepare kernel itself
+      if (p.group == 0 && mp.n_ext > 0) grid_dep_wait();
       grid_dep_launch();                 // the next kernel's CTAs may come in as SMs fall free
       producer_loop(&tmapK, &tmapQ, p, it, tail, q_s, k_s, true);
     }
@@ -620,9 +648,12 @@ __device__ __forceinline__ void pair_producer_loop(const CUtensorMap* tmapK, con
   if (rank == 0) mbar_arrive_expect_tx(qf, 2u * MT * 128 * 256);
   for (int kb = 0; kb < 2; ++kb)
     for (int mt = 0; mt < MT; ++mt)
-      tma_load_2d_pair(q_s + kb * (MT * 16384) + mt * 16384, tmapQ, kb * 64,
-                       it.g * p.kv_rows + (it.group % p.n_rb) * p.rb_rows +
-                           (static_cast<int>(rank) * MT + mt) * 128, cluster_addr(qf, 0));
+    {
+      const int row = (it.group % p.n_rb) * p.rb_rows + (static_cast<int>(rank) * MT + mt) * 128;
+      const uint32_t dst = q_s + kb * (MT * 16384) + mt * 16384;
+      if (p.group > 0) tma_load_3d_pair(dst, tmapQ, kb * 64, it.g * p.group, row / p.group, cluster_addr(qf, 0));
+      else tma_load_2d_pair(dst, tmapQ, kb * 64, it.g * p.kv_rows + row, cluster_addr(qf, 0));
+    }
   for (; n < n_units && ok; ++n) ok = load_unit(n);
 }
 
@@ -723,10 +754,10 @@ scores_pair_kernel(const __grid_constant__ CUtensorMap tmapK,
   const bool run = (it.n_tiles > 0) && (*abort_flag == 0);
 
   if (warp == 0) {
-    // The query was packed by the kernel before the statistics kernel, which had completed before
+    // A packed query was made by the kernel before the statistics kernel, which had completed before
     // the statistics kernel let this one start.  A launch without the statistics kernel waits.
     if (lane == 0 && run)
-      pair_producer_loop<MT>(&tmapK, &tmapQ, p, it, mp.n_ext > 0, tail, rank, q_s, k_s);
+      pair_producer_loop<MT>(&tmapK, &tmapQ, p, it, p.group == 0 && mp.n_ext > 0, tail, rank, q_s, k_s);
   } else if (warp == 1 || warp == 2) {
     if (lane == 0 && run && rank == 0)
       pair_issue_loop<MT>(p, it, tail, tmem_base, q_s, k_s, static_cast<uint32_t>(warp - 1));
@@ -797,7 +828,8 @@ scores_pair_kernel(const __grid_constant__ CUtensorMap tmapK,
 // small kernels around the two passes
 // ---------------------------------------------------------------------------------------
 
-// Packs the query rows of every kv head contiguously, zero-padded to kv_rows,
+// Packs the query rows of every kv head contiguously, zero-padded to kv_rows (head groups whose rows a
+// TMA box cannot collect from the caller's array),
 // and clears the per-run state (encoded scores, empty bitmap, selection
 // state).
 __global__ void prepare_kernel(const uint4* __restrict__ q, uint4* __restrict__ qp, PrepParams p) {
@@ -817,16 +849,7 @@ __global__ void prepare_kernel(const uint4* __restrict__ q, uint4* __restrict__ 
     }
     qp[e] = val;
   }
-  for (long long t = tid; t < p.L; t += nthreads) p.enc[t] = 0u;
-  const long long n_words = (p.L + 31) / 32;
-  for (long long w = tid; w < n_words; w += nthreads) {
-    const long long left = p.L - p.n_sink - w * 32;       // bits past the end never look free
-    const uint32_t bits = (left >= 32) ? 0u : (left <= 0) ? 0xFFFFFFFFu : 0xFFFFFFFFu << left;
-    p.bitmap[w] = bits;
-  }
-  for (long long e = tid; e < p.hist_words; e += nthreads) p.hist[e] = 0u;
-  if (tid == 0) *p.grid_barrier = 0u;
-  for (long long c = tid; c < p.sel_state_words; c += nthreads) p.cand_count[c] = 0u;
+  if (p.clear) clear_state(p, tid, nthreads);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -859,23 +882,27 @@ size_t scores_smem_bytes(int rb_rows, int stages) {
 }
 
 template <int MT>
-static cudaError_t launch_row_stats_mt(const CUtensorMap& tk, const CUtensorMap& tq,
-                                       const QkParams& p, cudaStream_t st) {
+static cudaError_t launch_row_stats_mt(const CUtensorMap& tk, const CUtensorMap& tq, const QkParams& p,
+                                       const PrepParams& pp, bool first_kernel, cudaStream_t st) {
   const size_t smem = row_stats_smem_bytes(MT * 128, p.stages);
   cudaError_t e = cudaFuncSetAttribute(row_stats_kernel<MT, kRowStatsPolyPairs>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
+  if (first_kernel) {
+    row_stats_kernel<MT, kRowStatsPolyPairs><<<p.n_groups * p.cpg, kStatsThreads, smem, st>>>(tk, tq, p, pp);
+    return cudaGetLastError();
+  }
   return launch_after_previous(row_stats_kernel<MT, kRowStatsPolyPairs>, p.n_groups * p.cpg,
-                               kStatsThreads, smem, st, tk, tq, p);
+                               kStatsThreads, smem, st, tk, tq, p, pp);
 }
 
 cudaError_t launch_row_stats(const CUtensorMap& tk, const CUtensorMap& tq, const QkParams& p,
-                             cudaStream_t st) {
+                             const PrepParams& pp, bool first_kernel, cudaStream_t st) {
   switch (p.rb_rows / 128) {
-    case 1: return launch_row_stats_mt<1>(tk, tq, p, st);
-    case 2: return launch_row_stats_mt<2>(tk, tq, p, st);
-    case 3: return launch_row_stats_mt<3>(tk, tq, p, st);
-    case 4: return launch_row_stats_mt<4>(tk, tq, p, st);
+    case 1: return launch_row_stats_mt<1>(tk, tq, p, pp, first_kernel, st);
+    case 2: return launch_row_stats_mt<2>(tk, tq, p, pp, first_kernel, st);
+    case 3: return launch_row_stats_mt<3>(tk, tq, p, pp, first_kernel, st);
+    case 4: return launch_row_stats_mt<4>(tk, tq, p, pp, first_kernel, st);
     default: return cudaErrorInvalidValue;
   }
 }

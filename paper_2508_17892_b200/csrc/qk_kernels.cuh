@@ -45,6 +45,8 @@ struct QkParams {
   int rb_rows;       // rows per block: multiple of 128 up to kMaxRbRows (pair: of 256 up to kMaxPairRows)
   int kv_rows;       // rows of one kv head in the packed query (>= n_rb * rb_rows)
   int rows_per_kv;   // those that are not padding
+  int group;         // query heads per kv head when the query is loaded from the caller's array (a
+                     // box of 128 rows = `group` heads of 128 / group tokens); 0: from the packed copy
   int cpg;           // key chunks (CTAs or CTA pairs) per group
   int stages;        // ring depth in key tiles (pair: in units, set by the launcher)
   float c2;          // log2(e) / sqrt(d)
@@ -64,6 +66,7 @@ struct QkParams {
 
 struct PrepParams {
   int n_kv, n_q, group_size, q_len, kv_rows;   // kv_rows = 0: no query to pack
+  int clear;                // the state of the run is to be cleared
   long long L;
   int n_sink;
   uint32_t* enc;
@@ -91,8 +94,10 @@ size_t row_stats_smem_bytes(int rb_rows, int stages);
 size_t scores_smem_bytes(int rb_rows, int stages);
 
 cudaError_t launch_prepare(const void* q, void* qp, const PrepParams& p, int n_sm, cudaStream_t st);
+// first_kernel: no prepare kernel was launched before this one, which then clears the run's state itself
+// (pp.clear); else the launch overlaps the end of the prepare kernel.
 cudaError_t launch_row_stats(const CUtensorMap& tk, const CUtensorMap& tq, const QkParams& p,
-                             cudaStream_t st);
+                             const PrepParams& pp, bool first_kernel, cudaStream_t st);
 // (max in log2 units, sum of exponentials) of every query row over the keys of this launch,
 // rows in the caller's order i * n_q + h.
 cudaError_t launch_export_stats(const MergeParams& p, float2* out, cudaStream_t st);
