@@ -19,6 +19,7 @@
 #include <cuda_bf16.h>
 
 #include "attn_kernels.cuh"
+#include "launch.cuh"
 #include "sm100_ptx.cuh"
 
 namespace ilre {
@@ -120,6 +121,8 @@ chunk_attention_kernel(const __grid_constant__ CUtensorMap map_q,
   tc_fence_after();
   const uint32_t tmem_base = tail->tmem_base;
   const bool run = (*abort_flag == 0);
+  grid_dep_wait();                         // everything above overlaps the kernel before this one
+  grid_dep_launch();
 
   // TMEM columns: S of stream x at 128 x, O of stream x at 256 + 128 x.
   // Ring items (key and value tiles) are each used by both streams.
@@ -412,8 +415,8 @@ cudaError_t launch_chunk_attention(const CUtensorMap& map_q, const CUtensorMap& 
     --p.split_from;
     n_cta += p.n_q - per_qt;
   }
-  chunk_attention_kernel<<<static_cast<unsigned>(n_cta), kAttnThreads, smem, st>>>(map_q, map_k, map_v, p);
-  return cudaGetLastError();
+  return launch_after_previous(chunk_attention_kernel, static_cast<int>(n_cta), kAttnThreads, smem, st,
+                               map_q, map_k, map_v, p);
 }
 
 }  // namespace ilre

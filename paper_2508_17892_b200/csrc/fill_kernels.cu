@@ -17,6 +17,7 @@
 #include <cuda_bf16.h>
 
 #include "fill_kernels.cuh"
+#include "launch.cuh"
 #include "sm100_ptx.cuh"
 
 namespace ilre {
@@ -125,6 +126,8 @@ fill_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ C
   tc_fence_after();
   const uint32_t tmem_base = tail->tmem_base;
   const bool run = (*abort_flag == 0);
+  grid_dep_wait();                         // everything above overlaps the kernel before this one
+  grid_dep_launch();
 
   // The loading and issuing threads test the barriers of up to kFillBatch blocks at once: a test
   // waits behind the copies or MMAs that the thread has issued before it and what follows waits for
@@ -341,14 +344,17 @@ cudaError_t launch_rope_pos_tables(float2* lo, float2* hi, int hi_rows, double t
 }
 
 cudaError_t launch_fill(const CUtensorMap& map_x, const CUtensorMap& map_w, const CUtensorMap& map_w_tail,
-                        const FillParams& p, int n_sm, cudaStream_t st) {
+                        const FillParams& p, bool new_tables, int n_sm, cudaStream_t st) {
   constexpr int kSmem = kFillStages * 2 * 128 * kFillBlockK * 2 + kFillTailBytes;
   cudaError_t e = cudaFuncSetAttribute(fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
   if (e != cudaSuccess) return e;
   const int workers = n_sm / 2 > 0 ? n_sm / 2 : 1;
   const int grid = 2 * (p.n_tiles < workers ? p.n_tiles : workers);
-  fill_kernel<<<grid, kFillThreads, kSmem, st>>>(map_x, map_w, map_w_tail, p);
-  return cudaGetLastError();
+  if (new_tables) {                        // read through the non-coherent path: no overlap with their kernel
+    fill_kernel<<<grid, kFillThreads, kSmem, st>>>(map_x, map_w, map_w_tail, p);
+    return cudaGetLastError();
+  }
+  return launch_after_previous(fill_kernel, grid, kFillThreads, kSmem, st, map_x, map_w, map_w_tail, p);
 }
 
 }  // namespace ilre

@@ -34,6 +34,6 @@ cudaError_t launch_rope_pos_tables(float2* lo, float2* hi, int hi_rows, double t
                                    cudaStream_t st);
 // The box of map_w has unit_width / 2 weight rows, that of map_w_tail tail_width / 2.
 cudaError_t launch_fill(const CUtensorMap& map_x, const CUtensorMap& map_w, const CUtensorMap& map_w_tail,
-                        const FillParams& p, int n_sm, cudaStream_t st);
+                        const FillParams& p, bool new_tables, int n_sm, cudaStream_t st);
 
 }  // namespace ilre

@@ -562,7 +562,7 @@ int recall_impl(ilre_recall_t* h, const void* k_cache_dev, int64_t L, const void
   if (io.stages & kStageStats) {
     TraceRange r("ilre: row statistics (Eq. 4)");
     set_pass(g.stats);
-    ILRE_CUDA(launch_row_stats(map_k, map_q, qk, pp, !prepare, st)); ++launches;
+    ILRE_CUDA(launch_row_stats(map_k, map_q, qk, pp, st)); ++launches;
     if (io.stats_out) { ILRE_CUDA(launch_export_stats(mp, io.stats_out, st)); ++launches; }
   }
   ILRE_MARK(2);
@@ -762,7 +762,7 @@ int ilre_recall_fill_keys(ilre_recall_t* h, const void* x_dev, int64_t n_tok, in
       !encode_2d(h->encode, &map_w, w_k_dev, inner, static_cast<uint64_t>(n_out), inner * 2, fp.unit_width / 2) ||
       !encode_2d(h->encode, &map_w_tail, w_k_dev, inner, static_cast<uint64_t>(n_out), inner * 2, fp.tail_width / 2))
     return ILRE_ERR_CUDA;
-  ILRE_CUDA(launch_fill(map_x, map_w, map_w_tail, fp, h->n_sm, st)); ++launches;
+  ILRE_CUDA(launch_fill(map_x, map_w, map_w_tail, fp, launches > 0, h->n_sm, st)); ++launches;
   h->last_launches = launches;
   return ILRE_OK;
 }
@@ -803,7 +803,7 @@ int ilre_recall_rerope_keys(ilre_recall_t* h, const void* k_cache_dev, void* k_o
   rp.k_out = static_cast<uint4*>(k_out_dev);
   rp.L = L; rp.n_kv = h->cfg.n_kv_heads; rp.chunk = chunk_size; rp.n_sink = n_sink;
   rp.n_chunks = n_chunks; rp.table = h->rope_table;
-  ILRE_CUDA(launch_rerope(rp, h->n_sm, st)); ++launches;
+  ILRE_CUDA(launch_rerope(rp, launches > 0, h->n_sm, st)); ++launches;
   h->last_launches = launches;
   return ILRE_OK;
 }

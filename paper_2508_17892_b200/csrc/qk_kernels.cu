@@ -6,6 +6,7 @@
 //   scores:         D[key, row] tiles (operands swapped), one thread per context position keeps
 //                   max over rows of (logit - lse_row); exp is monotone, so one exp per position
 //                   is taken afterwards.
+#include "launch.cuh"
 #include "qk_kernels.cuh"
 #include <utility>
 #include "sm100_ptx.cuh"
@@ -241,9 +242,9 @@ row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
 
   if (warp == 0) {
     if (lane == 0 && run) {
-      // The packed query comes from the kernel before this one, which may still be running (as the
-      // first kernel of a run this one does not overlap anything and the wait returns at once).
-      // After that the next kernel's CTAs may come in as SMs fall free.
+      // The packed query (or, as the first kernel of a run, whatever else this one reads) comes from
+      // the kernel before this one, which may still be running.  After that the next kernel's CTAs
+      // may come in as SMs fall free.
       grid_dep_wait();
       grid_dep_launch();
       producer_loop(&tmapK, &tmapQ, p, it, tail, q_s, k_s, false, p.skip_tiles);
@@ -288,9 +289,11 @@ row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
     // at L = 1M, q_len 256 -- more registers' worth of independent work beats the prefetch).
     const int wg = (warp - 2) >> 2;
     const int quad = warp & 3;               // TMEM lane quadrant this warp may read
-    if (pp.clear)                            // while the first tiles are on their way
+    if (pp.clear) {                          // while the first tiles are on their way
+      grid_dep_wait();                       // the run before this one may still read that state
       clear_state(pp, static_cast<long long>(blockIdx.x) * (kStatsConsumerWarps * 32) + threadIdx.x - 64,
                   static_cast<long long>(gridDim.x) * (kStatsConsumerWarps * 32));
+    }
     // Accumulator u belongs to warpgroup u % 4 and holds row tile u % MT.  With 1, 2 or 4 row
     // tiles a warpgroup therefore always meets the same row tile (wg % MT) and a thread keeps
     // one (max, sum) pair; only with 3 row tiles does it meet all of them in turn.
@@ -833,7 +836,8 @@ scores_pair_kernel(const __grid_constant__ CUtensorMap tmapK,
 // and clears the per-run state (encoded scores, empty bitmap, selection
 // state).
 __global__ void prepare_kernel(const uint4* __restrict__ q, uint4* __restrict__ qp, PrepParams p) {
-  grid_dep_launch();                     // the statistics kernel sets itself up meanwhile
+  grid_dep_wait();                       // the run before this one may still use the buffers
+  grid_dep_launch();                     // the next kernel sets itself up meanwhile
   const long long tid = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   const long long nthreads = static_cast<long long>(gridDim.x) * blockDim.x;
   // packed query: 16 x uint4 per 128-element row
@@ -855,24 +859,6 @@ __global__ void prepare_kernel(const uint4* __restrict__ q, uint4* __restrict__ 
 // ---------------------------------------------------------------------------------------
 // host-side launchers
 // ---------------------------------------------------------------------------------------
-// Launch that may overlap the end of the kernel before it in the stream (programmatic
-// dependent launch): the kernel itself waits (grid_dep_wait) before it touches that kernel's output.
-template <typename... Params, typename... Args>
-static cudaError_t launch_after_previous(void (*kernel)(Params...), int grid, int block, size_t smem,
-                                         cudaStream_t st, Args&&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
-}
-
 size_t row_stats_smem_bytes(int rb_rows, int stages) {
   return static_cast<size_t>(rb_rows) * 256 + static_cast<size_t>(stages) * kStageBytes +
          kSmemTailBytes;
@@ -883,26 +869,22 @@ size_t scores_smem_bytes(int rb_rows, int stages) {
 
 template <int MT>
 static cudaError_t launch_row_stats_mt(const CUtensorMap& tk, const CUtensorMap& tq, const QkParams& p,
-                                       const PrepParams& pp, bool first_kernel, cudaStream_t st) {
+                                       const PrepParams& pp, cudaStream_t st) {
   const size_t smem = row_stats_smem_bytes(MT * 128, p.stages);
   cudaError_t e = cudaFuncSetAttribute(row_stats_kernel<MT, kRowStatsPolyPairs>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  if (first_kernel) {
-    row_stats_kernel<MT, kRowStatsPolyPairs><<<p.n_groups * p.cpg, kStatsThreads, smem, st>>>(tk, tq, p, pp);
-    return cudaGetLastError();
-  }
   return launch_after_previous(row_stats_kernel<MT, kRowStatsPolyPairs>, p.n_groups * p.cpg,
                                kStatsThreads, smem, st, tk, tq, p, pp);
 }
 
 cudaError_t launch_row_stats(const CUtensorMap& tk, const CUtensorMap& tq, const QkParams& p,
-                             const PrepParams& pp, bool first_kernel, cudaStream_t st) {
+                             const PrepParams& pp, cudaStream_t st) {
   switch (p.rb_rows / 128) {
-    case 1: return launch_row_stats_mt<1>(tk, tq, p, pp, first_kernel, st);
-    case 2: return launch_row_stats_mt<2>(tk, tq, p, pp, first_kernel, st);
-    case 3: return launch_row_stats_mt<3>(tk, tq, p, pp, first_kernel, st);
-    case 4: return launch_row_stats_mt<4>(tk, tq, p, pp, first_kernel, st);
+    case 1: return launch_row_stats_mt<1>(tk, tq, p, pp, st);
+    case 2: return launch_row_stats_mt<2>(tk, tq, p, pp, st);
+    case 3: return launch_row_stats_mt<3>(tk, tq, p, pp, st);
+    case 4: return launch_row_stats_mt<4>(tk, tq, p, pp, st);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -951,8 +933,8 @@ cudaError_t launch_scores(const CUtensorMap& tk, const CUtensorMap& tq, const Qk
 
 cudaError_t launch_prepare(const void* q, void* qp, const PrepParams& p, int n_sm,
                            cudaStream_t st) {
-  prepare_kernel<<<n_sm * 4, 256, 0, st>>>(static_cast<const uint4*>(q), static_cast<uint4*>(qp), p);
-  return cudaGetLastError();
+  return launch_after_previous(prepare_kernel, n_sm * 4, 256, 0, st, static_cast<const uint4*>(q),
+                               static_cast<uint4*>(qp), p);
 }
 
 }  // namespace ilre

@@ -97,7 +97,7 @@ cudaError_t launch_prepare(const void* q, void* qp, const PrepParams& p, int n_s
 // first_kernel: no prepare kernel was launched before this one, which then clears the run's state itself
 // (pp.clear); else the launch overlaps the end of the prepare kernel.
 cudaError_t launch_row_stats(const CUtensorMap& tk, const CUtensorMap& tq, const QkParams& p,
-                             const PrepParams& pp, bool first_kernel, cudaStream_t st);
+                             const PrepParams& pp, cudaStream_t st);
 // (max in log2 units, sum of exponentials) of every query row over the keys of this launch,
 // rows in the caller's order i * n_q + h.
 cudaError_t launch_export_stats(const MergeParams& p, float2* out, cudaStream_t st);

@@ -6,6 +6,8 @@
 #include <cuda_bf16.h>
 
 #include "rerope_kernels.cuh"
+#include "launch.cuh"
+#include "sm100_ptx.cuh"
 
 namespace ilre {
 
@@ -49,6 +51,8 @@ __global__ void __launch_bounds__(kReropeThreads)
 rerope_kernel(const ReropeParams p) {
   // One item = one 16-byte segment pair (low half, high half) of one (position, kv head) row;
   // eight consecutive threads cover a row, a warp four rows = 1 KB of contiguous cache.
+  grid_dep_wait();
+  grid_dep_launch();
   const long long n_items = p.L * p.n_kv * 8;
   const bool copy_tail = p.k_out != p.k_in;
   const long long rot_end = (p.n_chunks >= 2)                // first position of chunk N_C - 1
@@ -144,11 +148,14 @@ cudaError_t launch_rope_table(float2* table, int n_rows, int chunk, double theta
   return cudaGetLastError();
 }
 
-cudaError_t launch_rerope(const ReropeParams& p, int n_sm, cudaStream_t st) {
+cudaError_t launch_rerope(const ReropeParams& p, bool new_table, int n_sm, cudaStream_t st) {
   // Four CTAs of 256 threads per SM, all resident, one item per thread in flight: measured
   // fastest (0.70 ms for a 2 GiB cache; 8 CTAs or 2-8 items in flight: 0.72-1.17 ms).
-  rerope_kernel<<<n_sm * kReropeCtasPerSm, kReropeThreads, 0, st>>>(p);
-  return cudaGetLastError();
+  if (new_table) {                         // read through the non-coherent path: no overlap with its kernel
+    rerope_kernel<<<n_sm * kReropeCtasPerSm, kReropeThreads, 0, st>>>(p);
+    return cudaGetLastError();
+  }
+  return launch_after_previous(rerope_kernel, n_sm * kReropeCtasPerSm, kReropeThreads, 0, st, p);
 }
 
 }  // namespace ilre

@@ -23,7 +23,7 @@ struct ReropeParams {
 cudaError_t launch_rope_table(float2* table, int n_rows, int chunk, double theta,
                               cudaStream_t st);
 // K~ = R(D_i) K for the chunks before the last two; the last two are copied when out != in.
-cudaError_t launch_rerope(const ReropeParams& p, int n_sm, cudaStream_t st);
+cudaError_t launch_rerope(const ReropeParams& p, bool new_table, int n_sm, cudaStream_t st);
 
 // Every (row, kv head) vector of k_in [n_rows][128] turned by the distance of `table_row`
 // ([64] (cos, sin)); a null row copies.  k_out may alias k_in.

@@ -444,3 +444,65 @@ def test_recalls_in_a_row_on_a_side_stream_keep_their_own_results():
         assert np.array_equal(sc.cpu().numpy(), ref_sc), f"scores of recall {n}"
     assert eng.check_guards() == 0, "a kernel wrote past the end of a workspace buffer"
     eng.close()
+
+
+@pytest.mark.parametrize("n_kv,n_q,L,q_len", [(8, 32, 1500, 8), (4, 28, 1500, 8), (8, 32, 40000, 130)])
+@pytest.mark.parametrize("captured", [False, True])
+def test_every_kernel_waits_for_the_call_before_it(n_kv, n_q, L, q_len, captured):
+    """Each kernel may start while the one before it ends.  Fill, Eq. 7, recall, attention and the
+    allocation of given scores, in a row through the same buffers, give what they give with a
+    synchronisation after every call; in a graph, behind a join of two streams too."""
+    from paper_2508_17892_b200 import IlreRecall
+    rounds, d_model, chunk = 4, 64, 256
+    g = torch.Generator(device="cuda").manual_seed(5)
+    rand = lambda *s: torch.randn(*s, generator=g, device="cuda").to(torch.bfloat16)
+    X = [rand(L, d_model) for _ in range(rounds)]
+    Q = [rand(q_len, n_q, 128) for _ in range(rounds)]
+    A = rand(chunk, n_q, 128)
+    W = rand(n_kv * 128, d_model) / 8
+    eng = IlreRecall(max_L=L, max_q_len=q_len, max_budget=128, n_kv_heads=n_kv, n_q_heads=n_q)
+    cache = torch.zeros(L, n_kv, 128, dtype=torch.bfloat16, device="cuda")
+    turned = torch.zeros_like(cache)
+    given = torch.zeros(L, device="cuda")
+    side, other = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+
+    def sequence(after):
+        results = []
+        for i in range(rounds):
+            eng.fill_keys(X[i], W, cache, 0, stream=side)
+            after()
+            eng.rerope_keys(cache, chunk, out=turned, stream=side)
+            after()
+            idx, _ = eng.run(turned, Q[i], 128, (1,), (1, 7), 1, 4, out_scores=given, stream=side)
+            after()
+            again = eng.allocate(given, 100, (2,), (5,), 1, stream=side)
+            after()
+            out = eng.chunk_attention(A, cache[:chunk + 100], turned[:chunk + 100], 100, stream=side)
+            after()
+            results.append((idx, again, out, given.clone(), cache.clone()))
+        return results
+
+    with torch.cuda.stream(side):
+        want = sequence(torch.cuda.synchronize)
+        if captured:
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=side):
+                other.wait_stream(side)
+                with torch.cuda.stream(other):
+                    cache.zero_()
+                given.zero_()
+                side.wait_stream(other)
+                got = sequence(lambda: None)
+            graph.replay()
+        else:
+            got = sequence(lambda: None)
+    torch.cuda.synchronize()
+    eng.check_status()
+    for a, b in zip(want, got):
+        for x, y in zip(a, b):
+            assert torch.equal(x, y)
+    assert eng.check_guards() == 0, "a kernel wrote past the end of a workspace buffer"
+    if captured:
+        del graph
+    eng.close()
