@@ -188,9 +188,11 @@ chunk_attention_kernel(const __grid_constant__ CUtensorMap map_q,
           const int t = next[x];
           if (t >= n_tiles) continue;
           if (s_role) {
-            // S_x(t): needs the key tile and, after the first, S_x(t-1) read out of tensor memory
-            if (ring_ready(k_item(t)) &&
-                (t == 0 || mbar_test_wait(smem_u32(&tail->s_empty[x]), static_cast<uint32_t>(t - 1) & 1u))) {
+            // S_x(t): needs, after the first, S_x(t-1) read out of tensor memory and the key tile (asked
+            // second: S_x(t-1) read means O += P V of tile t-3 done, so that the value tile which had the
+            // key tile's ring slot before it has arrived and the parity of the slot means this phase)
+            if ((t == 0 || mbar_test_wait(smem_u32(&tail->s_empty[x]), static_cast<uint32_t>(t - 1) & 1u)) &&
+                ring_ready(k_item(t))) {
               tc_fence_after();
               const uint32_t k_s = ring_s + (k_item(t) % kAttnStages) * kAttnTileBytes;
               const uint32_t qx = q_s + x * kAttnTileBytes;

@@ -179,7 +179,7 @@ Geometry make_geometry(const ilre_recall_config_t& c, int n_sm, long long L, int
   // Scores by CTA pairs, which pad the rows of a kv head to a multiple of 256 (single CTAs: to 32), where
   // there are more than kPairMinRows rows, and where a pair has at least kPairMinTiles accumulators to
   // compute, which pay for the cluster launch.  Scores pass, pairs / single CTAs, us:
-  //   rows, 128K keys: 148: 53.4 / 47.4; 192: 53.5 / 50.0; 256: 53.7 / 56.1; 280: 93.7 / 100.6;
+  //   rows, 128K keys: 148: 53.4 / 49.0; 192: 53.5 / 50.0; 256: 53.7 / 56.1; 280: 93.7 / 100.6;
   //   400: 94.6 / 101.7; 560: 129.7 / 194.8; 800: 169 / 189 (a second tile of few rows starves the two
   //   issuing threads of the single form); L = 1M, 1024 rows: 1414 / 1568.
   //   accumulators: 57 (32K keys, 1024 rows) 55.2 / 56.4; 28 (32K, 512) 37.9 / 37.7; 14 (8K, 1024)
@@ -192,6 +192,9 @@ Geometry make_geometry(const ilre_recall_config_t& c, int n_sm, long long L, int
   const long long accumulators = static_cast<long long>(pair.n_tiles) * (pair.rb_rows / 256);
   const bool use_pair = rg > kPairMinRows && accumulators >= static_cast<long long>(kPairMinTiles) * pair.cpg;
   g.scores = use_pair ? pair : g.stats;
+  // Where the two issuing threads take the key tiles in turn, a stage of the ring must always meet the
+  // same one: a parity wait is only sound for a thread that has seen the stage's phase before.
+  if (!use_pair && g.scores.rb_rows <= 256) g.scores.stages &= ~1;
   const int a = g.stats.n_rb * g.stats.rb_rows, b = g.scores.n_rb * g.scores.rb_rows;
   g.kv_rows = a > b ? a : b;
   return g;

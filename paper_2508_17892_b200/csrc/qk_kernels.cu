@@ -904,8 +904,11 @@ template <int MT>
 static cudaError_t launch_scores_pair_mt(const CUtensorMap& tk, const CUtensorMap& tq, QkParams p,
                                          const MergeParams& mp, cudaStream_t st) {
   constexpr int kFixed = MT * 128 * 256 + kSmemTailBytes + MT * 256 * static_cast<int>(sizeof(float));
-  constexpr int kUnits = (kMaxDynSmem - kFixed) / kUnitBytes;
-  p.stages = kUnits > kMaxUnits ? kMaxUnits : kUnits;
+  constexpr int kUnits = (kMaxDynSmem - kFixed) / kUnitBytes < kMaxUnits ? (kMaxDynSmem - kFixed) / kUnitBytes
+                                                                         : kMaxUnits;
+  // the issuing threads take the tiles of two units in turn with one row tile; see make_geometry
+  static_assert(MT > 1 || kUnits % 4 == 0, "a ring unit must always meet the same issuing thread");
+  p.stages = kUnits;
   const size_t smem = static_cast<size_t>(kFixed) + static_cast<size_t>(p.stages) * kUnitBytes;
   cudaError_t e = cudaFuncSetAttribute(scores_pair_kernel<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);

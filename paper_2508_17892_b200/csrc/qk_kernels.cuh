@@ -94,8 +94,7 @@ size_t row_stats_smem_bytes(int rb_rows, int stages);
 size_t scores_smem_bytes(int rb_rows, int stages);
 
 cudaError_t launch_prepare(const void* q, void* qp, const PrepParams& p, int n_sm, cudaStream_t st);
-// first_kernel: no prepare kernel was launched before this one, which then clears the run's state itself
-// (pp.clear); else the launch overlaps the end of the prepare kernel.
+// Where no prepare kernel was launched before it, this one clears the run's state (pp.clear).
 cudaError_t launch_row_stats(const CUtensorMap& tk, const CUtensorMap& tq, const QkParams& p,
                              const PrepParams& pp, cudaStream_t st);
 // (max in log2 units, sum of exponentials) of every query row over the keys of this launch,
