@@ -218,7 +218,7 @@ __device__ __forceinline__ void row_update64(const float (&va)[32], const float 
 // Pass A: row statistics.  MT = number of 128-row tiles of the resident Q block.
 // ---------------------------------------------------------------------------------------
 template <int MT, int NPOLY>
-__global__ void __launch_bounds__(kStatsThreads, 1)
+__global__ void __launch_bounds__(kStatsThreads<MT>, 1)
 row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
                  const __grid_constant__ CUtensorMap tmapQ, const QkParams p, const PrepParams pp) {
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -230,7 +230,8 @@ row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const CtaItem it = decode_item(p, blockIdx.x);
 
-  const uint32_t tmem_base = cta_setup(tail, smem_base, p.stages, 4, 4, p.status);
+  constexpr uint32_t kIssuers = kStatsIssuers<MT>;       // every one reads every key tile
+  const uint32_t tmem_base = cta_setup(tail, smem_base, p.stages, 4, 4, p.status, kIssuers);
   const bool run = (it.n_tiles > 0) && (*abort_flag == 0);
   const bool stamp = (p.clk != nullptr) && blockIdx.x == 0 && threadIdx.x == 0;
   if (stamp) {
@@ -249,8 +250,13 @@ row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
       grid_dep_launch();
       producer_loop(&tmapK, &tmapQ, p, it, tail, q_s, k_s, false, p.skip_tiles);
     }
-  } else if (warp == 1) {
+  } else if (warp == 1 || warp >= 2 + kStatsConsumerWarps) {
     if (lane == 0 && run) {
+      // Accumulator u is filled by issuing thread u % kIssuers.  A barrier test waits behind the MMAs that
+      // its thread has issued: one thread took 1030 cycles per accumulator for 512 cycles of MMAs, and
+      // the consumers waited 1700 of 4160 cycles for each of theirs; with two threads 450 of 4010
+      // (row statistics at 256K keys, 512 rows per kv head: 278 -> 272 us; 1M keys, 1024 rows: 2489 -> 2424 us).
+      const uint32_t mine = (warp == 1) ? 0u : 1u;
       constexpr uint32_t idesc = umma_idesc_bf16(128, kTileKeys);
       bool ok = mbar_wait(smem_u32(&tail->q_full), 0, abort_flag, p.status, kDevWaitQFull, p.wait_limit);
       tc_fence_after();
@@ -262,6 +268,7 @@ row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
         if (!ok) break;
         tc_fence_after();
         for (int mt = 0; mt < MT; ++mt, ++u) {
+          if (u % kIssuers != mine) continue;
           const uint32_t b = u & 3u, use = u >> 2;
           ok = mbar_wait(smem_u32(&tail->acc_empty[b]), (use & 1u) ^ 1u, abort_flag, p.status,
                          kDevWaitAccEmpty, p.wait_limit);
@@ -281,7 +288,7 @@ row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
         if (++s == p.stages) { s = 0; kphase ^= 1u; }
       }
     }
-  } else if (warp >= 2) {
+  } else {
     // Consumer warpgroups take the accumulator buffers in turn, so that they sit in different
     // phases (waiting, loading, taking maxima, exponentials) and keep the special-function
     // and FMA pipes fed.  Each thread owns one query row of the buffer and takes its 128 columns
@@ -875,7 +882,7 @@ static cudaError_t launch_row_stats_mt(const CUtensorMap& tk, const CUtensorMap&
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   return launch_after_previous(row_stats_kernel<MT, kRowStatsPolyPairs>, p.n_groups * p.cpg,
-                               kStatsThreads, smem, st, tk, tq, p, pp);
+                               kStatsThreads<MT>, smem, st, tk, tq, p, pp);
 }
 
 cudaError_t launch_row_stats(const CUtensorMap& tk, const CUtensorMap& tq, const QkParams& p,
