@@ -51,8 +51,9 @@ __global__ void __launch_bounds__(kReropeThreads)
 rerope_kernel(const ReropeParams p) {
   // One item = one 16-byte segment pair (low half, high half) of one (position, kv head) row;
   // eight consecutive threads cover a row, a warp four rows = 1 KB of contiguous cache.
-  grid_dep_wait();
-  grid_dep_launch();
+  grid_dep_wait();                         // and no early release of the next kernel: a re-rotation whose
+                                           // CTAs came in beside these ran unevenly placed (128K keys, calls
+                                           // in a row: 88 -> 124 us; plain launches 90)
   const long long n_items = p.L * p.n_kv * 8;
   const bool copy_tail = p.k_out != p.k_in;
   const long long rot_end = (p.n_chunks >= 2)                // first position of chunk N_C - 1
