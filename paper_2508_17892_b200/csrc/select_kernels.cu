@@ -24,6 +24,12 @@
 //
 // Work of phase B is cut into tiles of cells of one group of windows, work of phase D into tiles of
 // kSelTile cells of one combination; every CTA owns a contiguous run of tiles.
+//
+// Bound by the chain of its phases: barriers, one CTA's walk, code met cold in the instruction cache
+// (everything it reads is in L2).  The stage by itself, events around it after an L2 flush, with a
+// selection inside the threshold bin, one window per pooling tile and scattered candidates -> as it
+// stands: 4K positions 39 -> 34 us, 32K 52 -> 42, 128K 59 -> 48, 512K 89 -> 66, 1M 117..131 -> 88, 1M with
+// 48 combinations 270..280 -> 218.
 #include "select_kernels.cuh"
 #include "sm100_ptx.cuh"
 
