@@ -13,8 +13,9 @@ static constexpr int kMaxStages = 6;
 static constexpr int kMaxRbRows = 512;             // query rows resident in shared memory
 static constexpr int kQkThreads = 384;             // scores: warp 0 TMA, warps 1-2 MMA, warps 4..11 consumers
 static constexpr int kConsumerWarps = 8;
-// Row statistics: warp 0 TMA, warp 1 MMA, then kStatsWarpgroups consumer warpgroups of four
-// warps (one per TMEM lane quadrant); accumulator buffer u belongs to warpgroup u % kStatsWarpgroups.
+// Row statistics: warp 0 TMA, warp 1 MMA, kStatsWarpgroups consumer warpgroups of four
+// warps (one per TMEM lane quadrant), perhaps a second MMA warp; accumulator buffer u belongs to warpgroup
+// u % kStatsWarpgroups.
 static constexpr int kStatsWarpgroups = 4;
 // A warpgroup's first accumulator must be one of the first four (the number of TMEM buffers):
 // a parity wait on a buffer that has not completed its first phase yet would pass at once.

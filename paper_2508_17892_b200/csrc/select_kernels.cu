@@ -1123,8 +1123,7 @@ select_kernel(const ComboTable tbl, const SelectParams p) {
 // ---------------------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------------------
-size_t select_smem_bytes(long long L, int max_km, int budget, SelectParams* p) {
-  (void)budget;                                             // the output list (<= kMaxKm) fits the work area
+size_t select_smem_bytes(long long L, int max_km, SelectParams* p) {
   // quota walk: one or two staging buffers of max_km cell ids in the work area, the bitmap and its
   // summary (when they fit) behind it
   const size_t cap = (static_cast<size_t>(max_km < 1 ? 1 : max_km) + 3) & ~size_t(3);
