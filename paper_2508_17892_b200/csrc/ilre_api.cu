@@ -13,6 +13,7 @@
 #include "../../include/ilre_recall.h"
 #include "attn_kernels.cuh"
 #include "fill_kernels.cuh"
+#include "qk_geometry.cuh"
 #include "qk_kernels.cuh"
 #include "rerope_kernels.cuh"
 #include "sweep_kernels.cuh"
@@ -31,18 +32,8 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 constexpr int kNumStages = 4;            // timed stages (see ilre_recall_stage_times)
 constexpr int kProfRing = 32;            // runs whose stage events are kept for averaging
 constexpr int kMaxSinkStaging = 65536;
-constexpr int kPairMinRows = 192;        // query rows per kv head above which the paired scores pass is used
-constexpr int kPairMinTiles = 32;        // accumulators per CTA pair from which the paired scores pass is used
 static constexpr int kHostPieces = 16;              // most pieces of a pipelined host upload
 static constexpr long long kHostPieceMinKeys = 65536;   // no piece shorter than this (128-key multiple)
-
-struct PassGeometry {
-  int pair, n_rb, rb_rows, n_groups, cpg, n_tiles, stages;
-};
-struct Geometry {
-  int group_size, kv_rows;             // kv_rows: rows of one kv head in the packed query
-  PassGeometry stats, scores;
-};
 
 }  // namespace
 
@@ -142,63 +133,6 @@ struct DeviceGuard {
   }
   ~DeviceGuard() { if (prev >= 0) cudaSetDevice(prev); }
 };
-
-// Splits the rows of one kv head into blocks of at most max_rows, padded to a multiple of `unit`.
-void split_rows(int rows, int max_rows, int unit, PassGeometry* g) {
-  g->n_rb = (rows + max_rows - 1) / max_rows;
-  const int per = (rows + g->n_rb - 1) / g->n_rb;
-  g->rb_rows = ((per + unit - 1) / unit) * unit;
-}
-
-// Upper bound of the packed rows of one kv head, for any query of up to q_len tokens.
-int rows_padded_bound(int group_size, int q_len) {
-  const long long rg = static_cast<long long>(group_size) * q_len;
-  const long long n_rb = (rg + kMaxRbRows - 1) / kMaxRbRows, n_pair = (rg + kMaxPairRows - 1) / kMaxPairRows;
-  const long long stats = 128 * (n_rb + 1), pair = 256 * (n_pair + 1);     // paddings
-  return static_cast<int>(rg + (stats > pair ? stats : pair));
-}
-
-Geometry make_geometry(const ilre_recall_config_t& c, int n_sm, long long L, int q_len) {
-  Geometry g;
-  g.group_size = c.n_q_heads / c.n_kv_heads;
-  const int rg = g.group_size * q_len;
-  auto finish = [&](PassGeometry* p, int tile_keys, int workers) {
-    p->n_groups = c.n_kv_heads * p->n_rb;
-    p->n_tiles = static_cast<int>((L + tile_keys - 1) / tile_keys);
-    p->cpg = workers / p->n_groups;
-    if (p->cpg < 1) p->cpg = 1;
-    if (p->cpg > p->n_tiles) p->cpg = p->n_tiles;
-    const long long fixed = static_cast<long long>(p->rb_rows) * 256 + kSmemTailBytes +
-                            static_cast<long long>(p->rb_rows) * 4;
-    p->stages = static_cast<int>((kMaxDynSmem - fixed) / kStageBytes);
-    if (p->stages > kMaxStages) p->stages = kMaxStages;
-  };
-  g.stats.pair = 0;
-  split_rows(rg, kMaxRbRows, 128, &g.stats);
-  finish(&g.stats, kTileKeys, n_sm);
-  // Scores by CTA pairs, which pad the rows of a kv head to a multiple of 256 (single CTAs: to 32), where
-  // there are more than kPairMinRows rows, and where a pair has at least kPairMinTiles accumulators to
-  // compute, which pay for the cluster launch.  Scores pass, pairs / single CTAs, us:
-  //   rows, 128K keys: 148: 53.4 / 49.0; 192: 53.5 / 50.0; 256: 53.7 / 56.1; 280: 93.7 / 100.6;
-  //   400: 94.6 / 101.7; 560: 129.7 / 194.8; 800: 169 / 189 (a second tile of few rows starves the two
-  //   issuing threads of the single form); L = 1M, 1024 rows: 1414 / 1568.
-  //   accumulators: 57 (32K keys, 1024 rows) 55.2 / 56.4; 28 (32K, 512) 37.9 / 37.7; 14 (8K, 1024)
-  //   24.4 / 23.4.
-  PassGeometry pair;
-  split_rows(rg, kMaxPairRows, 256, &pair);
-  pair.pair = 1;
-  finish(&pair, kPairTileKeys, n_sm / 2);
-  pair.stages = 2;                       // the launcher sizes the ring
-  const long long accumulators = static_cast<long long>(pair.n_tiles) * (pair.rb_rows / 256);
-  const bool use_pair = rg > kPairMinRows && accumulators >= static_cast<long long>(kPairMinTiles) * pair.cpg;
-  g.scores = use_pair ? pair : g.stats;
-  // Where the two issuing threads take the key tiles in turn, a stage of the ring must always meet the
-  // same one: a parity wait is only sound for a thread that has seen the stage's phase before.
-  if (!use_pair && g.scores.rb_rows <= 256) g.scores.stages &= ~1;
-  const int a = g.stats.n_rb * g.stats.rb_rows, b = g.scores.n_rb * g.scores.rb_rows;
-  g.kv_rows = a > b ? a : b;
-  return g;
-}
 
 // One workspace buffer of the handle, followed by a guard zone of kGuardBytes that nothing may
 // write to (checked by ilre_recall_check_guards).
@@ -427,7 +361,7 @@ int recall_impl(ilre_recall_t* h, const void* k_cache_dev, int64_t L, const void
   DeviceGuard guard(h->cfg.device);
   if (!guard.ok) return ILRE_ERR_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-  const Geometry g = make_geometry(h->cfg, h->n_sm, L, q_len);
+  const Geometry g = make_geometry(h->cfg.n_kv_heads, h->cfg.n_q_heads, h->n_sm, L, q_len);
   if (g.stats.stages < 2 || g.scores.stages < 2) return ILRE_ERR_UNSUPPORTED;
 
   // combination table (Algorithm 1 loop order: max sizes outer, window sizes inner)

@@ -116,7 +116,7 @@ __device__ __forceinline__ void load_query_tile(const CUtensorMap* tmapQ, const 
 __device__ __forceinline__ void producer_loop(const CUtensorMap* tmapK, const CUtensorMap* tmapQ,
                                               const QkParams& p, const CtaItem& it,
                                               SmemTail* tail, uint32_t q_s, uint32_t k_s, bool down,
-                                              int skip_tiles = 0) {
+                                              int stages, int skip_tiles = 0) {
   volatile int* abort_flag = &tail->abort_flag;
   const uint32_t qf = smem_u32(&tail->q_full);
   mbar_arrive_expect_tx(qf, static_cast<uint32_t>(p.rb_rows) * 256u);
@@ -135,7 +135,7 @@ __device__ __forceinline__ void producer_loop(const CUtensorMap* tmapK, const CU
     const int row = (down ? it.tile_down(i) : it.tile_begin + i) * kTileKeys;
     tma_load_2d(k_s + s * kStageBytes, tmapK, it.g * 128, row, kf);
     tma_load_2d(k_s + s * kStageBytes + 16384, tmapK, it.g * 128 + 64, row, kf);
-    if (++s == p.stages) { s = 0; phase ^= 1u; }
+    if (++s == stages) { s = 0; phase ^= 1u; }
   }
 }
 
@@ -248,7 +248,7 @@ row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
       // may come in as SMs fall free.
       grid_dep_wait();
       grid_dep_launch();
-      producer_loop(&tmapK, &tmapQ, p, it, tail, q_s, k_s, false, p.skip_tiles);
+      producer_loop(&tmapK, &tmapQ, p, it, tail, q_s, k_s, false, p.stages, p.skip_tiles);
     }
   } else if (warp == 1 || warp >= 2 + kStatsConsumerWarps) {
     if (lane == 0 && run) {
@@ -492,8 +492,9 @@ scores_kernel(const __grid_constant__ CUtensorMap tmapK,
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const CtaItem it = decode_item(p, blockIdx.x);
   // query rows of the block, rounded up to the consumers' step of 32: the tensor time goes with them
-  const int n_rows = (min(p.rb_rows, p.rows_per_kv - (it.group % p.n_rb) * p.rb_rows) + 31) & ~31;
-  const int n_nh = (n_rows + 255) / 256;
+  const int n_rows = scores_block_rows(p.rb_rows, p.rows_per_kv, it.group % p.n_rb);
+  const int n_nh = scores_row_halves(n_rows);
+  const int stages = scores_ring_stages(p.stages, n_nh);
 
   // Two MMA-issuing threads (warps 1 and 2), one per accumulator buffer: tcgen05.mma holds its
   // issuing thread until the tensor pipe takes the instruction, so the waits and commits of
@@ -501,8 +502,7 @@ scores_kernel(const __grid_constant__ CUtensorMap tmapK,
   // issues one half of every tile and both release the tile's stage; with one, the threads
   // take the tiles in turn.
   const int k_releasers = (n_nh >= 2) ? 2 : 1;
-  const uint32_t tmem_base = cta_setup(tail, smem_base, p.stages, 2, kConsumerWarps, p.status,
-                                       k_releasers);
+  const uint32_t tmem_base = cta_setup(tail, smem_base, stages, 2, kConsumerWarps, p.status, k_releasers);
   const bool run = (it.n_tiles > 0) && (*abort_flag == 0);
 
   if (warp == 0) {
@@ -511,7 +511,7 @@ scores_kernel(const __grid_constant__ CUtensorMap tmapK,
       // one waited for, unless that was the prepare kernel itself
       if (p.group == 0 && mp.n_ext > 0) grid_dep_wait();
       grid_dep_launch();                 // the next kernel's CTAs may come in as SMs fall free
-      producer_loop(&tmapK, &tmapQ, p, it, tail, q_s, k_s, true);
+      producer_loop(&tmapK, &tmapQ, p, it, tail, q_s, k_s, true, stages);
     }
   } else if (warp == 1 || warp == 2) {
     if (lane == 0 && run) {
@@ -522,7 +522,7 @@ scores_kernel(const __grid_constant__ CUtensorMap tmapK,
       int s = -1;
       uint32_t kphase = 1;
       for (int i = 0; i < it.n_tiles && ok; ++i) {
-        if (++s == p.stages) s = 0;                      // stage and phase of key tile i
+        if (++s == stages) s = 0;                        // stage and phase of key tile i
         if (s == 0) kphase ^= 1u;
         if (n_nh == 1 && ((static_cast<uint32_t>(i) & 1u) != mine)) { ++u; continue; }
         ok = mbar_wait(smem_u32(&tail->k_full[s]), kphase, abort_flag, p.status, kDevWaitKFull);
@@ -913,7 +913,7 @@ static cudaError_t launch_scores_pair_mt(const CUtensorMap& tk, const CUtensorMa
   constexpr int kFixed = MT * 128 * 256 + kSmemTailBytes + MT * 256 * static_cast<int>(sizeof(float));
   constexpr int kUnits = (kMaxDynSmem - kFixed) / kUnitBytes < kMaxUnits ? (kMaxDynSmem - kFixed) / kUnitBytes
                                                                          : kMaxUnits;
-  // the issuing threads take the tiles of two units in turn with one row tile; see make_geometry
+  // the issuing threads take the tiles of two units in turn with one row tile; see scores_ring_stages
   static_assert(MT > 1 || kUnits % 4 == 0, "a ring unit must always meet the same issuing thread");
   p.stages = kUnits;
   const size_t smem = static_cast<size_t>(kFixed) + static_cast<size_t>(p.stages) * kUnitBytes;

@@ -39,6 +39,22 @@ static constexpr int kPairThreads = 640;           // warp 0 TMA, warps 1-2 MMA,
 // instead of the special-function unit (0 = none).  Balances the two pipes.
 static constexpr int kRowStatsPolyPairs = 4;
 
+// Scores by single CTAs: row halves of 256 (accumulators per key tile) of row block `block`, whose rows past
+// those of its kv head are left out, in steps of 32.
+__host__ __device__ constexpr int scores_block_rows(int rb_rows, int rows_per_kv, int block) {
+  const int left = rows_per_kv - block * rb_rows;
+  return ((left < rb_rows ? left : rb_rows) + 31) & ~31;
+}
+__host__ __device__ constexpr int scores_row_halves(int block_rows) { return (block_rows + 255) / 256; }
+// ... and the stages of the ring that such a block uses.  With one row half the two issuing threads take the
+// key tiles in turn.  A parity wait is only sound for a thread that has seen the stage's phase before, so
+// there a stage must always meet the same thread: an even ring.  A last block of few rows beside full
+// ones, whose ring may be odd, has at most half of their work, so the stage it gives up costs nothing
+// (1190 rows per kv head, 16384 keys: 29.4 us; all blocks with two row halves and three stages 29.1).
+__host__ __device__ constexpr int scores_ring_stages(int stages, int row_halves) {
+  return row_halves == 1 ? stages & ~1 : stages;
+}
+
 // Geometry of one pass.
 struct QkParams {
   long long L;

@@ -131,12 +131,14 @@ BIG = [
 
 # Query and key sizes of the paired scores pass: 1 to 4 row tiles per CTA, two row blocks per kv
 # head, contexts that end in the first or the second CTA's keys of the last tile, padded rows, and
-# the sizes one step below the dispatch's line (single CTAs).  (L, q_len, n_kv, n_q)
+# single CTAs of one and of several row blocks.  (L, q_len, n_kv, n_q)
 PAIRED = [(75777, 64, 8, 32), (75649, 33, 8, 64), (39001, 128, 8, 32), (26113, 192, 8, 32),
           (25801, 100, 4, 28), (20479, 256, 8, 32), (16640, 511, 4, 16), (9472, 512, 4, 16),
           # padded to more rows than the statistics pass; up to 192 rows single CTAs, in steps of 32 rows
           (40001, 70, 8, 32), (60001, 129, 2, 8), (75001, 48, 8, 32), (75001, 49, 8, 32), (20001, 8, 8, 32),
-          (20001, 9, 8, 32), (20001, 37, 8, 32), (3001, 24, 4, 28), (3001, 19, 1, 7)]
+          (20001, 9, 8, 32), (20001, 37, 8, 32), (3001, 24, 4, 28), (3001, 19, 1, 7),
+          # single CTAs, several row blocks of 512 whose last one has at most 256 live rows
+          (20001, 170, 4, 28), (15001, 230, 4, 28), (9001, 300, 8, 32)]
 
 
 @pytest.mark.parametrize("case", PAIRED, ids=lambda c: f"L{c[0]}_q{c[1]}_kv{c[2]}_h{c[3]}")

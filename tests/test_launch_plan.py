@@ -1,0 +1,67 @@
+"""Host-side launch rules, compiled from the library's headers with the host compiler and checked over
+ranges of sizes.  No GPU."""
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2508_17892_b200", "csrc")
+CUDA = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+
+
+def _run(tmp_path, body):
+    src, exe = tmp_path / "check.cpp", tmp_path / "check"
+    src.write_text(body)
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-I", CSRC, "-I", os.path.join(CUDA, "include"),
+                           "-x", "c++", str(src), "-o", str(exe)])
+    r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, r.stdout[-2000:]
+    return r.stdout
+
+
+RINGS = r"""
+#include <cstdio>
+#include <cstring>
+#include "qk_geometry.cuh"
+using namespace ilre;
+int main() {
+  const int heads[][2] = {{8, 32}, {4, 28}, {8, 64}, {2, 16}, {4, 16}, {1, 7}, {2, 8}, {7, 7}};
+  const long long lengths[] = {1, 129, 1000, 4096, 9001, 16384, 24001, 49001, 131072, 1048576};
+  long long blocks = 0, in_turn = 0, short_last = 0, bad = 0;
+  for (const auto& h : heads)
+    for (long long L : lengths)
+      for (int q_len = 1; q_len <= 640; ++q_len) {
+        const Geometry g = make_geometry(h[0], h[1], 148, L, q_len);
+        if (g.scores.pair) continue;
+        const int rows = g.group_size * q_len;
+        int covered = 0;
+        for (int b = 0; b < g.scores.n_rb; ++b, ++blocks) {
+          const int block_rows = scores_block_rows(g.scores.rb_rows, rows, b);
+          const int halves = scores_row_halves(block_rows);
+          const int ring = scores_ring_stages(g.scores.stages, halves);
+          covered += block_rows;
+          bool ok = block_rows > 0 && block_rows <= g.scores.rb_rows && halves <= 2 && ring >= 2 &&
+                    ring <= g.scores.stages;
+          if (halves == 1) {             // tile i: issuing thread i % 2, stage i % ring
+            ++in_turn;
+            short_last += g.scores.rb_rows > 256;
+            for (int i = 0; i < 4 * ring; ++i) ok = ok && ((i % ring) & 1) == (i & 1);
+          }
+          if (!ok && bad++ < 5)
+            std::printf("heads %d/%d L %lld q_len %d block %d: %d rows, ring %d\n", h[0], h[1], L, q_len, b,
+                        block_rows, ring);
+        }
+        if (covered < rows && bad++ < 5) std::printf("rows not covered: %d of %d\n", covered, rows);
+      }
+  std::printf("%lld blocks, %lld in turn, %lld of them short last blocks\n", blocks, in_turn, short_last);
+  return bad || !in_turn || !short_last;
+}
+"""
+
+
+def test_a_ring_stage_always_meets_the_same_issuing_thread(tmp_path):
+    """Single-CTA scores pass: where the two issuing threads take the key tiles in turn, a stage must not
+    change hands (a parity wait is only sound for a thread that has seen the phase before), in every
+    row block of a launch: the last one may have few live rows beside full ones."""
+    _run(tmp_path, RINGS)
