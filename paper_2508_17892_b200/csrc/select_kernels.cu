@@ -190,8 +190,8 @@ __device__ __forceinline__ float score_at(const SelectParams& p, long long t) {
 
 // Phase A for one tile of source `src`: cells of MaxPooling(size = stride = m), a shorter
 // last cell where m does not divide the length.  The tokens are read coalesced into `buf`
-// (kSrcTileTokens words), all loads in flight together; the maximum is taken of the encoded
-// scores, whose order is the scores', and one exponential per cell.
+// (kSrcTileTokens words), all loads in flight together; of encoded scores the maximum is taken before
+// they are decoded (their order is the scores'), one exponential per cell.
 __device__ __forceinline__ void maxpool_tile(const ComboTable& tbl, const SelectParams& p, int src,
                                              int tile_in_src, uint32_t* buf) {
   const int m = tbl.src_m[src], len = tbl.src_len[src];
@@ -203,24 +203,35 @@ __device__ __forceinline__ void maxpool_tile(const ComboTable& tbl, const Select
   const long long t0 = static_cast<long long>(c0) * m;
   const int n_tok = static_cast<int>(min(static_cast<long long>(n_cells) * m, Lp - t0));
   constexpr int kLd = kSrcTileTokens / kSelThreads;
+  const uint32_t pad = p.scores_given ? __float_as_uint(-INFINITY) : 0u;        // below every score
   uint32_t v[kLd];
 #pragma unroll
   for (int k = 0; k < kLd; ++k) {
     const int i = k * kSelThreads + threadIdx.x;
-    v[k] = (i < n_tok) ? __ldcg(a + t0 + i) : 0u;
-    if (p.scores_given && i < n_tok) v[k] = float_to_ordered(__uint_as_float(v[k]));
+    v[k] = (i < n_tok) ? __ldcg(a + t0 + i) : pad;
   }
 #pragma unroll
-  for (int k = 0; k < kLd; ++k) buf[k * kSelThreads + threadIdx.x] = v[k];      // 0: below every score
+  for (int k = 0; k < kLd; ++k) buf[k * kSelThreads + threadIdx.x] = v[k];
   __syncthreads();
   float* out = p.maxpooled + static_cast<long long>(src) * p.maxpooled_stride;
   for (int c = threadIdx.x; c < n_cells; c += kSelThreads) {
-    uint32_t acc = buf[c * m];
-    for (int j = 1; j < m; ++j) acc = max(acc, buf[c * m + j]);
-    out[c0 + c] = p.scores_given ? ordered_to_float(acc) : exp2f(ordered_to_float(acc));
+    if (p.scores_given) {                  // as floats: a NaN does not win
+      float acc = __uint_as_float(buf[c * m]);
+      for (int j = 1; j < m; ++j) acc = fmaxf(acc, __uint_as_float(buf[c * m + j]));
+      out[c0 + c] = acc;
+    } else {
+      uint32_t acc = buf[c * m];
+      for (int j = 1; j < m; ++j) acc = max(acc, buf[c * m + j]);
+      out[c0 + c] = exp2f(ordered_to_float(acc));
+    }
   }
   __syncthreads();
 }
+
+// A pooled value as it is stored: no NaN, since the histogram, the gather and the ranking must agree on
+// where every cell belongs (a cell counted and not found leaves a hole in the candidate list).  A NaN (of
+// given scores, or of positions that a scores pass which gave up never reached) ranks below every score.
+__device__ __forceinline__ float ranked_value(float v) { return (v == v) ? v : -0.f; }
 
 // Counts the bin of one cell per lane (-1: none).  Neighbouring cells of a window maximum are often
 // equal: the first lane of a run of equal bins adds the whole run.
@@ -287,7 +298,7 @@ __device__ __forceinline__ void pool_tile(const ComboTable& tbl, const SelectPar
         const int i = base + threadIdx.x;
         int bin = -1;
         if (i < n_out) {
-          const float acc = fmaxf(s0[i], s0[i + n - w]);
+          const float acc = ranked_value(fmaxf(s0[i], s0[i + n - w]));
           out[i] = acc;
           bin = bin_of_ordered(float_to_ordered(acc));
         }
@@ -315,7 +326,7 @@ __device__ __forceinline__ void pool_tile(const ComboTable& tbl, const SelectPar
         const int c = i - (n_max / 2 - n / 2);             // cell of the window that starts here
         int bin = -1;
         if (c >= 0 && c < n_out) {
-          const float avg = acc / static_cast<float>(n);
+          const float avg = ranked_value(acc / static_cast<float>(n));
           p.pooled[static_cast<long long>(combo) * p.pooled_stride + c0 + c] = avg;
           bin = bin_of_ordered(float_to_ordered(avg));
         }

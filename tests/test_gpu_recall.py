@@ -197,6 +197,44 @@ def test_window_groups_match_oracle(case):
     eng.close()
 
 
+# Given scores with NaNs: a window average with a NaN in it ranks below every score, a maximum takes the
+# numbers beside it.  Few NaNs, more than are ranked, NaNs among the chosen cells, more NaNs at the
+# threshold than its bin may bring.  (L, budget, NaNs, max_size, win_size, win_op)
+NANS = [(5000, 300, 3, 1, 1, 1), (40001, 300, 301, 1, 1, 1), (40001, 300, 6000, 3, 1, 1), (40001, 300, 40, 1, 5, 0),
+        (5000, 300, 400, 1, 7, 1), (40001, 900, 9000, 2, 4, 0), (5000, 4990, 300, 1, 1, 0), (9000, 4000, 6000, 1, 1, 1),
+        (5000, 0, 9, 1, 1, 1)]
+
+
+def _one_combination(scores, budget, m, n, win_op):
+    """Algorithm 1 with one combination in numpy, fp32."""
+    a = np.concatenate([scores, np.full(-len(scores) % m, np.nan, np.float32)])
+    cells = np.fmax.reduce(a.reshape(-1, m), axis=1)
+    pad = np.float32(-np.inf if win_op else 0.0)
+    w = np.concatenate([np.full(n // 2, pad), cells, np.full(n, pad)]).astype(np.float32)
+    v = w[:len(cells)].copy() if win_op else np.zeros(len(cells), np.float32) + w[:len(cells)]
+    for j in range(1, n):
+        v = np.fmax(v, w[j:j + len(cells)]) if win_op else v + w[j:j + len(cells)]
+    v = v if win_op else v / np.float32(n)
+    order = np.argsort(-np.where(np.isnan(v), np.float32(-1), v), kind="stable")
+    tokens = (order[:, None] * m + np.arange(m)[None, :]).ravel()
+    return np.sort(tokens[tokens < len(scores)][:budget])
+
+
+@pytest.mark.parametrize("case", NANS, ids=lambda c: f"L{c[0]}_B{c[1]}_{c[2]}nans_m{c[3]}_n{c[4]}_op{c[5]}")
+def test_nans_in_given_scores_rank_last(case):
+    from paper_2508_17892_b200 import IlreRecall
+    L, budget, n_nan, m, n, op = case
+    rng = np.random.default_rng(L + n_nan)
+    scores = (rng.random(L) ** 8).astype(np.float32) + np.float32(1e-12)
+    scores[rng.permutation(L)[:n_nan]] = np.nan
+    eng = IlreRecall(max_L=L, max_q_len=1, max_budget=budget, n_kv_heads=1, n_q_heads=1)
+    got = eng.allocate(torch.from_numpy(scores).cuda(), budget, (m,), (n,), op)
+    eng.check_status()
+    assert np.array_equal(got.cpu().numpy(), _one_combination(scores, budget, m, n, op))
+    assert eng.check_guards() == 0, "a kernel wrote past the end of a workspace buffer"
+    eng.close()
+
+
 @pytest.mark.parametrize("pattern", ["all_equal", "two_levels", "blocks_of_equal", "all_equal_40k",
                                      "blocks_of_equal_40k", "all_equal_40k_B6000",
                                      "blocks_of_equal_40k_B6000"])
