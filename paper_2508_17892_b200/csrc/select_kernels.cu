@@ -163,8 +163,6 @@ __device__ __forceinline__ int combo_of_tile(const ComboTable& tbl, int tile, in
 
 static constexpr int kTilePer = kSelTile / kSelThreads;
 static constexpr int kMaxWalkWarps = kSelThreads / 32;
-static constexpr int kWalkCells = 2;      // ranked cells per thread of the quota walk, for the longest list
-static constexpr int kMinWalkers = 128;   // fewest threads that walk
 static constexpr int kScanGroup = 4;      // tiles whose loads are issued together (long way)
 static constexpr int kGatherGroup = 4;    // the same in the gather
 
@@ -549,8 +547,8 @@ enum : int {
 };
 
 // Tokens of cell `cell` (size m) that are not allocated yet, as a bit mask (bit j = token j).  Positions
-// fit 32 bits (L < 2^31).  Words past the bitmap's end may be read (there is memory behind it) but
-// their bits are masked.
+// fit 32 bits (L < 2^31).  Up to two words past the bitmap's end may be read (kSelBitmapSlackWords of
+// memory lie behind it) but their bits are masked.
 template <int kCells, bool kSmem>
 __device__ __forceinline__ auto fresh_tokens(const uint32_t* bm, int cell, int m, int Lp) {
   const int t0 = cell * m;
@@ -1134,19 +1132,6 @@ select_kernel(const ComboTable tbl, const SelectParams p) {
 // ---------------------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------------------
-size_t select_smem_bytes(long long L, int max_km, SelectParams* p) {
-  // quota walk: one or two staging buffers of max_km cell ids in the work area, the bitmap and its
-  // summary (when they fit) behind it
-  const size_t cap = (static_cast<size_t>(max_km < 1 ? 1 : max_km) + 3) & ~size_t(3);
-  const size_t words = (static_cast<size_t>((L + 31) / 32) + 3) & ~size_t(3);
-  p->bitmap_in_smem = words * sizeof(uint32_t) <= static_cast<size_t>(kSelBitmapSmemBytes) ? 1 : 0;
-  int walkers = ((max_km + kWalkCells - 1) / kWalkCells + 31) & ~31;
-  p->walk_threads = walkers < kMinWalkers ? kMinWalkers : (walkers > kSelThreads ? kSelThreads : walkers);
-  p->stage_capacity = static_cast<int>(cap);
-  p->stage_double = (2 * cap * sizeof(int) <= static_cast<size_t>(kSelWorkBytes)) ? 1 : 0;
-  return kSelWorkBytes + (p->bitmap_in_smem ? (words + (words + 31) / 32) * sizeof(uint32_t) : 0);
-}
-
 cudaError_t select_max_grid(int n_sm, int* max_grid) {
   cudaError_t e = cudaFuncSetAttribute(select_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kSelMaxDynSmemBytes);

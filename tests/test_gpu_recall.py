@@ -181,6 +181,7 @@ def test_selection_kernel_edge_paths(case):
 # number of tiles.  (L, budget, max_sizes, win_sizes, win_op, n_sink)
 GROUPS = [(5000, 300, (1,), (63, 1, 200, 7, 31, 15), 1, 0), (3073, 200, (3, 1, 2), (16, 5, 1, 9, 2, 1024), 0, 4),
           (260, 20, (4, 1), (1024, 3, 2, 600, 1, 5, 9), 1, 3), (40, 9, (1, 64), (7, 100, 1), 0, 0),
+          (128, 30, (33, 63), (1, 3), 1, 0), (1024, 90, (33, 49), (2,), 0, 0),    # last cells that end with a bitmap word
           (33025, 700, (1, 2), (31, 4, 8, 16, 2, 64, 1, 128, 256, 512, 1024), 1, 1),
           (150000, 4096, (1,), (5, 4, 3, 2, 1, 6, 7), 0, 0)]
 

@@ -65,3 +65,39 @@ def test_a_ring_stage_always_meets_the_same_issuing_thread(tmp_path):
     change hands (a parity wait is only sound for a thread that has seen the phase before), in every
     row block of a launch: the last one may have few live rows beside full ones."""
     _run(tmp_path, RINGS)
+
+
+WALK = r"""
+#include <cstdio>
+#include "select_kernels.cuh"
+using namespace ilre;
+int main() {
+  int bad = 0;
+  long long past_end = 0;
+  for (long long L = 1; L <= 5000; L += (L < 1100 ? 1 : 97))
+    for (int n_sink = 0; n_sink < 5 && n_sink < L; n_sink += 4) {
+      SelectParams p;
+      const size_t bytes = select_smem_bytes(L, 1, &p);
+      const int Lp = static_cast<int>(L) - n_sink;
+      if (!p.bitmap_in_smem || bytes > static_cast<size_t>(kSelMaxDynSmemBytes)) ++bad;
+      for (int m = 1; m <= kMaxMaxSize; ++m) {
+        int last = 0;                    // last bitmap word that the walk reads for any cell
+        for (int t0 = 0; t0 < Lp; t0 += m) {
+          const int w = (t0 >> 5) + (32 % m == 0 ? 0 : m <= 32 ? 1 : (t0 & 31) ? 2 : 1);
+          last = w > last ? w : last;
+        }
+        past_end += last >= (L + 31) / 32;
+        if (kSelWorkBytes + 4 * static_cast<size_t>(last + 1) > bytes && bad++ < 5)
+          std::printf("L %lld sink %d m %d: word %d read, %zu bytes\n", L, n_sink, m, last, bytes);
+      }
+    }
+  std::printf("%lld cases read past the bitmap\n", past_end);
+  return bad || !past_end;
+}
+"""
+
+
+def test_the_quota_walk_reads_inside_its_shared_memory(tmp_path):
+    """A cell of more than 32 tokens is read as three bitmap words, the last of which may lie behind the
+    bitmap: the launch asks for that memory too."""
+    _run(tmp_path, WALK)
