@@ -274,11 +274,12 @@ fill_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ C
         for (int j = 0; j < 16; j += 2) {
           float l0 = v_lo[j], l1 = v_lo[j + 1], h0 = v_hi[j], h1 = v_hi[j + 1];
           if (p.bias) {
+            // ordinary loads: the kernel before this one may have written the bias
             const uint16_t* bp = p.bias + head * 128 + c0 + j;
-            l0 += __uint_as_float(static_cast<uint32_t>(__ldg(bp)) << 16);
-            l1 += __uint_as_float(static_cast<uint32_t>(__ldg(bp + 1)) << 16);
-            h0 += __uint_as_float(static_cast<uint32_t>(__ldg(bp + 64)) << 16);
-            h1 += __uint_as_float(static_cast<uint32_t>(__ldg(bp + 65)) << 16);
+            l0 += __uint_as_float(static_cast<uint32_t>(bp[0]) << 16);
+            l1 += __uint_as_float(static_cast<uint32_t>(bp[1]) << 16);
+            h0 += __uint_as_float(static_cast<uint32_t>(bp[64]) << 16);
+            h1 += __uint_as_float(static_cast<uint32_t>(bp[65]) << 16);
           }
           const __nv_bfloat162 pl = __floats2bfloat162_rn(fmaf(l0, cs[j], -h0 * sn[j]),
                                                           fmaf(l1, cs[j + 1], -h1 * sn[j + 1]));

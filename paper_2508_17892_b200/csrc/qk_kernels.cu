@@ -842,8 +842,10 @@ scores_pair_kernel(const __grid_constant__ CUtensorMap tmapK,
 // TMA box cannot collect from the caller's array),
 // and clears the per-run state (encoded scores, empty bitmap, selection
 // state).
-__global__ void prepare_kernel(const uint4* __restrict__ q, uint4* __restrict__ qp, PrepParams p) {
-  grid_dep_wait();                       // the run before this one may still use the buffers
+__global__ void prepare_kernel(const uint4* q, uint4* qp, PrepParams p) {
+  // The run before this one may still use the buffers, and whatever was before it may have written the
+  // query: no read through the non-coherent path.
+  grid_dep_wait();
   grid_dep_launch();                     // the next kernel sets itself up meanwhile
   const long long tid = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   const long long nthreads = static_cast<long long>(gridDim.x) * blockDim.x;
@@ -856,7 +858,7 @@ __global__ void prepare_kernel(const uint4* __restrict__ q, uint4* __restrict__ 
     uint4 val = make_uint4(0, 0, 0, 0);
     if (rg < p.group_size * p.q_len) {
       const int i = rg / p.group_size, j = rg % p.group_size;
-      val = q[(static_cast<long long>(i) * p.n_q + g * p.group_size + j) * 16 + part];
+      val = __ldcg(q + (static_cast<long long>(i) * p.n_q + g * p.group_size + j) * 16 + part);
     }
     qp[e] = val;
   }

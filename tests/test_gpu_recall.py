@@ -492,7 +492,8 @@ def test_recalls_in_a_row_on_a_side_stream_keep_their_own_results():
 def test_every_kernel_waits_for_the_call_before_it(n_kv, n_q, L, q_len, captured):
     """Each kernel may start while the one before it ends.  Fill, Eq. 7, recall, attention and the
     allocation of given scores, in a row through the same buffers, give what they give with a
-    synchronisation after every call; in a graph, behind a join of two streams too."""
+    synchronisation after every call; in a graph, behind a join of two streams too.  The bias and the
+    query are rewritten in place by the kernel just before the call that reads them."""
     from paper_2508_17892_b200 import IlreRecall
     rounds, d_model, chunk = 4, 64, 256
     g = torch.Generator(device="cuda").manual_seed(5)
@@ -501,6 +502,8 @@ def test_every_kernel_waits_for_the_call_before_it(n_kv, n_q, L, q_len, captured
     Q = [rand(q_len, n_q, 128) for _ in range(rounds)]
     A = rand(chunk, n_q, 128)
     W = rand(n_kv * 128, d_model) / 8
+    bias = [rand(n_kv * 128) for _ in range(rounds)]
+    q_now, bias_now = torch.empty_like(Q[0]), torch.empty_like(bias[0])
     eng = IlreRecall(max_L=L, max_q_len=q_len, max_budget=128, n_kv_heads=n_kv, n_q_heads=n_q)
     cache = torch.zeros(L, n_kv, 128, dtype=torch.bfloat16, device="cuda")
     turned = torch.zeros_like(cache)
@@ -511,11 +514,15 @@ def test_every_kernel_waits_for_the_call_before_it(n_kv, n_q, L, q_len, captured
     def sequence(after):
         results = []
         for i in range(rounds):
-            eng.fill_keys(X[i], W, cache, 0, stream=side)
+            bias_now.copy_(bias[i])
+            bias_now.neg_()
+            eng.fill_keys(X[i], W, cache, 0, bias=bias_now, stream=side)
             after()
+            q_now.copy_(Q[i])
             eng.rerope_keys(cache, chunk, out=turned, stream=side)
             after()
-            idx, _ = eng.run(turned, Q[i], 128, (1,), (1, 7), 1, 4, out_scores=given, stream=side)
+            q_now.neg_()
+            idx, _ = eng.run(turned, q_now, 128, (1,), (1, 7), 1, 4, out_scores=given, stream=side)
             after()
             again = eng.allocate(given, 100, (2,), (5,), 1, stream=side)
             after()
