@@ -173,6 +173,12 @@ fill_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ C
           }
         }
       }
+      // The releases of the last blocks, which no load waits for, arrive in both CTAs' barriers: this CTA
+      // must not leave before they have.
+      for (int j = 0; j < kFillStages && ok; ++j) {
+        ok = mbar_wait(smem_u32(&tail->empty[s]), phase ^ 1u, abort_flag, p.status, kDevWaitKEmpty);
+        if (++s == kFillStages) { s = 0; phase ^= 1u; }
+      }
     }
   } else if (warp == 1) {
     if (lane == 0 && run && rank == 0) {
@@ -302,7 +308,8 @@ fill_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ C
       }
     }
   }
-  // Neither CTA may leave while the other can still signal its barriers or read its operands.
+  // Neither CTA may leave while the other can still signal its barriers or read its operands (every commit
+  // has been waited for, by the epilogue warps or by the loading threads).
   tc_fence_before();
   __syncwarp();
   cluster_sync_all();

@@ -665,6 +665,12 @@ __device__ __forceinline__ void pair_producer_loop(const CUtensorMap* tmapK, con
       else tma_load_2d_pair(dst, tmapQ, kb * 64, it.g * p.kv_rows + row, cluster_addr(qf, 0));
     }
   for (; n < n_units && ok; ++n) ok = load_unit(n);
+  // The releases of the last units, which no load waits for, arrive in both CTAs' barriers: this CTA must
+  // not leave before they have.
+  for (int j = 0; j < units && ok; ++j) {
+    ok = mbar_wait(smem_u32(&tail->k_empty[s]), phase ^ 1u, abort_flag, p.status, kDevWaitKEmpty);
+    if (++s == units) { s = 0; phase ^= 1u; }
+  }
 }
 
 // One of the two MMA-issuing threads of a pair (first CTA, warps 1 and 2), one per accumulator:
@@ -824,7 +830,8 @@ scores_pair_kernel(const __grid_constant__ CUtensorMap tmapK,
       if (ok && t < p.L) atomicMax(p.enc + t, float_to_ordered(fmaxf(fmaxf(b0, b1), fmaxf(b2, b3))));
     }
   }
-  // Neither CTA may leave while the other can still signal its barriers or read its operands.
+  // Neither CTA may leave while the other can still signal its barriers or read its operands (every commit
+  // has been waited for, by the consumers or by the loading thread).
   tc_fence_before();
   __syncwarp();
   cluster_sync_all();
