@@ -55,7 +55,7 @@ __device__ __forceinline__ int bin_of_ordered(uint32_t o) {
 }
 
 struct SelShared {
-  uint32_t hist[kHistBins];
+  alignas(8) uint32_t hist[kHistBins];     // (the ranking's scratch after the scans)
   uint32_t above[kHistBins + 1];           // of one combination: [b + 1] values in the bins above bin b; [0] all
   uint32_t scan[33];
   int flag;
@@ -459,16 +459,102 @@ __device__ __forceinline__ void bin_search(const SelectParams& p, const uint32_t
 
 // Phase E: ranks the candidates [lo, hi) of `combo`, which are sorted by bin: the rank of a candidate is
 // where its bin's segment begins plus the keys of the segment above its own (keys are distinct).  The
-// segments that the range touches are staged in shared memory, kRankChunk keys at a time; several
+// segments that the range touches (`unsorted`, after the long way: all is one segment) are staged in
+// shared memory, kRankChunk keys at a time; several
 // threads share a candidate when there are threads to spare.  Ranks past K_m are not wanted.
+//
+// A bin may hold thousands of candidates (scores that lie close together, ties), and one CTA may have all
+// of them: the early combinations want few cells and get one CTA, and the threshold bin brings up to
+// kCandSlack.  Comparing them all costs 20 us per million comparisons and CTA, so from kRankDense
+// comparisons on, the keys of the range's segments are first dealt out to kRankBuckets value ranges
+// between as many sampled keys (taken at even strides, ranked among themselves), and a candidate is compared
+// with its own range only.  The line: 4096 positions in [1/2, 1), 3 windows, 12.3 us compared, 9.1 dealt
+// out; 131072 positions that took the long way 16.7 and 11.6.  Phase E with everything compared -> as it
+// stands: 4096 positions within 0.1 % of each other, 3 windows, 127 -> 17 us; 131072 in [1/2, 1), 48
+// combinations, 472 -> 27; log-normal scores 4.3 and 7.2 us -> 4.6 and 4.7 (the CTA's list is found by all threads).
 static constexpr int kRankChunk = 8192;
+static constexpr int kRankBuckets = 256;
+static constexpr int kRankDense = 150000;
+
+struct RankScratch {
+  unsigned long long samp[kRankBuckets];
+  unsigned long long spl[kRankBuckets];    // the samples in descending order; the last entry is unused
+  uint32_t rank[kRankBuckets];
+  uint32_t count[kRankBuckets];
+  uint32_t start[kRankBuckets + 1];
+};
+static_assert(sizeof(RankScratch) <= sizeof(SelShared::hist), "the scratch takes the histogram's place");
+
+// Ranks the keys [lo, hi) of cand[0 .. n), kRankBuckets <= n <= kRankChunk; ranks from `limit` on are not wanted.
+__device__ __noinline__ void rank_dense(const unsigned long long* cand, int* ranked, int n, int lo, int hi, int limit,
+                                        unsigned long long* grouped, SelShared* sh) {
+  RankScratch* rs = reinterpret_cast<RankScratch*>(sh->hist);
+  constexpr int kLd = kRankChunk / kSelThreads;
+  const int tid = threadIdx.x;
+  unsigned long long v[kLd];
+#pragma unroll
+  for (int k = 0; k < kLd; ++k) {
+    const int i = k * kSelThreads + tid;
+    v[k] = (i < n) ? __ldcg(&cand[i]) : 0ull;
+  }
+  if (tid < kRankBuckets) {                                 // (the caller's vote freed the scratch and the chunk)
+    rs->samp[tid] = __ldcg(&cand[tid * n / kRankBuckets]);
+    rs->rank[tid] = 0;
+    rs->count[tid] = 0;
+  }
+  __syncthreads();
+  {                                                         // rank the samples among themselves
+    constexpr int kPer = kRankBuckets / (kSelThreads / kRankBuckets);
+    const int si = tid % kRankBuckets, j0 = (tid / kRankBuckets) * kPer;
+    const unsigned long long mine = rs->samp[si];
+    uint32_t above = 0;
+#pragma unroll 8
+    for (int j = 0; j < kPer; ++j) above += (rs->samp[j0 + j] > mine) ? 1u : 0u;
+    if (above) atomicAdd(&rs->rank[si], above);
+  }
+  __syncthreads();
+  if (tid < kRankBuckets) rs->spl[rs->rank[tid]] = rs->samp[tid];
+  __syncthreads();
+  uint32_t where[kLd];                                      // bucket << 16 | slot inside the bucket
+#pragma unroll
+  for (int k = 0; k < kLd; ++k) {
+    const int i = k * kSelThreads + tid;
+    if (i < n) {
+      int b = 0;                                            // samples above the key, the last one left out
+#pragma unroll
+      for (int step = kRankBuckets / 2; step >= 1; step >>= 1)
+        if (rs->spl[b + step - 1] > v[k]) b += step;
+      where[k] = (static_cast<uint32_t>(b) << 16) | atomicAdd(&rs->count[b], 1u);
+    }
+  }
+  __syncthreads();
+  uint32_t total;
+  const uint32_t before = block_exclusive_scan(tid < kRankBuckets ? rs->count[tid] : 0u, sh->scan, &total);
+  if (tid <= kRankBuckets) rs->start[tid] = before;
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < kLd; ++k) {
+    const int i = k * kSelThreads + tid;
+    if (i < n) grouped[rs->start[where[k] >> 16] + (where[k] & 0xFFFFu)] = v[k];
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < kLd; ++k) {
+    const int i = k * kSelThreads + tid;
+    if (i < lo || i >= hi) continue;
+    const int first = static_cast<int>(rs->start[where[k] >> 16]), last = static_cast<int>(rs->start[(where[k] >> 16) + 1]);
+    int rank = first;
+#pragma unroll 4
+    for (int j = first; j < last; ++j) rank += (grouped[j] > v[k]) ? 1 : 0;
+    if (rank < limit) ranked[rank] = static_cast<int>(0xFFFFFFFFu - static_cast<uint32_t>(v[k] & 0xFFFFFFFFull));
+  }
+}
 
 __device__ __forceinline__ void rank_range(const SelectParams& p, const ComboTable& tbl, int combo, int n, int lo, int hi,
-                                           unsigned long long* chunk) {
+                                           bool unsorted, unsigned long long* chunk, SelShared* sh) {
   const unsigned long long* cand = p.cand + static_cast<long long>(combo) * p.cand_stride;
   const uint32_t* seg = p.cand_seg + static_cast<long long>(combo) * p.cand_stride;
   int* ranked = p.ranked + static_cast<long long>(combo) * p.cand_stride;
-  const bool unsorted = __ldcg(&p.cand_count[kMaxCombos + combo]) != 0u;     // came the long way: one segment
   const int k_m = tbl.k_m[combo];
   for (int c0 = lo; c0 < hi; c0 += kSelThreads) {
     const int nc = min(kSelThreads, hi - c0);
@@ -484,10 +570,19 @@ __device__ __forceinline__ void rank_range(const SelectParams& p, const ComboTab
     const int begin = static_cast<int>(s_first & 0xFFFFu);
     const int end = static_cast<int>((s_last & 0xFFFFu) + (s_last >> 16));
     const int first = static_cast<int>(s_mine & 0xFFFFu), last = first + static_cast<int>(s_mine >> 16);
+    // the vote is also the barrier behind the previous users of the chunk
+    if (__syncthreads_or(active && (last - first) * (hi - c0) > kRankDense)) {
+      const uint32_t s_end = unsorted ? whole : __ldcg(&seg[hi - 1]);
+      const int len = static_cast<int>((s_end & 0xFFFFu) + (s_end >> 16)) - begin;
+      if (len >= kRankBuckets && len <= kRankChunk) {       // uniform
+        rank_dense(cand + begin, ranked + begin, len, c0 - begin, hi - begin, k_m - begin, chunk, sh);
+        return;
+      }
+    }
     int above = 0;
     for (int base = begin; base < end; base += kRankChunk) {
       const int cnt = min(kRankChunk, end - base);
-      __syncthreads();                                      // previous users of the chunk
+      if (base > begin) __syncthreads();                    // previous users of the chunk
       for (int i = threadIdx.x; i < cnt; i += kSelThreads) chunk[i] = __ldcg(&cand[base + i]);
       __syncthreads();
       if (active) {
@@ -1083,34 +1178,35 @@ select_kernel(const ComboTable tbl, const SelectParams p) {
   // ---- E: ranking ----
   {
     unsigned long long* chunk = reinterpret_cast<unsigned long long*>(dyn_smem);
-    for (int combo = threadIdx.x; combo < tbl.n_comb; combo += kSelThreads)
-      sh.state[combo] = min(__ldcg(&p.cand_count[combo]), static_cast<uint32_t>(p.cand_stride));
-    __syncthreads();
     const int grid = static_cast<int>(gridDim.x), bid = static_cast<int>(blockIdx.x);
-    if (tbl.rank_by_list) {
-      // Enough CTAs: each serves one combination only (a CTA that met two would stage and
-      // split both lists, and the whole grid would wait for it).  The host has dealt the CTAs
-      // out: combination c has [rank_cta_begin[c], rank_cta_begin[c + 1]).
-      for (int combo = 0; combo < tbl.n_comb; ++combo) {
-        const int b0 = tbl.rank_cta_begin[combo], b1 = tbl.rank_cta_begin[combo + 1];
-        if (bid < b0 || bid >= b1) continue;
-        const uint32_t n = sh.state[combo], share = b1 - b0, k = bid - b0;
-        const int lo = static_cast<int>(n * k / share), hi = static_cast<int>(n * (k + 1) / share);
-        if (lo < hi) rank_range(p, tbl, combo, static_cast<int>(n), lo, hi, chunk);
+    for (int combo = threadIdx.x; combo < tbl.n_comb; combo += kSelThreads) {
+      const uint32_t n = min(__ldcg(&p.cand_count[combo]), static_cast<uint32_t>(p.cand_stride));
+      sh.state[combo] = n;
+      sh.mode[combo] = static_cast<uint8_t>(__ldcg(&p.cand_count[kMaxCombos + combo]));     // came the long way
+      const int b0 = tbl.rank_cta_begin[combo], share = tbl.rank_cta_begin[combo + 1] - b0;
+      if (tbl.rank_by_list && bid >= b0 && bid < b0 + share) {
+        sh.flag = combo;
+        sh.krem[0] = n * static_cast<uint32_t>(bid - b0) / static_cast<uint32_t>(share);
+        sh.krem[1] = n * static_cast<uint32_t>(bid - b0 + 1) / static_cast<uint32_t>(share);
       }
-    } else {
-      // fewer CTAs than lists: every CTA takes a contiguous run of all candidates
-      long long n_cand = 0;
-      for (int combo = 0; combo < tbl.n_comb; ++combo) n_cand += sh.state[combo];
-      const int i_begin = static_cast<int>(static_cast<long long>(bid) * n_cand / grid);
-      const int i_end = static_cast<int>(static_cast<long long>(bid + 1) * n_cand / grid);
-      int first = 0;
-      for (int combo = 0; combo < tbl.n_comb; ++combo) {
-        const int n = static_cast<int>(sh.state[combo]);
-        const int lo = max(i_begin, first) - first, hi = min(i_end, first + n) - first;
-        if (lo < hi) rank_range(p, tbl, combo, n, lo, hi, chunk);
-        first += n;
-      }
+    }
+    __syncthreads();
+    // Enough CTAs: each serves one combination only (a CTA that met two would stage and split both lists,
+    // and the whole grid would wait for it).  The host has dealt the CTAs out: combination c has
+    // [rank_cta_begin[c], rank_cta_begin[c + 1]).  Fewer CTAs than lists: every CTA takes a contiguous run
+    // of all candidates.
+    const int only = tbl.rank_by_list ? sh.flag : -1;
+    long long n_cand = 0;
+    for (int combo = 0; combo < tbl.n_comb && only < 0; ++combo) n_cand += sh.state[combo];
+    const int i_begin = static_cast<int>(static_cast<long long>(bid) * n_cand / grid);
+    const int i_end = static_cast<int>(static_cast<long long>(bid + 1) * n_cand / grid);
+    int first = 0;
+    for (int combo = max(only, 0); combo < (only < 0 ? tbl.n_comb : only + 1); ++combo) {
+      const int n = static_cast<int>(sh.state[combo]);
+      const int lo = only < 0 ? max(i_begin, first) - first : static_cast<int>(sh.krem[0]);
+      const int hi = only < 0 ? min(i_end, first + n) - first : static_cast<int>(sh.krem[1]);
+      if (lo < hi) rank_range(p, tbl, combo, n, lo, hi, sh.mode[combo] != 0, chunk, &sh);
+      first += n;
     }
   }
   if (!grid_sync<kCluster>(p, &sh, epoch)) return;

@@ -236,6 +236,33 @@ def test_nans_in_given_scores_rank_last(case):
     eng.close()
 
 
+# Given scores that lie close together, so that thousands of candidates share a bin: lists of a few hundred
+# to 8192 keys and more, shared by several CTAs or several lists to a CTA, ties inside them, lists that
+# came the long way.  (L, budget, max_sizes, win_sizes, scores)
+DENSE = [(500, 200, (1,), (1,), "narrow"), (4096, 1024, (1,), (1, 7, 15), "narrow"), (4096, 1024, (1,), (1, 7, 15), "levels"),
+         (4096, 1024, (2, 4, 8), tuple(range(1, 17)), "narrow"), (8192, 4097, (1,), (1,), "narrow"),
+         (8193, 4097, (1,), (1,), "levels"), (12000, 6000, (1, 2), (3,), "narrow"), (20000, 4096, (2, 4, 8), (1, 2, 5), "half"),
+         (60000, 3000, (1,), (1, 7), "half"), (60000, 3000, (1,), (1, 7), "levels"), (60000, 9000, (1,), (1,), "levels")]
+
+
+@pytest.mark.parametrize("case", DENSE, ids=lambda c: f"L{c[0]}_B{c[1]}_m{len(c[2])}_n{len(c[3])}_{c[4]}")
+def test_dense_bins_match_oracle(case):
+    from paper_2508_17892_b200 import IlreRecall
+    L, budget, max_sizes, win_sizes, kind = case
+    rng = np.random.default_rng(L + budget)
+    u = rng.random(L).astype(np.float32)
+    scores = {"narrow": np.float32(1e-3) * (1 + np.float32(1e-3) * u), "half": np.float32(0.5) + np.float32(0.5) * u,
+              "levels": np.floor(64 * u) / np.float32(4096) + np.float32(0.25)}[kind].astype(np.float32)
+    eng = IlreRecall(max_L=L, max_q_len=1, max_budget=budget, max_combinations=48, n_kv_heads=1, n_q_heads=1)
+    for win_op in (0, 1):
+        got = eng.allocate(torch.from_numpy(scores).cuda(), budget, max_sizes, win_sizes, win_op)
+        eng.check_status()
+        want = oracle.allocate(scores, budget, max_sizes, win_sizes, win_op, avg_single=True)
+        assert np.array_equal(got.cpu().numpy(), np.asarray(want))
+    assert eng.check_guards() == 0, "a kernel wrote past the end of a workspace buffer"
+    eng.close()
+
+
 @pytest.mark.parametrize("pattern", ["all_equal", "two_levels", "blocks_of_equal", "all_equal_40k",
                                      "blocks_of_equal_40k", "all_equal_40k_B6000",
                                      "blocks_of_equal_40k_B6000"])
