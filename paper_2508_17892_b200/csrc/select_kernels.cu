@@ -46,14 +46,6 @@ __device__ __forceinline__ void pass_bits(int pass, int& shift, int& bits) {
   bits = bt[pass];
 }
 
-// Bin of a pooled value: kHistBins logarithmic bins, 32 per power of two, from 2^-63 to 2 (the scores are
-// probabilities); values outside fall into the first and the last one.
-static constexpr int kBinShift = 18;
-static constexpr int kFirstBin = (64 << 5) + 8192;       // float_to_ordered(2^-63) >> kBinShift
-__device__ __forceinline__ int bin_of_ordered(uint32_t o) {
-  return min(max(static_cast<int>(o >> kBinShift) - kFirstBin, 0), kHistBins - 1);
-}
-
 struct SelShared {
   alignas(8) uint32_t hist[kHistBins];     // (the ranking's scratch after the scans)
   uint32_t above[kHistBins + 1];           // of one combination: [b + 1] values in the bins above bin b; [0] all
@@ -298,7 +290,7 @@ __device__ __forceinline__ void pool_tile(const ComboTable& tbl, const SelectPar
         if (i < n_out) {
           const float acc = ranked_value(fmaxf(s0[i], s0[i + n - w]));
           out[i] = acc;
-          bin = bin_of_ordered(float_to_ordered(acc));
+          bin = bin_of_bits(__float_as_int(acc));
         }
         count_bins(hist, bin);
       }
@@ -326,7 +318,7 @@ __device__ __forceinline__ void pool_tile(const ComboTable& tbl, const SelectPar
         if (c >= 0 && c < n_out) {
           const float avg = ranked_value(acc / static_cast<float>(n));
           p.pooled[static_cast<long long>(combo) * p.pooled_stride + c0 + c] = avg;
-          bin = bin_of_ordered(float_to_ordered(avg));
+          bin = bin_of_bits(__float_as_int(avg));
         }
         count_bins((k == 0) ? hist0 : hist1 + (k - 1) * kHistBins, bin);
       }
@@ -376,11 +368,11 @@ __device__ __forceinline__ void gather_combination(const SelectParams& p, const 
   uint32_t* seg = p.cand_seg + static_cast<long long>(combo) * p.cand_stride;
   uint32_t* slots = p.hist + static_cast<long long>(tbl.n_comb + combo) * kHistBins;
   const int len = tbl.len[combo], threshold = sh->threshold;
-  const float lowest = (threshold == 0) ? -INFINITY
-                                        : ordered_to_float(static_cast<uint32_t>(threshold + kFirstBin) << kBinShift);
+  const float lowest = (threshold == 0) ? -INFINITY : __int_as_float(bin_floor_bits(threshold));
   auto place = [&](int cell) {
-    const uint32_t o = float_to_ordered(__ldcg(w + cell));
-    const int bin = bin_of_ordered(o);
+    const float value = __ldcg(w + cell);
+    const uint32_t o = float_to_ordered(value);
+    const int bin = bin_of_bits(__float_as_int(value));
     const uint32_t start = sh->above[bin + 1], count = sh->above[bin] - start;
     const uint32_t at = start + atomicAdd(&slots[bin], 1u);
     if (at < static_cast<uint32_t>(p.cand_stride)) {

@@ -8,6 +8,23 @@ namespace ilre {
 
 static constexpr int kMaxCombos = 64;
 static constexpr int kHistBins = 2048;
+// Bin of a pooled value, from its bit pattern: 32 bins per power of two for probabilities from 2^-35 to 2,
+// where the scores that are selected lie, 4 per power of two below and above (given scores may have any
+// scale).  Values below zero go to bin 0.
+static constexpr int kFineExponent = 92, kFineEnd = 128;      // biased exponents of 2^-35 and of 2
+static constexpr int kFineBin = 4 * kFineExponent, kCoarseBin = kFineBin + 32 * (kFineEnd - kFineExponent);
+static_assert(kCoarseBin + 4 * (255 - kFineEnd) < kHistBins, "infinity has the last bin");
+__host__ __device__ constexpr int bin_of_bits(int bits) {
+  const int u = bits < 0 ? 0 : bits;
+  return u < (kFineExponent << 23) ? u >> 21
+       : u < (kFineEnd << 23) ? (u >> 18) - (kFineExponent << 5) + kFineBin
+                                                                      : (u >> 21) - (kFineEnd << 2) + kCoarseBin;
+}
+// Bit pattern of the lowest value of bin b > 0.
+__host__ __device__ constexpr int bin_floor_bits(int b) {
+  return b < kFineBin ? b << 21
+       : b < kCoarseBin ? (b - kFineBin + (kFineExponent << 5)) << 18 : (b - kCoarseBin + (kFineEnd << 2)) << 21;
+}
 static constexpr int kMaxWin = 1024;        // largest stride-1 window size
 static constexpr int kMaxMaxSize = 64;      // largest strided max-pool size
 static constexpr int kMaxKm = 16384;        // largest K_m (bounds the candidate lists)

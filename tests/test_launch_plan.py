@@ -101,3 +101,34 @@ def test_the_quota_walk_reads_inside_its_shared_memory(tmp_path):
     """A cell of more than 32 tokens is read as three bitmap words, the last of which may lie behind the
     bitmap: the launch asks for that memory too."""
     _run(tmp_path, WALK)
+
+
+BINS = r"""
+#include <cstdio>
+#include <cstring>
+#include "select_kernels.cuh"
+using namespace ilre;
+static int bits_of(float f) { int b; std::memcpy(&b, &f, 4); return b; }
+int main() {
+  int bad = 0;
+  // every bin that holds a value: it begins where the one before it ends
+  for (int b = 1; b <= bin_of_bits(0x7F800000); ++b)
+    if (bin_of_bits(bin_floor_bits(b)) != b || bin_of_bits(bin_floor_bits(b) - 1) != b - 1)
+      if (bad++ < 5) std::printf("bin %d begins at %08x\n", b, bin_floor_bits(b));
+  bad += bin_of_bits(0) != 0 || bin_of_bits(bits_of(-0.0f)) != 0 || bin_of_bits(bits_of(-3.0f)) != 0;
+  bad += bin_of_bits(0x7F800000) >= kHistBins;
+  // 11-bit digits of the long way are unions of whole bins
+  for (int u = 1; u < (0x7F800000 >> 21); ++u) {
+    const int b = bin_of_bits(u << 21);
+    bad += bin_floor_bits(b) != (u << 21);
+  }
+  // 32 bins per power of two for probabilities from 2^-35 on
+  float v = 1.0f;
+  for (int e = 0; e < 35; ++e, v *= 0.5f) bad += bin_of_bits(bits_of(v)) - bin_of_bits(bits_of(v * 0.5f)) != 32;
+  return bad;
+}
+"""
+
+
+def test_histogram_bins_cover_every_value_in_order(tmp_path):
+    _run(tmp_path, BINS)
