@@ -13,7 +13,7 @@
 //      bin: the place of a cell is the number of values in higher bins plus a counter of its own
 //      bin.  The threshold bin brings a few cells more than K_m; only when it brings more than
 //      kCandSlack of them (a plateau of equal values, mostly) does the combination take the long
-//      way: a radix select of the K_m-th value in three histogram passes over the array, then the
+//      way: a radix select of the K_m-th value in two more histogram passes over the array, then the
 //      ties in cell order (the tiles are in cell order, so a count of the holders per tile plus an
 //      ordered rank inside the tile settle which cells win);
 //   E  ranking (value descending, cell ascending): a candidate is compared with the candidates of
@@ -46,6 +46,8 @@ __device__ __forceinline__ void pass_bits(int pass, int& shift, int& bits) {
   bits = bt[pass];
 }
 
+enum : uint8_t { kFirstDigitKnown = 1, kAllPasses = 2 };       // SelShared::mode
+
 struct SelShared {
   alignas(8) uint32_t hist[kHistBins];     // (the ranking's scratch after the scans)
   uint32_t above[kHistBins + 1];           // of one combination: [b + 1] values in the bins above bin b; [0] all
@@ -55,9 +57,9 @@ struct SelShared {
   int plateau;                             // it brings too many cells: full-scan passes
   uint32_t n_listed;                       // candidates of this CTA listed in shared memory
   unsigned long long prefix[kMaxCombos];   // full-scan passes, per combination: radix prefix found so far,
-  uint32_t state[kMaxCombos];              // whether the K_m-th value is settled,
+  uint32_t state[kMaxCombos];              // 1: the K_m-th value is settled, 2: the first pass is left out,
   uint32_t krem[kMaxCombos];               // and the keys still wanted inside the prefix
-  uint8_t mode[kMaxCombos];                // 1: the combination takes the full-scan passes
+  uint8_t mode[kMaxCombos];                // 0, or how the combination takes the full-scan passes
   uint32_t tot[2][32];                     // warp totals of the one-barrier block scan
 };
 
@@ -290,7 +292,7 @@ __device__ __forceinline__ void pool_tile(const ComboTable& tbl, const SelectPar
         if (i < n_out) {
           const float acc = ranked_value(fmaxf(s0[i], s0[i + n - w]));
           out[i] = acc;
-          bin = bin_of_bits(__float_as_int(acc));
+          bin = bin_of_bits(__float_as_int(acc), p.scores_given != 0);
         }
         count_bins(hist, bin);
       }
@@ -318,7 +320,7 @@ __device__ __forceinline__ void pool_tile(const ComboTable& tbl, const SelectPar
         if (c >= 0 && c < n_out) {
           const float avg = ranked_value(acc / static_cast<float>(n));
           p.pooled[static_cast<long long>(combo) * p.pooled_stride + c0 + c] = avg;
-          bin = bin_of_bits(__float_as_int(avg));
+          bin = bin_of_bits(__float_as_int(avg), p.scores_given != 0);
         }
         count_bins((k == 0) ? hist0 : hist1 + (k - 1) * kHistBins, bin);
       }
@@ -357,6 +359,23 @@ __device__ __forceinline__ void find_threshold(const SelectParams& p, const Comb
   __syncthreads();
 }
 
+// Where the long way begins for a combination whose threshold bin is known (one thread): the bin settles the
+// first digit of the K_m-th value's key, so that pass is left out (1048576 given scores in [1/2, 1), 3 windows:
+// 58 -> 48 us of long way).  A bin with several first digits (the first one, of the values below zero among
+// others): all passes.
+__device__ __noinline__ uint8_t start_long_way(uint32_t k, bool given, uint32_t* all_passes, int combo, SelShared* sh) {
+  const int digit = bin_digit(sh->threshold, given);
+  if (digit < 0) {
+    sh->prefix[combo] = 0ull;
+    sh->krem[combo] = k;
+    *all_passes = 1u;
+    return kAllPasses;
+  }
+  sh->prefix[combo] = static_cast<unsigned long long>(digit) << 53;
+  sh->krem[combo] = k - sh->above[last_bin_of_digit(digit, given) + 1];
+  return kFirstDigitKnown;
+}
+
 // Phase D for the tiles [tile0, tile1) of one combination: the cells of its threshold bin and of the bins
 // above, sorted by bin.  Four consecutive cells per thread and tile; few of them are candidates, and
 // those come in runs, so they are listed in shared memory first and then placed a cell per thread
@@ -368,11 +387,11 @@ __device__ __forceinline__ void gather_combination(const SelectParams& p, const 
   uint32_t* seg = p.cand_seg + static_cast<long long>(combo) * p.cand_stride;
   uint32_t* slots = p.hist + static_cast<long long>(tbl.n_comb + combo) * kHistBins;
   const int len = tbl.len[combo], threshold = sh->threshold;
-  const float lowest = (threshold == 0) ? -INFINITY : __int_as_float(bin_floor_bits(threshold));
+  const float lowest = (threshold == 0) ? -INFINITY : __int_as_float(bin_floor_bits(threshold, p.scores_given != 0));
   auto place = [&](int cell) {
     const float value = __ldcg(w + cell);
     const uint32_t o = float_to_ordered(value);
-    const int bin = bin_of_bits(__float_as_int(value));
+    const int bin = bin_of_bits(__float_as_int(value), p.scores_given != 0);
     const uint32_t start = sh->above[bin + 1], count = sh->above[bin] - start;
     const uint32_t at = start + atomicAdd(&slots[bin], 1u);
     if (at < static_cast<uint32_t>(p.cand_stride)) {
@@ -939,9 +958,176 @@ __device__ __forceinline__ void allocate(const ComboTable& tbl, const SelectPara
   if (threadIdx.x == 0 && total != static_cast<uint32_t>(p.budget)) atomicCAS(p.status, 0, kDevQuota);
 }
 
+// The long way, for the combinations whose threshold bin is a plateau: the K_m-th value, then the ties and
+// the gather.  Out of line, as it is hardly ever needed and the kernel meets its code cold: recalls of 4096
+// tokens in a row 46.3 us with it inline, 45.3 so (it costs the long way itself 2 to 8 us).  tbl and p are
+// references into the kernel's parameters (__grid_constant__; a copy in local memory took 60 us).
+// Returns the barrier's epoch, kGaveUp when a barrier gave up.
+static constexpr uint32_t kGaveUp = 0xFFFFFFFFu;
+template <bool kCluster>
+__device__ __noinline__ uint32_t long_way(const ComboTable& tbl, const SelectParams& p, SelShared* sh, int t_begin,
+                                      int t_end, int c_lo, int c_hi, uint32_t epoch) {
+  uint32_t* pass_hist = p.hist + 2ll * tbl.n_comb * kHistBins;
+  const long long n_hist = static_cast<long long>(kSelectPasses) * tbl.n_comb * kHistBins;
+  const int first_pass = __ldcg(&p.cand_count[3 * kMaxCombos + 1]) != 0u ? 0 : 1;       // the same for every CTA
+  for (long long i = static_cast<long long>(blockIdx.x) * kSelThreads + threadIdx.x; i < n_hist;
+       i += static_cast<long long>(gridDim.x) * kSelThreads)
+    pass_hist[i] = 0u;
+  for (int combo = c_lo + threadIdx.x; combo <= c_hi; combo += kSelThreads) {
+    // nothing left to do for those that do not go the long way
+    sh->state[combo] = sh->mode[combo] == 0 ? 1u : (sh->mode[combo] == kFirstDigitKnown && first_pass == 0) ? 2u : 0u;
+  }
+  if (!grid_sync<kCluster>(p, sh, epoch)) return kGaveUp;
+  for (int pass = first_pass; pass < kSelectPasses; ++pass) {
+    if (pass == 1) {
+      for (int combo = c_lo + threadIdx.x; combo <= c_hi; combo += kSelThreads)
+        if (sh->state[combo] == 2u) sh->state[combo] = 0u;
+      __syncthreads();
+    }
+    int shift, bits;
+    pass_bits(pass, shift, bits);
+    const uint32_t mask = (1u << bits) - 1u;
+    uint32_t* hist_pass = pass_hist + static_cast<long long>(pass) * tbl.n_comb * kHistBins;
+    int cur = -1, load_cursor = 0, cursor = 0;
+    for (int t0 = t_begin; t0 < t_end; t0 += kScanGroup) {
+      float wv[kScanGroup][kTilePer];
+#pragma unroll
+      for (int g = 0; g < kScanGroup; ++g)
+        if (t0 + g < t_end) fetch_tile(tbl, p, t0 + g, load_cursor, sh->state, wv[g]);
+#pragma unroll
+      for (int g = 0; g < kScanGroup; ++g) {
+        const int tile = t0 + g;
+        if (tile >= t_end) break;
+        const int combo = combo_of_tile(tbl, tile, cursor);
+        if (sh->state[combo]) continue;
+        if (combo != cur && cur >= 0)
+          hist_flush(sh->hist, hist_pass + static_cast<long long>(cur) * kHistBins);
+        cur = combo;
+        const unsigned long long prefix = sh->prefix[combo];
+        const int c0 = (tile - tbl.tile_begin[combo]) * kSelTile;
+        const int c1 = min(tbl.len[combo], c0 + kSelTile);
+#pragma unroll
+        for (int k = 0; k < kTilePer; ++k) {
+          const int c = c0 + k * kSelThreads + threadIdx.x;
+          uint32_t digit = 0xFFFFFFFFu;                    // sentinel: does not take part
+          if (c < c1) {
+            const unsigned long long key = make_key(wv[g][k], static_cast<uint32_t>(c));
+            if (pass == 0 || ((key ^ prefix) >> (shift + bits)) == 0ull)
+              digit = static_cast<uint32_t>(key >> shift) & mask;
+          }
+          hist_add(sh->hist, digit);
+        }
+      }
+    }
+    if (cur >= 0) hist_flush(sh->hist, hist_pass + static_cast<long long>(cur) * kHistBins);
+    if (!grid_sync<kCluster>(p, sh, epoch)) return kGaveUp;
+    for (int combo = c_lo; combo <= c_hi; ++combo)
+      if (sh->state[combo] == 0u)
+        bin_search(p, hist_pass + static_cast<long long>(combo) * kHistBins, combo, pass, sh);
+  }
+
+  // ---- D: ties at the K_m-th value, then the gather ----
+  // A combination that is not settled by now has its K_m-th value v (upper half of the
+  // prefix) and wants krem of the cells that hold exactly v: the ones with the lowest index.
+  {
+    int load_cursor = 0, cursor = 0;
+    for (int t0 = t_begin; t0 < t_end; t0 += kScanGroup) {
+      float wv[kScanGroup][kTilePer];
+#pragma unroll
+      for (int g = 0; g < kScanGroup; ++g)
+        if (t0 + g < t_end) fetch_tile(tbl, p, t0 + g, load_cursor, sh->state, wv[g]);
+#pragma unroll
+      for (int g = 0; g < kScanGroup; ++g) {
+        const int tile = t0 + g;
+        if (tile >= t_end) break;
+        const int combo = combo_of_tile(tbl, tile, cursor);
+        if (sh->state[combo]) continue;
+        const uint32_t v_star = static_cast<uint32_t>(sh->prefix[combo] >> 32);
+        const int c0 = (tile - tbl.tile_begin[combo]) * kSelTile;
+        const int c1 = min(tbl.len[combo], c0 + kSelTile);
+        int mine = 0;
+#pragma unroll
+        for (int k = 0; k < kTilePer; ++k) {
+          const int c = c0 + k * kSelThreads + threadIdx.x;
+          mine += (c < c1 && float_to_ordered(wv[g][k]) == v_star) ? 1 : 0;
+        }
+        const int holders = __syncthreads_count(mine & 1) + 2 * __syncthreads_count(mine & 2) +
+                            4 * __syncthreads_count(mine & 4);
+        if (threadIdx.x == 0) p.tile_ties[tile] = holders;
+      }
+    }
+  }
+  if (!grid_sync<kCluster>(p, sh, epoch)) return kGaveUp;
+  {
+    const int lane = threadIdx.x & 31;
+    int load_cursor = 0, cursor = 0;
+    for (int t0 = t_begin; t0 < t_end; t0 += kScanGroup) {
+      float wv[kScanGroup][kTilePer];
+#pragma unroll
+      for (int g = 0; g < kScanGroup; ++g)
+        if (t0 + g < t_end) fetch_tile(tbl, p, t0 + g, load_cursor, nullptr, wv[g]);
+#pragma unroll
+      for (int g = 0; g < kScanGroup; ++g) {
+        const int tile = t0 + g;
+        if (tile >= t_end) break;
+        const int combo = combo_of_tile(tbl, tile, cursor);
+        if (!sh->mode[combo]) continue;                       // gathered in the first scan
+        const bool settled = sh->state[combo] != 0u;
+        const unsigned long long threshold = sh->prefix[combo];
+        const uint32_t v_star = static_cast<uint32_t>(threshold >> 32);
+        const uint32_t wanted = sh->krem[combo];
+        unsigned long long* cand = p.cand + static_cast<long long>(combo) * p.cand_stride;
+        const int c0 = (tile - tbl.tile_begin[combo]) * kSelTile;
+        const int c1 = min(tbl.len[combo], c0 + kSelTile);
+        // holders of v in the earlier tiles of this combination (tiles are in cell order)
+        uint32_t before = 0;
+        bool ties_here = false;
+        if (!settled) {
+          ties_here = __ldcg(&p.tile_ties[tile]) > 0;      // uniform
+          if (ties_here) {
+            uint32_t part = 0;
+            for (int t = tbl.tile_begin[combo] + threadIdx.x; t < tile; t += kSelThreads)
+              part += static_cast<uint32_t>(__ldcg(&p.tile_ties[t]));
+            block_exclusive_scan_1(part, sh->tot, 0, &before);
+            __syncthreads();
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < kTilePer; ++k) {
+          const int c = c0 + k * kSelThreads + threadIdx.x;
+          unsigned long long key = 0ull;
+          bool take = false, holder = false;
+          if (c < c1) {
+            key = make_key(wv[g][k], static_cast<uint32_t>(c));
+            const uint32_t v = static_cast<uint32_t>(key >> 32);
+            if (settled) take = key >= threshold;
+            else { take = v > v_star; holder = v == v_star; }
+          }
+          if (ties_here) {                                 // uniform
+            uint32_t in_row;
+            const uint32_t rank = before + block_exclusive_scan_1(holder ? 1u : 0u, sh->tot, 1, &in_row);
+            __syncthreads();
+            if (holder && rank < wanted) take = true;
+            before += in_row;
+          }
+          const uint32_t votes = __ballot_sync(0xFFFFFFFFu, take);
+          if (votes) {
+            uint32_t slot = 0;
+            if (lane == __ffs(votes) - 1) slot = atomicAdd(&p.cand_count[combo], __popc(votes));
+            slot = __shfl_sync(0xFFFFFFFFu, slot, __ffs(votes) - 1) +
+                   __popc(votes & ((1u << lane) - 1u));
+            if (take && slot < static_cast<uint32_t>(tbl.k_m[combo])) cand[slot] = key;
+          }
+        }
+      }
+    }
+  }
+  return epoch;
+}
+
 template <bool kCluster>
 __global__ void __launch_bounds__(kSelThreads, 1)
-select_kernel(const ComboTable tbl, const SelectParams p) {
+select_kernel(const __grid_constant__ ComboTable tbl, const __grid_constant__ SelectParams p) {
   extern __shared__ __align__(16) uint8_t dyn_smem[];
   __shared__ SelShared sh;
   const int n_tiles = tbl.tile_begin[tbl.n_comb];
@@ -1003,7 +1189,11 @@ select_kernel(const ComboTable tbl, const SelectParams p) {
   }
   for (int combo = c_lo; combo <= c_hi; ++combo) {
     find_threshold(p, tbl, combo, &sh);
-    if (threadIdx.x == 0) sh.mode[combo] = static_cast<uint8_t>(sh.plateau);
+    if (threadIdx.x == 0) {
+      sh.mode[combo] = sh.plateau ? start_long_way(static_cast<uint32_t>(tbl.k_m[combo]), p.scores_given != 0,
+                                                   p.cand_count + 3 * kMaxCombos + 1, combo, &sh)
+                                  : 0;
+    }
     if (!sh.plateau)                                         // uniform
       gather_combination(p, tbl, combo, max(t_begin, tbl.tile_begin[combo]), min(t_end, tbl.tile_begin[combo + 1]), &sh,
                          reinterpret_cast<int*>(dyn_smem));
@@ -1011,159 +1201,10 @@ select_kernel(const ComboTable tbl, const SelectParams p) {
   }
   if (!grid_sync<kCluster>(p, &sh, epoch)) return;
 
-  // The long way, for the combinations whose threshold bin is a plateau.  The flag is the same for every
-  // CTA.  The histograms of its passes are cleared here: they are hardly ever needed.
+  // The long way, for the combinations whose threshold bin is a plateau.  The flag is the same for every CTA.
   if (__ldcg(&p.cand_count[3 * kMaxCombos]) != 0u) {
-    uint32_t* pass_hist = p.hist + 2ll * tbl.n_comb * kHistBins;
-    const long long n_hist = static_cast<long long>(kSelectPasses) * tbl.n_comb * kHistBins;
-    for (long long i = static_cast<long long>(blockIdx.x) * kSelThreads + threadIdx.x; i < n_hist;
-         i += static_cast<long long>(gridDim.x) * kSelThreads)
-      pass_hist[i] = 0u;
-    for (int combo = c_lo + threadIdx.x; combo <= c_hi; combo += kSelThreads) {
-      sh.prefix[combo] = 0ull;
-      sh.krem[combo] = static_cast<uint32_t>(tbl.k_m[combo]);
-      sh.state[combo] = sh.mode[combo] ? 0u : 1u;            // nothing left to do for the others
-    }
-    if (!grid_sync<kCluster>(p, &sh, epoch)) return;
-    for (int pass = 0; pass < kSelectPasses; ++pass) {
-      int shift, bits;
-      pass_bits(pass, shift, bits);
-      const uint32_t mask = (1u << bits) - 1u;
-      uint32_t* hist_pass = pass_hist + static_cast<long long>(pass) * tbl.n_comb * kHistBins;
-      int cur = -1, load_cursor = 0, cursor = 0;
-      for (int t0 = t_begin; t0 < t_end; t0 += kScanGroup) {
-        float wv[kScanGroup][kTilePer];
-#pragma unroll
-        for (int g = 0; g < kScanGroup; ++g)
-          if (t0 + g < t_end) fetch_tile(tbl, p, t0 + g, load_cursor, sh.state, wv[g]);
-#pragma unroll
-        for (int g = 0; g < kScanGroup; ++g) {
-          const int tile = t0 + g;
-          if (tile >= t_end) break;
-          const int combo = combo_of_tile(tbl, tile, cursor);
-          if (sh.state[combo]) continue;
-          if (combo != cur && cur >= 0)
-            hist_flush(sh.hist, hist_pass + static_cast<long long>(cur) * kHistBins);
-          cur = combo;
-          const unsigned long long prefix = sh.prefix[combo];
-          const int c0 = (tile - tbl.tile_begin[combo]) * kSelTile;
-          const int c1 = min(tbl.len[combo], c0 + kSelTile);
-#pragma unroll
-          for (int k = 0; k < kTilePer; ++k) {
-            const int c = c0 + k * kSelThreads + threadIdx.x;
-            uint32_t digit = 0xFFFFFFFFu;                    // sentinel: does not take part
-            if (c < c1) {
-              const unsigned long long key = make_key(wv[g][k], static_cast<uint32_t>(c));
-              if (pass == 0 || ((key ^ prefix) >> (shift + bits)) == 0ull)
-                digit = static_cast<uint32_t>(key >> shift) & mask;
-            }
-            hist_add(sh.hist, digit);
-          }
-        }
-      }
-      if (cur >= 0) hist_flush(sh.hist, hist_pass + static_cast<long long>(cur) * kHistBins);
-      if (!grid_sync<kCluster>(p, &sh, epoch)) return;
-      for (int combo = c_lo; combo <= c_hi; ++combo)
-        if (sh.state[combo] == 0u)
-          bin_search(p, hist_pass + static_cast<long long>(combo) * kHistBins, combo, pass, &sh);
-    }
-
-    // ---- D: ties at the K_m-th value, then the gather ----
-    // A combination that is not settled by now has its K_m-th value v (upper half of the
-    // prefix) and wants krem of the cells that hold exactly v: the ones with the lowest index.
-    {
-      int load_cursor = 0, cursor = 0;
-      for (int t0 = t_begin; t0 < t_end; t0 += kScanGroup) {
-        float wv[kScanGroup][kTilePer];
-#pragma unroll
-        for (int g = 0; g < kScanGroup; ++g)
-          if (t0 + g < t_end) fetch_tile(tbl, p, t0 + g, load_cursor, sh.state, wv[g]);
-#pragma unroll
-        for (int g = 0; g < kScanGroup; ++g) {
-          const int tile = t0 + g;
-          if (tile >= t_end) break;
-          const int combo = combo_of_tile(tbl, tile, cursor);
-          if (sh.state[combo]) continue;
-          const uint32_t v_star = static_cast<uint32_t>(sh.prefix[combo] >> 32);
-          const int c0 = (tile - tbl.tile_begin[combo]) * kSelTile;
-          const int c1 = min(tbl.len[combo], c0 + kSelTile);
-          int mine = 0;
-#pragma unroll
-          for (int k = 0; k < kTilePer; ++k) {
-            const int c = c0 + k * kSelThreads + threadIdx.x;
-            mine += (c < c1 && float_to_ordered(wv[g][k]) == v_star) ? 1 : 0;
-          }
-          const int holders = __syncthreads_count(mine & 1) + 2 * __syncthreads_count(mine & 2) +
-                              4 * __syncthreads_count(mine & 4);
-          if (threadIdx.x == 0) p.tile_ties[tile] = holders;
-        }
-      }
-    }
-    if (!grid_sync<kCluster>(p, &sh, epoch)) return;
-    {
-      const int lane = threadIdx.x & 31;
-      int load_cursor = 0, cursor = 0;
-      for (int t0 = t_begin; t0 < t_end; t0 += kScanGroup) {
-        float wv[kScanGroup][kTilePer];
-#pragma unroll
-        for (int g = 0; g < kScanGroup; ++g)
-          if (t0 + g < t_end) fetch_tile(tbl, p, t0 + g, load_cursor, nullptr, wv[g]);
-#pragma unroll
-        for (int g = 0; g < kScanGroup; ++g) {
-          const int tile = t0 + g;
-          if (tile >= t_end) break;
-          const int combo = combo_of_tile(tbl, tile, cursor);
-          if (!sh.mode[combo]) continue;                       // gathered in the first scan
-          const bool settled = sh.state[combo] != 0u;
-          const unsigned long long threshold = sh.prefix[combo];
-          const uint32_t v_star = static_cast<uint32_t>(threshold >> 32);
-          const uint32_t wanted = sh.krem[combo];
-          unsigned long long* cand = p.cand + static_cast<long long>(combo) * p.cand_stride;
-          const int c0 = (tile - tbl.tile_begin[combo]) * kSelTile;
-          const int c1 = min(tbl.len[combo], c0 + kSelTile);
-          // holders of v in the earlier tiles of this combination (tiles are in cell order)
-          uint32_t before = 0;
-          bool ties_here = false;
-          if (!settled) {
-            ties_here = __ldcg(&p.tile_ties[tile]) > 0;      // uniform
-            if (ties_here) {
-              uint32_t part = 0;
-              for (int t = tbl.tile_begin[combo] + threadIdx.x; t < tile; t += kSelThreads)
-                part += static_cast<uint32_t>(__ldcg(&p.tile_ties[t]));
-              block_exclusive_scan_1(part, sh.tot, 0, &before);
-              __syncthreads();
-            }
-          }
-#pragma unroll
-          for (int k = 0; k < kTilePer; ++k) {
-            const int c = c0 + k * kSelThreads + threadIdx.x;
-            unsigned long long key = 0ull;
-            bool take = false, holder = false;
-            if (c < c1) {
-              key = make_key(wv[g][k], static_cast<uint32_t>(c));
-              const uint32_t v = static_cast<uint32_t>(key >> 32);
-              if (settled) take = key >= threshold;
-              else { take = v > v_star; holder = v == v_star; }
-            }
-            if (ties_here) {                                 // uniform
-              uint32_t in_row;
-              const uint32_t rank = before + block_exclusive_scan_1(holder ? 1u : 0u, sh.tot, 1, &in_row);
-              __syncthreads();
-              if (holder && rank < wanted) take = true;
-              before += in_row;
-            }
-            const uint32_t votes = __ballot_sync(0xFFFFFFFFu, take);
-            if (votes) {
-              uint32_t slot = 0;
-              if (lane == __ffs(votes) - 1) slot = atomicAdd(&p.cand_count[combo], __popc(votes));
-              slot = __shfl_sync(0xFFFFFFFFu, slot, __ffs(votes) - 1) +
-                     __popc(votes & ((1u << lane) - 1u));
-              if (take && slot < static_cast<uint32_t>(tbl.k_m[combo])) cand[slot] = key;
-            }
-          }
-        }
-      }
-    }
+    epoch = long_way<kCluster>(tbl, p, &sh, t_begin, t_end, c_lo, c_hi, epoch);
+    if (epoch == kGaveUp) return;
     if (!grid_sync<kCluster>(p, &sh, epoch)) return;
   }
 

@@ -242,7 +242,9 @@ def test_nans_in_given_scores_rank_last(case):
 DENSE = [(500, 200, (1,), (1,), "narrow"), (4096, 1024, (1,), (1, 7, 15), "narrow"), (4096, 1024, (1,), (1, 7, 15), "levels"),
          (4096, 1024, (2, 4, 8), tuple(range(1, 17)), "narrow"), (8192, 4097, (1,), (1,), "narrow"),
          (8193, 4097, (1,), (1,), "levels"), (12000, 6000, (1, 2), (3,), "narrow"), (20000, 4096, (2, 4, 8), (1, 2, 5), "half"),
-         (60000, 3000, (1,), (1, 7), "half"), (60000, 3000, (1,), (1, 7), "levels"), (60000, 9000, (1,), (1,), "levels")]
+         (60000, 3000, (1,), (1, 7), "half"), (60000, 3000, (1,), (1, 7), "levels"), (60000, 9000, (1,), (1,), "levels"),
+         # long way: the K_m-th value in a crowded bin in one combination, among zeros in the other
+         (60000, 16000, (1,), (1, 1), "mostly zero"), (60000, 16000, (1,), (1, 1), "1e-30"), (60000, 3000, (1, 2), (2, 1), "1e30")]
 
 
 @pytest.mark.parametrize("case", DENSE, ids=lambda c: f"L{c[0]}_B{c[1]}_m{len(c[2])}_n{len(c[3])}_{c[4]}")
@@ -252,7 +254,10 @@ def test_dense_bins_match_oracle(case):
     rng = np.random.default_rng(L + budget)
     u = rng.random(L).astype(np.float32)
     scores = {"narrow": np.float32(1e-3) * (1 + np.float32(1e-3) * u), "half": np.float32(0.5) + np.float32(0.5) * u,
-              "levels": np.floor(64 * u) / np.float32(4096) + np.float32(0.25)}[kind].astype(np.float32)
+              "levels": np.floor(64 * u) / np.float32(4096) + np.float32(0.25),
+              "mostly zero": (0.25 + 1e-3 * u) * (rng.permutation(L) < 14000),
+              "1e-30": 1e-30 * (1 + 1e-3 * u) * (1 + (rng.permutation(L) < 14000)),
+              "1e30": 1e30 * (1 + 1e-3 * u)}[kind].astype(np.float32)
     eng = IlreRecall(max_L=L, max_q_len=1, max_budget=budget, max_combinations=48, n_kv_heads=1, n_q_heads=1)
     for win_op in (0, 1):
         got = eng.allocate(torch.from_numpy(scores).cuda(), budget, max_sizes, win_sizes, win_op)

@@ -111,20 +111,30 @@ using namespace ilre;
 static int bits_of(float f) { int b; std::memcpy(&b, &f, 4); return b; }
 int main() {
   int bad = 0;
-  // every bin that holds a value: it begins where the one before it ends
-  for (int b = 1; b <= bin_of_bits(0x7F800000); ++b)
-    if (bin_of_bits(bin_floor_bits(b)) != b || bin_of_bits(bin_floor_bits(b) - 1) != b - 1)
-      if (bad++ < 5) std::printf("bin %d begins at %08x\n", b, bin_floor_bits(b));
-  bad += bin_of_bits(0) != 0 || bin_of_bits(bits_of(-0.0f)) != 0 || bin_of_bits(bits_of(-3.0f)) != 0;
-  bad += bin_of_bits(0x7F800000) >= kHistBins;
-  // 11-bit digits of the long way are unions of whole bins
-  for (int u = 1; u < (0x7F800000 >> 21); ++u) {
-    const int b = bin_of_bits(u << 21);
-    bad += bin_floor_bits(b) != (u << 21);
+  for (int given = 0; given < 2; ++given) {
+    const bool r = given;
+    const int last = bin_of_bits(0x7F800000, r);         // infinity
+    bad += bin_of_bits(0, r) != 0 || bin_of_bits(bits_of(-0.0f), r) != 0 || bin_of_bits(bits_of(-3.0f), r) != 0;
+    bad += last >= kHistBins || (given && last == kHistBins - 1);
+    // a bin begins where the one before it ends
+    for (int b = 1; b <= last; ++b)
+      if (bin_of_bits(bin_floor_bits(b, r), r) != b || bin_of_bits(bin_floor_bits(b, r) - 1, r) != b - 1)
+        if (bad++ < 5) std::printf("given %d: bin %d begins at %08x\n", given, b, bin_floor_bits(b, r));
+    // a digit's bins hold that digit only, and none of it lies above the last of them
+    for (int b = 0; b <= last; ++b) {
+      const int digit = bin_digit(b, r);
+      if (digit < 0) { bad += b != 0 && (given || b < kHistBins - 8); continue; }
+      const int top = last_bin_of_digit(digit, r);
+      bad += top < b || bin_digit(top, r) != digit;
+      bad += top < last && bin_digit(top + 1, r) == digit;
+      const int end = top < kHistBins - 1 ? bin_floor_bits(top + 1, r) - 1 : 0x7F800000;
+      bad += ((end >> 21) | 0x400) != digit;
+    }
   }
-  // 32 bins per power of two for probabilities from 2^-35 on
+  // 32 bins per power of two for probabilities
   float v = 1.0f;
-  for (int e = 0; e < 35; ++e, v *= 0.5f) bad += bin_of_bits(bits_of(v)) - bin_of_bits(bits_of(v * 0.5f)) != 32;
+  for (int e = 0; e < 62; ++e, v *= 0.5f)
+    bad += bin_of_bits(bits_of(v), false) - bin_of_bits(bits_of(v * 0.5f), false) != 32;
   return bad;
 }
 """
