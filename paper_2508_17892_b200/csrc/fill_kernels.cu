@@ -325,7 +325,10 @@ void fill_plan(int n_sm, FillParams* p) {
   // so that they spread over more pairs.  A narrow tile costs more per channel, since the 128
   // tokens of each CTA are loaded whatever the width: `cost` is the measured time of one pass over
   // 4096 model channels in units of the widest tile's (25, 17, 14 and 12 us and about 7 us of
-  // launch, set-up and output in each call).
+  // launch, set-up and output in each call).  Fewer than 16 tokens: every pair loads the same few rows, and
+  // dozens of pairs hold one another up at them, so there are no more than 16 tiles narrower than a head
+  // (4096 model channels, 16 heads: 64 tiles 30 to 34 us, 16 tiles 25 to 28; 32 heads: 64 tiles 32 to 34, 32
+  // tiles 27 to 34; from 16 tokens on 64 tiles 24 to 26 and the wider ones no faster).
   const int widths[4] = {256, 128, 64, 32};
   const int cost[4] = {100, 70, 55, 50};
   const int workers = n_sm / 2 > 0 ? n_sm / 2 : 1;
@@ -337,6 +340,7 @@ void fill_plan(int n_sm, FillParams* p) {
   long long best = -1;
   for (int i = 0; i < 4; ++i) {
     if (widths[i] > p->unit_width) continue;
+    if (p->n_tok < 16 && widths[i] < 128 && p->n_kv * 128 / widths[i] > 16) continue;
     const long long tiles = rest * (p->unit_width / widths[i]);
     const long long c = (tiles + workers - 1) / workers * cost[i];
     if (best < 0 || c < best) { best = c; p->tail_width = widths[i]; }

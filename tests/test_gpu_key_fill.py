@@ -74,7 +74,8 @@ def test_fill_matches_oracle(case):
 # loading thread tests at once.  (n_tok, d_model, n_kv, pos0, bias)
 SPLITS = [(127, 192, 3, 5, True), (129, 320, 8, 0, False), (256, 64, 7, 5, True), (257, 128, 5, 5, False),
           (1000, 192, 8, 1000, True), (2047, 64, 8, 5, False), (4400, 64, 8, 5, True),
-          (4865, 192, 8, 5, True), (9800, 64, 7, 5, False), (5121, 448, 4, 5, False)]
+          (4865, 192, 8, 5, True), (9800, 64, 7, 5, False), (5121, 448, 4, 5, False),
+          (15, 192, 16, 5, True), (16, 192, 16, 5, False), (1, 64, 8, 5, False)]            # few tokens, many heads
 
 
 @pytest.mark.parametrize("case", SPLITS, ids=lambda c: f"n{c[0]}_d{c[1]}_kv{c[2]}")
