@@ -10,12 +10,12 @@ static constexpr int kMaxCombos = 64;
 static constexpr int kHistBins = 2048;
 // Histogram bins of the pooled values, from their bit patterns (values below zero: the first bin).
 // Probabilities from the scores pass: 32 bins per power of two from 2^-63 to 2.  Given scores may have any
-// scale: 32 per power of two from 2^-35 to 2, where the probabilities that are selected lie, 4 per power of two
-// below and above.  (With the first rule log-normal scores scaled to 1e4 all share a bin: allocation of 131072
-// positions 90 us, so 61; with 8 bins per power of two throughout, one rank's part of a sharded recall of 1M
-// tokens 620 us, so 605.)
-static constexpr int kFineExponent = 92, kFineEnd = 128;      // biased exponents of 2^-35 and of 2
-static constexpr int kFineBin = 4 * kFineExponent, kCoarseBin = kFineBin + 32 * (kFineEnd - kFineExponent);
+// scale: 32 per power of two from 2^-35, below which hardly a selected probability lies, to 2^8, 2 below and
+// 4 above.  (With the first rule log-normal scores scaled to 1e4 all share a bin: allocation of 131072
+// positions 77 us, so 48; with 4 bins from 2 on, 32768 raw logits 72, so 40; with 8 bins per power of two
+// throughout, one rank's part of a sharded recall of 1M tokens 620 us, so 600.)
+static constexpr int kFineExponent = 92, kFineEnd = 135;      // biased exponents of 2^-35 and of 2^8
+static constexpr int kFineBin = 2 * kFineExponent, kCoarseBin = kFineBin + 32 * (kFineEnd - kFineExponent);
 static_assert(kCoarseBin + 4 * (255 - kFineEnd) < kHistBins, "infinity has a bin of its own");
 __host__ __device__ constexpr int bin_of_bits(int bits, bool given) {
   const int u = bits < 0 ? 0 : bits;
@@ -23,13 +23,13 @@ __host__ __device__ constexpr int bin_of_bits(int bits, bool given) {
     const int b = (u >> 18) - (64 << 5);
     return b < 0 ? 0 : b < kHistBins ? b : kHistBins - 1;
   }
-  return u < (kFineExponent << 23) ? u >> 21
+  return u < (kFineExponent << 23) ? u >> 22
        : u < (kFineEnd << 23) ? (u >> 18) - (kFineExponent << 5) + kFineBin : (u >> 21) - (kFineEnd << 2) + kCoarseBin;
 }
 // Bit pattern of the lowest value of bin b > 0.
 __host__ __device__ constexpr int bin_floor_bits(int b, bool given) {
   if (!given) return (b + (64 << 5)) << 18;
-  return b < kFineBin ? b << 21
+  return b < kFineBin ? b << 22
        : b < kCoarseBin ? (b - kFineBin + (kFineExponent << 5)) << 18 : (b - kCoarseBin + (kFineEnd << 2)) << 21;
 }
 // The last bin with values of a first digit of the long way (the upper 11 of a positive value's 32 key bits).
@@ -39,7 +39,7 @@ __host__ __device__ constexpr int last_bin_of_digit(int digit, bool given) {
 // That digit of all values of bin b; -1: the bin, or the digit's last one, holds several.
 __host__ __device__ constexpr int bin_digit(int b, bool given) {
   const int digit = (bin_floor_bits(b, given) >> 21) | 0x400;
-  return b == 0 || last_bin_of_digit(digit, given) == kHistBins - 1 ? -1 : digit;
+  return b == 0 || (given && b < kFineBin) || last_bin_of_digit(digit, given) == kHistBins - 1 ? -1 : digit;
 }
 static constexpr int kMaxWin = 1024;        // largest stride-1 window size
 static constexpr int kMaxMaxSize = 64;      // largest strided max-pool size

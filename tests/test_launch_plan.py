@@ -123,7 +123,7 @@ int main() {
     // a digit's bins hold that digit only, and none of it lies above the last of them
     for (int b = 0; b <= last; ++b) {
       const int digit = bin_digit(b, r);
-      if (digit < 0) { bad += b != 0 && (given || b < kHistBins - 8); continue; }
+      if (digit < 0) { bad += b != 0 && b >= (given ? kFineBin : 1) && (given || b < kHistBins - 8); continue; }
       const int top = last_bin_of_digit(digit, r);
       bad += top < b || bin_digit(top, r) != digit;
       bad += top < last && bin_digit(top + 1, r) == digit;
