@@ -438,7 +438,6 @@ int recall_impl(ilre_recall_t* h, const void* k_cache_dev, int64_t L, const void
   pp.n_kv = h->cfg.n_kv_heads; pp.n_q = h->cfg.n_q_heads; pp.group_size = g.group_size;
   pp.q_len = q_len; pp.kv_rows = g.kv_rows; pp.L = L; pp.n_sink = spec->n_sink;
   pp.enc = h->enc; pp.bitmap = h->bitmap; pp.hist = h->hist;
-  pp.n_comb = tbl.n_comb;
   pp.hist_words = 2ll * tbl.n_comb * kHistBins;
   pp.cand_count = h->cand_count; pp.grid_barrier = h->grid_barrier;
   pp.sel_state_words = 4 * kMaxCombos;

@@ -44,7 +44,6 @@ __device__ __forceinline__ void rotate8(uint4& lo, uint4& hi, const float2* __re
 }
 
 static constexpr int kReropeThreads = 256;
-static constexpr int kReropeUnroll = 1;        // (row, segment) items per thread in flight
 static constexpr int kReropeCtasPerSm = 4;
 
 __global__ void __launch_bounds__(kReropeThreads)
@@ -60,35 +59,19 @@ rerope_kernel(const ReropeParams p) {
       ? static_cast<long long>(p.n_sink) + (p.n_chunks - 2) * p.chunk : 0;
   const long long stride = static_cast<long long>(gridDim.x) * kReropeThreads;
   const long long limit = copy_tail ? n_items : rot_end * p.n_kv * 8;
-  for (long long base = static_cast<long long>(blockIdx.x) * kReropeThreads + threadIdx.x;
-       base < limit; base += stride * kReropeUnroll) {
-    uint4 lo[kReropeUnroll], hi[kReropeUnroll];
-#pragma unroll
-    for (int u = 0; u < kReropeUnroll; ++u) {
-      const long long item = base + u * stride;
-      if (item < limit) {
-        const long long row = item >> 3;
-        const int seg = static_cast<int>(item & 7);
-        lo[u] = p.k_in[row * 16 + seg];
-        hi[u] = p.k_in[row * 16 + 8 + seg];
-      }
+  for (long long item = static_cast<long long>(blockIdx.x) * kReropeThreads + threadIdx.x; item < limit;
+       item += stride) {
+    const long long row = item >> 3;
+    const int seg = static_cast<int>(item & 7);
+    uint4 lo = p.k_in[row * 16 + seg], hi = p.k_in[row * 16 + 8 + seg];
+    const long long t = row / p.n_kv;
+    if (t < rot_end) {
+      const long long i = (t < p.n_sink) ? 1 : 1 + (t - p.n_sink) / p.chunk;   // 1-based chunk
+      const long long dist_row = p.n_chunks - 1 - i - 1;                       // D / chunk - 1
+      rotate8(lo, hi, p.table + dist_row * kRopeHalfDim + seg * 8);
     }
-#pragma unroll
-    for (int u = 0; u < kReropeUnroll; ++u) {
-      const long long item = base + u * stride;
-      if (item < limit) {
-        const long long row = item >> 3;
-        const int seg = static_cast<int>(item & 7);
-        const long long t = row / p.n_kv;
-        if (t < rot_end) {
-          const long long i = (t < p.n_sink) ? 1 : 1 + (t - p.n_sink) / p.chunk;   // 1-based chunk
-          const long long dist_row = p.n_chunks - 1 - i - 1;                       // D / chunk - 1
-          rotate8(lo[u], hi[u], p.table + dist_row * kRopeHalfDim + seg * 8);
-        }
-        p.k_out[row * 16 + seg] = lo[u];
-        p.k_out[row * 16 + 8 + seg] = hi[u];
-      }
-    }
+    p.k_out[row * 16 + seg] = lo;
+    p.k_out[row * 16 + 8 + seg] = hi;
   }
 }
 
