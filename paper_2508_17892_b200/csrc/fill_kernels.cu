@@ -11,9 +11,10 @@
 // one token block are neighbours in that order, so the block's activations are read from HBM once
 // and served from L2 to the other heads.
 //
-// Tensor pipe and board power bound long calls (100001 tokens x 4096 -> 1024 channels: 641 -> 595 us =
-// 1.41 PFLOP/s, the measured sustained rate), the chain of one CTA's 64 blocks short ones (1024
-// tokens 25.4 -> 20.8 us, 4096 tokens 46 -> 33.9; one CTA per 128-token tile before).
+// Tensor pipe and board power bound long calls (100001 tokens x 4096 -> 1024 channels, one CTA per
+// 128-token tile -> pairs: single calls on a cool board 641 -> 595 us = 1.41 PFLOP/s, calls in a row at the
+// power cap 752 -> 679 = 1.24), the chain of one CTA's 64 blocks short ones (1024 tokens 25.4 -> 20.8 us,
+// 4096 tokens 46 -> 33.9).
 #include <cuda_bf16.h>
 
 #include "fill_kernels.cuh"

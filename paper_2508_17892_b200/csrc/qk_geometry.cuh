@@ -53,7 +53,7 @@ inline Geometry make_geometry(int n_kv_heads, int n_q_heads, int n_sm, long long
   // compute, which pay for the cluster launch.  Scores pass, pairs / single CTAs, us:
   //   rows, 128K keys: 148: 53.4 / 49.0; 192: 53.5 / 50.0; 256: 53.7 / 56.1; 280: 93.7 / 100.6;
   //   400: 94.6 / 101.7; 560: 129.7 / 194.8; 800: 169 / 189 (a second tile of few rows starves the two
-  //   issuing threads of the single form); L = 1M, 1024 rows: 1414 / 1568.
+  //   issuing threads of the single form); L = 1M, 1024 rows: 1414 / 1568 (single calls).
   //   accumulators: 57 (32K keys, 1024 rows) 55.2 / 56.4; 28 (32K, 512) 37.9 / 37.7; 14 (8K, 1024)
   //   24.4 / 23.4.
   PassGeometry pair;

@@ -612,8 +612,9 @@ scores_kernel(const __grid_constant__ CUtensorMap tmapK,
 // 256-key tile.  Per instruction an SM reads 8 KB of operands for 128 cycles of math where the
 // one-CTA form reads 12 KB, a key tile crosses from L2 to the SMs once per pair instead of once
 // per CTA, and twice the query rows stay resident, so that half as many CTAs read each key tile.
-// Bound by the tensor pipe and the board's power: L = 1M, 1024 rows per kv head 1414 us = 1.56
-// PFLOP/s (one-CTA kernel 1568 us = 1.40).
+// Bound by the tensor pipe and the board's power: L = 1M, 1024 rows per kv head, single calls on a cool
+// board 1414 us = 1.56 PFLOP/s (one-CTA kernel 1568 us = 1.40), at the power cap of a long run 1470 to
+// 1540 us = 1.43 to 1.49.
 struct PairTail {
   uint64_t q_full;                   // q_full, k_full and acc_empty: used in the first CTA only
   uint64_t k_full[kMaxUnits];

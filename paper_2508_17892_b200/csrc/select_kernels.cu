@@ -17,7 +17,7 @@
 //      ties in cell order (the tiles are in cell order, so a count of the holders per tile plus an
 //      ordered rank inside the tile settle which cells win);
 //   E  ranking (value descending, cell ascending): a candidate is compared with the candidates of
-//      its own bin only, spread over the grid;
+//      its own bin only (a crowded bin's are dealt out first), spread over the grid;
 //   F  one CTA walks the combinations in loop order: maps cells back to tokens, skips tokens
 //      already allocated, stops each combination at its quota B_c, then writes the allocated
 //      positions in ascending order.
@@ -28,8 +28,8 @@
 // Bound by the chain of its phases: barriers, one CTA's walk, code met cold in the instruction cache
 // (everything it reads is in L2).  The stage by itself, events around it after an L2 flush, with a
 // selection inside the threshold bin, one window per pooling tile and scattered candidates -> as it
-// stands: 4K positions 39 -> 34 us, 32K 52 -> 42, 128K 59 -> 48, 512K 89 -> 66, 1M 117..131 -> 88, 1M with
-// 48 combinations 270..280 -> 218.
+// stands: 4K positions 39 -> 29 us, 32K 52 -> 38, 128K 59 -> 44, 512K 89 -> 63, 1M 117..131 -> 84, 1M with
+// 48 combinations 270..280 -> 210.
 #include "select_kernels.cuh"
 #include "sm100_ptx.cuh"
 
