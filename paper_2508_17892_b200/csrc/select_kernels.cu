@@ -52,7 +52,8 @@ struct SelShared {
   alignas(8) uint32_t hist[kHistBins];     // (the ranking's scratch after the scans)
   uint32_t above[kHistBins + 1];           // of one combination: [b + 1] values in the bins above bin b; [0] all
   uint32_t scan[33];
-  int flag;
+  int flag;                                // of the grid barrier: written and read there only
+  int list;                                // ranking: the combination that this CTA serves
   int threshold;                           // the bin of its K_m-th largest value
   int plateau;                             // it brings too many cells: full-scan passes
   uint32_t n_listed;                       // candidates of this CTA listed in shared memory
@@ -1218,7 +1219,7 @@ select_kernel(const __grid_constant__ ComboTable tbl, const __grid_constant__ Se
       sh.mode[combo] = static_cast<uint8_t>(__ldcg(&p.cand_count[kMaxCombos + combo]));     // came the long way
       const int b0 = tbl.rank_cta_begin[combo], share = tbl.rank_cta_begin[combo + 1] - b0;
       if (tbl.rank_by_list && bid >= b0 && bid < b0 + share) {
-        sh.flag = combo;
+        sh.list = combo;
         sh.krem[0] = n * static_cast<uint32_t>(bid - b0) / static_cast<uint32_t>(share);
         sh.krem[1] = n * static_cast<uint32_t>(bid - b0 + 1) / static_cast<uint32_t>(share);
       }
@@ -1228,7 +1229,7 @@ select_kernel(const __grid_constant__ ComboTable tbl, const __grid_constant__ Se
     // and the whole grid would wait for it).  The host has dealt the CTAs out: combination c has
     // [rank_cta_begin[c], rank_cta_begin[c + 1]).  Fewer CTAs than lists: every CTA takes a contiguous run
     // of all candidates.
-    const int only = tbl.rank_by_list ? sh.flag : -1;
+    const int only = tbl.rank_by_list ? sh.list : -1;
     long long n_cand = 0;
     for (int combo = 0; combo < tbl.n_comb && only < 0; ++combo) n_cand += sh.state[combo];
     const int i_begin = static_cast<int>(static_cast<long long>(bid) * n_cand / grid);
