@@ -51,7 +51,7 @@ enum : uint8_t { kFirstDigitKnown = 1, kAllPasses = 2 };       // SelShared::mod
 struct SelShared {
   alignas(8) uint32_t hist[kHistBins];     // (the ranking's scratch after the scans)
   uint32_t above[kHistBins + 1];           // of one combination: [b + 1] values in the bins above bin b; [0] all
-  uint32_t scan[33];
+  uint32_t scan[32];
   int flag;                                // of the grid barrier: written and read there only
   int list;                                // ranking: the combination that this CTA serves
   int threshold;                           // the bin of its K_m-th largest value
@@ -62,6 +62,9 @@ struct SelShared {
   uint32_t krem[kMaxCombos];               // and the keys still wanted inside the prefix
   uint8_t mode[kMaxCombos];                // 0, or how the combination takes the full-scan passes
   uint32_t tot[2][32];                     // warp totals of the one-barrier block scan
+  // quota walk, per combination: (m, quota, ranked cells, kind of cells); an indexed read of the kernel's
+  // parameters costs hundreds of cycles in the walk's dependent chain
+  int4 walk[kMaxCombos];
 };
 
 // Grid-wide barrier (all CTAs are co-resident: cooperative launch).  The arrival counter is
@@ -115,20 +118,9 @@ __device__ __noinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* sh_w
   __syncthreads();                       // protects sh_warp from the previous call's readers
   if (lane == 31) sh_warp[warp] = incl;
   __syncthreads();
-  if (warp == 0) {
-    uint32_t w = sh_warp[lane];
-    uint32_t wi = w;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, wi, o);
-      if (lane >= o) wi += t;
-    }
-    sh_warp[lane] = wi - w;              // exclusive warp offsets
-    if (lane == 31) sh_warp[32] = wi;    // grand total
-  }
-  __syncthreads();
-  *total = sh_warp[32];
-  return sh_warp[warp] + incl - v;
+  const uint32_t w = sh_warp[lane];      // every warp adds up the warps' totals itself
+  *total = __reduce_add_sync(0xFFFFFFFFu, w);
+  return __reduce_add_sync(0xFFFFFFFFu, lane < warp ? w : 0u) + incl - v;
 }
 
 // Adds one digit per thread (0xFFFFFFFF = none) to the shared histogram, one atomic per
@@ -609,13 +601,10 @@ __device__ __forceinline__ void rank_range(const SelectParams& p, const ComboTab
   }
 }
 
-// Shared memory of the allocation phase: the bitmap and its summary lie behind the work area of the
-// other phases, which the staged cells and the output list reuse.
+// Shared memory of the allocation phase: the bitmap lies behind the work area of the other phases, which
+// the output lists reuse.
 __device__ __forceinline__ uint32_t* smem_bitmap(uint8_t* dyn_smem) {
   return reinterpret_cast<uint32_t*>(dyn_smem + kSelWorkBytes);
-}
-__device__ __forceinline__ uint32_t* smem_summary(uint8_t* dyn_smem, long long L) {
-  return reinterpret_cast<uint32_t*>(dyn_smem + kSelWorkBytes) + (((L + 31) / 32 + 3) & ~3ll);
 }
 
 // Bitmap word access of the quota walk.  The bitmap lives in shared memory on the common path;
@@ -630,12 +619,15 @@ __device__ __forceinline__ uint32_t bitmap_word(const uint32_t* bm, int w) {
     return *reinterpret_cast<const volatile uint32_t*>(bm + w);
   }
 }
+// Sets bits where there are any: a predicated atomic, since a branch around each costs more than it saves.
 template <bool kSmem>
 __device__ __forceinline__ void bitmap_set(uint32_t* bm, int w, uint32_t bits) {
   if constexpr (kSmem) {
-    asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(smem_u32(bm + w)), "r"(bits) : "memory");
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p red.shared.or.b32 [%0], %1;\n\t}"
+                 ::"r"(smem_u32(bm + w)), "r"(bits) : "memory");
   } else {
-    atomicOr(bm + w, bits);
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t@p red.global.or.b32 [%0], %1;\n\t}"
+                 ::"l"(__cvta_generic_to_global(bm + w)), "r"(bits) : "memory");
   }
 }
 
@@ -652,6 +644,9 @@ enum : int {
   kCellsShort = 1,        // m <= 32: in at most two words (one funnel shift)
   kCellsLong = 2          // m <= 64: in at most three words
 };
+__device__ __forceinline__ int cells_kind(int m) {
+  return (m & (m - 1)) == 0 && m <= 32 ? kCellsAligned : m <= 32 ? kCellsShort : kCellsLong;
+}
 
 // Tokens of cell `cell` (size m) that are not allocated yet, as a bit mask (bit j = token j).  Positions
 // fit 32 bits (L < 2^31).  Up to two words past the bitmap's end may be read (kSelBitmapSlackWords of
@@ -674,83 +669,132 @@ __device__ __forceinline__ auto fresh_tokens(const uint32_t* bm, int cell, int m
   }
 }
 
-// Marks the fresh tokens `f` of a cell that starts at token t0, and in the summary (one bit per bitmap
-// word; null: none) the words that were touched.
+// Marks the fresh tokens `f` of a cell that starts at token t0 and may lie in several words.
 template <int kCells, bool kSmem, class Mask>
-__device__ __forceinline__ void mark_tokens(uint32_t* bm, uint32_t* summary, int t0, Mask f) {
+__device__ __forceinline__ void mark_tokens(uint32_t* bm, int t0, Mask f) {
   const int w0 = t0 >> 5, sft = t0 & 31;
-  auto set = [&](int w, uint32_t bits) {
-    if (!bits) return;
-    bitmap_set<kSmem>(bm, w, bits);
-    if constexpr (kSmem) {
-      if (summary) bitmap_set<true>(summary, w >> 5, 1u << (w & 31));
-    }
-  };
-  if constexpr (kCells == kCellsAligned) {
-    set(w0, f << sft);
-  } else if constexpr (kCells == kCellsShort) {
-    set(w0, f << sft);
-    set(w0 + 1, __funnelshift_l(f, 0u, sft));
+  if constexpr (kCells == kCellsShort) {
+    bitmap_set<kSmem>(bm, w0, f << sft);
+    bitmap_set<kSmem>(bm, w0 + 1, __funnelshift_l(f, 0u, sft));
   } else {
     const unsigned long long shifted = f << sft;
-    set(w0, static_cast<uint32_t>(shifted));
-    set(w0 + 1, static_cast<uint32_t>(shifted >> 32));
-    set(w0 + 2, sft ? static_cast<uint32_t>(f >> (64 - sft)) : 0u);
+    bitmap_set<kSmem>(bm, w0, static_cast<uint32_t>(shifted));
+    bitmap_set<kSmem>(bm, w0 + 1, static_cast<uint32_t>(shifted >> 32));
+    bitmap_set<kSmem>(bm, w0 + 2, sft ? static_cast<uint32_t>(f >> (64 - sft)) : 0u);
   }
 }
 
-// One combination of the quota walk.  Thread t owns the ranks [t * per, (t + 1) * per).  Only the warp in
-// which the quota ends needs the order of its cells' tokens: the warps before it take all of theirs,
-// so the counts are added up with one reduction per warp instead of a prefix sum.  `totals`: one word
-// per walking warp, of this combination only.  The barrier separates counting from marking.  The
-// loops are not unrolled: the kernel meets every instruction cold, and the fetch of unrolled code
-// costs more than the loops do.
+// One round of the quota walk over a combination: kWalkCells consecutive ranks per lane, r0 on, a warp those of
+// its lanes in turn; c: their cells.  The cells of a combination are disjoint, so all of a round's
+// cells are counted before any is marked, and a round's marks do not change another round's counts: one
+// barrier per round, `tot`: the warps' counts, two buffers that the rounds use in turn.  `taken`: tokens of
+// the combination's rounds before (kept up to date when another round follows; in warp 0 always).
+//
+// What a round costs is the instructions that each warp has to fetch and issue (about three cycles each) and
+// the chain of its steps (B200, cycles: shuffle 40, warp reduction 52, block barrier 35 with one warp and 104
+// with 32; several lanes' atomics on one word 31 per lane; a divergent branch about 50).  So only the warp in which
+// the quota ends looks at the order of its lanes, warps behind it mark nothing, and a lane's
+// neighbouring cells mark a bitmap word together (a plateau's cells are ranked one behind the other).
+// The walk of 3 / 4 / 5 / 48 combinations (4K, 128K, 1M, 200003 positions), one cell after another in each lane
+// and lists copied to shared memory a step ahead -> as it stands: 4.6, 10, 13, 66 -> 2.8, 6.2, 8.5, 42 us.
 template <int kCells, bool kSmem, class Barrier>
-__device__ __forceinline__ void walk_combination(const SelectParams& p, const int* cells, int K, int m, uint32_t quota,
-                                                 uint32_t* bm, uint32_t* summary, uint32_t* totals, int n_walk,
-                                                 Barrier walk_barrier) {
+__device__ __forceinline__ void walk_round(const SelectParams& p, const int (&c)[kWalkCells], int r0, int K, int m,
+                                           uint32_t quota, uint32_t* bm, uint32_t* tot, uint32_t& taken, bool last_round,
+                                           int n_walk, Barrier walk_barrier) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int Lp = static_cast<int>(p.L - p.n_sink);
   auto count = [](auto f) -> uint32_t {
     if constexpr (kCells == kCellsLong) return __popcll(f); else return __popc(f);
   };
-  const int per = (K + n_walk - 1) / n_walk;
-  const int r0 = min(K, static_cast<int>(threadIdx.x) * per), r1 = min(K, r0 + per);
-  uint32_t mine = 0;
-#pragma unroll 1
-  for (int r = r0; r < r1; ++r) mine += count(fresh_tokens<kCells, kSmem>(bm, cells[r], m, Lp));
-  const uint32_t warp_sum = __reduce_add_sync(0xFFFFFFFFu, mine);
-  if (lane == 0) totals[warp] = warp_sum;
+  decltype(fresh_tokens<kCells, kSmem>(bm, 0, m, Lp)) f[kWalkCells];
+  uint32_t mine = 0, sum = 0;                                  // of this lane, of the warp
+  if (r0 - kWalkCells * lane < K) {                            // uniform
+#pragma unroll
+    for (int j = 0; j < kWalkCells; ++j) {
+      f[j] = fresh_tokens<kCells, kSmem>(bm, (r0 + j < K) ? c[j] : 0, m, Lp);
+      if (r0 + j >= K) f[j] = 0;
+      mine += count(f[j]);
+    }
+    sum = __reduce_add_sync(0xFFFFFFFFu, mine);
+  }
+  if (lane == 0) tot[warp] = sum;
   walk_barrier();
-  const uint32_t wt = (lane < n_walk / 32) ? totals[lane] : 0u;
-  const uint32_t before = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? wt : 0u);
-  if (warp == 0 && __reduce_add_sync(0xFFFFFFFFu, wt) < quota && lane == 0) atomicCAS(p.status, 0, kDevQuota);
-  if (before >= quota) return;
-  uint32_t room = 0xFFFFFFFFu;                                 // tokens that this thread may take
-  if (before + warp_sum > quota) {                             // the quota ends inside this warp
+  const uint32_t wt = (lane < n_walk / 32) ? tot[lane] : 0u;
+  const uint32_t before = taken + __reduce_add_sync(0xFFFFFFFFu, lane < warp ? wt : 0u);
+  if (!last_round || warp == 0) taken += __reduce_add_sync(0xFFFFFFFFu, wt);
+  if (before >= quota || sum == 0) return;                     // uniform
+  if (before + sum > quota) {                                  // the quota ends inside this warp
     uint32_t incl = mine;
-#pragma unroll 1
+#pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
       if (lane >= o) incl += t;
     }
     const uint32_t ord = before + incl - mine;
-    room = (ord < quota) ? quota - ord : 0u;
-  }
-  // rank order; inside a cell in ascending position
-#pragma unroll 1
-  for (int r = r0; r < r1 && room > 0; ++r) {
-    const int c = cells[r];
-    auto f = fresh_tokens<kCells, kSmem>(bm, c, m, Lp);
-    const uint32_t n_new = count(f);
-    if (n_new == 0) continue;
-    if (n_new > room) {                                        // the quota ends inside this cell
-      auto rest = f;
-      for (uint32_t k = 0; k < room; ++k) rest &= rest - 1;    // without its lowest `room` tokens
-      f ^= rest;
+    uint32_t room = ord < quota ? quota - ord : 0u;
+    auto end = f[0];                                           // the cell in which the quota ends
+    uint32_t end_room = 0;
+    int end_cell = 0;
+#pragma unroll
+    for (int j = 0; j < kWalkCells; ++j) {
+      const uint32_t n_new = count(f[j]);
+      const bool all = n_new <= room;
+      if (!all && room) { end = f[j]; end_room = room; end_cell = c[j]; }
+      f[j] = all ? f[j] : 0;
+      room = all ? room - n_new : 0;
     }
-    room = (n_new > room) ? 0u : room - n_new;
-    mark_tokens<kCells, kSmem>(bm, summary, c * m, f);
+    if (end_room) {                                            // its lowest tokens
+      auto rest = end;
+      for (uint32_t k = 0; k < end_room; ++k) rest &= rest - 1;
+      const int t0 = end_cell * m;
+      if constexpr (kCells == kCellsAligned) bitmap_set<kSmem>(bm, t0 >> 5, (end ^ rest) << (t0 & 31));
+      else mark_tokens<kCells, kSmem>(bm, t0, end ^ rest);
+    }
+  }
+  if constexpr (kCells == kCellsAligned) {
+    uint32_t bits = 0;
+#pragma unroll
+    for (int j = 0; j < kWalkCells; ++j) {
+      const int t0 = c[j] * m;
+      bits |= f[j] << (t0 & 31);
+      const bool goes_on = j + 1 < kWalkCells && (c[(j + 1) % kWalkCells] * m) >> 5 == t0 >> 5;
+      bitmap_set<kSmem>(bm, t0 >> 5, goes_on ? 0u : bits);
+      bits = goes_on ? bits : 0u;
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < kWalkCells; ++j) mark_tokens<kCells, kSmem>(bm, c[j] * m, f[j]);
+  }
+}
+
+// Writes the positions of one bitmap word per lane (`bits` of word `w`, its first position at `place`).  A
+// lane writes its word's positions itself where they are few, the warp together, a lane each, those of
+// a word with more: quoted passages fill whole words, and a lane by itself takes 32 steps for one.
+__device__ __forceinline__ void emit_words(const SelectParams& p, uint32_t bits, int w, uint32_t place, uint32_t cap) {
+  constexpr uint32_t kAlone = 4;
+  const uint32_t lane = threadIdx.x & 31, n = __popc(bits);
+  const int pos0 = p.n_sink + w * 32;
+  uint32_t together = __ballot_sync(0xFFFFFFFFu, n > kAlone);
+  while (together) {
+    const int a = __ffs(together) - 1;                         // two words per turn
+    together &= together - 1;
+    const int b = together ? __ffs(together) - 1 : a;
+    together &= together - 1;                                  // (0 stays 0)
+    const uint32_t bits_a = __shfl_sync(0xFFFFFFFFu, bits, a), bits_b = __shfl_sync(0xFFFFFFFFu, bits, b);
+    const uint32_t place_a = __shfl_sync(0xFFFFFFFFu, place, a), place_b = __shfl_sync(0xFFFFFFFFu, place, b);
+    const int pos_a = __shfl_sync(0xFFFFFFFFu, pos0, a), pos_b = __shfl_sync(0xFFFFFFFFu, pos0, b);
+    const uint32_t lt = (1u << lane) - 1u;
+    const uint32_t at_a = place_a + __popc(bits_a & lt), at_b = place_b + __popc(bits_b & lt);
+    if (((bits_a >> lane) & 1u) && at_a < cap) p.out_idx[at_a] = pos_a + lane;
+    if (((bits_b >> lane) & 1u) && at_b < cap) p.out_idx[at_b] = pos_b + lane;
+  }
+  if (n <= kAlone) {
+    while (bits) {
+      const int k = __ffs(bits) - 1;
+      bits &= bits - 1;
+      if (place < cap) p.out_idx[place] = pos0 + k;
+      ++place;
+    }
   }
 }
 
@@ -790,173 +834,140 @@ __device__ __forceinline__ void allocate(const ComboTable& tbl, const SelectPara
   // Two instantiations, so that the compiler knows the bitmap's address space on the common
   // path (shared memory) instead of going through generic loads and atomics.
   uint32_t* bm = kBitmapInSmem ? smem_bitmap(dyn_smem) : p.bitmap;
-  // (the output pass takes a thread per bitmap word, without the summary, up to kSelThreads words)
-  uint32_t* summary = (kBitmapInSmem && (p.L - p.n_sink + 31) / 32 > kSelThreads) ? smem_summary(dyn_smem, p.L) : nullptr;
-  int* staged = reinterpret_cast<int*>(dyn_smem);
   __shared__ uint32_t warp_totals[2][kMaxWalkWarps];
   const int n_walk = p.walk_threads;                       // multiple of 32, <= kSelThreads
-  // (m, quota, ranked cells) per combination: an indexed read of the kernel's parameters costs
-  // hundreds of cycles in the walk's dependent chain
-  __shared__ int4 walk_table[kMaxCombos];
-  for (int combo = threadIdx.x; combo < tbl.n_comb; combo += kSelThreads)
-    walk_table[combo] = make_int4(tbl.m[combo], tbl.quota[combo],
-                                  min(static_cast<int>(min(__ldcg(&p.cand_count[combo]), static_cast<uint32_t>(kMaxKm))),
-                                      tbl.k_m[combo]), 0);
-  __syncthreads();
-  // The walk is a chain of short dependent steps per combination, so what it costs is the
-  // number of warps that have to issue them and the length of the chain: walk_threads threads walk
-  // (kWalkCells ranked cells each for the longest list), the others wait for the output pass.  The
-  // ranked cells of a combination reach shared memory by 16-byte asynchronous copies, one
-  // combination ahead when two staging buffers fit.
+  // The walk is a chain of short dependent rounds, at least one per combination: walk_threads threads walk
+  // (kWalkCells ranked cells each for the longest list, as long as there are so many threads), the others
+  // wait for the output pass.  A thread fetches its cells of a round while it walks the one before.
   if (static_cast<int>(threadIdx.x) < n_walk) {
     auto walk_barrier = [&] { asm volatile("bar.sync 1, %0;" ::"r"(n_walk) : "memory"); };
-    const bool two = p.stage_double != 0;
-    auto issue_copy = [&](int combo) {
-      const int K = walk_table[combo].z;
-      const int* ranked = p.ranked + static_cast<long long>(combo) * p.cand_stride;
-      int* dst = staged + ((two && (combo & 1)) ? p.stage_capacity : 0);
-      for (int r = 4 * threadIdx.x; r < K; r += 4 * n_walk)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst + r)),
-                     "l"(ranked + r) : "memory");
-      asm volatile("cp.async.commit_group;" ::: "memory");
+    const int n_comb = tbl.n_comb, first = kWalkCells * static_cast<int>(threadIdx.x);
+    static_assert(kWalkCells == 4, "one 16-byte load per round");
+    auto fetch = [&](int combo, int r0, int K) -> int4 {
+      return (r0 < K) ? __ldcg(reinterpret_cast<const int4*>(p.ranked + static_cast<long long>(combo) * p.cand_stride + r0))
+                      : make_int4(0, 0, 0, 0);
     };
-    if (tbl.n_comb > 0) issue_copy(0);
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    walk_barrier();
-    const int n_comb = tbl.n_comb;
+    int4 entry = n_comb > 0 ? sh->walk[0] : make_int4(1, 0, 0, 0);
+    int4 next = fetch(0, first, entry.z);
+    uint32_t round = 0;
+#pragma unroll 1
     for (int combo = 0; combo < n_comb; ++combo) {
-      const int4 entry = walk_table[combo];
-      const int m = entry.x, K = entry.z;
+      const int m = entry.x, K = entry.z, kind = entry.w;
       const uint32_t quota = static_cast<uint32_t>(entry.y);
-      const int* cells = staged + ((two && (combo & 1)) ? p.stage_capacity : 0);
-      // the other buffer last served combination combo - 1, which every thread has left
-      if (two && combo + 1 < n_comb) issue_copy(combo + 1);
-      uint32_t* totals = warp_totals[combo & 1];
-      if (32 % m == 0)
-        walk_combination<kCellsAligned, kBitmapInSmem>(p, cells, K, m, quota, bm, summary, totals, n_walk, walk_barrier);
-      else if (m <= 32)
-        walk_combination<kCellsShort, kBitmapInSmem>(p, cells, K, m, quota, bm, summary, totals, n_walk, walk_barrier);
-      else
-        walk_combination<kCellsLong, kBitmapInSmem>(p, cells, K, m, quota, bm, summary, totals, n_walk, walk_barrier);
-      if (!two) {                                              // one buffer: copy only once it is free
-        walk_barrier();
-        if (combo + 1 < n_comb) issue_copy(combo + 1);
+      entry = combo + 1 < n_comb ? sh->walk[combo + 1] : make_int4(1, 0, 0, 0);
+      uint32_t taken = 0;
+      int base = 0;
+#pragma unroll 1
+      for (;;) {
+        const int c[kWalkCells] = {next.x, next.y, next.z, next.w};
+        const int r0 = base + first;
+        uint32_t* tot = warp_totals[round++ & 1u];
+        base += kWalkCells * n_walk;
+        const bool last_round = base >= K;
+        next = last_round ? fetch(combo + 1, first, entry.z) : fetch(combo, base + first, K);
+        if (kind == kCellsAligned)
+          walk_round<kCellsAligned, kBitmapInSmem>(p, c, r0, K, m, quota, bm, tot, taken, last_round, n_walk, walk_barrier);
+        else if (kind == kCellsShort)
+          walk_round<kCellsShort, kBitmapInSmem>(p, c, r0, K, m, quota, bm, tot, taken, last_round, n_walk, walk_barrier);
+        else
+          walk_round<kCellsLong, kBitmapInSmem>(p, c, r0, K, m, quota, bm, tot, taken, last_round, n_walk, walk_barrier);
+        if (last_round) break;
+        if (taken >= quota) {                                  // met before the list's end: the wrong cells were fetched
+          next = fetch(combo + 1, first, entry.z);
+          break;
+        }
       }
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-      walk_barrier();                                          // bitmap updates and the next cells visible
+      if (threadIdx.x == 0 && taken < quota) atomicCAS(p.status, 0, kDevQuota);
+      walk_barrier();                                          // bitmap updates visible
     }
+  }
+  // The bits past the end, which had to look taken, stand for nothing from here on.
+  const int Lp = static_cast<int>(p.L - p.n_sink), n_quads = (Lp + 127) / 128;     // bitmap words by fours
+  if (threadIdx.x < 4) {
+    const int w = Lp / 32 + static_cast<int>(threadIdx.x);
+    const uint32_t keep = (threadIdx.x == 0) ? (1u << (Lp & 31)) - 1u : 0u;
+    if (w < 4 * n_quads) bm[w] = bitmap_word<kBitmapInSmem>(bm, w) & keep;
   }
   __syncthreads();
 
-  // Ascending output.  One SM does this, so what counts is the number of instructions it has
-  // to issue.  The sink part is the identity.  Up to kSelThreads bitmap words (32K positions) a thread
-  // takes one word.  Longer contexts: the words that hold an allocated position
-  // (at most `budget`, usually a few hundred) are listed in ascending order in shared memory (where
-  // the staged cells were; they are done with): from the summary, 32 words per summary word, or,
-  // with the bitmap in global memory, from the bitmap, four words per lane and load, read twice.
-  // The threads share the list out evenly, take the prefix of the words' position counts and
-  // write the positions.
-  const int Lp = static_cast<int>(p.L - p.n_sink);
-  const long long n_words = (Lp + 31ll) / 32;
+  // Ascending output.  One SM does this, so what counts is the number of instructions it has to issue (with 32
+  // warps a shuffle takes 6 cycles of a scheduler, a vote 3.6, a population count 2.7) and that it meets
+  // them cold (a line that is not in its cache costs some 300 cycles).  The sink part is the identity.
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t cap = static_cast<uint32_t>(p.n_sink + p.budget);
   for (int j = threadIdx.x; j < p.n_sink; j += kSelThreads) p.out_idx[j] = j;
-  if (n_words <= kSelThreads) {
-    // short context: a thread per bitmap word, one prefix sum
-    const int w = static_cast<int>(threadIdx.x);
-    uint32_t bits = (w < n_words) ? bitmap_word<kBitmapInSmem>(bm, w) & ~empty_bitmap_word(w, Lp) : 0u;
-    uint32_t total;
-    uint32_t at = p.n_sink + block_exclusive_scan(__popc(bits), sh->scan, &total);
-    while (bits) {
-      const int b = __ffs(bits) - 1;
-      bits &= bits - 1;
-      if (at < cap) p.out_idx[at] = p.n_sink + w * 32 + b;
-      ++at;
-    }
+  uint32_t total;
+  if (4 * n_quads <= kSelThreads) {
+    // up to 32K positions: a lane per bitmap word, the words shared out evenly over the warps (32K: 3.5 -> 2.4 us)
+    const int per = (4 * n_quads + kMaxWalkWarps - 1) / kMaxWalkWarps, w = warp * per + lane;
+    const uint32_t bits = (lane < per && w < 4 * n_quads) ? bitmap_word<kBitmapInSmem>(bm, w) : 0u;
+    const uint32_t before = block_exclusive_scan(__popc(bits), sh->scan, &total);
+    emit_words(p, bits, w, p.n_sink + before, cap);
     if (threadIdx.x == 0 && total != static_cast<uint32_t>(p.budget)) atomicCAS(p.status, 0, kDevQuota);
     return;
   }
-  const int n_w = static_cast<int>(n_words);                // L < 2^31: word and quad numbers fit an int
-  int* list = staged;
-  uint32_t n_entries;
-  if constexpr (kBitmapInSmem) {
-    const int n_sum = (n_w + 31) / 32, per = (n_sum + kSelThreads - 1) / kSelThreads;
-    const int s0 = min(n_sum, static_cast<int>(threadIdx.x) * per), s1 = min(n_sum, s0 + per);
-    uint32_t n_mine = 0;
-    for (int k = s0; k < s1; ++k) n_mine += __popc(bitmap_word<true>(summary, k));
-    uint32_t at = block_exclusive_scan(n_mine, sh->scan, &n_entries);
-    for (int k = s0; k < s1; ++k) {
-      uint32_t words = bitmap_word<true>(summary, k);
-      while (words) {
-        const int b = __ffs(words) - 1;
-        words &= words - 1;
-        if (at < static_cast<uint32_t>(p.budget)) list[at] = k * 32 + b;    // never short unless a quota was overrun
-        ++at;
-      }
-    }
-  } else {
-    const int n_quads = (n_w + 3) / 4;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int rounds = (n_quads + kSelThreads - 1) / kSelThreads;      // per warp
-    const int q_begin = warp * rounds * 32;
-    const int plain_to = Lp / 128;                            // quads that lie inside the context
-    auto load_quad = [&](int q) -> uint4 {
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (q >= n_quads) return v;
-      v = __ldcg(reinterpret_cast<const uint4*>(bm) + q);
-      if (q < plain_to) return v;
-      const int w0 = 4 * q;                                   // bits past the end stand for nothing
-      v.x &= ~empty_bitmap_word(w0, Lp);
-      v.y &= ~empty_bitmap_word(w0 + 1, Lp);
-      v.z &= ~empty_bitmap_word(w0 + 2, Lp);
-      v.w &= ~empty_bitmap_word(w0 + 3, Lp);
-      return v;
-    };
-    uint32_t n_mine = 0;
-    for (int k = 0; k < rounds; ++k) {
-      const uint4 v = load_quad(q_begin + k * 32 + lane);
-      n_mine += (v.x != 0u) + (v.y != 0u) + (v.z != 0u) + (v.w != 0u);
-    }
-    uint32_t running = block_exclusive_scan(n_mine, sh->scan, &n_entries);
-    running = __shfl_sync(0xFFFFFFFFu, running, 0);            // entries of the warps before this one
-    const uint32_t lt = (1u << lane) - 1u;
-    for (int k = 0; k < rounds; ++k) {
-      const int q = q_begin + k * 32 + lane;
-      const uint4 v = load_quad(q);
-      if (__ballot_sync(0xFFFFFFFFu, (v.x | v.y | v.z | v.w) != 0u) == 0u) continue;
-      const uint32_t b0 = __ballot_sync(0xFFFFFFFFu, v.x != 0u), b1 = __ballot_sync(0xFFFFFFFFu, v.y != 0u);
-      const uint32_t b2 = __ballot_sync(0xFFFFFFFFu, v.z != 0u), b3 = __ballot_sync(0xFFFFFFFFu, v.w != 0u);
-      uint32_t at = running + __popc(b0 & lt) + __popc(b1 & lt) + __popc(b2 & lt) + __popc(b3 & lt);
-      const uint32_t room = static_cast<uint32_t>(p.budget);  // the list's size; never short unless a quota was overrun
-      if (v.x) { if (at < room) list[at] = 4 * q; ++at; }
-      if (v.y) { if (at < room) list[at] = 4 * q + 1; ++at; }
-      if (v.z) { if (at < room) list[at] = 4 * q + 2; ++at; }
-      if (v.w) { if (at < room) list[at] = 4 * q + 3; ++at; }
-      running += __popc(b0) + __popc(b1) + __popc(b2) + __popc(b3);
-    }
-  }
-  __syncthreads();
-  n_entries = min(n_entries, static_cast<uint32_t>(p.budget));
-  const int per = static_cast<int>((n_entries + kSelThreads - 1) / kSelThreads);
-  const int e_begin = min(static_cast<int>(n_entries), static_cast<int>(threadIdx.x) * per);
-  const int e_end = min(static_cast<int>(n_entries), e_begin + per);
+  // Longer contexts: every warp takes an equal run of the bitmap and counts its positions; with the sum of the
+  // warps' before it, it goes through the run again, lists the words that are not empty (a few in a hundred,
+  // neighbours for the most part) in order and writes their positions, a lane per word (128K: 7.8 -> 5.4 us; 1M
+  // 8.6 and 9.1).
+  const int per = ((n_quads + kMaxWalkWarps - 1) / kMaxWalkWarps + 31) & ~31;
+  const int q_begin = min(n_quads, warp * per), q_end = min(n_quads, q_begin + per);
+  auto load_quad = [&](int q) -> uint4 {
+    if (q >= q_end) return make_uint4(0u, 0u, 0u, 0u);
+    if constexpr (kBitmapInSmem) return reinterpret_cast<const uint4*>(bm)[q];
+    else return __ldcg(reinterpret_cast<const uint4*>(bm) + q);
+  };
   uint32_t mine = 0;
-  for (int e = e_begin; e < e_end; ++e) {
-    const int w = list[e];
-    mine += __popc(bitmap_word<kBitmapInSmem>(bm, w) & ~empty_bitmap_word(w, Lp));
+#pragma unroll 4
+  for (int q = q_begin; q < q_end; q += 32) {
+    const uint4 v = load_quad(q + lane);
+    if (__any_sync(0xFFFFFFFFu, (v.x | v.y | v.z | v.w) != 0u)) mine += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
   }
-  uint32_t total;
-  uint32_t at = static_cast<uint32_t>(p.n_sink) + block_exclusive_scan(mine, sh->scan, &total);
-  for (int e = e_begin; e < e_end; ++e) {
-    const int w = list[e];
-    uint32_t bits = bitmap_word<kBitmapInSmem>(bm, w) & ~empty_bitmap_word(w, Lp);
-    while (bits) {
-      const int b = __ffs(bits) - 1;
-      bits &= bits - 1;
-      if (at < cap) p.out_idx[at] = p.n_sink + w * 32 + b;
-      ++at;
+  uint32_t at = p.n_sink + block_exclusive_scan(mine, sh->scan, &total);
+  at = __shfl_sync(0xFFFFFFFFu, at, 0);
+  if (threadIdx.x == 0 && total != static_cast<uint32_t>(p.budget)) atomicCAS(p.status, 0, kDevQuota);
+  constexpr int kList = kSelWorkBytes / 4 / kMaxWalkWarps;      // words that a warp's list holds
+  int* list = reinterpret_cast<int*>(dyn_smem) + warp * kList;
+  int listed = 0;
+#pragma unroll 1
+  for (int q = q_begin; q < q_end; q += 32) {
+    const uint4 v = load_quad(q + lane);
+    const uint32_t full = (v.x ? 1u : 0u) | (v.y ? 2u : 0u) | (v.z ? 4u : 0u) | (v.w ? 8u : 0u);
+    if (__any_sync(0xFFFFFFFFu, full != 0u)) {
+      // a word's place in the list: behind the words of the lanes before, by votes, and those of its own lane
+      const uint32_t lt = (1u << lane) - 1u;
+      int before = 0, found = 0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const uint32_t votes = __ballot_sync(0xFFFFFFFFu, (full >> k) & 1u);
+        before += __popc(votes & lt);
+        found += __popc(votes);
+      }
+      int to = listed + before;
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if ((full >> k) & 1u) list[to++] = 4 * (q + lane) + k;
+      listed += found;
+    }
+    if (listed + 128 > kList || q + 32 >= q_end) {              // uniform: the next 32 quads might not fit, or the end
+      __syncwarp();
+#pragma unroll 1
+      for (int e = lane; e - lane < listed; e += 32) {
+        const int w = (e < listed) ? list[e] : 0;
+        const uint32_t bits = (e < listed) ? bitmap_word<kBitmapInSmem>(bm, w) : 0u, n = __popc(bits);
+        uint32_t incl = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+          if (lane >= o) incl += t;
+        }
+        emit_words(p, bits, w, at + incl - n, cap);
+        at += __shfl_sync(0xFFFFFFFFu, incl, 31);
+      }
+      listed = 0;
+      __syncwarp();
     }
   }
-  if (threadIdx.x == 0 && total != static_cast<uint32_t>(p.budget)) atomicCAS(p.status, 0, kDevQuota);
 }
 
 // The long way, for the combinations whose threshold bin is a plateau: the K_m-th value, then the ties and
@@ -1139,8 +1150,6 @@ select_kernel(const __grid_constant__ ComboTable tbl, const __grid_constant__ Se
     uint32_t* bm = smem_bitmap(dyn_smem);
     const int n_words = static_cast<int>((p.L + 31) / 32), Lp = static_cast<int>(p.L - p.n_sink);
     for (int w = threadIdx.x; w < n_words; w += kSelThreads) bm[w] = empty_bitmap_word(w, Lp);
-    uint32_t* summary = smem_summary(dyn_smem, p.L);
-    for (int k = threadIdx.x; k < (n_words + 31) / 32; k += kSelThreads) summary[k] = 0u;
   }
   uint32_t epoch = 0;
   grid_dep_wait();       // the kernel before this one (scores, state cleared for this run) is done
@@ -1217,6 +1226,9 @@ select_kernel(const __grid_constant__ ComboTable tbl, const __grid_constant__ Se
       const uint32_t n = min(__ldcg(&p.cand_count[combo]), static_cast<uint32_t>(p.cand_stride));
       sh.state[combo] = n;
       sh.mode[combo] = static_cast<uint8_t>(__ldcg(&p.cand_count[kMaxCombos + combo]));     // came the long way
+      sh.walk[combo] = make_int4(tbl.m[combo], tbl.quota[combo],
+                                 min(static_cast<int>(min(n, static_cast<uint32_t>(kMaxKm))), tbl.k_m[combo]),
+                                 cells_kind(tbl.m[combo]));
       const int b0 = tbl.rank_cta_begin[combo], share = tbl.rank_cta_begin[combo + 1] - b0;
       if (tbl.rank_by_list && bid >= b0 && bid < b0 + share) {
         sh.list = combo;

@@ -52,16 +52,16 @@ static constexpr int kPoolTileMax = 3072;   // cells of a group of windows per w
 static constexpr int kSrcTileTokens = 8192; // tokens per work tile of the strided max-pool
 static constexpr int kSelClusterMax = 8;     // grids up to this size run as one thread-block cluster
 static constexpr int kCandSlack = 4096;      // candidates past K_m that the threshold bin may bring
-static constexpr int kWalkCells = 2;         // ranked cells per thread of the quota walk, for the longest list
-static constexpr int kMinWalkers = 128;      // fewest threads that walk
+static constexpr int kWalkCells = 4;         // ranked cells per thread and round of the quota walk
+static constexpr int kMinWalkers = 64;       // fewest threads that walk
 static constexpr int kSelBitmapSmemBytes = 136 * 1024;   // bitmap kept in shared memory up to this
-static constexpr int kSelBitmapSlackWords = 4;           // behind the bitmap and its summary
-// Work area in front of the bitmap: pooling tiles, the keys of a ranking list, the staged cells of the
-// quota walk and the list of the output pass, one after another.
+static constexpr int kSelBitmapSlackWords = 4;           // behind the bitmap
+// Work area in front of the bitmap: pooling tiles, the keys of a ranking list and the warps' output
+// lists, one after another.
 static constexpr int kSelWorkBytes = 64 * 1024;
-static_assert(kSelWorkBytes >= (kPoolGroup - 1) * kHistBins * 4 + 2 * (kPoolTileMax + kMaxWin) * 4 && kSelWorkBytes >= kSrcTileTokens * 4 &&
-              kSelWorkBytes >= kMaxKm * 4, "work area too small");
-static constexpr int kSelMaxDynSmemBytes = kSelWorkBytes + kSelBitmapSmemBytes + kSelBitmapSmemBytes / 32 + 64;
+static_assert(kSelWorkBytes >= (kPoolGroup - 1) * kHistBins * 4 + 2 * (kPoolTileMax + kMaxWin) * 4 && kSelWorkBytes >= kSrcTileTokens * 4,
+              "work area too small");
+static constexpr int kSelMaxDynSmemBytes = kSelWorkBytes + kSelBitmapSmemBytes + 4 * kSelBitmapSlackWords;
 
 // One entry per (m_i, n_j) combination, in Algorithm 1's loop order.
 struct ComboTable {
@@ -116,8 +116,6 @@ struct SelectParams {
   int* ranked;             // [n_comb][cand_stride] cell ids in rank order (cand_stride: multiple of 4)
   uint32_t* bitmap;        // [ceil(L/32)] in global memory, used when it does not fit shared memory
   int bitmap_in_smem;
-  int stage_capacity;      // cell ids per staging buffer of the quota walk (>= largest K_m, multiple of 4)
-  int stage_double;        // two staging buffers fit shared memory
   int walk_threads;        // threads that walk the combinations in the allocation phase
   int* out_idx;            // [n_sink + budget]
   int budget;
@@ -130,20 +128,14 @@ struct SelectParams {
   int barrier_extra;
 };
 
-// Dynamic shared memory the kernel needs for a context of L positions (the output list, <= kMaxKm, fits
-// the work area).
-// Also fills p->bitmap_in_smem, p->stage_capacity, p->stage_double and p->walk_threads.
+// Dynamic shared memory the kernel needs for a context of L positions.  Also fills p->bitmap_in_smem and p->walk_threads.
 inline size_t select_smem_bytes(long long L, int max_km, SelectParams* p) {
-  // quota walk: one or two staging buffers of max_km cell ids in the work area, the bitmap and its
-  // summary (when they fit) behind it
-  const size_t cap = (static_cast<size_t>(max_km < 1 ? 1 : max_km) + 3) & ~size_t(3);
+  // the bitmap, when it fits, lies behind the work area
   const size_t words = (static_cast<size_t>((L + 31) / 32) + 3) & ~size_t(3);
   p->bitmap_in_smem = words * sizeof(uint32_t) <= static_cast<size_t>(kSelBitmapSmemBytes) ? 1 : 0;
   int walkers = ((max_km + kWalkCells - 1) / kWalkCells + 31) & ~31;
   p->walk_threads = walkers < kMinWalkers ? kMinWalkers : (walkers > kSelThreads ? kSelThreads : walkers);
-  p->stage_capacity = static_cast<int>(cap);
-  p->stage_double = (2 * cap * sizeof(int) <= static_cast<size_t>(kSelWorkBytes)) ? 1 : 0;
-  return kSelWorkBytes + (p->bitmap_in_smem ? (words + (words + 31) / 32 + kSelBitmapSlackWords) * sizeof(uint32_t) : 0);
+  return kSelWorkBytes + (p->bitmap_in_smem ? (words + kSelBitmapSlackWords) * sizeof(uint32_t) : 0);
 }
 // Largest grid that is co-resident on the device (the kernel's CTAs wait on one another).
 cudaError_t select_max_grid(int n_sm, int* max_grid);

@@ -1,0 +1,49 @@
+"""GPU: quota walk and ascending output where their paths change.
+
+A walking thread takes four ranked cells per round, at most 1024 threads walk: lists of more than
+4096 cells take several rounds, and may meet the quota before their last one.  Cells lie in one,
+two or three bitmap words.  The output pass takes a lane per bitmap word up to 32768 positions,
+warp lists behind; above 1 114 112 positions the bitmap lives in global memory.
+"""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    # L, budget, max sizes, window sizes, n_sink
+    (1, 1, (1,), (1,), 0),
+    (129, 125, (1,), (3, 5), 4),
+    (32768, 4097, (1,), (1, 7, 15), 0),             # a lane per word, the last such length
+    (32773, 5, (2, 64), (1, 2), 5),                 # 32768 positions behind the sink part
+    (32769, 16382, (1,), (1, 31), 0),               # warp lists; four rounds, met before the last
+    (40001, 16000, (3, 1, 48), (1, 9), 1),          # cells of one, two and three words
+    (131072, 12289, (1, 2, 32, 33, 64), (1, 4), 0),
+    (1114113, 9000, (1, 5, 64), (1, 15), 0),        # bitmap in global memory
+]
+
+
+@pytest.mark.parametrize("dense", [False, True])
+@pytest.mark.parametrize("L,budget,max_sizes,win_sizes,n_sink", CASES)
+def test_walk_and_output(L, budget, max_sizes, win_sizes, n_sink, dense):
+    """Windows take the maximum, so every value is exact on both sides: identical positions."""
+    from paper_2508_17892_b200 import IlreRecall
+    rng = np.random.default_rng(L + budget)
+    a = (rng.random(L) ** 4).astype(np.float32)
+    if dense:                                       # whole runs of high and equal scores
+        for p in rng.integers(0, L, size=max(1, L // 4000)):
+            a[p:p + 300] = np.float32(0.5 + 0.4 * rng.random())
+    eng = IlreRecall(max_L=L, max_q_len=1, max_budget=budget, n_kv_heads=1, n_q_heads=1,
+                     max_combinations=len(max_sizes) * len(win_sizes))
+    idx = eng.allocate(torch.from_numpy(a).cuda(), budget, max_sizes, win_sizes, 1, n_sink)
+    torch.cuda.synchronize()
+    eng.check_status()
+    assert eng.check_guards() == 0
+    ref = oracle.allocate(a.astype(np.float64), budget, max_sizes, win_sizes, 1, n_sink)
+    assert np.array_equal(idx.cpu().numpy(), ref)
+    eng.close()
