@@ -177,11 +177,12 @@ bool encode_2d(EncodeTiledFn fn, CUtensorMap* map, const void* base, uint64_t in
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The query [q_len][n_q][128] as boxes of 64 channels x `group` heads x 128 / group tokens.
-bool encode_query(EncodeTiledFn fn, CUtensorMap* map, const void* base, uint64_t n_q, uint64_t q_len, uint32_t group) {
+// The query [q_len][n_q][128] as boxes of 64 channels x `group` heads x box_rows / group tokens.
+bool encode_query(EncodeTiledFn fn, CUtensorMap* map, const void* base, uint64_t n_q, uint64_t q_len, uint32_t group,
+                  uint32_t box_rows) {
   const cuuint64_t gdim[3] = {kHeadDim, n_q, q_len};
   const cuuint64_t gstride[2] = {kHeadDim * 2, n_q * kHeadDim * 2};
-  const cuuint32_t box[3] = {64, group, 128 / group};
+  const cuuint32_t box[3] = {64, group, box_rows / group};
   const cuuint32_t estride[3] = {1, 1, 1};
   return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), gdim, gstride, box,
             estride, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -408,17 +409,22 @@ int recall_impl(ilre_recall_t* h, const void* k_cache_dev, int64_t L, const void
       }
     }
 
-  CUtensorMap map_k, map_q;
+  CUtensorMap map_k, map_q, map_q32;                     // map_q32: in boxes of 32 rows, for copied row tiles
   std::memset(&map_k, 0, sizeof(map_k));
   std::memset(&map_q, 0, sizeof(map_q));
   // Groups of 1, 2, 4, ... 128 query heads per kv head: a TMA box collects 128 rows of a kv head from the
   // caller's query, and no packed copy is made.
   const int direct = (with_qk && 128 % g.group_size == 0) ? g.group_size : 0;
+  auto encode_rows = [&](CUtensorMap* map, int box_rows) {
+    return direct ? encode_query(h->encode, map, query_dev, h->cfg.n_q_heads, q_len, direct, box_rows)
+                  : encode_2d(h->encode, map, h->qp, 128, static_cast<uint64_t>(h->cfg.n_kv_heads) * g.kv_rows, 256, box_rows);
+  };
+  const int rows_per_kv = g.group_size * q_len;
+  const bool tail = (io.stages & kStageStats) && g.stats_tail;
   if (with_qk &&
       (!encode_2d(h->encode, &map_k, k_cache_dev, static_cast<uint64_t>(h->cfg.n_kv_heads) * 128,
                   static_cast<uint64_t>(L), static_cast<uint64_t>(h->cfg.n_kv_heads) * 256) ||
-       !(direct ? encode_query(h->encode, &map_q, query_dev, h->cfg.n_q_heads, q_len, direct)
-                : encode_2d(h->encode, &map_q, h->qp, 128, static_cast<uint64_t>(h->cfg.n_kv_heads) * g.kv_rows, 256))))
+       !encode_rows(&map_q, 128) || (tail && !encode_rows(&map_q32, 32))))
     return ILRE_ERR_CUDA;
 
   QkParams qk;
@@ -426,7 +432,8 @@ int recall_impl(ilre_recall_t* h, const void* k_cache_dev, int64_t L, const void
     qk.pair = pg.pair; qk.n_tiles = pg.n_tiles; qk.n_groups = pg.n_groups; qk.n_rb = pg.n_rb;
     qk.rb_rows = pg.rb_rows; qk.cpg = pg.cpg; qk.stages = pg.stages;
   };
-  qk.L = L; qk.kv_rows = g.kv_rows; qk.group = direct; qk.rows_per_kv = g.group_size * q_len;
+  qk.L = L; qk.kv_rows = g.kv_rows; qk.group = direct; qk.rows_per_kv = rows_per_kv;
+  qk.tail = 0;
   qk.c2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(kHeadDim)));
   qk.partial = h->partial; qk.enc = h->enc; qk.status = h->status;
   qk.clk = h->profiling ? h->clk : nullptr;
@@ -498,7 +505,9 @@ int recall_impl(ilre_recall_t* h, const void* k_cache_dev, int64_t L, const void
   if (io.stages & kStageStats) {
     TraceRange r("ilre: row statistics (Eq. 4)");
     set_pass(g.stats);
-    ILRE_CUDA(launch_row_stats(map_k, map_q, qk, pp, st)); ++launches;
+    qk.tail = tail ? 1 : 0;
+    ILRE_CUDA(launch_row_stats(map_k, map_q, tail ? map_q32 : map_q, qk, pp, st)); ++launches;
+    qk.tail = 0;
     if (io.stats_out) { ILRE_CUDA(launch_export_stats(mp, io.stats_out, st)); ++launches; }
   }
   ILRE_MARK(2);

@@ -104,7 +104,7 @@ __device__ __forceinline__ void cta_teardown(uint32_t tmem_base) {
   }
 }
 
-// 128 query rows of kv head g from row `row` on, channels 64 kb ..: from the packed copy, or straight from
+// A box of query rows of kv head g from row `row` on, channels 64 kb ..: from the packed copy, or straight from
 // the caller's [q_len][n_q][128] array, whose rows of one kv head are `group` heads of consecutive tokens.
 __device__ __forceinline__ void load_query_tile(const CUtensorMap* tmapQ, const QkParams& p, int g, int row, int kb,
                                                 uint32_t dst, uint32_t bar) {
@@ -112,18 +112,24 @@ __device__ __forceinline__ void load_query_tile(const CUtensorMap* tmapQ, const 
   else tma_load_2d(dst, tmapQ, kb * 64, g * p.kv_rows + row, bar);
 }
 
-// TMA producer: the resident Q block once, then the K tiles of this CTA's key range.
-__device__ __forceinline__ void producer_loop(const CUtensorMap* tmapK, const CUtensorMap* tmapQ,
+// TMA producer: the resident Q block of mts row tiles once, then the K tiles of this CTA's key range.  Row tile
+// `copied` (-1: none) is made of copies of its first copy_rows rows, in boxes of 32 rows (tmapQ32).
+__device__ __forceinline__ void producer_loop(const CUtensorMap* tmapK, const CUtensorMap* tmapQ, const CUtensorMap* tmapQ32,
                                               const QkParams& p, const CtaItem& it,
                                               SmemTail* tail, uint32_t q_s, uint32_t k_s, bool down,
-                                              int stages, int skip_tiles = 0) {
+                                              int stages, int mts, int copied = -1, int copy_rows = 128, int skip_tiles = 0) {
   volatile int* abort_flag = &tail->abort_flag;
   const uint32_t qf = smem_u32(&tail->q_full);
-  mbar_arrive_expect_tx(qf, static_cast<uint32_t>(p.rb_rows) * 256u);
+  mbar_arrive_expect_tx(qf, static_cast<uint32_t>(mts) * (128u * 256u));
+  const int row0 = (it.group % p.n_rb) * p.rb_rows;
   for (int kb = 0; kb < 2; ++kb)
-    for (int mt = 0; mt < p.rb_rows / 128; ++mt)
-      load_query_tile(tmapQ, p, it.g, (it.group % p.n_rb) * p.rb_rows + mt * 128, kb,
-                      q_s + kb * p.rb_rows * 128 + mt * 16384, qf);
+    for (int mt = 0; mt < mts; ++mt) {
+      const uint32_t dst = q_s + kb * mts * 16384 + mt * 16384;
+      if (mt != copied) load_query_tile(tmapQ, p, it.g, row0 + mt * 128, kb, dst, qf);
+      else                                                   // the same rows again in each copy
+        for (int quad = 0; quad < 4; ++quad)
+          load_query_tile(tmapQ32, p, it.g, row0 + mt * 128 + quad * 32 % copy_rows, kb, dst + quad * 4096, qf);
+    }
   // ring position as (stage, phase) counters: no division by the run-time stage count
   int s = 0;
   uint32_t phase = 0;
@@ -217,10 +223,20 @@ __device__ __forceinline__ void row_update64(const float (&va)[32], const float 
 // ---------------------------------------------------------------------------------------
 // Pass A: row statistics.  MT = number of 128-row tiles of the resident Q block.
 // ---------------------------------------------------------------------------------------
-template <int MT, int NPOLY>
+// Row tile of accumulator j of key tile i.  A warpgroup always meets the same accumulator of four; where the last
+// row tile is short it would have less to do than the others (TAIL), so the tiles take turns.
+template <int MT, bool TAIL>
+__device__ __forceinline__ int row_tile(int i, int j) {
+  if constexpr (!TAIL || MT == 1 || MT == 3) return j;
+  if constexpr (MT == 2) return j ^ ((i >> 1) & 1);
+  return (i + j) & 3;
+}
+
+template <int MT, int NPOLY, bool TAIL>
 __global__ void __launch_bounds__(kStatsThreads<MT>, 1)
 row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
-                 const __grid_constant__ CUtensorMap tmapQ, const QkParams p, const PrepParams pp) {
+                 const __grid_constant__ CUtensorMap tmapQ, const __grid_constant__ CUtensorMap tmapQ32, const QkParams p,
+             const PrepParams pp) {
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t smem_base = smem_u32(smem);
   const uint32_t q_s = smem_base;
@@ -230,6 +246,10 @@ row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const CtaItem it = decode_item(p, blockIdx.x);
 
+  const int live_rows = min(p.rb_rows, p.rows_per_kv - (it.group % p.n_rb) * p.rb_rows);
+  // the last live row tile: its rows' copies, rows per copy
+  const int tail_tile = (live_rows - 1) / 128, copies = TAIL ? stats_tail_copies(live_rows) : 1;
+  const int copy_rows = 128 / copies;
   constexpr uint32_t kIssuers = kStatsIssuers<MT>;       // every one reads every key tile
   const uint32_t tmem_base = cta_setup(tail, smem_base, p.stages, 4, 4, p.status, kIssuers);
   const bool run = (it.n_tiles > 0) && (*abort_flag == 0);
@@ -248,7 +268,8 @@ row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
       // may come in as SMs fall free.
       grid_dep_wait();
       grid_dep_launch();
-      producer_loop(&tmapK, &tmapQ, p, it, tail, q_s, k_s, false, p.stages, p.skip_tiles);
+      producer_loop(&tmapK, &tmapQ, &tmapQ32, p, it, tail, q_s, k_s, false, p.stages, MT, copies > 1 ? tail_tile : -1,
+                    copy_rows, p.skip_tiles);
     }
   } else if (warp == 1 || warp >= 2 + kStatsConsumerWarps) {
     if (lane == 0 && run) {
@@ -267,8 +288,9 @@ row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
         ok = mbar_wait(smem_u32(&tail->k_full[s]), kphase, abort_flag, p.status, kDevWaitKFull, p.wait_limit);
         if (!ok) break;
         tc_fence_after();
-        for (int mt = 0; mt < MT; ++mt, ++u) {
+        for (int j = 0; j < MT; ++j, ++u) {
           if (u % kIssuers != mine) continue;
+          const int mt = row_tile<MT, TAIL>(i, j);
           const uint32_t b = u & 3u, use = u >> 2;
           ok = mbar_wait(smem_u32(&tail->acc_empty[b]), (use & 1u) ^ 1u, abort_flag, p.status,
                          kDevWaitAccEmpty, p.wait_limit);
@@ -303,20 +325,20 @@ row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
     }
     // Accumulator u belongs to warpgroup u % 4 and holds row tile u % MT.  With 1, 2 or 4 row
     // tiles a warpgroup therefore always meets the same row tile (wg % MT) and a thread keeps
-    // one (max, sum) pair; only with 3 row tiles does it meet all of them in turn.
-    constexpr int kStates = (MT == 3) ? 3 : 1;
+    // one (max, sum) pair; only with 3 row tiles, or tiles that take turns, does it meet all of them.
+    constexpr int kStates = (MT == 3 || (TAIL && MT > 1)) ? MT : 1;
     float m[kStates], z[kStates];
 #pragma unroll
     for (int j = 0; j < kStates; ++j) { m[j] = -1e30f; z[j] = 0.f; }
     const float c2 = p.c2;
-    const int live_rows = min(p.rb_rows, p.rows_per_kv - (it.group % p.n_rb) * p.rb_rows);
+    const int tail_col = quad * 32 / copy_rows * copy_rows;      // this warp's columns of a copied row tile
     const uint32_t n_acc = run ? static_cast<uint32_t>(it.n_tiles) * MT : 0u;
     // One copy of the loop body serves every (key tile, row tile): the warpgroups run at
     // different places of the loop, and a body unrolled over the row tiles would not fit the
     // instruction cache between them.
 #pragma unroll 1
     for (uint32_t u = wg; u < n_acc; u += kStatsWarpgroups) {
-      const int i = static_cast<int>(u / MT), mt = static_cast<int>(u % MT);
+      const int i = static_cast<int>(u / MT), mt = row_tile<MT, TAIL>(i, static_cast<int>(u % MT));
       const long long key0 = static_cast<long long>(it.tile_begin + i) * kTileKeys;
       const int valid = static_cast<int>(min(static_cast<long long>(kTileKeys), p.L - key0));
       const uint32_t b = u & 3u, use = u >> 2;
@@ -324,7 +346,8 @@ row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
                      kDevWaitAccFull, p.wait_limit))
         break;
       tc_fence_after();
-      if (mt * 128 + quad * 32 >= live_rows) {                 // padding rows only: nothing to compute
+      const bool shared = TAIL && mt == tail_tile;
+      if (mt * 128 + (shared ? quad * 32 % copy_rows : quad * 32) >= live_rows) {    // padding rows only: nothing to compute
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&tail->acc_empty[b]));
@@ -337,23 +360,24 @@ row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
           if (j == mt) { mr = m[j]; zr = z[j]; }
       }
       const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16) + b * 128;
-      if (valid >= kTileKeys) {
+      const int col0 = shared ? tail_col : 0, col1 = shared ? col0 + copy_rows : kTileKeys;
+      if (valid >= kTileKeys && (!TAIL || col1 - col0 >= 64)) {
 #pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
+        for (int c = col0; c < col1; c += 64) {
           float va[32], vb[32];
-          tmem_ld32(taddr + 64 * h, va);
-          tmem_ld32(taddr + 64 * h + 32, vb);
+          tmem_ld32(taddr + c, va);
+          tmem_ld32(taddr + c + 32, vb);
           tmem_ld_wait();
-          if (h == 1) {                      // read completely: back to the MMA thread
+          if (c + 64 == col1) {                      // read completely: back to the MMA thread
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&tail->acc_empty[b]));
           }
           row_update64<NPOLY>(va, vb, c2, mr, zr);
         }
-      } else {                               // the context ends inside this tile
+      } else {                               // the context ends inside this tile, or four copies
 #pragma unroll 1
-        for (int c = 0; c < kTileKeys; c += 32) {
+        for (int c = col0; c < col1; c += 32) {
           float v[32];
           tmem_ld32(taddr + c, v);
           tmem_ld_wait();
@@ -394,19 +418,23 @@ row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
     asm volatile("bar.sync 1, %0;" ::"r"(kStatsConsumerWarps * 32) : "memory");
     if (wg == 0) {
       float2* out = reinterpret_cast<float2*>(p.partial) +
-                    (static_cast<size_t>(it.group) * p.cpg + it.chunk) * (MT * 128);
+                    (static_cast<size_t>(it.group) * p.cpg + it.chunk) * p.rb_rows;
 #pragma unroll
       for (int mt = 0; mt < MT; ++mt) {
+        if (mt * 128 + row_in_tile >= live_rows) break;
+        const int n_copy = (TAIL && mt == tail_tile) ? copies : 1;
         float mm = -1e30f;
+        for (int x = 0; x < n_copy; ++x)
 #pragma unroll
-        for (int w = 0; w < kStatsWarpgroups; ++w)
-          mm = fmaxf(mm, scratch[(w * MT + mt) * 128 + row_in_tile].x);
+          for (int w = 0; w < kStatsWarpgroups; ++w)
+            mm = fmaxf(mm, scratch[(w * MT + mt) * 128 + x * copy_rows + row_in_tile].x);
         float zz = 0.f;
+        for (int x = 0; x < n_copy; ++x)
 #pragma unroll
-        for (int w = 0; w < kStatsWarpgroups; ++w) {
-          const float2 o = scratch[(w * MT + mt) * 128 + row_in_tile];
-          zz += o.y * exp2f((o.x - mm) * c2);
-        }
+          for (int w = 0; w < kStatsWarpgroups; ++w) {
+            const float2 o = scratch[(w * MT + mt) * 128 + x * copy_rows + row_in_tile];
+            zz += o.y * exp2f((o.x - mm) * c2);
+          }
         out[mt * 128 + row_in_tile] = make_float2(mm * c2, zz);
       }
     }
@@ -511,7 +539,7 @@ scores_kernel(const __grid_constant__ CUtensorMap tmapK,
       // one waited for, unless that was the prepare kernel itself
       if (p.group == 0 && mp.n_ext > 0) grid_dep_wait();
       grid_dep_launch();                 // the next kernel's CTAs may come in as SMs fall free
-      producer_loop(&tmapK, &tmapQ, p, it, tail, q_s, k_s, true, stages);
+      producer_loop(&tmapK, &tmapQ, nullptr, p, it, tail, q_s, k_s, true, stages, p.rb_rows / 128);
     }
   } else if (warp == 1 || warp == 2) {
     if (lane == 0 && run) {
@@ -885,23 +913,22 @@ size_t scores_smem_bytes(int rb_rows, int stages) {
 }
 
 template <int MT>
-static cudaError_t launch_row_stats_mt(const CUtensorMap& tk, const CUtensorMap& tq, const QkParams& p,
-                                       const PrepParams& pp, cudaStream_t st) {
+static cudaError_t launch_row_stats_mt(const CUtensorMap& tk, const CUtensorMap& tq, const CUtensorMap& tq32,
+                                       const QkParams& p, const PrepParams& pp, cudaStream_t st) {
   const size_t smem = row_stats_smem_bytes(MT * 128, p.stages);
-  cudaError_t e = cudaFuncSetAttribute(row_stats_kernel<MT, kRowStatsPolyPairs>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const auto kernel = p.tail ? row_stats_kernel<MT, kRowStatsPolyPairs, true> : row_stats_kernel<MT, kRowStatsPolyPairs, false>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return launch_after_previous(row_stats_kernel<MT, kRowStatsPolyPairs>, p.n_groups * p.cpg,
-                               kStatsThreads<MT>, smem, st, tk, tq, p, pp);
+  return launch_after_previous(kernel, p.n_groups * p.cpg, kStatsThreads<MT>, smem, st, tk, tq, tq32, p, pp);
 }
 
-cudaError_t launch_row_stats(const CUtensorMap& tk, const CUtensorMap& tq, const QkParams& p,
+cudaError_t launch_row_stats(const CUtensorMap& tk, const CUtensorMap& tq, const CUtensorMap& tq32, const QkParams& p,
                              const PrepParams& pp, cudaStream_t st) {
-  switch (p.rb_rows / 128) {
-    case 1: return launch_row_stats_mt<1>(tk, tq, p, pp, st);
-    case 2: return launch_row_stats_mt<2>(tk, tq, p, pp, st);
-    case 3: return launch_row_stats_mt<3>(tk, tq, p, pp, st);
-    case 4: return launch_row_stats_mt<4>(tk, tq, p, pp, st);
+  switch ((p.rb_rows + 127) / 128) {
+    case 1: return launch_row_stats_mt<1>(tk, tq, tq32, p, pp, st);
+    case 2: return launch_row_stats_mt<2>(tk, tq, tq32, p, pp, st);
+    case 3: return launch_row_stats_mt<3>(tk, tq, tq32, p, pp, st);
+    case 4: return launch_row_stats_mt<4>(tk, tq, tq32, p, pp, st);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -55,6 +55,19 @@ __host__ __device__ constexpr int scores_ring_stages(int stages, int row_halves)
   return row_halves == 1 ? stages & ~1 : stages;
 }
 
+// Statistics pass: copies of the rows of a block's last live row tile.  A tile's rows lie in the four lane
+// quadrants of tensor memory, each read by the warps of one scheduler: 20 rows are one scheduler's work, as long
+// as 128 rows are, while the others wait.  So a tile of up to 32 rows is loaded four times, one of up to
+// 64 twice, and each copy takes its share of the key tile's columns (148 rows, 1M keys: 521 -> 468 us).
+__host__ __device__ constexpr int stats_tail_rows(int live_rows) { return (live_rows - 1) % 128 + 1; }
+__host__ __device__ constexpr int stats_tail_copies(int live_rows) {
+  return stats_tail_rows(live_rows) <= 32 ? 4 : stats_tail_rows(live_rows) <= 64 ? 2 : 1;
+}
+// Rows that a TMA box collects for such a tile: those of whole tokens.  (Head groups of more than 32: no copies.)
+__host__ __device__ constexpr int stats_box_rows(int group_size) {
+  return 128 % group_size == 0 && group_size > 32 ? 128 : 32;
+}
+
 // Geometry of one pass.
 struct QkParams {
   long long L;
@@ -62,12 +75,14 @@ struct QkParams {
   int n_tiles;       // key tiles of kTileKeys keys (pair: of kPairTileKeys)
   int n_groups;      // n_kv_heads * n_rb
   int n_rb;          // row blocks per kv head
-  int rb_rows;       // rows per block: multiple of 128 up to kMaxRbRows (pair: of 256 up to kMaxPairRows)
+  int rb_rows;       // rows per block: multiple of 128 up to kMaxRbRows (statistics: of 32; pair: of 256 up to
+                     // kMaxPairRows)
   int kv_rows;       // rows of one kv head in the packed query (>= n_rb * rb_rows)
   int rows_per_kv;   // those that are not padding
   int group;         // query heads per kv head when the query is loaded from the caller's array (a
                      // box of 128 rows = `group` heads of 128 / group tokens); 0: from the packed copy
   int cpg;           // key chunks (CTAs or CTA pairs) per group
+  int tail;          // statistics: some block's last row tile is short and loaded in copies (stats_tail_copies)
   int stages;        // ring depth in key tiles (pair: in units, set by the launcher)
   float c2;          // log2(e) / sqrt(d)
   float* partial;    // [n_groups][cpg][rb_rows][2]: (max * c2, sum-exp) per key chunk
@@ -114,7 +129,8 @@ size_t scores_smem_bytes(int rb_rows, int stages);
 
 cudaError_t launch_prepare(const void* q, void* qp, const PrepParams& p, int n_sm, cudaStream_t st);
 // Where no prepare kernel was launched before it, this one clears the run's state (pp.clear).
-cudaError_t launch_row_stats(const CUtensorMap& tk, const CUtensorMap& tq, const QkParams& p,
+// tq32: the query in boxes of 32 rows, read with p.tail.
+cudaError_t launch_row_stats(const CUtensorMap& tk, const CUtensorMap& tq, const CUtensorMap& tq32, const QkParams& p,
                              const PrepParams& pp, cudaStream_t st);
 // (max in log2 units, sum of exponentials) of every query row over the keys of this launch,
 // rows in the caller's order i * n_q + h.
