@@ -96,6 +96,7 @@ struct ilre_recall {
   int cand_stride;
   long long pooled_stride;
   int select_max_grid;                  // co-resident CTAs of the selection kernel
+  bool select_wide;                     // the device takes a cluster of kSelClusterWide of them
   long long wait_limit;                 // spin budget of the device waits, SM cycles
   int inject;                           // failure-detection self test: which wait cannot complete
 };
@@ -317,7 +318,7 @@ int ilre_recall_create(const ilre_recall_config_t* cfg, ilre_recall_t** out) {
   if (ok) ok = (cudaMemset(h->status, 0, sizeof(int)) == cudaSuccess);
   if (ok) ok = (cudaMemset(h->clk, 0, 2 * sizeof(unsigned long long)) == cudaSuccess);
   if (ok) ok = (cudaMemset(h->grid_barrier, 0, sizeof(uint32_t)) == cudaSuccess);
-  if (ok) ok = (select_max_grid(h->n_sm, &h->select_max_grid) == cudaSuccess);
+  if (ok) ok = (select_max_grid(h->n_sm, &h->select_max_grid, &h->select_wide) == cudaSuccess);
   if (ok) ok = (cudaDeviceSynchronize() == cudaSuccess);
   if (!ok) {
     cudaGetLastError();
@@ -479,7 +480,9 @@ int recall_impl(ilre_recall_t* h, const void* k_cache_dev, int64_t L, const void
   if (want_grid < 1) want_grid = 1;
   // a grid just above the cluster size: the cluster barrier is worth more than the extra CTAs
   if (want_grid > kSelClusterMax && want_grid <= 2 * kSelClusterMax) want_grid = kSelClusterMax;
+  if (want_grid > kSelClusterMax && h->select_wide && select_wide_cluster(tbl)) want_grid = kSelClusterWide;
   if (want_grid > h->select_max_grid) want_grid = h->select_max_grid;
+  sp.cluster = (want_grid <= kSelClusterMax || (want_grid == kSelClusterWide && h->select_wide)) ? 1 : 0;
   const int select_grid = static_cast<int>(want_grid);
 
   const bool prof = h->profiling != 0;

@@ -30,6 +30,8 @@
 // selection inside the threshold bin, one window per pooling tile and scattered candidates -> as it
 // stands: 4K positions 39 -> 29 us, 32K 52 -> 38, 128K 59 -> 44, 512K 89 -> 63, 1M 117..131 -> 84, 1M with
 // 48 combinations 270..280 -> 210.
+#include <atomic>
+
 #include "select_kernels.cuh"
 #include "sm100_ptx.cuh"
 
@@ -132,12 +134,16 @@ __device__ __forceinline__ void hist_add(uint32_t* hist, uint32_t digit) {
     atomicAdd(&hist[digit], __popc(peers));
 }
 
-__device__ __forceinline__ void hist_flush(uint32_t* sh_hist, uint32_t* gh) {
-  __syncthreads();
+// Adds the shared histogram to the global one and clears it.
+__device__ __forceinline__ void hist_drain(uint32_t* sh_hist, uint32_t* gh) {
   for (int b = threadIdx.x; b < kHistBins; b += kSelThreads) {
     const uint32_t v = sh_hist[b];
     if (v) { atomicAdd(&gh[b], v); sh_hist[b] = 0u; }
   }
+}
+__device__ __forceinline__ void hist_flush(uint32_t* sh_hist, uint32_t* gh) {
+  __syncthreads();
+  hist_drain(sh_hist, gh);
   __syncthreads();
 }
 
@@ -1182,10 +1188,12 @@ select_kernel(const __grid_constant__ ComboTable tbl, const __grid_constant__ Se
       while (grp + 1 < tbl.n_grp && tile >= tbl.grp_tile_begin[grp + 1]) ++grp;
       const int c0 = (tile - tbl.grp_tile_begin[grp]) * per, first = tbl.grp_first[grp];
       pool_tile(tbl, p, grp, c0, min(per, tbl.len[tbl.grp_combo[first]] - c0), buf0, buf1, sh.hist, hist1);
-      if (tile + 1 == p_end || tile + 1 == tbl.grp_tile_begin[grp + 1])        // the CTA's last tile of this group
-        for (int k = 0; first + k < tbl.grp_first[grp + 1]; ++k)
-          hist_flush((k == 0) ? sh.hist : hist1 + (k - 1) * kHistBins,
+      if (tile + 1 == p_end || tile + 1 == tbl.grp_tile_begin[grp + 1]) {      // the CTA's last tile of this group
+        for (int k = 0; first + k < tbl.grp_first[grp + 1]; ++k)               // (which ended with a barrier)
+          hist_drain((k == 0) ? sh.hist : hist1 + (k - 1) * kHistBins,
                      p.hist + static_cast<long long>(tbl.grp_combo[first + k]) * kHistBins);
+        __syncthreads();
+      }
     }
   }
   if (!grid_sync<kCluster>(p, &sh, epoch)) return;
@@ -1274,7 +1282,7 @@ select_kernel(const __grid_constant__ ComboTable tbl, const __grid_constant__ Se
 // ---------------------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------------------
-cudaError_t select_max_grid(int n_sm, int* max_grid) {
+cudaError_t select_max_grid(int n_sm, int* max_grid, bool* wide_cluster) {
   cudaError_t e = cudaFuncSetAttribute(select_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kSelMaxDynSmemBytes);
   if (e != cudaSuccess) return e;
@@ -1287,6 +1295,35 @@ cudaError_t select_max_grid(int n_sm, int* max_grid) {
   if (e != cudaSuccess) return e;
   if (per_sm < 1) return cudaErrorLaunchOutOfResources;
   *max_grid = n_sm;                      // one CTA per SM is plenty for these phases
+  // A cluster of more than 8 CTAs is the device's to grant.  The answer is kept, since asking takes 0.2 ms.
+  const bool allowed = n_sm > kSelClusterWide &&
+      cudaFuncSetAttribute(select_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+  static std::atomic<int> granted[64];             // per device: 0 not asked yet, 1 no, 2 yes
+  int dev = 0;
+  e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  int known = dev < 64 ? granted[dev].load() : 0;
+  if (known == 0) {
+    int n = 0;
+    if (allowed) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(kSelClusterWide);
+      cfg.blockDim = dim3(kSelThreads);
+      cfg.dynamicSmemBytes = kSelMaxDynSmemBytes;
+      cudaLaunchAttribute attr;
+      attr.id = cudaLaunchAttributeClusterDimension;
+      attr.val.clusterDim.x = kSelClusterWide;
+      attr.val.clusterDim.y = 1;
+      attr.val.clusterDim.z = 1;
+      cfg.attrs = &attr;
+      cfg.numAttrs = 1;
+      if (cudaOccupancyMaxActiveClusters(&n, select_kernel<true>, &cfg) != cudaSuccess) n = 0;
+    }
+    known = n > 0 ? 2 : 1;
+    if (dev < 64) granted[dev].store(known);
+  }
+  *wide_cluster = allowed && known == 2;
+  cudaGetLastError();
   return cudaSuccess;
 }
 
@@ -1354,12 +1391,12 @@ cudaError_t launch_select(const ComboTable& table, const SelectParams& p, int gr
   ComboTable tbl = table;
   assign_pooling(&tbl, grid);
   assign_ranking(&tbl, grid);
-  // Short contexts need few CTAs: up to kSelClusterMax of them run as one thread-block cluster,
+  // Short contexts need few CTAs: up to kSelClusterMax of them, or kSelClusterWide, run as one thread-block cluster,
   // whose hardware barrier costs a fraction of a trip to the L2 (not with the self test's
   // barrier that cannot complete: that one is the counter's).  Longer ones: a cooperative
   // launch (every CTA resident: they wait on one another).  Either way the launch may overlap
   // the end of the kernel before it in the stream; the kernel waits before it reads anything.
-  const bool cluster = grid <= kSelClusterMax && p.barrier_extra == 0;
+  const bool cluster = p.cluster != 0 && p.barrier_extra == 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(kSelThreads);

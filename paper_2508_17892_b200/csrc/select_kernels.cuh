@@ -51,6 +51,7 @@ static constexpr int kPoolGroup = 5;        // window sizes of one strided max-p
 static constexpr int kPoolTileMax = 3072;   // cells of a group of windows per work tile, at most
 static constexpr int kSrcTileTokens = 8192; // tokens per work tile of the strided max-pool
 static constexpr int kSelClusterMax = 8;     // grids up to this size run as one thread-block cluster
+static constexpr int kSelClusterWide = 16;   // and those of this size where select_wide_cluster says so
 static constexpr int kCandSlack = 4096;      // candidates past K_m that the threshold bin may bring
 static constexpr int kWalkCells = 4;         // ranked cells per thread and round of the quota walk
 static constexpr int kMinWalkers = 64;       // fewest threads that walk
@@ -116,6 +117,7 @@ struct SelectParams {
   int* ranked;             // [n_comb][cand_stride] cell ids in rank order (cand_stride: multiple of 4)
   uint32_t* bitmap;        // [ceil(L/32)] in global memory, used when it does not fit shared memory
   int bitmap_in_smem;
+  int cluster;             // the grid runs as one thread-block cluster
   int walk_threads;        // threads that walk the combinations in the allocation phase
   int* out_idx;            // [n_sink + budget]
   int budget;
@@ -137,8 +139,20 @@ inline size_t select_smem_bytes(long long L, int max_km, SelectParams* p) {
   p->walk_threads = walkers < kMinWalkers ? kMinWalkers : (walkers > kSelThreads ? kSelThreads : walkers);
   return kSelWorkBytes + (p->bitmap_in_smem ? (words + kSelBitmapSlackWords) * sizeof(uint32_t) : 0);
 }
-// Largest grid that is co-resident on the device (the kernel's CTAs wait on one another).
-cudaError_t select_max_grid(int n_sm, int* max_grid);
+// Which contexts of more than one small cluster's work run as one cluster of kSelClusterWide CTAs (where the device
+// takes such a cluster): it starts under the end of the scores pass, and its barriers cost half of the
+// counter's, which a cooperative grid of 50 to 100 CTAs gains back on many cells, on many candidates to rank, or on
+// many combinations.  Whole recalls (16 query tokens), cooperative / cluster of 16, us: 3 windows, budget 512, 8K
+// positions 31.2 / 30.6, 16K 40.2 / 37.4, 24K 42.5 / 40.6, 32K 47.3 / 48.0; budget 4096, 16K 43.5 / 43.3, 24K
+// 46.4 / 49.8; 5 windows, budget 2048, 12K 44.1 / 42.4, 16K 44.2 / 47.5; 48 combinations, 8K 80 / 103.
+inline bool select_wide_cluster(const ComboTable& t) {
+  long long cells = 0, cand = 0;
+  for (int c = 0; c < t.n_comb; ++c) { cells += t.len[c]; cand += t.k_m[c]; }
+  return t.n_comb <= 8 && cells > 20480 && cells + 5 * cand <= 95000;
+}
+// Largest grid that is co-resident on the device (the kernel's CTAs wait on one another), and whether it takes a
+// cluster of kSelClusterWide CTAs.
+cudaError_t select_max_grid(int n_sm, int* max_grid, bool* wide_cluster);
 // One cooperative launch: A^C from the encoded maxima, then all of Algorithm 1.
 cudaError_t launch_select(const ComboTable& tbl, const SelectParams& p, int grid, size_t smem,
                           cudaStream_t st);

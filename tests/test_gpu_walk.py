@@ -1,4 +1,4 @@
-"""GPU: quota walk and ascending output where their paths change.
+"""GPU: selection, quota walk and ascending output where their paths change.
 
 A walking thread takes four ranked cells per round, at most 1024 threads walk: lists of more than
 4096 cells take several rounds, and may meet the quota before their last one.  Cells lie in one,
@@ -19,6 +19,10 @@ CASES = [
     # L, budget, max sizes, window sizes, n_sink
     (1, 1, (1,), (1,), 0),
     (129, 125, (1,), (3, 5), 4),
+    (6830, 512, (1,), (1, 7, 15), 2),               # one cluster of 16 CTAs: fewest and most cells, odd lengths
+    (16384, 512, (1,), (1, 7, 15), 0),
+    (12289, 2047, (1,), (1, 7, 15, 31, 63), 3),
+    (20001, 300, (1, 2), (1, 9), 0),
     (32768, 4097, (1,), (1, 7, 15), 0),             # a lane per word, the last such length
     (32773, 5, (2, 64), (1, 2), 5),                 # 32768 positions behind the sink part
     (32769, 16382, (1,), (1, 31), 0),               # warp lists; four rounds, met before the last
