@@ -28,6 +28,10 @@ static constexpr int kAttnStages = 3;
 static constexpr int kAttnTileBytes = 128 * 128 * 2;       // one 128 x 128 bf16 tile
 static constexpr int kAttnTailBytes = 256;
 static constexpr int kAttnPolyPairs = 2;                   // of every 16 pairs of exponentials
+// Of a tile's four groups of exponentials, those computed before the wait for the P buffer.  Us at 1024 / 2048 /
+// 16384 tokens behind 516 rows, calls in a row, 0 to 4 of them: 28.9 / 58.1 / 2122, 27.4 / 55.3 / 2078, 26.4 / 53.8 /
+// 1998, 27.0 / 54.8 / 1982, 30.3 / 60.3 / 1968 (all: nothing is left that the stores could overlap with).
+static constexpr int kAttnEarly = 2;
 static constexpr int kAttnSoftmaxWarps = 4;                // per stream: one per TMEM lane quadrant
 
 struct AttnTail {
@@ -309,18 +313,13 @@ chunk_attention_kernel(const __grid_constant__ CUtensorMap map_q,
         ref = (cm == -INFINITY) ? ref : cm;
       }
       const float nr = (ref == -INFINITY) ? 0.f : -ref * c2;
-      // the previous tile's P must have been consumed (and O updated) by its MMAs
-      ok = mbar_wait(smem_u32(&tail->p_empty[x]), (static_cast<uint32_t>(t) & 1u) ^ 1u, abort_flag,
-                     p.status, kDevWaitAccEmpty);
-      if (!ok) break;
-      // Exponentials in groups of 32 keys; each group's bf16 pairs go straight to P[row][key]
-      // (two halves of 64 keys, rows of 128 bytes, 16-byte groups XOR-swizzled by the row index:
-      // the layout TMA's 128-byte swizzle produces for the other operands), so the stores
-      // drain while the next group is computed.
+      // Exponentials in groups of 32 keys; each group's bf16 pairs go to P[row][key] (two halves of 64 keys, rows
+      // of 128 bytes, 16-byte groups XOR-swizzled by the row index: the layout TMA's 128-byte swizzle produces
+      // for the other operands), so the stores drain while the next group is computed.  The first kAttnEarly groups
+      // are computed before the previous tile's P is known to have been consumed by its MMAs, which takes
+      // until some 600 cycles after the maximum.
       float2 sum2 = make_float2(0.f, 0.f);
-#pragma unroll
-      for (int g32 = 0; g32 < 4; ++g32) {
-        uint32_t w[16];
+      auto exponentials = [&](int g32, uint32_t (&w)[16]) {
 #pragma unroll
         for (int i = 0; i < 32; i += 2) {
           const float2 a = ffma2(make_float2(V(g32 * 32 + i), V(g32 * 32 + i + 1)), make_float2(c2, c2),
@@ -334,12 +333,34 @@ chunk_attention_kernel(const __grid_constant__ CUtensorMap map_q,
           const __nv_bfloat162 pr = __floats2bfloat162_rn(pp.x, pp.y);
           w[i >> 1] = *reinterpret_cast<const uint32_t*>(&pr);
         }
+      };
+      auto store = [&](int g32, const uint32_t (&w)[16]) {
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
           const int c16 = g32 * 4 + c;
           uint4* dst = reinterpret_cast<uint4*>(p_mine + (c16 >> 3) * 16384 + row * 128 +
                                                 (((c16 & 7) ^ (row & 7)) << 4));
           *dst = make_uint4(w[c * 4], w[c * 4 + 1], w[c * 4 + 2], w[c * 4 + 3]);
+        }
+      };
+      uint32_t early[kAttnEarly][16];
+#pragma unroll
+      for (int g32 = 0; g32 < kAttnEarly; ++g32) {
+        exponentials(g32, early[g32]);
+#pragma unroll
+        for (int i = 0; i < 16; ++i) asm volatile("" : "+r"(early[g32][i]));     // not after the wait
+      }
+      ok = mbar_wait(smem_u32(&tail->p_empty[x]), (static_cast<uint32_t>(t) & 1u) ^ 1u, abort_flag,
+                     p.status, kDevWaitAccEmpty);
+      if (!ok) break;
+#pragma unroll
+      for (int g32 = 0; g32 < 4; ++g32) {
+        uint32_t w[16];
+        if (g32 < kAttnEarly) {
+          store(g32, early[g32 < kAttnEarly ? g32 : 0]);
+        } else {
+          exponentials(g32, w);
+          store(g32, w);
         }
       }
       l = fmaf(l, scale, sum2.x + sum2.y);
