@@ -17,14 +17,14 @@ struct AttnParams {
   int n_qt;          // query tiles of 128 tokens
   int split_from;    // query tiles >= split_from get one CTA per head (n_qt = none)
   float c2;          // log2(e) / sqrt(d)
-  uint16_t* out;     // bf16 [c][n_q][128]
   int* status;
 };
 
 size_t attn_smem_bytes();
 // One CTA per (query tile, head pair) -- or per head, for the query tiles from split_from on;
-// fills p.n_qt and p.split_from (n_sm: SMs of the device).
+// fills p.n_qt and p.split_from (n_sm: SMs of the device).  map_o: the output, bf16 [c][n_q][128], in boxes of 32 rows.
 cudaError_t launch_chunk_attention(const CUtensorMap& map_q, const CUtensorMap& map_k,
-                                   const CUtensorMap& map_v, AttnParams p, int n_sm, cudaStream_t st);
+                                   const CUtensorMap& map_v, const CUtensorMap& map_o, AttnParams p, int n_sm,
+                                   cudaStream_t st);
 
 }  // namespace ilre

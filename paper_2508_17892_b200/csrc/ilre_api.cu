@@ -654,16 +654,17 @@ int ilre_recall_chunk_attention(ilre_recall_t* h, const void* q_dev, const void*
   const uint64_t n_rows = static_cast<uint64_t>(n_prefix) + chunk_len;
   const uint64_t q_inner = static_cast<uint64_t>(h->cfg.n_q_heads) * kHeadDim;
   const uint64_t kv_inner = static_cast<uint64_t>(h->cfg.n_kv_heads) * kHeadDim;
-  CUtensorMap map_q, map_k, map_v;
+  CUtensorMap map_q, map_k, map_v, map_o;
   if (!encode_2d(h->encode, &map_q, q_dev, q_inner, chunk_len, q_inner * 2, 128) ||
       !encode_2d(h->encode, &map_k, k_dev, kv_inner, n_rows, kv_inner * 2, 128) ||
-      !encode_2d(h->encode, &map_v, v_dev, kv_inner, n_rows, kv_inner * 2, 128))
+      !encode_2d(h->encode, &map_v, v_dev, kv_inner, n_rows, kv_inner * 2, 128) ||
+      !encode_2d(h->encode, &map_o, out_dev, q_inner, chunk_len, q_inner * 2, 32))
     return ILRE_ERR_CUDA;
   AttnParams ap;
   ap.c = chunk_len; ap.n_prefix = n_prefix; ap.n_q = h->cfg.n_q_heads; ap.n_kv = h->cfg.n_kv_heads;
   ap.c2 = static_cast<float>(1.4426950408889634 / std::sqrt(static_cast<double>(kHeadDim)));
-  ap.out = static_cast<uint16_t*>(out_dev); ap.status = h->status;
-  ILRE_CUDA(launch_chunk_attention(map_q, map_k, map_v, ap, h->n_sm, st));
+  ap.status = h->status;
+  ILRE_CUDA(launch_chunk_attention(map_q, map_k, map_v, map_o, ap, h->n_sm, st));
   h->last_launches = 1;
   return ILRE_OK;
 }
