@@ -26,7 +26,8 @@
 // kSelTile cells of one combination; every CTA owns a contiguous run of tiles.
 //
 // Bound by the chain of its phases: barriers, one CTA's walk, code met cold in the instruction cache
-// (everything it reads is in L2).  The stage by itself, events around it after an L2 flush, with a
+// (everything it reads is in L2).  Hence `unroll 1` on loops of few turns: the compiler's fourfold copies with their
+// remainders are lines fetched for one turn (with its own choice 128K positions 33.1 us, so 28.9; 1M 71, 64).  The stage by itself, events around it after an L2 flush, with a
 // selection inside the threshold bin, one window per pooling tile and scattered candidates -> as it
 // stands: 4K positions 39 -> 29 us, 32K 52 -> 38, 128K 59 -> 44, 512K 89 -> 63, 1M 117..131 -> 84, 1M with
 // 48 combinations 270..280 -> 210.
@@ -150,6 +151,7 @@ __device__ __forceinline__ void hist_flush(uint32_t* sh_hist, uint32_t* gh) {
 // Combination that owns `tile`.  Tiles are visited in increasing order, so the search resumes
 // from the previous answer (`cur`, 0 at first).
 __device__ __forceinline__ int combo_of_tile(const ComboTable& tbl, int tile, int& cur) {
+#pragma unroll 1
   while (cur + 1 < tbl.n_comb && tile >= tbl.tile_begin[cur + 1]) ++cur;
   return cur;
 }
@@ -247,21 +249,28 @@ __device__ __forceinline__ void pool_tile(const ComboTable& tbl, const SelectPar
   const int some = tbl.grp_combo[first];
   const int n_max = tbl.n[tbl.grp_combo[first + n_win - 1]], len = tbl.len[some];
   const int source = tbl.src[some];
-  const float* a = (source < 0) ? nullptr : p.maxpooled + static_cast<long long>(source) * p.maxpooled_stride;
+  // the cells: pooled ones, given scores, or encoded ones, which are decoded here
+  const bool encoded = source < 0 && !p.scores_given;
+  const uint32_t* a = source >= 0 ? reinterpret_cast<const uint32_t*>(p.maxpooled + static_cast<long long>(source) * p.maxpooled_stride)
+                                  : (encoded ? p.enc : reinterpret_cast<const uint32_t*>(p.scores)) + p.n_sink;
   const int lo = c0 - n_max / 2;
   const int span = n_out + n_max - 1;
   const float pad = (p.win_op == 0) ? 0.f : -INFINITY;
+  const int first_cell = lo + static_cast<int>(threadIdx.x), last_cell = min(len, lo + span);
+#pragma unroll 1
   for (int base = 0; base < span; base += 4 * kSelThreads) {
-    float v[4];                                            // all loads in flight together
+    uint32_t raw[4];                                       // all loads in flight together
 #pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int u = first_cell + base + k * kSelThreads;
+      raw[k] = (u >= 0 && u < last_cell) ? __ldcg(a + u) : 0u;
+    }
+#pragma unroll 1
     for (int k = 0; k < 4; ++k) {
       const int idx = base + k * kSelThreads + threadIdx.x, u = lo + idx;
-      v[k] = (idx < span && u >= 0 && u < len) ? (a ? __ldcg(a + u) : score_at(p, p.n_sink + u)) : pad;
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int idx = base + k * kSelThreads + threadIdx.x;
-      if (idx < span) buf0[idx] = v[k];
+      if (idx >= span) break;
+      buf0[idx] = (u < 0 || u >= len) ? pad : encoded ? exp2f(ordered_to_float(raw[0])) : __uint_as_float(raw[0]);
+      raw[0] = raw[1]; raw[1] = raw[2]; raw[2] = raw[3];
     }
   }
   __syncthreads();
@@ -276,7 +285,7 @@ __device__ __forceinline__ void pool_tile(const ComboTable& tbl, const SelectPar
 #pragma unroll 1
       for (; 2 * w <= n; w *= 2) {
         const int cnt = span - 2 * w + 1;
-#pragma unroll 4
+#pragma unroll 1
         for (int i = threadIdx.x; i < cnt; i += kSelThreads) dst[i] = fmaxf(src[i], src[i + w]);
         __syncthreads();
         float* t = src; src = dst; dst = t;
@@ -398,6 +407,7 @@ __device__ __forceinline__ void gather_combination(const SelectParams& p, const 
       seg[at] = start | (count << 16);
     }
   };
+#pragma unroll 1
   for (int tile = tile0; tile < tile1; tile += kGatherGroup) {
     const int cell0 = (tile - tbl.tile_begin[combo]) * kSelTile + 4 * static_cast<int>(threadIdx.x);
     const int end = min(len, (tile1 - tbl.tile_begin[combo]) * kSelTile);
@@ -414,6 +424,7 @@ __device__ __forceinline__ void gather_combination(const SelectParams& p, const 
                 (v[g].w >= lowest ? 8u : 0u)) << (4 * g);
     if (!found) continue;
     int at = static_cast<int>(atomicAdd(&sh->n_listed, static_cast<uint32_t>(__popc(found))));
+#pragma unroll 1
     while (found) {
       const int e = __ffs(found) - 1;
       found &= found - 1;
@@ -424,6 +435,7 @@ __device__ __forceinline__ void gather_combination(const SelectParams& p, const 
   }
   __syncthreads();
   const int n = static_cast<int>(min(sh->n_listed, static_cast<uint32_t>(kSelWorkBytes / 4)));
+#pragma unroll 1
   for (int i = threadIdx.x; i < n; i += kSelThreads)
     if (list[i] >= 0) place(list[i]);
 }
@@ -566,9 +578,11 @@ __device__ __forceinline__ void rank_range(const SelectParams& p, const ComboTab
   const uint32_t* seg = p.cand_seg + static_cast<long long>(combo) * p.cand_stride;
   int* ranked = p.ranked + static_cast<long long>(combo) * p.cand_stride;
   const int k_m = tbl.k_m[combo];
+#pragma unroll 1
   for (int c0 = lo; c0 < hi; c0 += kSelThreads) {
     const int nc = min(kSelThreads, hi - c0);
     int g = 1;                                              // threads per candidate
+#pragma unroll 1
     while (g < 32 && 2 * g * nc <= kSelThreads) g <<= 1;
     const int local = threadIdx.x / g, sub = threadIdx.x % g;
     const bool active = local < nc;
@@ -590,9 +604,11 @@ __device__ __forceinline__ void rank_range(const SelectParams& p, const ComboTab
       }
     }
     int above = 0;
+#pragma unroll 1
     for (int base = begin; base < end; base += kRankChunk) {
       const int cnt = min(kRankChunk, end - base);
       if (base > begin) __syncthreads();                    // previous users of the chunk
+#pragma unroll 1
       for (int i = threadIdx.x; i < cnt; i += kSelThreads) chunk[i] = __ldcg(&cand[base + i]);
       __syncthreads();
       if (active) {
@@ -601,6 +617,7 @@ __device__ __forceinline__ void rank_range(const SelectParams& p, const ComboTab
         for (int j = max(first, base) - base + sub; j < j1; j += g) above += (chunk[j] > key) ? 1 : 0;
       }
     }
+#pragma unroll 1
     for (int d = 1; d < g; d <<= 1) above += __shfl_xor_sync(0xFFFFFFFFu, above, d);
     if (active && sub == 0 && first + above < k_m)
       ranked[first + above] = static_cast<int>(0xFFFFFFFFu - static_cast<uint32_t>(key & 0xFFFFFFFFull));
@@ -751,6 +768,7 @@ __device__ __forceinline__ void walk_round(const SelectParams& p, const int (&c)
     }
     if (end_room) {                                            // its lowest tokens
       auto rest = end;
+#pragma unroll 1
       for (uint32_t k = 0; k < end_room; ++k) rest &= rest - 1;
       const int t0 = end_cell * m;
       if constexpr (kCells == kCellsAligned) bitmap_set<kSmem>(bm, t0 >> 5, (end ^ rest) << (t0 & 31));
@@ -781,6 +799,7 @@ __device__ __forceinline__ void emit_words(const SelectParams& p, uint32_t bits,
   const uint32_t lane = threadIdx.x & 31, n = __popc(bits);
   const int pos0 = p.n_sink + w * 32;
   uint32_t together = __ballot_sync(0xFFFFFFFFu, n > kAlone);
+#pragma unroll 1
   while (together) {
     const int a = __ffs(together) - 1;                         // two words per turn
     together &= together - 1;
@@ -795,6 +814,7 @@ __device__ __forceinline__ void emit_words(const SelectParams& p, uint32_t bits,
     if (((bits_b >> lane) & 1u) && at_b < cap) p.out_idx[at_b] = pos_b + lane;
   }
   if (n <= kAlone) {
+#pragma unroll 1
     while (bits) {
       const int k = __ffs(bits) - 1;
       bits &= bits - 1;
@@ -901,6 +921,7 @@ __device__ __forceinline__ void allocate(const ComboTable& tbl, const SelectPara
   // them cold (a line that is not in its cache costs some 300 cycles).  The sink part is the identity.
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t cap = static_cast<uint32_t>(p.n_sink + p.budget);
+#pragma unroll 1
   for (int j = threadIdx.x; j < p.n_sink; j += kSelThreads) p.out_idx[j] = j;
   uint32_t total;
   if (4 * n_quads <= kSelThreads) {
@@ -924,7 +945,7 @@ __device__ __forceinline__ void allocate(const ComboTable& tbl, const SelectPara
     else return __ldcg(reinterpret_cast<const uint4*>(bm) + q);
   };
   uint32_t mine = 0;
-#pragma unroll 4
+#pragma unroll 1
   for (int q = q_begin; q < q_end; q += 32) {
     const uint4 v = load_quad(q + lane);
     if (__any_sync(0xFFFFFFFFu, (v.x | v.y | v.z | v.w) != 0u)) mine += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
@@ -1155,6 +1176,7 @@ select_kernel(const __grid_constant__ ComboTable tbl, const __grid_constant__ Se
   if (blockIdx.x == 0 && p.bitmap_in_smem) {               // for phase F: empty
     uint32_t* bm = smem_bitmap(dyn_smem);
     const int n_words = static_cast<int>((p.L + 31) / 32), Lp = static_cast<int>(p.L - p.n_sink);
+#pragma unroll 1
     for (int w = threadIdx.x; w < n_words; w += kSelThreads) bm[w] = empty_bitmap_word(w, Lp);
   }
   uint32_t epoch = 0;
@@ -1166,7 +1188,9 @@ select_kernel(const __grid_constant__ ComboTable tbl, const __grid_constant__ Se
     const int s_begin = static_cast<int>(static_cast<long long>(blockIdx.x) * n_st / gridDim.x);
     const int s_end = static_cast<int>(static_cast<long long>(blockIdx.x + 1) * n_st / gridDim.x);
     int src = 0;
+#pragma unroll 1
     for (int tile = s_begin; tile < s_end; ++tile) {
+#pragma unroll 1
       while (src + 1 < tbl.n_src && tile >= tbl.src_tile_begin[src + 1]) ++src;
       maxpool_tile(tbl, p, src, tile - tbl.src_tile_begin[src], reinterpret_cast<uint32_t*>(dyn_smem));
     }
@@ -1184,11 +1208,14 @@ select_kernel(const __grid_constant__ ComboTable tbl, const __grid_constant__ Se
     const int p_begin = static_cast<int>(static_cast<long long>(blockIdx.x) * n_pt / gridDim.x);
     const int p_end = static_cast<int>(static_cast<long long>(blockIdx.x + 1) * n_pt / gridDim.x);
     int grp = 0;
+#pragma unroll 1
     for (int tile = p_begin; tile < p_end; ++tile) {
+#pragma unroll 1
       while (grp + 1 < tbl.n_grp && tile >= tbl.grp_tile_begin[grp + 1]) ++grp;
       const int c0 = (tile - tbl.grp_tile_begin[grp]) * per, first = tbl.grp_first[grp];
       pool_tile(tbl, p, grp, c0, min(per, tbl.len[tbl.grp_combo[first]] - c0), buf0, buf1, sh.hist, hist1);
       if (tile + 1 == p_end || tile + 1 == tbl.grp_tile_begin[grp + 1]) {      // the CTA's last tile of this group
+#pragma unroll 1
         for (int k = 0; first + k < tbl.grp_first[grp + 1]; ++k)               // (which ended with a barrier)
           hist_drain((k == 0) ? sh.hist : hist1 + (k - 1) * kHistBins,
                      p.hist + static_cast<long long>(tbl.grp_combo[first + k]) * kHistBins);
@@ -1205,6 +1232,7 @@ select_kernel(const __grid_constant__ ComboTable tbl, const __grid_constant__ Se
     c_lo = combo_of_tile(tbl, t_begin, cursor);
     c_hi = combo_of_tile(tbl, t_end - 1, cursor);
   }
+#pragma unroll 1
   for (int combo = c_lo; combo <= c_hi; ++combo) {
     find_threshold(p, tbl, combo, &sh);
     if (threadIdx.x == 0) {
@@ -1230,6 +1258,7 @@ select_kernel(const __grid_constant__ ComboTable tbl, const __grid_constant__ Se
   {
     unsigned long long* chunk = reinterpret_cast<unsigned long long*>(dyn_smem);
     const int grid = static_cast<int>(gridDim.x), bid = static_cast<int>(blockIdx.x);
+#pragma unroll 1
     for (int combo = threadIdx.x; combo < tbl.n_comb; combo += kSelThreads) {
       const uint32_t n = min(__ldcg(&p.cand_count[combo]), static_cast<uint32_t>(p.cand_stride));
       sh.state[combo] = n;
@@ -1251,10 +1280,12 @@ select_kernel(const __grid_constant__ ComboTable tbl, const __grid_constant__ Se
     // of all candidates.
     const int only = tbl.rank_by_list ? sh.list : -1;
     long long n_cand = 0;
+#pragma unroll 1
     for (int combo = 0; combo < tbl.n_comb && only < 0; ++combo) n_cand += sh.state[combo];
     const int i_begin = static_cast<int>(static_cast<long long>(bid) * n_cand / grid);
     const int i_end = static_cast<int>(static_cast<long long>(bid + 1) * n_cand / grid);
     int first = 0;
+#pragma unroll 1
     for (int combo = max(only, 0); combo < (only < 0 ? tbl.n_comb : only + 1); ++combo) {
       const int n = static_cast<int>(sh.state[combo]);
       const int lo = only < 0 ? max(i_begin, first) - first : static_cast<int>(sh.krem[0]);
@@ -1268,6 +1299,7 @@ select_kernel(const __grid_constant__ ComboTable tbl, const __grid_constant__ Se
   // ---- F: allocation and ascending output (one CTA); the others write the scores if asked ----
   if (p.user_scores && (blockIdx.x != 0 || gridDim.x == 1)) {
     const long long writers = gridDim.x == 1 ? 1 : gridDim.x - 1, mine = gridDim.x == 1 ? 0 : blockIdx.x - 1;
+#pragma unroll 1
     for (long long t = mine * kSelThreads + threadIdx.x; t < p.L; t += writers * kSelThreads)
       p.user_scores[t] = score_at(p, t);
   }
