@@ -167,12 +167,11 @@ __device__ __forceinline__ void fetch_tile(const ComboTable& tbl, const SelectPa
   const int combo = combo_of_tile(tbl, tile, cur);
   if (skip && skip[combo]) return;
   const float* w = p.pooled + static_cast<long long>(combo) * p.pooled_stride;
-  const int c0 = (tile - tbl.tile_begin[combo]) * kSelTile;
-  const int c1 = min(tbl.len[combo], c0 + kSelTile);
+  const int c0 = (tile - tbl.tile_begin[combo]) * kSelTile, n = cells_from(tbl.len[combo], c0, kSelTile);
 #pragma unroll
   for (int k = 0; k < kTilePer; ++k) {
-    const int c = c0 + k * kSelThreads + threadIdx.x;
-    wv[k] = (c < c1) ? __ldcg(&w[c]) : 0.f;
+    const int i = k * kSelThreads + threadIdx.x;
+    wv[k] = (i < n) ? __ldcg(&w[c0 + i]) : 0.f;
   }
 }
 
@@ -256,20 +255,20 @@ __device__ __forceinline__ void pool_tile(const ComboTable& tbl, const SelectPar
   const int lo = c0 - n_max / 2;
   const int span = n_out + n_max - 1;
   const float pad = (p.win_op == 0) ? 0.f : -INFINITY;
-  const int first_cell = lo + static_cast<int>(threadIdx.x), last_cell = min(len, lo + span);
+  const int in_begin = -lo, in_end = cells_from(len, c0, span) + n_max / 2;      // of the tile and its margins, what lies inside
 #pragma unroll 1
   for (int base = 0; base < span; base += 4 * kSelThreads) {
     uint32_t raw[4];                                       // all loads in flight together
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const int u = first_cell + base + k * kSelThreads;
-      raw[k] = (u >= 0 && u < last_cell) ? __ldcg(a + u) : 0u;
+      const int idx = base + k * kSelThreads + threadIdx.x;
+      raw[k] = (idx >= in_begin && idx < min(span, in_end)) ? __ldcg(a + lo + idx) : 0u;
     }
 #pragma unroll 1
     for (int k = 0; k < 4; ++k) {
-      const int idx = base + k * kSelThreads + threadIdx.x, u = lo + idx;
+      const int idx = base + k * kSelThreads + threadIdx.x;
       if (idx >= span) break;
-      buf0[idx] = (u < 0 || u >= len) ? pad : encoded ? exp2f(ordered_to_float(raw[0])) : __uint_as_float(raw[0]);
+      buf0[idx] = (idx < in_begin || idx >= in_end) ? pad : encoded ? exp2f(ordered_to_float(raw[0])) : __uint_as_float(raw[0]);
       raw[0] = raw[1]; raw[1] = raw[2]; raw[2] = raw[3];
     }
   }
@@ -409,13 +408,13 @@ __device__ __forceinline__ void gather_combination(const SelectParams& p, const 
   };
 #pragma unroll 1
   for (int tile = tile0; tile < tile1; tile += kGatherGroup) {
-    const int cell0 = (tile - tbl.tile_begin[combo]) * kSelTile + 4 * static_cast<int>(threadIdx.x);
-    const int end = min(len, (tile1 - tbl.tile_begin[combo]) * kSelTile);
+    const int first = (tile - tbl.tile_begin[combo]) * kSelTile, i0 = 4 * static_cast<int>(threadIdx.x);
+    const int n = cells_from(len, first, min(kGatherGroup, tile1 - tile) * kSelTile);
     float4 v[kGatherGroup];
 #pragma unroll
     for (int g = 0; g < kGatherGroup; ++g) {
       v[g] = make_float4(NAN, NAN, NAN, NAN);
-      if (cell0 + g * kSelTile < end) v[g] = __ldcg(reinterpret_cast<const float4*>(w + cell0 + g * kSelTile));
+      if (i0 + g * kSelTile < n) v[g] = __ldcg(reinterpret_cast<const float4*>(w + first + i0 + g * kSelTile));
     }
     uint32_t found = 0;
 #pragma unroll
@@ -428,9 +427,9 @@ __device__ __forceinline__ void gather_combination(const SelectParams& p, const 
     while (found) {
       const int e = __ffs(found) - 1;
       found &= found - 1;
-      const int cell = cell0 + (e >> 2) * kSelTile + (e & 3);
-      if (at < kSelWorkBytes / 4) list[at++] = (cell < len) ? cell : -1;
-      else if (cell < len) place(cell);                      // more than the list holds
+      const int i = i0 + (e >> 2) * kSelTile + (e & 3);
+      if (at < kSelWorkBytes / 4) list[at++] = (i < n) ? first + i : -1;
+      else if (i < n) place(first + i);                      // more than the list holds
     }
   }
   __syncthreads();
@@ -1043,14 +1042,13 @@ __device__ __noinline__ uint32_t long_way(const ComboTable& tbl, const SelectPar
           hist_flush(sh->hist, hist_pass + static_cast<long long>(cur) * kHistBins);
         cur = combo;
         const unsigned long long prefix = sh->prefix[combo];
-        const int c0 = (tile - tbl.tile_begin[combo]) * kSelTile;
-        const int c1 = min(tbl.len[combo], c0 + kSelTile);
+        const int c0 = (tile - tbl.tile_begin[combo]) * kSelTile, n = cells_from(tbl.len[combo], c0, kSelTile);
 #pragma unroll
         for (int k = 0; k < kTilePer; ++k) {
-          const int c = c0 + k * kSelThreads + threadIdx.x;
+          const int i = k * kSelThreads + threadIdx.x;
           uint32_t digit = 0xFFFFFFFFu;                    // sentinel: does not take part
-          if (c < c1) {
-            const unsigned long long key = make_key(wv[g][k], static_cast<uint32_t>(c));
+          if (i < n) {
+            const unsigned long long key = make_key(wv[g][k], static_cast<uint32_t>(c0 + i));
             if (pass == 0 || ((key ^ prefix) >> (shift + bits)) == 0ull)
               digit = static_cast<uint32_t>(key >> shift) & mask;
           }
@@ -1082,13 +1080,12 @@ __device__ __noinline__ uint32_t long_way(const ComboTable& tbl, const SelectPar
         const int combo = combo_of_tile(tbl, tile, cursor);
         if (sh->state[combo]) continue;
         const uint32_t v_star = static_cast<uint32_t>(sh->prefix[combo] >> 32);
-        const int c0 = (tile - tbl.tile_begin[combo]) * kSelTile;
-        const int c1 = min(tbl.len[combo], c0 + kSelTile);
+        const int c0 = (tile - tbl.tile_begin[combo]) * kSelTile, n = cells_from(tbl.len[combo], c0, kSelTile);
         int mine = 0;
 #pragma unroll
         for (int k = 0; k < kTilePer; ++k) {
-          const int c = c0 + k * kSelThreads + threadIdx.x;
-          mine += (c < c1 && float_to_ordered(wv[g][k]) == v_star) ? 1 : 0;
+          const int i = k * kSelThreads + threadIdx.x;
+          mine += (i < n && float_to_ordered(wv[g][k]) == v_star) ? 1 : 0;
         }
         const int holders = __syncthreads_count(mine & 1) + 2 * __syncthreads_count(mine & 2) +
                             4 * __syncthreads_count(mine & 4);
@@ -1116,8 +1113,7 @@ __device__ __noinline__ uint32_t long_way(const ComboTable& tbl, const SelectPar
         const uint32_t v_star = static_cast<uint32_t>(threshold >> 32);
         const uint32_t wanted = sh->krem[combo];
         unsigned long long* cand = p.cand + static_cast<long long>(combo) * p.cand_stride;
-        const int c0 = (tile - tbl.tile_begin[combo]) * kSelTile;
-        const int c1 = min(tbl.len[combo], c0 + kSelTile);
+        const int c0 = (tile - tbl.tile_begin[combo]) * kSelTile, n = cells_from(tbl.len[combo], c0, kSelTile);
         // holders of v in the earlier tiles of this combination (tiles are in cell order)
         uint32_t before = 0;
         bool ties_here = false;
@@ -1133,11 +1129,11 @@ __device__ __noinline__ uint32_t long_way(const ComboTable& tbl, const SelectPar
         }
 #pragma unroll
         for (int k = 0; k < kTilePer; ++k) {
-          const int c = c0 + k * kSelThreads + threadIdx.x;
+          const int i = k * kSelThreads + threadIdx.x;
           unsigned long long key = 0ull;
           bool take = false, holder = false;
-          if (c < c1) {
-            key = make_key(wv[g][k], static_cast<uint32_t>(c));
+          if (i < n) {
+            key = make_key(wv[g][k], static_cast<uint32_t>(c0 + i));
             const uint32_t v = static_cast<uint32_t>(key >> 32);
             if (settled) take = key >= threshold;
             else { take = v > v_star; holder = v == v_star; }
@@ -1384,38 +1380,6 @@ static void assign_ranking(ComboTable* t, int grid) {
     b0 = b1;
   }
   t->rank_cta_begin[t->n_comb] = b0;
-}
-
-// Groups the combinations for the pooling phase and cuts the groups into tiles: equal shares of the
-// grid's CTAs, rounded up to whole warps.
-static void assign_pooling(ComboTable* t, int grid) {
-  t->n_grp = 0;
-  int n = 0;
-  long long cells = 0;
-  for (int src = -1; src < t->n_src; ++src) {
-    int list[kMaxCombos], cnt = 0;
-    for (int c = 0; c < t->n_comb; ++c)
-      if (t->src[c] == src) list[cnt++] = c;
-    for (int i = 1; i < cnt; ++i)                           // by window size
-      for (int j = i; j > 0 && t->n[list[j]] < t->n[list[j - 1]]; --j) {
-        const int x = list[j]; list[j] = list[j - 1]; list[j - 1] = x;
-      }
-    const int n_groups = (cnt + kPoolGroup - 1) / kPoolGroup;
-    for (int g = 0; g < n_groups; ++g) {                    // groups of even size
-      t->grp_first[t->n_grp++] = n;
-      for (int i = g * cnt / n_groups; i < (g + 1) * cnt / n_groups; ++i) t->grp_combo[n++] = list[i];
-      cells += t->len[list[0]];
-    }
-  }
-  t->grp_first[t->n_grp] = n;
-  const long long rounds = (cells + static_cast<long long>(grid) * kPoolTileMax - 1) / (static_cast<long long>(grid) * kPoolTileMax);
-  const long long workers = static_cast<long long>(grid) * (rounds < 1 ? 1 : rounds);
-  long long tile = ((cells + workers - 1) / workers + 31) & ~31ll;
-  t->pool_tile = static_cast<int>(tile < 256 ? 256 : (tile > kPoolTileMax ? kPoolTileMax : tile));
-  t->grp_tile_begin[0] = 0;
-  for (int g = 0; g < t->n_grp; ++g)
-    t->grp_tile_begin[g + 1] = t->grp_tile_begin[g] +
-        (t->len[t->grp_combo[t->grp_first[g]]] + t->pool_tile - 1) / t->pool_tile;
 }
 
 cudaError_t launch_select(const ComboTable& table, const SelectParams& p, int grid, size_t smem,

@@ -81,7 +81,7 @@ struct ComboTable {
   int src_len[kMaxCombos];
   int src_tile_begin[kMaxCombos + 1];   // tiles of kSrcTileTokens / m cells each
   // Groups of combinations of one source (up to kPoolGroup, ascending window sizes) that are pooled
-  // together, and their work tiles of pool_tile cells (filled in by launch_select).
+  // together, and their work tiles of pool_tile cells (filled in by assign_pooling).
   int n_grp, pool_tile;
   int grp_first[kMaxCombos + 1];        // first entry of each group in grp_combo
   int grp_combo[kMaxCombos];
@@ -91,6 +91,42 @@ struct ComboTable {
   int rank_by_list;
   int rank_cta_begin[kMaxCombos + 1];
 };
+
+// Of a combination's cells, those from `first` on, at most `most`.  (Lengths go up to 2^31 - 257: the end of a work tile
+// may not fit an int, and where a cell lies in its tile is compared instead.)
+__host__ __device__ constexpr int cells_from(int len, int first, int most) { return len - first < most ? len - first : most; }
+
+// Groups the combinations for the pooling phase and cuts the groups into tiles: equal shares of the
+// grid's CTAs, rounded up to whole warps.
+inline void assign_pooling(ComboTable* t, int grid) {
+  t->n_grp = 0;
+  int n = 0;
+  long long cells = 0;
+  for (int src = -1; src < t->n_src; ++src) {
+    int list[kMaxCombos], cnt = 0;
+    for (int c = 0; c < t->n_comb; ++c)
+      if (t->src[c] == src) list[cnt++] = c;
+    for (int i = 1; i < cnt; ++i)                           // by window size
+      for (int j = i; j > 0 && t->n[list[j]] < t->n[list[j - 1]]; --j) {
+        const int x = list[j]; list[j] = list[j - 1]; list[j - 1] = x;
+      }
+    const int n_groups = (cnt + kPoolGroup - 1) / kPoolGroup;
+    for (int g = 0; g < n_groups; ++g) {                    // groups of even size
+      t->grp_first[t->n_grp++] = n;
+      for (int i = g * cnt / n_groups; i < (g + 1) * cnt / n_groups; ++i) t->grp_combo[n++] = list[i];
+      cells += t->len[list[0]];
+    }
+  }
+  t->grp_first[t->n_grp] = n;
+  const long long rounds = (cells + static_cast<long long>(grid) * kPoolTileMax - 1) / (static_cast<long long>(grid) * kPoolTileMax);
+  const long long workers = static_cast<long long>(grid) * (rounds < 1 ? 1 : rounds);
+  long long tile = ((cells + workers - 1) / workers + 31) & ~31ll;
+  t->pool_tile = static_cast<int>(tile < 256 ? 256 : (tile > kPoolTileMax ? kPoolTileMax : tile));
+  t->grp_tile_begin[0] = 0;
+  for (int g = 0; g < t->n_grp; ++g)
+    t->grp_tile_begin[g + 1] = t->grp_tile_begin[g] +
+        static_cast<int>((static_cast<long long>(t->len[t->grp_combo[t->grp_first[g]]]) + t->pool_tile - 1) / t->pool_tile);
+}
 
 struct SelectParams {
   const uint32_t* enc;     // [L] order-preserving uint of max_r log2 p_rt (scores pass output)

@@ -51,3 +51,29 @@ def test_walk_and_output(L, budget, max_sizes, win_sizes, n_sink, dense):
     ref = oracle.allocate(a.astype(np.float64), budget, max_sizes, win_sizes, 1, n_sink)
     assert np.array_equal(idx.cpu().numpy(), ref)
     eng.close()
+
+
+@pytest.mark.parametrize("win_op,win_sizes", [(1, (1, 1023)), (0, (8, 64))])
+def test_the_longest_context(win_op, win_sizes):
+    """2^31 - 257 positions, scores above zero among the last 20000 only: what is chosen there is what a
+    context that begins behind the zeros gives.  (Values are multiples of 2^-17 below 1, window sizes of the
+    averages powers of two: every sum and quotient is exact.)"""
+    from paper_2508_17892_b200 import IlreRecall
+    L, tail, budget = 2 ** 31 - 257, 20000, 2000
+    if torch.cuda.mem_get_info()[0] < 80 << 30:
+        pytest.skip("needs 80 GB of free device memory")
+    rng = np.random.default_rng(7)
+    a = (rng.integers(1, 2 ** 17, size=tail) / 2 ** 17).astype(np.float32)
+    a[:2000] = 0
+    eng = IlreRecall(max_L=L, max_q_len=1, max_budget=budget, n_kv_heads=1, n_q_heads=1, max_combinations=2)
+    scores = torch.zeros(L, device="cuda")
+    scores[-tail:] = torch.from_numpy(a).cuda()
+    idx = eng.allocate(scores, budget, (1,), win_sizes, win_op)
+    torch.cuda.synchronize()
+    eng.check_status()
+    assert eng.check_guards() == 0
+    ref = oracle.allocate(a.astype(np.float64), budget, (1,), win_sizes, win_op)
+    eng.close()
+    del scores
+    torch.cuda.empty_cache()
+    assert np.array_equal(idx.cpu().numpy(), ref + (L - tail))

@@ -10,10 +10,10 @@ CSRC = os.path.join(ROOT, "paper_2508_17892_b200", "csrc")
 CUDA = os.environ.get("CUDA_HOME", "/usr/local/cuda")
 
 
-def _run(tmp_path, body):
+def _run(tmp_path, body, *flags):
     src, exe = tmp_path / "check.cpp", tmp_path / "check"
     src.write_text(body)
-    subprocess.check_call(["g++", "-std=c++17", "-O1", "-I", CSRC, "-I", os.path.join(CUDA, "include"),
+    subprocess.check_call(["g++", "-std=c++17", "-O1", *flags, "-I", CSRC, "-I", os.path.join(CUDA, "include"),
                            "-x", "c++", str(src), "-o", str(exe)])
     r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stdout[-2000:]
@@ -142,3 +142,47 @@ int main() {
 
 def test_histogram_bins_cover_every_value_in_order(tmp_path):
     _run(tmp_path, BINS)
+
+
+LONGEST = r"""
+#include <algorithm>
+#include <cstdio>
+#include <cstring>
+#include "select_kernels.cuh"
+using namespace ilre;
+int main() {
+  int bad = 0;
+  for (long long L : {2147483647LL - 256, 2147483647LL - 256 - 2 * kPoolTileMax, 2147479553LL, 2147479552LL, 5000LL, 1LL})
+    for (int m : {1, 2, 64})
+      for (int grid : {1, 8, 148}) {
+        ComboTable t;
+        std::memset(&t, 0, sizeof(t));
+        t.n_comb = 2;
+        t.n_src = m > 1;
+        const int len = static_cast<int>((L + m - 1) / m);
+        for (int c = 0; c < 2; ++c) { t.m[c] = m; t.n[c] = c ? kMaxWin : 1; t.len[c] = len; t.src[c] = m > 1 ? 0 : -1; }
+        assign_pooling(&t, grid);
+        const long long end = static_cast<long long>(t.grp_tile_begin[1]) * t.pool_tile;
+        bool ok = t.n_grp == 1 && t.pool_tile <= kPoolTileMax && end >= len && end - t.pool_tile < len;
+        // the last tiles of the pooling and of the gather hold the last cell and nothing behind it
+        for (int size : {t.pool_tile, kSelTile, kSelTile * 4}) {
+          const int first = (len - 1) / size * size;
+          ok = ok && first + static_cast<long long>(cells_from(len, first, size)) == len;
+          ok = ok && (first == 0 || cells_from(len, first - size, size) == size);
+        }
+        // and of a tile with its margins, idx < cells_from(..) + margin are the cells of the context
+        for (int c0 : {0, std::max(0, len - 1), std::max(0, len / 2)}) {
+          const int span = std::min(t.pool_tile, len - c0) + kMaxWin - 1, margin = kMaxWin / 2;
+          const long long inside = std::min<long long>(span, static_cast<long long>(len) - c0 + margin);
+          ok = ok && std::min(span, cells_from(len, c0, span) + margin) == inside;
+        }
+        if (!ok && bad++ < 5) std::printf("L %lld m %d grid %d: tiles end at %lld\n", L, m, grid, end);
+      }
+  return bad;
+}
+"""
+
+
+def test_tiles_of_the_longest_contexts_end_where_the_context_does(tmp_path):
+    """Lengths go up to 2^31 - 257, where the end of a tile may not fit 32 bits with a sign."""
+    _run(tmp_path, LONGEST, "-fsanitize=signed-integer-overflow", "-fno-sanitize-recover")
