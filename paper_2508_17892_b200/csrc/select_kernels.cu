@@ -932,10 +932,12 @@ __device__ __forceinline__ void allocate(const ComboTable& tbl, const SelectPara
     if (threadIdx.x == 0 && total != static_cast<uint32_t>(p.budget)) atomicCAS(p.status, 0, kDevQuota);
     return;
   }
-  // Longer contexts: every warp takes an equal run of the bitmap and counts its positions; with the sum of the
-  // warps' before it, it goes through the run again, lists the words that are not empty (a few in a hundred,
-  // neighbours for the most part) in order and writes their positions, a lane per word (128K: 7.8 -> 5.4 us; 1M
-  // 8.6 and 9.1).
+  // Longer contexts: every warp takes an equal run of the bitmap and counts the words that are not empty (a few in a
+  // hundred, neighbours for the most part); with the sum of the warps' before it, it goes through the run
+  // again and enters them, in order, in the block's list.  The warps then take equal shares of the list, whose
+  // positions they count and write, a lane per word: passages may lie anywhere, all of them in one warp's run too.
+  // (Each warp writing what lies in its own run: allocation of 524288 positions, budget 4096, chosen from one 32nd of the
+  // context 80.9 us, so 64.5, spread evenly 110 and 113; 4000000 positions 150 and 112, spread 112 and 112.)
   const int per = ((n_quads + kMaxWalkWarps - 1) / kMaxWalkWarps + 31) & ~31;
   const int q_begin = min(n_quads, warp * per), q_end = min(n_quads, q_begin + per);
   auto load_quad = [&](int q) -> uint4 {
@@ -947,52 +949,60 @@ __device__ __forceinline__ void allocate(const ComboTable& tbl, const SelectPara
 #pragma unroll 1
   for (int q = q_begin; q < q_end; q += 32) {
     const uint4 v = load_quad(q + lane);
-    if (__any_sync(0xFFFFFFFFu, (v.x | v.y | v.z | v.w) != 0u)) mine += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+    mine += (v.x ? 1u : 0u) + (v.y ? 1u : 0u) + (v.z ? 1u : 0u) + (v.w ? 1u : 0u);
   }
-  uint32_t at = p.n_sink + block_exclusive_scan(mine, sh->scan, &total);
-  at = __shfl_sync(0xFFFFFFFFu, at, 0);
-  if (threadIdx.x == 0 && total != static_cast<uint32_t>(p.budget)) atomicCAS(p.status, 0, kDevQuota);
-  constexpr int kList = kSelWorkBytes / 4 / kMaxWalkWarps;      // words that a warp's list holds
-  int* list = reinterpret_cast<int*>(dyn_smem) + warp * kList;
-  int listed = 0;
+  constexpr uint32_t kList = kSelWorkBytes / 4;
+  static_assert(kList >= kMaxKm, "the list holds a word per position");
+  int* list = reinterpret_cast<int*>(dyn_smem);
+  uint32_t n_words;
+  uint32_t to = block_exclusive_scan(mine, sh->scan, &n_words);
+  to = __shfl_sync(0xFFFFFFFFu, to, 0);
 #pragma unroll 1
   for (int q = q_begin; q < q_end; q += 32) {
     const uint4 v = load_quad(q + lane);
     const uint32_t full = (v.x ? 1u : 0u) | (v.y ? 2u : 0u) | (v.z ? 4u : 0u) | (v.w ? 8u : 0u);
-    if (__any_sync(0xFFFFFFFFu, full != 0u)) {
-      // a word's place in the list: behind the words of the lanes before, by votes, and those of its own lane
-      const uint32_t lt = (1u << lane) - 1u;
-      int before = 0, found = 0;
+    if (!__any_sync(0xFFFFFFFFu, full != 0u)) continue;
+    // a word's place in the list: behind the words of the lanes before, by votes, and those of its own lane
+    const uint32_t lt = (1u << lane) - 1u;
+    uint32_t at = to;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const uint32_t votes = __ballot_sync(0xFFFFFFFFu, (full >> k) & 1u);
-        before += __popc(votes & lt);
-        found += __popc(votes);
-      }
-      int to = listed + before;
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        if ((full >> k) & 1u) list[to++] = 4 * (q + lane) + k;
-      listed += found;
+    for (int k = 0; k < 4; ++k) {
+      const uint32_t votes = __ballot_sync(0xFFFFFFFFu, (full >> k) & 1u);
+      at += __popc(votes & lt);
+      to += __popc(votes);
     }
-    if (listed + 128 > kList || q + 32 >= q_end) {              // uniform: the next 32 quads might not fit, or the end
-      __syncwarp();
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if ((full >> k) & 1u) {
+        if (at < kList) list[at] = 4 * (q + lane) + k;           // never past it unless a quota was overrun
+        ++at;
+      }
+  }
+  __syncthreads();
+  const int n_listed = static_cast<int>(min(n_words, kList)), share = (n_listed + kMaxWalkWarps - 1) / kMaxWalkWarps;
+  const int e_begin = min(n_listed, warp * share), e_end = min(n_listed, e_begin + share);
+  mine = 0;
 #pragma unroll 1
-      for (int e = lane; e - lane < listed; e += 32) {
-        const int w = (e < listed) ? list[e] : 0;
-        const uint32_t bits = (e < listed) ? bitmap_word<kBitmapInSmem>(bm, w) : 0u, n = __popc(bits);
-        uint32_t incl = n;
+  for (int e = e_begin + lane; e < e_end; e += 32) mine += __popc(bitmap_word<kBitmapInSmem>(bm, list[e]));
+  uint32_t at = p.n_sink + block_exclusive_scan(mine, sh->scan, &total);
+  if (threadIdx.x == 0 && total != static_cast<uint32_t>(p.budget)) atomicCAS(p.status, 0, kDevQuota);
+  if (share > 32) at = __shfl_sync(0xFFFFFFFFu, at, 0);          // else: already the place of the lane's one word
+#pragma unroll 1
+  for (int e = e_begin; e < e_end; e += 32) {
+    const int w = (e + lane < e_end) ? list[e + lane] : 0;
+    const uint32_t bits = (e + lane < e_end) ? bitmap_word<kBitmapInSmem>(bm, w) : 0u, n = __popc(bits);
+    uint32_t place = at;
+    if (share > 32) {
+      uint32_t incl = n;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-          if (lane >= o) incl += t;
-        }
-        emit_words(p, bits, w, at + incl - n, cap);
-        at += __shfl_sync(0xFFFFFFFFu, incl, 31);
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= o) incl += t;
       }
-      listed = 0;
-      __syncwarp();
+      place = at + incl - n;
+      at += __shfl_sync(0xFFFFFFFFu, incl, 31);
     }
+    emit_words(p, bits, w, place, cap);
   }
 }
 

@@ -3,7 +3,8 @@
 A walking thread takes four ranked cells per round, at most 1024 threads walk: lists of more than
 4096 cells take several rounds, and may meet the quota before their last one.  Cells lie in one,
 two or three bitmap words.  The output pass takes a lane per bitmap word up to 32768 positions,
-warp lists behind; above 1 114 112 positions the bitmap lives in global memory.
+a list of words shared out over the warps behind, in one round or many; above 1 114 112 positions the
+bitmap lives in global memory.
 """
 from __future__ import annotations
 
@@ -25,23 +26,27 @@ CASES = [
     (20001, 300, (1, 2), (1, 9), 0),
     (32768, 4097, (1,), (1, 7, 15), 0),             # a lane per word, the last such length
     (32773, 5, (2, 64), (1, 2), 5),                 # 32768 positions behind the sink part
-    (32769, 16382, (1,), (1, 31), 0),               # warp lists; four rounds, met before the last
+    (32769, 16382, (1,), (1, 31), 0),               # word list; four rounds, met before the last
     (40001, 16000, (3, 1, 48), (1, 9), 1),          # cells of one, two and three words
     (131072, 12289, (1, 2, 32, 33, 64), (1, 4), 0),
+    (1048576, 16000, (1,), (1, 7), 0),              # a list of many rounds per warp where spread out
     (1114113, 9000, (1, 5, 64), (1, 15), 0),        # bitmap in global memory
 ]
 
 
-@pytest.mark.parametrize("dense", [False, True])
+@pytest.mark.parametrize("lie", ["spread", "runs", "together"])
 @pytest.mark.parametrize("L,budget,max_sizes,win_sizes,n_sink", CASES)
-def test_walk_and_output(L, budget, max_sizes, win_sizes, n_sink, dense):
+def test_walk_and_output(L, budget, max_sizes, win_sizes, n_sink, lie):
     """Windows take the maximum, so every value is exact on both sides: identical positions."""
     from paper_2508_17892_b200 import IlreRecall
     rng = np.random.default_rng(L + budget)
     a = (rng.random(L) ** 4).astype(np.float32)
-    if dense:                                       # whole runs of high and equal scores
+    if lie == "runs":                               # whole runs of high and equal scores
         for p in rng.integers(0, L, size=max(1, L // 4000)):
             a[p:p + 300] = np.float32(0.5 + 0.4 * rng.random())
+    elif lie == "together":                         # a third of one 32nd of the context
+        part = a[5 * L // 32:6 * L // 32 + 1]
+        part += np.where(rng.random(len(part)) < 0.33, 1, 0).astype(np.float32)
     eng = IlreRecall(max_L=L, max_q_len=1, max_budget=budget, n_kv_heads=1, n_q_heads=1,
                      max_combinations=len(max_sizes) * len(win_sizes))
     idx = eng.allocate(torch.from_numpy(a).cuda(), budget, max_sizes, win_sizes, 1, n_sink)
