@@ -366,49 +366,8 @@ int recall_impl(ilre_recall_t* h, const void* k_cache_dev, int64_t L, const void
   const Geometry g = make_geometry(h->cfg.n_kv_heads, h->cfg.n_q_heads, h->n_sm, L, q_len);
   if (g.stats.stages < 2 || g.scores.stages < 2) return ILRE_ERR_UNSUPPORTED;
 
-  // combination table (Algorithm 1 loop order: max sizes outer, window sizes inner)
   ComboTable tbl;
-  std::memset(&tbl, 0, sizeof(tbl));
-  const long long Lp = L - spec->n_sink;
-  tbl.n_comb = (budget > 0) ? spec->n_max * spec->n_win : 0;
-  long long allocated_before = 0;
-  for (int i = 0, c = 0; i < spec->n_max && tbl.n_comb; ++i)
-    for (int j = 0; j < spec->n_win; ++j, ++c) {
-      const int m = spec->max_sizes[i];
-      const long long len = (Lp + m - 1) / m;
-      long long km = budget / m + 1 + ((Lp % m) != 0 ? 1 : 0);
-      if (km > len) km = len;
-      tbl.m[c] = m;
-      tbl.n[c] = spec->win_sizes[j];
-      tbl.len[c] = static_cast<int>(len);
-      tbl.quota[c] = budget / tbl.n_comb + (c < budget % tbl.n_comb ? 1 : 0);
-      // Algorithm 1 ranks K_m cells, but the quota walk of this combination cannot go further
-      // than quota cells that bring a new token plus the cells made up entirely of tokens the
-      // earlier combinations took (at most allocated / m full cells and the partial tail
-      // cell).  Ranking only that many gives the same walk and, for all but the last
-      // combinations, far fewer candidates to select and order.
-      long long reach = tbl.quota[c] + allocated_before / m + ((Lp % m) != 0 ? 1 : 0);
-      if (reach < 1) reach = 1;
-      if (km > reach) km = reach;
-      tbl.k_m[c] = static_cast<int>(km);
-      allocated_before += tbl.quota[c];
-      tbl.tile_begin[c + 1] = tbl.tile_begin[c] + static_cast<int>((len + kSelTile - 1) / kSelTile);
-      // the strided max-pool of size m is shared by all window sizes
-      tbl.src[c] = -1;
-      if (m > 1) {
-        int s = 0;
-        while (s < tbl.n_src && tbl.src_m[s] != m) ++s;
-        if (s == tbl.n_src) {
-          const int cells_per_tile = kSrcTileTokens / m;
-          tbl.src_m[s] = m;
-          tbl.src_len[s] = static_cast<int>(len);
-          tbl.src_tile_begin[s + 1] =
-              tbl.src_tile_begin[s] + static_cast<int>((len + cells_per_tile - 1) / cells_per_tile);
-          ++tbl.n_src;
-        }
-        tbl.src[c] = s;
-      }
-    }
+  make_combinations(L - spec->n_sink, budget, spec->max_sizes, spec->n_max, spec->win_sizes, spec->n_win, &tbl);
 
   CUtensorMap map_k, map_q, map_q32;                     // map_q32: in boxes of 32 rows, for copied row tiles
   std::memset(&map_k, 0, sizeof(map_k));
@@ -471,19 +430,8 @@ int recall_impl(ilre_recall_t* h, const void* k_cache_dev, int64_t L, const void
   int max_km = 1;
   for (int c = 0; c < tbl.n_comb; ++c) max_km = tbl.k_m[c] > max_km ? tbl.k_m[c] : max_km;
   const size_t select_smem = select_smem_bytes(L, max_km, &sp);
-  // Grid of the selection kernel: enough CTAs for the scan tiles and for the ranking (about a
-  // hundred candidates per CTA), but no more, since every grid barrier pays for them.
-  long long want_grid = tbl.tile_begin[tbl.n_comb];
-  long long n_cand = 0;
-  for (int c = 0; c < tbl.n_comb; ++c) n_cand += tbl.k_m[c];
-  if (n_cand / 96 > want_grid) want_grid = n_cand / 96;
-  if (want_grid < 1) want_grid = 1;
-  // a grid just above the cluster size: the cluster barrier is worth more than the extra CTAs
-  if (want_grid > kSelClusterMax && want_grid <= 2 * kSelClusterMax) want_grid = kSelClusterMax;
-  if (want_grid > kSelClusterMax && h->select_wide && select_wide_cluster(tbl)) want_grid = kSelClusterWide;
-  if (want_grid > h->select_max_grid) want_grid = h->select_max_grid;
-  sp.cluster = (want_grid <= kSelClusterMax || (want_grid == kSelClusterWide && h->select_wide)) ? 1 : 0;
-  const int select_grid = static_cast<int>(want_grid);
+  const SelectGrid select = select_grid(tbl, h->select_max_grid, h->select_wide);
+  sp.cluster = select.cluster ? 1 : 0;
 
   const bool prof = h->profiling != 0;
   int launches = 0;
@@ -525,7 +473,7 @@ int recall_impl(ilre_recall_t* h, const void* k_cache_dev, int64_t L, const void
   ILRE_MARK(3);
   if (with_select) {
     TraceRange r("ilre: selection (Algorithm 1)");
-    ILRE_CUDA(launch_select(tbl, sp, select_grid, select_smem, st)); ++launches;
+    ILRE_CUDA(launch_select(tbl, sp, select.ctas, select_smem, st)); ++launches;
   }
   ILRE_MARK(4);
 #undef ILRE_MARK

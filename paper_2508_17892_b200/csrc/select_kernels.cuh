@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cstring>
+
 namespace ilre {
 
 static constexpr int kMaxCombos = 64;
@@ -96,6 +98,51 @@ struct ComboTable {
 // may not fit an int, and where a cell lies in its tile is compared instead.)
 __host__ __device__ constexpr int cells_from(int len, int first, int most) { return len - first < most ? len - first : most; }
 
+// The combinations of Algorithm 1 in its loop order (max sizes outer, window sizes inner) over Lp positions.
+inline void make_combinations(long long Lp, int budget, const int32_t* max_sizes, int n_max, const int32_t* win_sizes,
+                              int n_win, ComboTable* t) {
+  std::memset(t, 0, sizeof(*t));
+  t->n_comb = (budget > 0) ? n_max * n_win : 0;
+  long long allocated_before = 0;
+  for (int i = 0, c = 0; i < n_max && t->n_comb; ++i)
+    for (int j = 0; j < n_win; ++j, ++c) {
+      const int m = max_sizes[i];
+      const long long len = (Lp + m - 1) / m;
+      long long km = budget / m + 1 + ((Lp % m) != 0 ? 1 : 0);
+      if (km > len) km = len;
+      t->m[c] = m;
+      t->n[c] = win_sizes[j];
+      t->len[c] = static_cast<int>(len);
+      t->quota[c] = budget / t->n_comb + (c < budget % t->n_comb ? 1 : 0);
+      // Algorithm 1 ranks K_m cells, but the quota walk of this combination cannot go further
+      // than quota cells that bring a new token plus the cells made up entirely of tokens the
+      // earlier combinations took (at most allocated / m full cells and the partial tail
+      // cell).  Ranking only that many gives the same walk and, for all but the last
+      // combinations, far fewer candidates to select and order.
+      long long reach = t->quota[c] + allocated_before / m + ((Lp % m) != 0 ? 1 : 0);
+      if (reach < 1) reach = 1;
+      if (km > reach) km = reach;
+      t->k_m[c] = static_cast<int>(km);
+      allocated_before += t->quota[c];
+      t->tile_begin[c + 1] = t->tile_begin[c] + static_cast<int>((len + kSelTile - 1) / kSelTile);
+      // the strided max-pool of size m is shared by all window sizes
+      t->src[c] = -1;
+      if (m > 1) {
+        int s = 0;
+        while (s < t->n_src && t->src_m[s] != m) ++s;
+        if (s == t->n_src) {
+          const int cells_per_tile = kSrcTileTokens / m;
+          t->src_m[s] = m;
+          t->src_len[s] = static_cast<int>(len);
+          t->src_tile_begin[s + 1] =
+              t->src_tile_begin[s] + static_cast<int>((len + cells_per_tile - 1) / cells_per_tile);
+          ++t->n_src;
+        }
+        t->src[c] = s;
+      }
+    }
+}
+
 // Groups the combinations for the pooling phase and cuts the groups into tiles: equal shares of the
 // grid's CTAs, rounded up to whole warps.
 inline void assign_pooling(ComboTable* t, int grid) {
@@ -175,16 +222,33 @@ inline size_t select_smem_bytes(long long L, int max_km, SelectParams* p) {
   p->walk_threads = walkers < kMinWalkers ? kMinWalkers : (walkers > kSelThreads ? kSelThreads : walkers);
   return kSelWorkBytes + (p->bitmap_in_smem ? (words + kSelBitmapSlackWords) * sizeof(uint32_t) : 0);
 }
-// Which contexts of more than one small cluster's work run as one cluster of kSelClusterWide CTAs (where the device
-// takes such a cluster): it starts under the end of the scores pass, and its barriers cost half of the
-// counter's, which a cooperative grid of 50 to 100 CTAs gains back on many cells, on many candidates to rank, or on
-// many combinations.  Whole recalls (16 query tokens), cooperative / cluster of 16, us: 3 windows, budget 512, 8K
-// positions 31.2 / 30.6, 16K 40.2 / 37.4, 24K 42.5 / 40.6, 32K 47.3 / 48.0; budget 4096, 16K 43.5 / 43.3, 24K
-// 46.4 / 49.8; 5 windows, budget 2048, 12K 44.1 / 42.4, 16K 44.2 / 47.5; 48 combinations, 8K 80 / 103.
-inline bool select_wide_cluster(const ComboTable& t) {
+// Grid of the selection kernel.
+struct SelectGrid {
+  int ctas;
+  bool cluster;            // one thread-block cluster, else a cooperative grid
+};
+
+// Enough CTAs for the scan tiles and for the ranking (about a hundred candidates per CTA), but no more, since every
+// barrier pays for them.  Up to kSelClusterMax CTAs, or kSelClusterWide where the device grants that, run as one
+// thread-block cluster: it starts under the end of the scores pass, and its barriers cost half of the counter's, which a
+// larger cooperative grid gains back on many cells, many candidates to rank, or many combinations.  Whole recalls in a
+// row (16 query tokens), us, cluster of 8 / cluster of 16 / cooperative (of 16, or of as many as are worth having):
+//   9 to 16 CTAs worth having: 3 windows, budget 512: 4K positions 29.3 / 29.2 / 32.9, 8K 31.6 / 31.2 / 34.5, 16K 39.1 / 35.4 /
+//   39.0, 20K 41.6 / 37.9 / 41.1; 5 windows 12K 42.1 / 37.6 / 40.8; 12 combinations (m = 1, 2, 4), 4K 50.3 / 42.6 / 46.8
+//   more: 3 windows, 24K positions, budget 512 44.3 / 40.7 / 43.6, 2048 48.6 / 44.1 / 45.1; 32K, 512 52.0 / 47.0 / 48.0; 40K
+//   60.4 / 54.2 / 53.9; one window, budget 2048, 8K 31.3 / 30.7 / 33.2, 40K 53.8 / 50.1 / 53.4
+//   more candidates than 5120: 3 windows, budget 4096, 12K 47.9 / 44.0 / 41.4; 5 windows, budget 2048, 6K 48.4 / 44.0 / 39.0
+inline SelectGrid select_grid(const ComboTable& t, int max_ctas, bool wide_granted) {
   long long cells = 0, cand = 0;
   for (int c = 0; c < t.n_comb; ++c) { cells += t.len[c]; cand += t.k_m[c]; }
-  return t.n_comb <= 8 && cells > 20480 && cells + 5 * cand <= 95000;
+  long long want = t.tile_begin[t.n_comb];
+  if (cand / 96 > want) want = cand / 96;
+  if (want < 1) want = 1;
+  if (want > kSelClusterMax && want <= kSelClusterWide) want = wide_granted ? kSelClusterWide : kSelClusterMax;
+  else if (want > kSelClusterWide && wide_granted && t.n_comb <= 8 && cand <= 5120 && cells + 5 * cand <= 95000)
+    want = kSelClusterWide;
+  if (want > max_ctas) want = max_ctas;
+  return {static_cast<int>(want), want <= kSelClusterMax || (want == kSelClusterWide && wide_granted)};
 }
 // Largest grid that is co-resident on the device (the kernel's CTAs wait on one another), and whether it takes a
 // cluster of kSelClusterWide CTAs.

@@ -13,17 +13,26 @@ import pytest
 import torch
 
 import oracle
+import parity
+from workloads import make_inputs, small_workload
 
 pytestmark = pytest.mark.gpu
 
-CASES = [
+# Contexts that run as one cluster of 16 CTAs (the host test of the launch rules checks that they do): the fewest
+# and the most cells, few and many candidates, a strided max-pool, more than 8 combinations.
+WIDE_CASES = [
     # L, budget, max sizes, window sizes, n_sink
+    (4096, 512, (1,), (1, 7, 15), 0),
+    (6830, 512, (1,), (1, 7, 15), 2),
+    (16384, 512, (1,), (1, 7, 15), 0),
+    (24001, 2040, (1,), (1, 7, 15), 3),
+    (20001, 300, (1, 2), (1, 9), 0),
+    (3003, 300, (1, 2, 4), (1, 4, 9, 15), 1),
+]
+CASES = WIDE_CASES + [
     (1, 1, (1,), (1,), 0),
     (129, 125, (1,), (3, 5), 4),
-    (6830, 512, (1,), (1, 7, 15), 2),               # one cluster of 16 CTAs: fewest and most cells, odd lengths
-    (16384, 512, (1,), (1, 7, 15), 0),
     (12289, 2047, (1,), (1, 7, 15, 31, 63), 3),
-    (20001, 300, (1, 2), (1, 9), 0),
     (32768, 4097, (1,), (1, 7, 15), 0),             # a lane per word, the last such length
     (32773, 5, (2, 64), (1, 2), 5),                 # 32768 positions behind the sink part
     (32769, 16382, (1,), (1, 31), 0),               # word list; four rounds, met before the last
@@ -55,6 +64,23 @@ def test_walk_and_output(L, budget, max_sizes, win_sizes, n_sink, lie):
     assert eng.check_guards() == 0
     ref = oracle.allocate(a.astype(np.float64), budget, max_sizes, win_sizes, 1, n_sink)
     assert np.array_equal(idx.cpu().numpy(), ref)
+    eng.close()
+
+
+@pytest.mark.parametrize("L,budget,max_sizes,win_sizes,n_sink", WIDE_CASES[2:5])
+def test_one_cluster_of_16_behind_the_scores_pass(L, budget, max_sizes, win_sizes, n_sink):
+    """Encoded scores, decoded by every CTA of the cluster, and the scores written for the caller."""
+    from paper_2508_17892_b200 import IlreRecall
+    w = small_workload(L, 3, n_kv_heads=2, n_q_heads=4, budget=budget, max_sizes=max_sizes, win_sizes=win_sizes,
+                       win_op=1, n_sink=n_sink, n_spans=3)
+    x = make_inputs(w)
+    eng = IlreRecall(max_L=L, max_q_len=3, max_budget=budget, n_kv_heads=2, n_q_heads=4,
+                     max_combinations=len(max_sizes) * len(win_sizes))
+    idx, sc = eng.run(x.K.cuda(), x.Q.cuda(), budget, max_sizes, win_sizes, 1, n_sink, want_scores=True)
+    torch.cuda.synchronize()
+    eng.check_status()
+    assert eng.check_guards() == 0
+    parity.check_recall(x.K, x.Q, w, idx.cpu().numpy(), sc.cpu().numpy())
     eng.close()
 
 

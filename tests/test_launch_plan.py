@@ -186,3 +186,59 @@ int main() {
 def test_tiles_of_the_longest_contexts_end_where_the_context_does(tmp_path):
     """Lengths go up to 2^31 - 257, where the end of a tile may not fit 32 bits with a sign."""
     _run(tmp_path, LONGEST, "-fsanitize=signed-integer-overflow", "-fno-sanitize-recover")
+
+
+GRIDS = r"""
+#include <cstdio>
+#include "select_kernels.cuh"
+using namespace ilre;
+static SelectGrid grid_of(long long L, int budget, int n_max, const int32_t* max_sizes, int n_win, const int32_t* win_sizes,
+                          int n_sink, bool granted, ComboTable* t) {
+  make_combinations(L - n_sink, budget, max_sizes, n_max, win_sizes, n_win, t);
+  return select_grid(*t, 148, granted);
+}
+int main() {
+  int bad = 0;
+  ComboTable t;
+  // {L, budget, n_sink, number of max sizes, max sizes .., number of window sizes, window sizes ..}, one cluster of 16
+  const int32_t wide[][32] = {%s};
+  for (const auto& w : wide) {
+    const int32_t* ms = w + 4;
+    const int32_t* ws = ms + w[3] + 1;
+    const SelectGrid g = grid_of(w[0], w[1], w[3], ms, ms[w[3]], ws, w[2], true, &t);
+    const SelectGrid no = grid_of(w[0], w[1], w[3], ms, ms[w[3]], ws, w[2], false, &t);
+    if ((!g.cluster || g.ctas != kSelClusterWide || (no.cluster && no.ctas > kSelClusterMax)) && bad++ < 5)
+      std::printf("L %%d budget %%d: %%d CTAs, cluster %%d\n", w[0], w[1], g.ctas, g.cluster);
+  }
+  const int32_t sizes[] = {1, 2, 4, 8, 16, 32}, wins[] = {1, 3, 7, 9, 15, 31, 47, 63};
+  int seen[4] = {0, 0, 0, 0};
+  for (long long L = 1; L < 5000000; L += 1 + L / 7)
+    for (int budget = 0; budget <= L && budget <= 16382; budget += 1 + budget)
+      for (int n_max = 1; n_max <= 6; ++n_max)
+        for (int n_win = 1; n_win <= 8; ++n_win)
+          for (int granted = 0; granted < 2; ++granted) {
+            const SelectGrid g = grid_of(L, budget, n_max, sizes, n_win, wins, 0, granted, &t);
+            long long cand = 0;
+            for (int c = 0; c < t.n_comb; ++c) cand += t.k_m[c];
+            bool ok = g.ctas >= 1 && g.ctas <= 148;
+            // a cluster is one that the device takes, and nothing of one cluster's size runs as a cooperative grid
+            ok = ok && (!g.cluster || g.ctas <= kSelClusterMax || (granted && g.ctas == kSelClusterWide));
+            ok = ok && (g.cluster || g.ctas > kSelClusterMax) && (g.cluster || !granted || g.ctas > kSelClusterWide);
+            // sixteen CTAs are not given the ranking of more candidates than they were measured with
+            ok = ok && (g.ctas != kSelClusterWide || cand <= 5120);
+            ++seen[g.cluster ? (g.ctas == kSelClusterWide ? 2 : 1) : 3];
+            if (!ok && bad++ < 5)
+              std::printf("L %%lld budget %%d %%d x %%d: %%d CTAs, cluster %%d\n", L, budget, n_max, n_win, g.ctas, g.cluster);
+          }
+  std::printf("%%d small clusters, %%d wide, %%d cooperative\n", seen[1], seen[2], seen[3]);
+  return bad || !seen[1] || !seen[2] || !seen[3];
+}
+"""
+
+
+def test_which_grid_the_selection_takes(tmp_path):
+    from test_gpu_walk import WIDE_CASES
+    rows = ",\n".join("{%d, %d, %d, %d, %s, %d, %s}" % (L, budget, n_sink, len(ms), ", ".join(map(str, ms)), len(ws),
+                                                        ", ".join(map(str, ws)))
+                      for L, budget, ms, ws, n_sink in WIDE_CASES)
+    _run(tmp_path, GRIDS % rows)
