@@ -14,7 +14,7 @@ struct PassGeometry {
 struct Geometry {
   int group_size, kv_rows;             // kv_rows: rows of one kv head in the packed query
   PassGeometry stats, scores;
-  bool stats_tail;                     // statistics: some block's last row tile is short and loaded in copies
+  bool stats_tail;                     // statistics: the last row tile of a full block is short; short ones are loaded in copies
 };
 
 // Splits the rows of one kv head into blocks of at most max_rows, padded to a multiple of `unit`.

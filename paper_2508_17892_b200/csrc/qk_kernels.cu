@@ -231,7 +231,8 @@ __device__ __forceinline__ void row_update64(const float (&va)[32], const float 
 // row tile is short it would have less to do than the others (TAIL), so the tiles take turns.
 template <int MT, bool TAIL>
 __device__ __forceinline__ int row_tile(int i, int j) {
-  if constexpr (!TAIL || MT == 1 || MT == 3) return j;
+  static_assert(!TAIL || MT > 1, "a short row tile is copied behind a full one only");
+  if constexpr (!TAIL || MT == 3) return j;
   if constexpr (MT == 2) return j ^ ((i >> 1) & 1);
   return (i + j) & 3;
 }
@@ -330,7 +331,7 @@ row_stats_kernel(const __grid_constant__ CUtensorMap tmapK,
     // Accumulator u belongs to warpgroup u % 4 and holds row tile u % MT.  With 1, 2 or 4 row
     // tiles a warpgroup therefore always meets the same row tile (wg % MT) and a thread keeps
     // one (max, sum) pair; only with 3 row tiles, or tiles that take turns, does it meet all of them.
-    constexpr int kStates = (MT == 3 || (TAIL && MT > 1)) ? MT : 1;
+    constexpr int kStates = (MT == 3 || TAIL) ? MT : 1;
     float m[kStates], z[kStates];
 #pragma unroll
     for (int j = 0; j < kStates; ++j) { m[j] = -1e30f; z[j] = 0.f; }
@@ -936,7 +937,9 @@ template <int MT>
 static cudaError_t launch_row_stats_mt(const CUtensorMap& tk, const CUtensorMap& tq, const CUtensorMap& tq32,
                                        const QkParams& p, const PrepParams& pp, cudaStream_t st) {
   const size_t smem = row_stats_smem_bytes(MT * 128, p.stages);
-  const auto kernel = p.tail ? row_stats_kernel<MT, kRowStatsPolyPairs, true> : row_stats_kernel<MT, kRowStatsPolyPairs, false>;
+  auto kernel = row_stats_kernel<MT, kRowStatsPolyPairs, false>;
+  if constexpr (MT > 1)
+    if (p.tail) kernel = row_stats_kernel<MT, kRowStatsPolyPairs, true>;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   return launch_after_previous(kernel, p.n_groups * p.cpg, kStatsThreads<MT>, smem, st, tk, tq, tq32, p, pp);

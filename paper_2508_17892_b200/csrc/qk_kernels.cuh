@@ -82,7 +82,7 @@ struct QkParams {
   int group;         // query heads per kv head when the query is loaded from the caller's array (a
                      // box of 128 rows = `group` heads of 128 / group tokens); 0: from the packed copy
   int cpg;           // key chunks (CTAs or CTA pairs) per group
-  int tail;          // statistics: some block's last row tile is short and loaded in copies (stats_tail_copies)
+  int tail;          // statistics: a block's last row tile is loaded in copies where it is short (stats_tail_copies)
   int stages;        // ring depth in key tiles (pair: in units, set by the launcher)
   float c2;          // log2(e) / sqrt(d)
   float* partial;    // [n_groups][cpg][rb_rows][2]: (max * c2, sum-exp) per key chunk
