@@ -42,3 +42,30 @@ int main() {
 
 def test_row_blocks_cover_the_query_and_stay_inside_its_packed_copy(tmp_path):
     _run(tmp_path, SPLIT)
+
+
+FORMS = r"""
+#include <cstdio>
+#include "qk_geometry.cuh"
+using namespace ilre;
+int main() {
+  const int cases[][5] = {%s};          // kv heads, heads per kv head, query tokens, keys; loaded in copies
+  int bad = 0, behind = 0;
+  for (const auto& c : cases) {
+    const int rows = c[1] * c[2];
+    const Geometry g = make_geometry(c[0], c[0] * c[1], 148, c[3], c[2]);
+    const int last = rows - (g.stats.n_rb - 1) * g.stats.rb_rows;
+    behind += g.stats_tail && stats_tail_copies(last) > 1 && (last + 127) / 128 < (g.stats.rb_rows + 127) / 128;
+    if (g.stats_tail != (c[4] != 0) && ++bad)
+      std::printf("%%d x %%d heads, %%d tokens, %%d keys: copies %%d\n", c[0], c[1], c[2], c[3], g.stats_tail);
+  }
+  return bad || behind < 2;
+}
+"""
+
+
+def test_gpu_cases_take_the_form_they_are_listed_under(tmp_path):
+    """And two of them copy a tile that is not the last of its block."""
+    from test_gpu_row_tails import COPIED, PLAIN
+    rows = ["{%d, %d, %d, %d, %d}" % (*c, form) for form, cases in ((1, COPIED), (0, PLAIN)) for c in cases]
+    _run(tmp_path, FORMS % ", ".join(rows))
