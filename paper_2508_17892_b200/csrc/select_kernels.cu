@@ -1,5 +1,5 @@
-// Algorithm 1 ("Context Allocation") on the device, as ONE cooperative kernel whose CTAs
-// meet at grid barriers between the phases:
+// Algorithm 1 ("Context Allocation") on the device, as ONE kernel, a thread-block cluster or a cooperative
+// grid, whose CTAs meet at barriers between the phases:
 //
 //   A  MaxPooling(size = stride = m), once per distinct m > 1;
 //   B  the stride-1 window pooling (average or max) of every (m, n) combination, up to kPoolGroup
@@ -108,7 +108,8 @@ __device__ __forceinline__ bool grid_sync(const SelectParams& p, SelShared* sh, 
 }
 
 // Exclusive prefix sum over the block of kSelThreads threads; *total receives the block sum.
-// Not inlined: the kernel meets its code cold, and every phase after the first use finds this one warm.
+// Begins with a barrier, and none follows the last reads of sh_warp: its next writer is the next call's, behind that
+// barrier.  Not inlined: the kernel meets its code cold, and every phase after the first use finds this one warm.
 __device__ __noinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* sh_warp,
                                                          uint32_t* total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -458,7 +459,7 @@ __device__ __forceinline__ void bin_search(const SelectParams& p, const uint32_t
     total += h[j];
   }
   uint32_t grand;
-  const uint32_t excl = block_exclusive_scan(total, sh->scan, &grand);   // ends with a barrier
+  const uint32_t excl = block_exclusive_scan(total, sh->scan, &grand);
   if (excl < k_rem && k_rem <= excl + total) {
     uint32_t cum = excl;
 #pragma unroll
@@ -851,8 +852,7 @@ __device__ __forceinline__ uint32_t block_exclusive_scan_1(uint32_t v, uint32_t 
 // Phase F (one CTA): quota walk over the ranked cells of every combination, then the
 // ascending list of allocated positions.  The bitmap lives in shared memory when it fits
 // (cleared at the start of the kernel, beside the memory of the other phases), else in global
-// memory.  Every thread owns a run of consecutive ranks; the cells of one combination are
-// disjoint, so the new-token counts of all its cells can be taken before any of them is marked.
+// memory.
 template <bool kBitmapInSmem>
 __device__ __forceinline__ void allocate(const ComboTable& tbl, const SelectParams& p,
                                          uint8_t* dyn_smem, SelShared* sh) {
@@ -933,11 +933,13 @@ __device__ __forceinline__ void allocate(const ComboTable& tbl, const SelectPara
     return;
   }
   // Longer contexts: every warp takes an equal run of the bitmap and counts the words that are not empty (a few in a
-  // hundred, neighbours for the most part); with the sum of the warps' before it, it goes through the run
-  // again and enters them, in order, in the block's list.  The warps then take equal shares of the list, whose
-  // positions they count and write, a lane per word: passages may lie anywhere, all of them in one warp's run too.
-  // (Each warp writing what lies in its own run: allocation of 524288 positions, budget 4096, chosen from one 32nd of the
-  // context 80.9 us, so 64.5, spread evenly 110 and 113; 4000000 positions 150 and 112, spread 112 and 112.)
+  // hundred, neighbours for the most part) and their positions; with the sums of the warps' before it, it goes
+  // through the run again and enters the words, in order, in the block's list.  Then it writes the positions of
+  // its own words, a lane per word.  But passages may lie anywhere, all of them in one warp's run too: where a
+  // warp would have a round of words more than an equal share of the list, all take equal shares, which
+  // costs two barriers and another sum.  (Own words always / shares always / as it stands, us: allocation, budget 4096,
+  // chosen from one 32nd of the context, 131072 positions 45.1 / 39.0 / 39.0, 524288 80.4 / 64.7 / 65.2, 4000000
+  // 143 / 102 / 103, spread out, 524288 91.5 / 92.2 / 91.9; recalls of 81690 positions, budget 1024, 118.6 / 120.2 / 118.8.)
   const int per = ((n_quads + kMaxWalkWarps - 1) / kMaxWalkWarps + 31) & ~31;
   const int q_begin = min(n_quads, warp * per), q_end = min(n_quads, q_begin + per);
   auto load_quad = [&](int q) -> uint4 {
@@ -945,18 +947,24 @@ __device__ __forceinline__ void allocate(const ComboTable& tbl, const SelectPara
     if constexpr (kBitmapInSmem) return reinterpret_cast<const uint4*>(bm)[q];
     else return __ldcg(reinterpret_cast<const uint4*>(bm) + q);
   };
-  uint32_t mine = 0;
+  uint32_t mine = 0;                                             // positions | words << 16
 #pragma unroll 1
   for (int q = q_begin; q < q_end; q += 32) {
     const uint4 v = load_quad(q + lane);
-    mine += (v.x ? 1u : 0u) + (v.y ? 1u : 0u) + (v.z ? 1u : 0u) + (v.w ? 1u : 0u);
+    if (__any_sync(0xFFFFFFFFu, (v.x | v.y | v.z | v.w) != 0u))
+      mine += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w) +
+              (((v.x ? 1u : 0u) + (v.y ? 1u : 0u) + (v.z ? 1u : 0u) + (v.w ? 1u : 0u)) << 16);
   }
   constexpr uint32_t kList = kSelWorkBytes / 4;
-  static_assert(kList >= kMaxKm, "the list holds a word per position");
+  static_assert(kList >= kMaxKm && kMaxKm < 65536, "the list holds a word per position, a count fits 16 bits");
   int* list = reinterpret_cast<int*>(dyn_smem);
-  uint32_t n_words;
-  uint32_t to = block_exclusive_scan(mine, sh->scan, &n_words);
-  to = __shfl_sync(0xFFFFFFFFu, to, 0);
+  uint32_t at = block_exclusive_scan(mine, sh->scan, &total);
+  at = __shfl_sync(0xFFFFFFFFu, at, 0);
+  if (threadIdx.x == 0 && (total & 0xFFFFu) != static_cast<uint32_t>(p.budget)) atomicCAS(p.status, 0, kDevQuota);
+  const int n_listed = static_cast<int>(min(total >> 16, kList)), share = (n_listed + kMaxWalkWarps - 1) / kMaxWalkWarps;
+  const bool own = __reduce_max_sync(0xFFFFFFFFu, sh->scan[lane] >> 16) <= static_cast<uint32_t>(share + 32);   // the same for all
+  uint32_t to = at >> 16;
+  int e_begin = min(static_cast<int>(to), n_listed);
 #pragma unroll 1
   for (int q = q_begin; q < q_end; q += 32) {
     const uint4 v = load_quad(q + lane);
@@ -964,45 +972,46 @@ __device__ __forceinline__ void allocate(const ComboTable& tbl, const SelectPara
     if (!__any_sync(0xFFFFFFFFu, full != 0u)) continue;
     // a word's place in the list: behind the words of the lanes before, by votes, and those of its own lane
     const uint32_t lt = (1u << lane) - 1u;
-    uint32_t at = to;
+    uint32_t place = to;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const uint32_t votes = __ballot_sync(0xFFFFFFFFu, (full >> k) & 1u);
-      at += __popc(votes & lt);
+      place += __popc(votes & lt);
       to += __popc(votes);
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k)
       if ((full >> k) & 1u) {
-        if (at < kList) list[at] = 4 * (q + lane) + k;           // never past it unless a quota was overrun
-        ++at;
+        if (place < kList) list[place] = 4 * (q + lane) + k;     // never past it unless a quota was overrun
+        ++place;
       }
   }
-  __syncthreads();
-  const int n_listed = static_cast<int>(min(n_words, kList)), share = (n_listed + kMaxWalkWarps - 1) / kMaxWalkWarps;
-  const int e_begin = min(n_listed, warp * share), e_end = min(n_listed, e_begin + share);
-  mine = 0;
+  int e_end = min(static_cast<int>(to), n_listed);
+  at = p.n_sink + (at & 0xFFFFu);
+  if (own) {
+    __syncwarp();
+  } else {
+    __syncthreads();
+    e_begin = min(n_listed, warp * share);
+    e_end = min(n_listed, e_begin + share);
+    mine = 0;
 #pragma unroll 1
-  for (int e = e_begin + lane; e < e_end; e += 32) mine += __popc(bitmap_word<kBitmapInSmem>(bm, list[e]));
-  uint32_t at = p.n_sink + block_exclusive_scan(mine, sh->scan, &total);
-  if (threadIdx.x == 0 && total != static_cast<uint32_t>(p.budget)) atomicCAS(p.status, 0, kDevQuota);
-  if (share > 32) at = __shfl_sync(0xFFFFFFFFu, at, 0);          // else: already the place of the lane's one word
+    for (int e = e_begin + lane; e < e_end; e += 32) mine += __popc(bitmap_word<kBitmapInSmem>(bm, list[e]));
+    at = p.n_sink + block_exclusive_scan(mine, sh->scan, &total);
+    at = __shfl_sync(0xFFFFFFFFu, at, 0);
+  }
 #pragma unroll 1
   for (int e = e_begin; e < e_end; e += 32) {
     const int w = (e + lane < e_end) ? list[e + lane] : 0;
     const uint32_t bits = (e + lane < e_end) ? bitmap_word<kBitmapInSmem>(bm, w) : 0u, n = __popc(bits);
-    uint32_t place = at;
-    if (share > 32) {
-      uint32_t incl = n;
+    uint32_t incl = n;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= o) incl += t;
-      }
-      place = at + incl - n;
-      at += __shfl_sync(0xFFFFFFFFu, incl, 31);
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+      if (lane >= o) incl += t;
     }
-    emit_words(p, bits, w, place, cap);
+    emit_words(p, bits, w, at + incl - n, cap);
+    at += __shfl_sync(0xFFFFFFFFu, incl, 31);
   }
 }
 
