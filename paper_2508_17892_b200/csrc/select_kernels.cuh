@@ -235,6 +235,8 @@ struct SelectGrid {
 // row (16 query tokens), us, cluster of 8 / cluster of 16 / cooperative (of 16, or of as many as are worth having):
 //   9 to 16 CTAs worth having: 3 windows, budget 512: 4K positions 29.3 / 29.2 / 32.9, 8K 31.6 / 31.2 / 34.5, 16K 39.1 / 35.4 /
 //   39.0, 20K 41.6 / 37.9 / 41.1; 5 windows 12K 42.1 / 37.6 / 40.8; 12 combinations (m = 1, 2, 4), 4K 50.3 / 42.6 / 46.8
+//   the same on fewer than 12288 cells: 2301 positions, 5 windows 43.4 / 44.4 / --, 2060, 3 windows 43.5 / 44.2 / --; but with more
+//   lists to rank than 8 CTAs: 1000 positions, 12 combinations 42.6 / 35.3 / 39.1
 //   more: 3 windows, 24K positions, budget 512 44.3 / 40.7 / 43.6, 2048 48.6 / 44.1 / 45.1; 32K, 512 52.0 / 47.0 / 48.0; 40K
 //   60.4 / 54.2 / 53.9; one window, budget 2048, 8K 31.3 / 30.7 / 33.2, 40K 53.8 / 50.1 / 53.4
 //   more candidates than 5120: 3 windows, budget 4096, 12K 47.9 / 44.0 / 41.4; 5 windows, budget 2048, 6K 48.4 / 44.0 / 39.0
@@ -244,7 +246,8 @@ inline SelectGrid select_grid(const ComboTable& t, int max_ctas, bool wide_grant
   long long want = t.tile_begin[t.n_comb];
   if (cand / 96 > want) want = cand / 96;
   if (want < 1) want = 1;
-  if (want > kSelClusterMax && want <= kSelClusterWide) want = wide_granted ? kSelClusterWide : kSelClusterMax;
+  if (want > kSelClusterMax && want <= kSelClusterWide)
+    want = wide_granted && (cells >= 12288 || t.n_comb > kSelClusterMax) ? kSelClusterWide : kSelClusterMax;
   else if (want > kSelClusterWide && wide_granted && t.n_comb <= 8 && cand <= 5120 && cells + 5 * cand <= 95000)
     want = kSelClusterWide;
   if (want > max_ctas) want = max_ctas;
@@ -253,7 +256,7 @@ inline SelectGrid select_grid(const ComboTable& t, int max_ctas, bool wide_grant
 // Largest grid that is co-resident on the device (the kernel's CTAs wait on one another), and whether it takes a
 // cluster of kSelClusterWide CTAs.
 cudaError_t select_max_grid(int n_sm, int* max_grid, bool* wide_cluster);
-// One cooperative launch: A^C from the encoded maxima, then all of Algorithm 1.
+// One launch: A^C from the encoded maxima, then all of Algorithm 1.
 cudaError_t launch_select(const ComboTable& tbl, const SelectParams& p, int grid, size_t smem,
                           cudaStream_t st);
 
