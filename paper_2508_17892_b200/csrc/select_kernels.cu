@@ -26,11 +26,12 @@
 // kSelTile cells of one combination; every CTA owns a contiguous run of tiles.
 //
 // Bound by the chain of its phases: barriers, one CTA's walk, code met cold in the instruction cache
-// (everything it reads is in L2).  Hence `unroll 1` on loops of few turns: the compiler's fourfold copies with their
-// remainders are lines fetched for one turn (with its own choice 128K positions 33.1 us, so 28.9; 1M 71, 64).  The stage by itself, events around it after an L2 flush, with a
+// (everything it reads is in L2).  Hence `unroll 1` on loops of few turns: the compiler's fourfold copies with
+// their remainders are lines fetched for one turn (the kernel between its own time stamps, with the compiler's choice
+// 128K positions 33.1 us, so 28.9; 1M 71, 64).  The stage by itself, events around it after an L2 flush, with a
 // selection inside the threshold bin, one window per pooling tile and scattered candidates -> as it
-// stands: 4K positions 39 -> 29 us, 32K 52 -> 38, 128K 59 -> 44, 512K 89 -> 63, 1M 117..131 -> 84, 1M with
-// 48 combinations 270..280 -> 210.
+// stands: 4K positions 39 -> 24 us, 32K 52 -> 31, 128K 59 -> 36, 512K 89 -> 55, 1M 117..131 -> 68, 1M with
+// 48 combinations 270..280 -> 188.
 #include <atomic>
 
 #include "select_kernels.cuh"
