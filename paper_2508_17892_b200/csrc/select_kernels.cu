@@ -626,7 +626,7 @@ __device__ __forceinline__ void rank_range(const SelectParams& p, const ComboTab
 }
 
 // Shared memory of the allocation phase: the bitmap lies behind the work area of the other phases, which
-// the output lists reuse.
+// the output list reuses.
 __device__ __forceinline__ uint32_t* smem_bitmap(uint8_t* dyn_smem) {
   return reinterpret_cast<uint32_t*>(dyn_smem + kSelWorkBytes);
 }

@@ -53,14 +53,14 @@ static constexpr int kPoolGroup = 5;        // window sizes of one strided max-p
 static constexpr int kPoolTileMax = 3072;   // cells of a group of windows per work tile, at most
 static constexpr int kSrcTileTokens = 8192; // tokens per work tile of the strided max-pool
 static constexpr int kSelClusterMax = 8;     // grids up to this size run as one thread-block cluster
-static constexpr int kSelClusterWide = 16;   // and those of this size where select_wide_cluster says so
+static constexpr int kSelClusterWide = 16;   // and those of this size where select_grid says so
 static constexpr int kCandSlack = 4096;      // candidates past K_m that the threshold bin may bring
 static constexpr int kWalkCells = 4;         // ranked cells per thread and round of the quota walk
 static constexpr int kMinWalkers = 64;       // fewest threads that walk
 static constexpr int kSelBitmapSmemBytes = 136 * 1024;   // bitmap kept in shared memory up to this
 static constexpr int kSelBitmapSlackWords = 4;           // behind the bitmap
-// Work area in front of the bitmap: pooling tiles, the keys of a ranking list and the warps' output
-// lists, one after another.
+// Work area in front of the bitmap: pooling tiles, the keys of a ranking list and the list of the output
+// pass, one after another.
 static constexpr int kSelWorkBytes = 64 * 1024;
 static_assert(kSelWorkBytes >= (kPoolGroup - 1) * kHistBins * 4 + 2 * (kPoolTileMax + kMaxWin) * 4 && kSelWorkBytes >= kSrcTileTokens * 4,
               "work area too small");
